@@ -54,6 +54,13 @@ phosim_status phosim_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* 
    CUDA. */
 phosim_status phosim_ds_eval(int op, const double* a, const double* b, double* out, int n);
 
+/* The helpers of the FP64 paths (reciprocal, roots and conversions that spare the FP64 pipe) applied element-wise,
+   for accuracy checks.  op: 0 1 / a, 1 1 / sqrt(a), 2 sqrt(a), 3 a truncated to single precision, 4 a rounded to
+   single precision, 5 the single-precision a as a double, 6 floor(a), 7 the integer floor(a), 8 (a + 1/2) 2^-32 of
+   the 32-bit integer a.  a, out: host, n values.  Errors: INVALID_ARGUMENT (unknown op, null pointer, n < 1),
+   OUT_OF_MEMORY, CUDA. */
+phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n);
+
 /* Per-kernel timing of phosim_trace.  While on, each phosim_trace call on the scene launches its kernels
    one by one (no CUDA graph) with a CUDA event recorded on the call's stream before and after each launch.
    phosim_stage_times waits for the events of the scene's last phosim_trace call and returns the summed

@@ -1,0 +1,79 @@
+// FP64 helpers of the photon path for a GPU whose FP64 pipe is its bottleneck.
+//
+// On GB300 a warp's FP64 instruction holds the SM's FP64 pipe for sixteen cycles (1.06 TFLOP/s measured, against
+// 77 for FP32), and a conversion to or from double or a double comparison costs as much as a fused
+// multiply-add; the FP64 kernels keep that pipe 86 % busy while the integer and FP32 pipes idle.  So reciprocals
+// and roots start from the hardware's approximations (PTX rcp.approx.ftz.f64 and rsqrt.approx.ftz.f64, about 20
+// bits, not on the FP64 pipe) and take one step of third order (Householder's iteration), which leaves a
+// relative error near 2^-60 before rounding, and conversions are integer operations on the words of a double.
+// Arguments are finite, non-zero and far from the ends of the exponent range where not said otherwise.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+namespace phosim {
+
+// 1 / b: with r = 1 - b x the exact reciprocal is x / (1 - r) = x (1 + r + r^2 + ...)
+__device__ __forceinline__ double rcp64(double b) {
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(b));
+    const double r = fma(-b, x, 1.0);
+    return fma(x, fma(r, r, r), x);
+}
+
+__device__ __forceinline__ double rsqrt_seed64(double a) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    return y;
+}
+// 1 / sqrt(a), a > 0: with e = 1 - a y^2 it is y (1 - e)^(-1/2) = y (1 + e / 2 + 3 e^2 / 8 + ...)
+__device__ __forceinline__ double rsqrt64(double a) {
+    const double y = rsqrt_seed64(a), e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+// sqrt(a), a > 0, from s = a y the same way
+__device__ __forceinline__ double sqrt64_pos(double a) {
+    const double y = rsqrt_seed64(a), s = a * y, e = fma(-s, y, 1.0);
+    return fma(s * e, fma(0.375, e, 0.5), s);
+}
+// sign tests on the high word (a double comparison takes the FP64 pipe)
+__device__ __forceinline__ bool negative64(double a) { return __double2hiint(a) < 0; }
+// sqrt(a) for a >= 0; numbers below 1e-290 give 0
+__device__ __forceinline__ double sqrt64(double a) { return __double2hiint(a) > 0x03c00000 ? sqrt64_pos(a) : 0.0; }
+
+// a double truncated to single precision; magnitudes below 1e-38 give a number of that size, those above 3e38 the
+// largest float (a start value or a comparison with a margin, never a result)
+__device__ __forceinline__ float f32_trunc(double v) {
+    const int hi = __double2hiint(v);
+    int m = hi & 0x7fffffff;
+    m = m < 0x38000000 ? 0x38000000 : (m > 0x47efffff ? 0x47efffff : m);
+    const uint32_t bits = __funnelshift_l((uint32_t)__double2loint(v), (uint32_t)(m - 0x38000000), 3);
+    return __uint_as_float((bits & 0x7fffffffu) | ((uint32_t)hi & 0x80000000u));
+}
+// (float)v, rounded to nearest even, for 0 or 1e-37 < v < 1e38
+__device__ __forceinline__ float f32_rn_pos(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    if (hi < 0x38100000u) return 0.f;
+    const unsigned long long b = ((unsigned long long)(hi - 0x38000000u) << 32) | lo;
+    return __uint_as_float((uint32_t)((b + 0x0fffffffull + ((lo >> 29) & 1u)) >> 29));
+}
+// (double)f, exact, for 0 and normal finite numbers
+__device__ __forceinline__ double f64_exact(float f) {
+    const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
+    const uint32_t hi = m ? (b & 0x80000000u) | ((m >> 3) + 0x38000000u) : b;
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+// (double)n of a non-negative n, exact: 2^52 + n by its bits, then 2^52 off
+__device__ __forceinline__ double f64_of_count(uint32_t n) { return __hiloint2double(0x43300000, (int)n) - 4503599627370496.0; }
+
+// floor(f) for |f| < 2^31 (floor_in_range) as a double and an integer: adding 1.5 2^52 rounded down leaves the
+// integer in the low word
+__device__ __forceinline__ bool floor_in_range(double f) { return (__double2hiint(f) & 0x7fffffff) < 0x41e00000; }
+__device__ __forceinline__ double floor64(double f, int& i) {
+    const double t = __dadd_rd(f, 6755399441055744.0);
+    i = __double2loint(t);
+    return t - 6755399441055744.0;
+}
+
+}  // namespace phosim

@@ -128,9 +128,10 @@ __device__ void surface_adjoint(const TraceParams& P, const GradParams& G, int s
     const double X[3] = {XD[0], XD[1], XD[2]}, D[3] = {XD[3], XD[4], XD[5]};
     double p[3], dl[3];
     to_surface(S, X, D, p, dl);
-    double l, Nfwd[3];
-    intersect(S, p, dl, l, Nfwd);
-    const double h[3] = {fma(l, dl[0], p[0]), fma(l, dl[1], p[1]), fma(l, dl[2], p[2])};
+    double h[3], Nfwd[3];
+    bool ahead;
+    intersect(S, P.surf_s[si], p, dl, h, Nfwd, ahead);
+    const double l = fma(h[0] - p[0], dl[0], fma(h[1] - p[1], dl[1], (h[2] - p[2]) * dl[2]));
     double zs, sx, sy, sxx, sxy, syy;
     sag_d2(S, nullptr, h[0], h[1], zs, sx, sy, sxx, sxy, syy);
     const double zx = sx, zy = sy;            // the slopes that define the normal, at the root

@@ -275,3 +275,41 @@ extern "C" phosim_status phosim_ds_eval(int op, const double* a, const double* b
     if (e != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_CUDA; }
     return PHOSIM_OK;
 }
+
+namespace {
+__global__ void fp64_eval_kernel(int op, const double* a, double* out, int n) {
+    using namespace phosim;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double x = a[i];
+    int k = 0;
+    switch (op) {
+        case 0: out[i] = rcp64(x); break;
+        case 1: out[i] = rsqrt64(x); break;
+        case 2: out[i] = sqrt64(x); break;
+        case 3: out[i] = (double)f32_trunc(x); break;
+        case 4: out[i] = (double)f32_rn_pos(x); break;
+        case 5: out[i] = f64_exact((float)x); break;
+        case 6: out[i] = floor64(x, k); break;
+        case 7: floor64(x, k); out[i] = (double)k; break;
+        case 8: out[i] = u64of((uint32_t)x); break;
+        default: break;
+    }
+}
+}  // namespace
+
+extern "C" phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n) {
+    if (op < 0 || op > 8 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
+    const size_t bytes = (size_t)n * sizeof(double);
+    double* d = nullptr;
+    if (cudaMalloc(&d, bytes) != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_OUT_OF_MEMORY; }
+    cudaError_t e = cudaMemcpy(d, a, bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        fp64_eval_kernel<<<(n + 127) / 128, 128>>>(op, d, d, n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(out, d, bytes, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_CUDA; }
+    return PHOSIM_OK;
+}

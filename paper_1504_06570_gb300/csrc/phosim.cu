@@ -156,6 +156,8 @@ phosim_status build_surface(const phosim_surface& s, DSurface& d) {
         d.ae[i] = s.alpha[2 * i + 1];    // alpha_4, 6, 8, 10
         if (d.ao[i] != 0.0) { flags |= SF_ODD; d.no = i + 1; }
         if (d.ae[i] != 0.0) { flags |= SF_EVEN; d.ne = i + 1; }
+        d.aed[i] = (2 * i + 4) * d.ae[i];
+        d.aod[i] = (2 * i + 3) * d.ao[i];
     }
     if (s.zern_rnorm > 0.0) d.zinv = 1.0 / s.zern_rnorm;
     if (s.n_zern > 0 && s.zern_rnorm > 0.0) {
@@ -248,7 +250,10 @@ __global__ void gradient_screen_kernel(const double* __restrict__ ph, int n, dou
     const double2 a = central_gradient(ph, n, two_pix, i, j), b = central_gradient(ph, n, two_pix, i1, j);
     const double2 c = central_gradient(ph, n, two_pix, i, j1), d = central_gradient(ph, n, two_pix, i1, j1);
     const size_t node = (size_t)j * n + i;
-    g64[4 * node] = a; g64[4 * node + 1] = b; g64[4 * node + 2] = c; g64[4 * node + 3] = d;
+    g64[4 * node] = a;
+    g64[4 * node + 1] = make_double2(b.x - a.x, b.y - a.y);
+    g64[4 * node + 2] = make_double2(c.x - a.x, c.y - a.y);
+    g64[4 * node + 3] = make_double2((a.x - b.x) + (d.x - c.x), (a.y - b.y) + (d.y - c.y));
     g32[2 * node] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
     g32[2 * node + 1] = make_float4((float)c.x, (float)c.y, (float)d.x, (float)d.y);
 }
@@ -465,6 +470,7 @@ phosim_status phosim_create_scene(const phosim_scene_desc* d, phosim_scene** out
     P.h_top = d->h_top;
     P.z_ent = d->z_entrance;
     P.lam_ref = d->lambda_ref;
+    P.inv_lam_ref = 1.0 / d->lambda_ref;
     P.kick0 = d->lambda_ref * 1e-6 / (2.0 * M_PI);
     P.nx = d->nx; P.ny = d->ny;
     P.pixel = d->pixel; P.inv_pixel = 1.0 / d->pixel;

@@ -44,36 +44,53 @@ __device__ __forceinline__ int wrap_index(long long i, int n) {
     return (int)(m < 0 ? m + n : m);
 }
 
+// node index of a floor beyond the integer range (a screen that many pixels from the origin)
+static __device__ __noinline__ int far_index(double fl, int n) { return wrap_index((long long)fl, n); }
+__device__ __forceinline__ int near_index(int i, int n) {
+    if ((n & (n - 1)) == 0) return i & (n - 1);
+    const int m = i % n;
+    return m < 0 ? m + n : m;
+}
+
 // Gradient of the phase at screen position (sx, sy), bilinear between central-difference nodes (Sec. 2.3.2)
 template <bool MIXED>
 __device__ __forceinline__ void screen_gradient(const DScale& S, double sx, double sy, double& gx, double& gy) {
     const double fx = sx * S.inv_pix, fy = sy * S.inv_pix;
-    const double flx = floor(fx), fly = floor(fy);
     const int n = S.n;
-    const int i0 = wrap_index((long long)flx, n), j0 = wrap_index((long long)fly, n);
+    double flx, fly;
+    int i0, j0;
+    if (floor_in_range(fx) && floor_in_range(fy)) {
+        flx = floor64(fx, i0);
+        fly = floor64(fy, j0);
+        i0 = near_index(i0, n);
+        j0 = near_index(j0, n);
+    } else {
+        flx = floor(fx);
+        fly = floor(fy);
+        i0 = far_index(flx, n);
+        j0 = far_index(fly, n);
+    }
     const size_t node = (size_t)j0 * n + i0;
     if constexpr (MIXED) {
-        const float tx = (float)(fx - flx), ty = (float)(fy - fly);
+        const float tx = f32_rn_pos(fx - flx), ty = f32_rn_pos(fy - fly);
         const float4 A = __ldg(S.g32 + 2 * node), B = __ldg(S.g32 + 2 * node + 1);
         const float w00 = (1.f - tx) * (1.f - ty), w10 = tx * (1.f - ty), w01 = (1.f - tx) * ty, w11 = tx * ty;
-        gx += (double)(w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z);
-        gy += (double)(w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w);
+        gx += f64_exact(w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z);
+        gy += f64_exact(w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w);
     } else {
         const double tx = fx - flx, ty = fy - fly;
         const double2* q = S.g64 + 4 * node;
         const double2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2), d = __ldg(q + 3);
-        const double w00 = (1.0 - tx) * (1.0 - ty), w10 = tx * (1.0 - ty), w01 = (1.0 - tx) * ty, w11 = tx * ty;
-        gx += w00 * a.x + w10 * b.x + w01 * c.x + w11 * d.x;
-        gy += w00 * a.y + w10 * b.y + w01 * c.y + w11 * d.y;
+        gx += fma(ty, fma(tx, d.x, c.x), fma(tx, b.x, a.x));
+        gy += fma(ty, fma(tx, d.y, c.y), fma(tx, b.y, a.y));
     }
 }
 
 __device__ __forceinline__ double lerp_table(const double* __restrict__ t, int n, double f) {
-    int k = (int)floor(f);
+    int k = __double2int_rd(f);
     k = k < 0 ? 0 : (k > n - 2 ? n - 2 : k);
-    double w = f - k;
-    w = w < 0.0 ? 0.0 : (w > 1.0 ? 1.0 : w);
-    return __ldg(t + k) * (1.0 - w) + __ldg(t + k + 1) * w;
+    const double w = fmin(fmax(f - (double)k, 0.0), 1.0), a = __ldg(t + k);
+    return fma(w, __ldg(t + k + 1) - a, a);
 }
 __device__ __forceinline__ float lerp_table_f(const float* __restrict__ t, int n, float f) {
     int k = (int)floorf(f);
@@ -156,13 +173,13 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
         }
         double p[3], dl[3];
         to_surface(S, X, D, p, dl);
-        double l, Nv[3];
-        const uint32_t why = intersect(S, p, dl, l, Nv);
+        double h[3], Nv[3];
+        bool ahead;
+        const uint32_t why = intersect(S, P.surf_s[si], p, dl, h, Nv, ahead);
         if (why) { R.flags = lost(why, si); return; }
-        if (GHOSTS && bounces > 0 && !(l > 0.0)) { R.flags = lost(PHOSIM_LOST_MISSED, si); return; }
-        p[0] = fma(l, dl[0], p[0]);
-        p[1] = fma(l, dl[1], p[1]);
-        p[2] = fma(l, dl[2], p[2]);
+        if (GHOSTS && bounces > 0 && !ahead) { R.flags = lost(PHOSIM_LOST_MISSED, si); return; }
+        p[0] = h[0]; p[1] = h[1]; p[2] = h[2];
+        const bool flat = (S.flags & SF_FLAT_ONLY) != 0;
         const double Nx = Nv[0], Ny = Nv[1], Nz = Nv[2];
         if (S.kind == PHOSIM_DETECTOR) {
             uint32_t w_conv = w1.w, w_diff_a = w2.x, w_diff_b = w2.y, w_back = w4.z;
@@ -183,7 +200,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 double L, sigma, gxd, gyd, r_back;
                 if constexpr (MIXED) {
                     const float n_si = silicon_index_f((float)lam);
-                    if (!refract(dl, Nx, Ny, Nz, n_cur / (double)n_si)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
+                    if (!refract(dl, Nx, Ny, Nz, n_cur * rcp64((double)n_si), flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
                     const float ell = lerp_table_f(P.ell32, P.n_ell, (float)((lam - P.ell_lam0) * P.inv_ell_dlam));
                     const float Lf = ell * -logf(u32of(w_conv));
                     L = (double)Lf;
@@ -191,7 +208,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     r_back = (double)(rf * rf);
                 } else {
                     const double n_si = silicon_index(lam);
-                    if (!refract(dl, Nx, Ny, Nz, n_cur / n_si)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
+                    if (!refract(dl, Nx, Ny, Nz, n_cur * rcp64(n_si), flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
                     const double ell = lerp_table(P.ell, P.n_ell, (lam - P.ell_lam0) * P.inv_ell_dlam);
                     L = ell * -log(u64of(w_conv));
                     const double rf = (n_si - 1.0) / (n_si + 1.0);
@@ -242,20 +259,28 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
             R.x = fx; R.y = fy;
             if (FULL) {
                 const double ux = fx - P.xlo, uy = fy - P.ylo;
-                const double px = floor(ux * P.inv_pixel), py = floor(uy * P.inv_pixel);
-                if (!(px >= 0.0 && py >= 0.0 && px < (double)P.nx && py < (double)P.ny)) {
+                // (conversions saturate; a NaN becomes the most negative integer)
+                const int px = __double2int_rd(ux * P.inv_pixel), py = __double2int_rd(uy * P.inv_pixel);
+                if (!(px >= 0 && py >= 0 && px < P.nx && py < P.ny)) {
                     R.flags = lost(PHOSIM_LOST_OFF_CHIP, si);
                     return;
                 }
-                R.pix = (int)py * P.nx + (int)px;
+                R.pix = py * P.nx + px;
             }
             R.flags = PHOSIM_F_DETECTED;
             return;
         }
         if (FULL) {
             // clear aperture
-            const double r2 = p[0] * p[0] + p[1] * p[1];
-            if (!(r2 <= S.r_out2 && r2 >= S.r_in2)) { R.flags = lost(PHOSIM_LOST_VIGNETTED, si); return; }
+            // (decided in single precision unless the radius is within 1e-5, relative, of a bound)
+            const float xf = f32_trunc(p[0]), yf = f32_trunc(p[1]), r2f = fmaf(xf, xf, yf * yf);
+            const float ro = P.surf_s[si].r_out2.hi, ri = P.surf_s[si].r_in2.hi;
+            bool clear = r2f <= ro && r2f >= ri;
+            if (!(fabsf(r2f - ro) > 1e-5f * ro && fabsf(r2f - ri) > 1e-5f * ri)) {
+                const double r2 = fma(p[0], p[0], p[1] * p[1]);
+                clear = r2 <= S.r_out2 && r2 >= S.r_in2;
+            }
+            if (!clear) { R.flags = lost(PHOSIM_LOST_VIGNETTED, si); return; }
             // coating accept-reject at the incidence angle and wavelength
             if (S.coat_slot >= 0) {
                 const DCoating& C = P.coat[S.coating];
@@ -266,10 +291,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     it = (int)floor((th - C.th0) * C.inv_dth);
                     it = it < 0 ? 0 : (it > C.nt - 1 ? C.nt - 1 : it);
                 }
-                int il = (int)floor((lam - C.lam0) * C.inv_dlam);
+                int il = __double2int_rd((lam - C.lam0) * C.inv_dlam);
                 il = il < 0 ? 0 : (il > C.nl - 1 ? C.nl - 1 : il);
                 const size_t ix = (size_t)il * C.nt + it;
-                const double T = __ldg(C.T + ix);
                 uint32_t w;
                 if (GHOSTS && bounces > 0) {
                     w = ghost_word(P, src, ray, n_ghost++);
@@ -277,9 +301,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     const int k = S.coat_slot;
                     w = k < 2 ? word(w2, 2 + k) : word(w3, k - 2);
                 }
-                if (!(u64of(w) < T)) {
+                if (!((unsigned long long)w < __ldg(C.T_thr + ix))) {    // (w + 1/2) 2^-32 < T
                     // reflected backwards (a ghost) with probability R, absorbed otherwise
-                    if (ghosts && S.kind != PHOSIM_MIRROR && C.TR && u64of(w) < __ldg(C.TR + ix)) {
+                    if (ghosts && S.kind != PHOSIM_MIRROR && C.TR && (unsigned long long)w < __ldg(C.TR_thr + ix)) {
                         const double dn = dl[0] * Nx + dl[1] * Ny + dl[2] * Nz;
                         dl[0] = fma(-2.0 * dn, Nx, dl[0]);
                         dl[1] = fma(-2.0 * dn, Ny, dl[1]);
@@ -309,17 +333,17 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 if (m.kind == PHOSIM_SELLMEIER) {
                     if (glass_mat != mi) {
                         glass_n = sellmeier(m, lam);
-                        glass_inv = 1.0 / glass_n;
+                        glass_inv = rcp64(glass_n);
                         glass_mat = mi;
                     }
                     n_next = glass_n;
                     inv_next = glass_inv;
                 } else if (m.kind == PHOSIM_SILICON) {
                     n_next = silicon_index(lam);
-                    inv_next = 1.0 / n_next;
+                    inv_next = rcp64(n_next);
                 }
             }
-            if (!refract(dl, Nx, Ny, Nz, n_cur * inv_next)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
+            if (!refract(dl, Nx, Ny, Nz, n_cur * inv_next, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
             n_cur = n_next;
         }
         from_surface(S, p, dl, X, D);
@@ -335,7 +359,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
 template <bool MIXED>
 __device__ __forceinline__ double sample_wavelength(const TraceParams& P, const DSource& s, const uint4& w0) {
     const int bin = sed_bin(P.thr + (size_t)s.sed * (P.n_bins - 1), P.sed_guide + (size_t)s.sed * (kSedGuide + 1), w0.z);
-    return fma(u64of(w0.w), P.sed_dlam, P.sed_lam0 + bin * P.sed_dlam) * s.zfac;
+    return fma(u64of(w0.w), P.sed_dlam, fma(f64_of_count((uint32_t)bin), P.sed_dlam, P.sed_lam0)) * s.zfac;
 }
 
 // Dynamic transmission (Sec. 3.2): the index of the first coated surface whose accept draw is not below the
@@ -349,10 +373,10 @@ __device__ __forceinline__ int early_coating_reject(const TraceParams& P, double
     for (int k = 0; k < nk; ++k) {
         const int si = P.coated_surface[k];
         const DCoating& C = P.coat[P.surf[si].coating];
-        int il = (int)floor((lam - C.lam0) * C.inv_dlam);
+        int il = __double2int_rd((lam - C.lam0) * C.inv_dlam);
         il = il < 0 ? 0 : (il > C.nl - 1 ? C.nl - 1 : il);
         const uint32_t w = k < 2 ? word(w2, 2 + k) : word(w3, k - 2);
-        if (!(u64of(w) < __ldg(C.Tmax + il))) return si;
+        if (!((unsigned long long)w < __ldg(C.Tmax_thr + il))) return si;
     }
     return -1;
 }
@@ -420,7 +444,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
     }
     // 1 / |n_z| = rsqrt(1 - n_x^2 - n_y^2): layer-to-layer distances are height differences times it
     double w = fma(-nx, nx, fma(-ny, ny, 1.0));
-    double rinv = rsqrt(w);
+    double rinv = rsqrt64(w);
     const uint4 w2 = philox(make_uint4(clo, chi, (uint32_t)src, 2u), P.k0, P.k1);
     uint4 w3 = make_uint4(0u, 0u, 0u, 0u);
     if (P.n_coated > 2) w3 = philox(make_uint4(clo, chi, (uint32_t)src, 3u), P.k0, P.k1);
@@ -429,12 +453,12 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
         if (si >= 0) { R.flags = lost(PHOSIM_LOST_COATING, si); return; }
     }
     // pupil point on the annulus, on the nominal first surface, moved back to the top of the atmosphere
-    const double r = sqrt(fma(u64of(w0.x), P.pr_dr2, P.pr_in2));
+    const double r = sqrt64(fma(u64of(w0.x), P.pr_dr2, P.pr_in2));
     double sp, cp;
     sincospi(2.0 * u64of(w0.y), &sp, &cp);
     double x = r * cp, y = r * sp;
     double zs = 0.0, zx, zy;
-    sag(P.pupil_surf, x, y, zs, zx, zy);
+    sag<false>(P.pupil_surf, nullptr, x, y, zs, zx, zy, nullptr);
     double z = P.pupil_z + zs;
     {
         const double l = (P.h_top - z) * rinv;
@@ -448,16 +472,14 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
     if (P.flags & PHOSIM_ATMOSPHERE) {
         double kick;
         if constexpr (MIXED) {
-            kick = (double)((float)P.kick0 * exp2f(-0.2f * log2f((float)(lam / P.lam_ref))));
+            kick = (double)((float)P.kick0 * exp2f(-0.2f * log2f(f32_rn_pos(lam * P.inv_lam_ref))));
         } else {
-            // (lambda / lambda_ref)^(-1/5): single-precision seed, then two Newton steps of y -> y (1 + (1 - a y^5) / 5)
-            const double a = lam / P.lam_ref;
-            double y5 = (double)powf((float)a, -0.2f);
-#pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const double y2 = y5 * y5;
-                y5 = fma(y5 * 0.2, fma(-a * y2, y2 * y5, 1.0), y5);
-            }
+            // (lambda / lambda_ref)^(-1/5): a single-precision seed y and one third-order step, with e = 1 - a y^5:
+            // y (1 - e)^(-1/5) = y (1 + e / 5 + 3 e^2 / 25 + ...)
+            const double a = lam * P.inv_lam_ref;
+            double y5 = f64_exact(powf(f32_trunc(a), -0.2f));
+            const double y2 = y5 * y5, e = fma(-(a * y5), y2 * y2, 1.0);
+            y5 = fma(y5 * e, fma(0.12, e, 0.2), y5);
             kick = P.kick0 * y5;
         }
 #pragma unroll 1
@@ -474,7 +496,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
             nx = fma(kick, gx, nx);
             ny = fma(kick, gy, ny);
             w = fma(-nx, nx, fma(-ny, ny, 1.0));
-            rinv = rsqrt(w);
+            rinv = rsqrt64(w);
         }
         // second kick (Sec. 2.3.2): a draw from the long-exposure PSF of the screens above kappa_crit,
         // scaled like the refractive kick by (lambda / lambda_ref)^(-1/5)
@@ -494,7 +516,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
                 ny = fma(ang, sp, ny);
             }
             w = fma(-nx, nx, fma(-ny, ny, 1.0));
-            rinv = rsqrt(w);
+            rinv = rsqrt64(w);
         }
     }
     const double nz = -w * rinv;

@@ -145,33 +145,6 @@ static __device__ PHOSIM_DS_STEP ds sellmeier_ds(const DMaterial& m, float lam_n
     return ds_sqrt(n2);
 }
 
-__device__ __forceinline__ void zern_eval_f(const float* __restrict__ zp, float u, float v, float& z, float& zu,
-                                            float& zv) {
-    float q[7], dq[7];
-    int off = 0;
-#pragma unroll
-    for (int b = 0; b <= 6; ++b) {
-        const int deg = 6 - b;
-        float acc = zp[off + deg], dacc = 0.f;
-#pragma unroll
-        for (int a = deg - 1; a >= 0; --a) {
-            dacc = fmaf(dacc, u, acc);
-            acc = fmaf(acc, u, zp[off + a]);
-        }
-        q[b] = acc;
-        dq[b] = dacc;
-        off += deg + 1;
-    }
-    float zz = q[6], zzu = dq[6], zzv = 0.f;
-#pragma unroll
-    for (int b = 5; b >= 0; --b) {
-        zzv = fmaf(zzv, v, zz);
-        zz = fmaf(zz, v, q[b]);
-        zzu = fmaf(zzu, v, dq[b]);
-    }
-    z = zz; zu = zzu; zv = zzv;
-}
-
 // Sag and slopes (Sec. 2.4.1).  The Zernike figure (tens of nanometres) is evaluated in single precision:
 // its absolute error is far below the 1e-8 mm the intersection resolves.  With the slopes S_x = x g(r^2),
 // S_y = y g(r^2) it returns, in single precision, g and, for the conic and even terms, g1 = dg / d(r^2), which
@@ -297,55 +270,6 @@ __device__ __forceinline__ uint32_t newton_ds(const DSurfaceS& E, int flags, con
         }
     }
     return PHOSIM_LOST_NEWTON;
-}
-
-// Sag and slopes in single precision (the hi parts of the surface's constants), for the first Newton steps
-__device__ __forceinline__ bool sag_f(const DSurfaceS& E, int flags, float x, float y, float& z, float& zx, float& zy) {
-    const float r2 = fmaf(x, x, y * y);
-    float g = 0.f;
-    z = 0.f;
-    if (flags & SF_CONIC) {
-        const float arg = fmaf(-E.k1c2.hi, r2, 1.f);
-        if (arg < 0.f) return false;
-        const float rs = rsqrtf(arg);
-        z = E.c.hi * r2 / fmaf(arg, rs, 1.f);
-        g = E.c.hi * rs;
-    }
-    if (flags & SF_EVEN) {
-        const float u = r2 * E.inv_rn2.hi;
-        int k = E.ne - 1;
-        float pe = E.ae[k].hi, pd = E.aed[k].hi;
-#pragma unroll 1
-        while (--k >= 0) {
-            pe = fmaf(pe, u, E.ae[k].hi);
-            pd = fmaf(pd, u, E.aed[k].hi);
-        }
-        z = fmaf(u * u, pe, z);
-        g = fmaf(u * E.inv_rn2.hi, pd, g);
-    }
-    if (flags & SF_ODD) {
-        const float rho = sqrtf(r2) * E.inv_rn.hi;
-        const float u = rho * rho;
-        int k = E.no - 1;
-        float po = E.ao[k].hi, pd = E.aod[k].hi;
-#pragma unroll 1
-        while (--k >= 0) {
-            po = fmaf(po, u, E.ao[k].hi);
-            pd = fmaf(pd, u, E.aod[k].hi);
-        }
-        z = fmaf(u * rho, po, z);
-        g = fmaf(rho * E.inv_rn2.hi, pd, g);
-    }
-    zx = x * g;
-    zy = y * g;
-    if (flags & SF_ZERN) {
-        float zz, zu, zv;
-        zern_eval_f(E.zp, x * E.zinv, y * E.zinv, zz, zu, zv);
-        z += zz;
-        zx = fmaf(zu, E.zinv, zx);
-        zy = fmaf(zv, E.zinv, zy);
-    }
-    return true;
 }
 
 // The unit normal of a conic at a point (x, y, z) on it: (-c x, -c y, 1 - kc z) normalised.  For a sphere
