@@ -1,4 +1,4 @@
-// Parameters of the adjoint kernel (grad.cu), filled by phosim_grad.
+// Parameters of the adjoint kernels (grad.cu), filled by phosim_grad.
 #pragma once
 
 #include "phosim_device.cuh"
@@ -6,21 +6,26 @@
 namespace phosim {
 
 constexpr int kMaxGradParams = 128;
+// Gradient sums of one source and surface, in the order the adjoint kernel reduces them: 32 for the monomials of
+// the Zernike figure (kZPoly of them), then 32 for the misalignments (field f in the words 32 + f + 8 g, g = 0..3)
+constexpr int kGradWords = 64;
 
 struct GradParams {
     int n_params;
-    int pert_p[PHOSIM_MAX_SURFACES][6];                  // parameter index of misalignment field f, or -1
-    int n_zp[PHOSIM_MAX_SURFACES];                       // Zernike parameters of each surface
-    int zp_j[PHOSIM_MAX_SURFACES][PHOSIM_MAX_ZERNIKE];   // their Noll index j (1-based)
-    int zp_p[PHOSIM_MAX_SURFACES][PHOSIM_MAX_ZERNIKE];   // their parameter index
-    int mat_before[PHOSIM_MAX_SURFACES];                 // medium in front of each surface (-1 = vacuum)
+    int first_surface;                                   // the first surface with a parameter: the sweep ends there
+    uint8_t shift[PHOSIM_MAX_SURFACES];                  // 1: a decenter of this surface is a parameter
+    uint8_t tilt[PHOSIM_MAX_SURFACES];                   // 1: a tilt is
+    uint8_t figure[PHOSIM_MAX_SURFACES];                 // 1: a Zernike coefficient is
+    int32_t param_surface[kMaxGradParams], param_field[kMaxGradParams];
     double dM[PHOSIM_MAX_SURFACES][3][9];                // dM/dtx, dM/dty, dM/dtz of each surface
     const double* zmono;                                 // PHOSIM_MAX_ZERNIKE x kZPoly monomials of Z_j
     const double* seeds;                                 // per source: Ax, Ay, Bxx, Bxy, Byy, mean x, mean y, 0
-    double* grad;                                        // n_src x n_params, added to
+    double* sums;                                        // n_src x n_surf x kGradWords, added to
+    double* grad;                                        // n_src x n_params, written by launch_grad_finish
 };
 
 cudaError_t launch_grad(const TraceParams& P, const GradParams& G, int blocks, cudaStream_t st);
+cudaError_t launch_grad_finish(const TraceParams& P, const GradParams& G, cudaStream_t st);
 cudaError_t grad_occupancy(int* blocks_per_sm);
 
 }  // namespace phosim

@@ -1212,30 +1212,23 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     GradParams G;
     std::memset(&G, 0, sizeof(G));
     G.n_params = n_params;
-    for (int s = 0; s < PHOSIM_MAX_SURFACES; ++s)
-        for (int f = 0; f < 6; ++f) G.pert_p[s][f] = -1;
+    G.first_surface = B.n_surf;
     for (int p = 0; p < n_params; ++p) {
         const int s = ps[p], f = pf[p];
         if (s < 0 || s >= B.n_surf) return PHOSIM_ERR_INVALID_ARGUMENT;
-        if (f >= 0 && f < 6) {
-            if (G.pert_p[s][f] >= 0) return PHOSIM_ERR_INVALID_ARGUMENT;
-            G.pert_p[s][f] = p;
-        } else if (f >= 100 && f < 100 + PHOSIM_MAX_ZERNIKE) {
-            if (!(sc->surfaces[s].zern_rnorm > 0.0)) return PHOSIM_ERR_INVALID_ARGUMENT;
-            for (int k = 0; k < G.n_zp[s]; ++k) if (G.zp_j[s][k] == f - 99) return PHOSIM_ERR_INVALID_ARGUMENT;
-            G.zp_j[s][G.n_zp[s]] = f - 99;
-            G.zp_p[s][G.n_zp[s]] = p;
-            ++G.n_zp[s];
-        } else {
-            return PHOSIM_ERR_INVALID_ARGUMENT;
-        }
+        const bool pert = f >= 0 && f < 6, zernike = f >= 100 && f < 100 + PHOSIM_MAX_ZERNIKE;
+        if (!pert && !zernike) return PHOSIM_ERR_INVALID_ARGUMENT;
+        if (zernike && !(sc->surfaces[s].zern_rnorm > 0.0)) return PHOSIM_ERR_INVALID_ARGUMENT;
+        for (int q = 0; q < p; ++q)
+            if (ps[q] == s && pf[q] == f) return PHOSIM_ERR_INVALID_ARGUMENT;
+        if (zernike) G.figure[s] = 1;
+        else if (f < 3) G.shift[s] = 1;
+        else G.tilt[s] = 1;
+        G.param_surface[p] = s;
+        G.param_field[p] = f;
+        G.first_surface = std::min(G.first_surface, s);
     }
-    int m = -1;
-    for (int s = 0; s < B.n_surf; ++s) {
-        G.mat_before[s] = m;
-        if (sc->surfaces[s].kind == PHOSIM_REFRACT) m = sc->surfaces[s].material;
-        rotation_derivatives(sc->surfaces[s].pert, G.dM[s]);
-    }
+    for (int s = 0; s < B.n_surf; ++s) rotation_derivatives(sc->surfaces[s].pert, G.dM[s]);
     G.zmono = sc->d_zmono;
     cudaStream_t st = (cudaStream_t)stream;
     // forward pass in FP64: moment sums about each source's chief ray
@@ -1285,7 +1278,8 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
             for (int k = 1; k < 6; ++k) o[k] = n > 0 ? D[k] : 0.0;
         }
     }
-    const size_t gbytes = ((size_t)n_src * 8 + (size_t)n_src * n_params) * sizeof(double);
+    const size_t sum_words = (size_t)n_src * B.n_surf * kGradWords;
+    const size_t gbytes = ((size_t)n_src * 8 + sum_words + (size_t)n_src * n_params) * sizeof(double);
     if (sc->cap_grad < gbytes) {
         cudaFree(sc->d_grad_scratch);
         sc->d_grad_scratch = nullptr; sc->cap_grad = 0;
@@ -1293,11 +1287,13 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
         sc->cap_grad = gbytes;
     }
     double* d_seeds = sc->d_grad_scratch;
-    double* d_grad = d_seeds + (size_t)n_src * 8;
+    double* d_sums = d_seeds + (size_t)n_src * 8;
+    double* d_grad = d_sums + sum_words;
     CU(cudaMemcpyAsync(d_seeds, seeds.data(), seeds.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    CU(cudaMemsetAsync(d_grad, 0, (size_t)n_src * n_params * sizeof(double), st));
+    CU(cudaMemsetAsync(d_sums, 0, sum_words * sizeof(double), st));
     CU(cudaMemsetAsync(sc->d_counters, 0, sizeof(unsigned long long), st));
     G.seeds = d_seeds;
+    G.sums = d_sums;
     G.grad = d_grad;
     // the trace left its source list (with chief-ray references) and tile prefix in the scene's scratch
     TraceParams P = sc->base;
@@ -1324,6 +1320,7 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     P.moments = nullptr;
     P.records = nullptr;
     CU(launch_grad(P, G, blocks, st));
+    CU(launch_grad_finish(P, G, st));
     CU(cudaMemcpyAsync(grad, d_grad, (size_t)n_src * n_params * sizeof(double), cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
     return PHOSIM_OK;

@@ -102,11 +102,15 @@ __device__ __forceinline__ float lerp_table_f(const float* __restrict__ t, int n
 
 // Surfaces in order (Sec. 2.4.2).  FULL = apertures, coatings and the sensor; otherwise the bare rays that
 // give each source's chief-ray reference.
-// Forward state kept for the adjoint sweep (RECORD): the telescope-frame position and direction entering
-// each surface, and the conversion length and diffusion offset of the sensor.
+// Forward state kept for the adjoint sweep (RECORD): at each surface, in its frame, the hit point, the direction
+// before it, the distance travelled to it, the normal and (refracting surfaces, the sensor) the index ratio n1 / n2;
+// and the conversion length of the sensor.
+struct SurfaceRecord {
+    double h[3], d[3], l, N[3], mu;
+};
 struct ForwardRecord {
-    double XD[PHOSIM_MAX_SURFACES][6];
-    double L, ox, oy;
+    SurfaceRecord s[PHOSIM_MAX_SURFACES];
+    double L;
 };
 
 // A photon of a bundle (Sec. 3.2 background optimisation): it follows its ray (the photon index divided by
@@ -167,10 +171,6 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
     for (;;) {
         if (si < 0 || si >= P.n_surf) break;
         const DSurface& S = P.surf[si];
-        if constexpr (RECORD) {
-            fr->XD[si][0] = X[0]; fr->XD[si][1] = X[1]; fr->XD[si][2] = X[2];
-            fr->XD[si][3] = D[0]; fr->XD[si][4] = D[1]; fr->XD[si][5] = D[2];
-        }
         double p[3], dl[3];
         to_surface(S, X, D, p, dl);
         double h[3], Nv[3];
@@ -178,6 +178,12 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
         const uint32_t why = intersect(S, P.surf_s[si], p, dl, h, Nv, ahead);
         if (why) { R.flags = lost(why, si); return; }
         if (GHOSTS && bounces > 0 && !ahead) { R.flags = lost(PHOSIM_LOST_MISSED, si); return; }
+        if constexpr (RECORD) {
+            SurfaceRecord& q = fr->s[si];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { q.h[k] = h[k]; q.d[k] = dl[k]; q.N[k] = Nv[k]; }
+            q.l = fma(h[0] - p[0], dl[0], fma(h[1] - p[1], dl[1], (h[2] - p[2]) * dl[2]));
+        }
         p[0] = h[0]; p[1] = h[1]; p[2] = h[2];
         const bool flat = (S.flags & SF_FLAT_ONLY) != 0;
         const double Nx = Nv[0], Ny = Nv[1], Nz = Nv[2];
@@ -207,8 +213,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     const float rf = (n_si - 1.f) / (n_si + 1.f);
                     r_back = (double)(rf * rf);
                 } else {
-                    const double n_si = silicon_index(lam);
-                    if (!refract(dl, Nx, Ny, Nz, n_cur * rcp64(n_si), flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
+                    const double n_si = silicon_index(lam), mu = n_cur * rcp64(n_si);
+                    if constexpr (RECORD) fr->s[si].mu = mu;
+                    if (!refract(dl, Nx, Ny, Nz, mu, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
                     const double ell = lerp_table(P.ell, P.n_ell, (lam - P.ell_lam0) * P.inv_ell_dlam);
                     L = ell * -log(u64of(w_conv));
                     const double rf = (n_si - 1.0) / (n_si + 1.0);
@@ -254,7 +261,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 }
                 fx = fma(sigma, gxd, fx);
                 fy = fma(sigma, gyd, fy);
-                if constexpr (RECORD) { fr->L = L; fr->ox = sigma * gxd; fr->oy = sigma * gyd; }
+                if constexpr (RECORD) fr->L = L;
             }
             R.x = fx; R.y = fy;
             if (FULL) {
@@ -343,7 +350,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     inv_next = rcp64(n_next);
                 }
             }
-            if (!refract(dl, Nx, Ny, Nz, n_cur * inv_next, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
+            const double mu = n_cur * inv_next;
+            if constexpr (RECORD) fr->s[si].mu = mu;
+            if (!refract(dl, Nx, Ny, Nz, mu, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
             n_cur = n_next;
         }
         from_surface(S, p, dl, X, D);
