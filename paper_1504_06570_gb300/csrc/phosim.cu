@@ -56,6 +56,8 @@ constexpr int kBatchWord = kHitCountWord + 1;      // next batch of states for t
 constexpr int kCounterWords = kBatchWord + 1;
 // photons per chunk of the two-kernel path: its state buffer holds one chunk (64 bytes a photon, 8.6 GB)
 constexpr uint64_t kStateChunk = 1ull << 27;
+// the same with reflecting coatings, whose turned rays take another 197 bytes a photon (3.3 GB)
+constexpr uint64_t kGhostChunk = 1ull << 24;
 
 // ----------------------------------------------------------------------------------------- Zernike figure
 // Noll index -> radial order n, |m| and whether the term is the cosine one (even j) or the sine one.
@@ -542,6 +544,8 @@ void phosim_destroy_scene(phosim_scene* sc) {
     cudaFree(sc->d_stage);
     cudaFree(sc->d_state);
     cudaFree(sc->d_hits);
+    cudaFree(sc->d_ghost);
+    cudaFree(sc->d_rounds);
     cudaFree(sc->d_mom_stripes);
     cudaFree(sc->d_grad_scratch);
     cudaFree(sc->d_mom_scratch);
@@ -1047,7 +1051,8 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     CU(cudaMemcpyAsync(sc->d_prefix, prefix.data(), prefix.size() * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
     // two-kernel path: the entrance-plane states of one chunk of tiles at most (kStateChunk photons)
     const uint64_t n_tiles = prefix[n_src];
-    const uint64_t chunk_tiles = staged ? std::max<uint64_t>(1, kStateChunk / T) : n_tiles;
+    const bool ghosts = staged && (sc->base.flags & kGhostFlag);
+    const uint64_t chunk_tiles = staged ? std::max<uint64_t>(1, (ghosts ? kGhostChunk : kStateChunk) / T) : n_tiles;
     if (staged) {
         const size_t need = (size_t)std::min<uint64_t>(total, chunk_tiles * T);
         if (sc->cap_state < need) {
@@ -1062,6 +1067,16 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
             sc->d_hits = nullptr; sc->cap_hits = 0;
             CU(cudaMalloc(&sc->d_hits, need_hits * sizeof(DSHit)));
             sc->cap_hits = need_hits;
+        }
+        if (ghosts) {
+            if (sc->cap_ghost < need) {
+                cudaFree(sc->d_ghost);
+                sc->d_ghost = nullptr; sc->cap_ghost = 0;
+                CU(cudaMalloc(&sc->d_ghost, need * (2 * sizeof(DSGhost) + sizeof(uint32_t) + 1)));
+                sc->cap_ghost = need;
+            }
+            if (!sc->d_rounds) CU(cudaMalloc(&sc->d_rounds, kGhostRounds * sizeof(GhostRound)));
+            CU(cudaMemsetAsync(sc->d_rounds, 0, kGhostRounds * sizeof(GhostRound), st));
         }
     }
     CU(cudaMemsetAsync(sc->d_counters, 0, kCounterWords * sizeof(unsigned long long), st));
@@ -1130,6 +1145,13 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         S.hits = sc->d_hits;
         S.n_hits = sc->d_counters + kHitCountWord;
         S.batch = sc->d_counters + kBatchWord;
+        S.ghost[0] = (DSGhost*)sc->d_ghost;
+        S.ghost[1] = S.ghost[0] + sc->cap_ghost;
+        S.ghost_order = (uint32_t*)(S.ghost[1] + sc->cap_ghost);
+        S.ghost_bin = (uint8_t*)(S.ghost_order + sc->cap_ghost);
+        S.rounds = sc->d_rounds;
+        S.round = 0;
+        const int walk = ghosts ? kWalkForward : kWalkPlain, n_rounds = ghosts ? kGhostRounds : 0;
         S.tile_begin = 0;
         S.tile_end = std::min(n_tiles, chunk_tiles);
         void* stage_args[2] = {&P, &S};
@@ -1142,25 +1164,37 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
             // the whole call as one graph: chief rays; per chunk the counter resets (after the first), the entry,
             // optics and bundle stages; the moment-stripe sum
             const uint64_t n_chunks = (n_tiles + chunk_tiles - 1) / chunk_tiles;
-            std::vector<DSStage> stages((size_t)n_chunks, S);
-            std::vector<std::array<void*, 2>> chunk_args((size_t)n_chunks);
+            const uint64_t per_chunk = 1 + n_rounds;      // the chunk's stage, and one for each round of ghosts
+            std::vector<DSStage> stages((size_t)(n_chunks * per_chunk), S);
+            std::vector<std::array<void*, 2>> chunk_args((size_t)(n_chunks * per_chunk));
+            std::vector<void*> order_args((size_t)(n_chunks * per_chunk));
             std::vector<LaunchOp> ops;
-            ops.reserve((size_t)n_chunks * 5 + 2);
+            ops.reserve((size_t)n_chunks * (6 + 2 * n_rounds) + 2);
             ops.push_back({chief_kernel_ptr(), chief_grid, chief_block, chief_args, nullptr, 0});
             for (uint64_t c = 0; c < n_chunks; ++c) {
-                DSStage& Sc = stages[(size_t)c];
-                Sc.tile_begin = c * chunk_tiles;
-                Sc.tile_end = std::min(n_tiles, Sc.tile_begin + chunk_tiles);
-                chunk_args[(size_t)c] = {&P, &Sc};
-                void** a = chunk_args[(size_t)c].data();
+                for (uint64_t k = c * per_chunk; k < (c + 1) * per_chunk; ++k) {
+                    DSStage& Sk = stages[(size_t)k];
+                    Sk.tile_begin = c * chunk_tiles;
+                    Sk.tile_end = std::min(n_tiles, Sk.tile_begin + chunk_tiles);
+                    Sk.round = (int)(k - c * per_chunk) - 1;
+                    chunk_args[(size_t)k] = {&P, &Sk};
+                    order_args[(size_t)k] = &Sk;
+                }
+                void** a = chunk_args[(size_t)(c * per_chunk)].data();
                 if (c > 0) {
                     ops.push_back({nullptr, dim3(), dim3(), nullptr, sc->d_counters, sizeof(unsigned long long)});
                     ops.push_back({nullptr, dim3(), dim3(), nullptr, sc->d_counters + kStateCountWord,
                                    3 * sizeof(unsigned long long)});
+                    if (ghosts) ops.push_back({nullptr, dim3(), dim3(), nullptr, sc->d_rounds, kGhostRounds * sizeof(GhostRound)});
                 }
                 ops.push_back({ds_entry_kernel_ptr(), dim3((unsigned)blocks), block, a, nullptr, 0});
-                ops.push_back({ds_optics_kernel_ptr(), dim3((unsigned)blocks_optics),
-                               dim3((unsigned)ds_optics_threads(sc->threads)), a, nullptr, 0});
+                const dim3 optics_grid((unsigned)blocks_optics), optics_block((unsigned)ds_optics_threads(sc->threads));
+                ops.push_back({ds_optics_kernel_ptr(walk), optics_grid, optics_block, a, nullptr, 0});
+                for (int r = 0; r < n_rounds; ++r) {
+                    const size_t k = (size_t)(c * per_chunk + 1 + r);
+                    ops.push_back({ghost_order_kernel_ptr(), optics_grid, dim3(256), &order_args[k], nullptr, 0});
+                    ops.push_back({ds_optics_kernel_ptr(kWalkGhosts), optics_grid, optics_block, chunk_args[k].data(), nullptr, 0});
+                }
                 if (bundles) ops.push_back({ds_members_kernel_ptr(), dim3((unsigned)blocks_members), block, a, nullptr, 0});
             }
             if (striped) ops.push_back(reduce);
@@ -1175,9 +1209,16 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
                 if (t0 > 0) {
                     CU(cudaMemsetAsync(sc->d_counters, 0, sizeof(unsigned long long), st));
                     CU(cudaMemsetAsync(sc->d_counters + kStateCountWord, 0, 3 * sizeof(unsigned long long), st));
+                    if (ghosts) CU(cudaMemsetAsync(sc->d_rounds, 0, kGhostRounds * sizeof(GhostRound), st));
                 }
                 ls = timed(2, [&] { return launch_ds_entry(P, S, blocks, sc->threads, st); });
-                if (ls == PHOSIM_OK) ls = timed(3, [&] { return launch_ds_optics(P, S, blocks_optics, sc->threads, st); });
+                if (ls == PHOSIM_OK) ls = timed(3, [&] { return launch_ds_optics(P, S, walk, blocks_optics, sc->threads, st); });
+                for (int r = 0; ls == PHOSIM_OK && r < n_rounds; ++r)
+                    ls = timed(3, [&] {
+                        S.round = r;
+                        const cudaError_t e = launch_ghost_order(S, blocks_optics, st);
+                        return e != cudaSuccess ? e : launch_ds_optics(P, S, kWalkGhosts, blocks_optics, sc->threads, st);
+                    });
                 if (ls == PHOSIM_OK && bundles)
                     ls = timed(4, [&] { return launch_ds_members(P, S, blocks_members, sc->threads, st); });
                 if (ls != PHOSIM_OK) return ls;

@@ -50,6 +50,9 @@ struct phosim_scene {
     size_t cap_state = 0;
     phosim::DSHit* d_hits = nullptr;            // detector hits of its bundle rays
     size_t cap_hits = 0;
+    void* d_ghost = nullptr;                    // rays turned round by coatings: two rounds, their bins and their order
+    size_t cap_ghost = 0;
+    phosim::GhostRound* d_rounds = nullptr;     // the rounds' counts
     double* d_mom_stripes = nullptr;            // its striped per-source moment accumulators
     size_t cap_mom_stripes = 0;
     size_t cap_stage = 0;
@@ -81,12 +84,15 @@ const void* chief_kernel_ptr();
 size_t source_s_bytes();                       // sizeof(SourceS), which the host code does not see
 // the two-kernel double-single path (PHOSIM_MIXED_DS in phosim_trace)
 cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
-cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
+cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_ds_members(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
 const void* ds_members_kernel_ptr();
 cudaError_t ds_stage_occupancy(int threads, int* entry_per_sm, int* optics_per_sm, int* members_per_sm);
 const void* ds_entry_kernel_ptr();
-const void* ds_optics_kernel_ptr();
+// kind of walk (WalkKind): 0 no reflecting coating, 1 forward with ghosts leaving, 2 a round of ghosts
+const void* ds_optics_kernel_ptr(int kind);
+const void* ghost_order_kernel_ptr();
+cudaError_t launch_ghost_order(const DSStage& S, int blocks, cudaStream_t st);
 const void* moment_stripes_kernel_ptr();
 cudaError_t launch_moment_stripes(const TraceParams& P, cudaStream_t st);
 int ds_optics_threads(int threads);      // the optics stage's block size for a schedule's block size

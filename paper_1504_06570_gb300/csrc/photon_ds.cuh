@@ -73,6 +73,8 @@ struct __align__(16) DSHit {
 
 // one chunk of the two-kernel path: tiles [tile_begin, tile_end) of the launch, their states and the
 // bundle rays' detector hits, with their counts
+struct DSGhost;
+struct GhostRound;
 struct DSStage {
     DSState* state;
     unsigned long long* n_state;
@@ -80,6 +82,12 @@ struct DSStage {
     unsigned long long* n_hits;
     unsigned long long* batch;    // the optics stage's blocks claim batches of states from this count
     uint64_t tile_begin, tile_end;
+    // ghosts (a coating reflects): the rays a coating turned round, in rounds (see GhostRound)
+    DSGhost* ghost[2];            // the rays of even and of odd rounds
+    uint8_t* ghost_bin;           // the coated surface that turned each ray of the round being filled
+    uint32_t* ghost_order;        // the round's rays by that surface
+    GhostRound* rounds;           // kGhostRounds
+    int round;                    // the round this launch walks (ghost launches)
 };
 
 // the per-source constants of a tile, converted once per tile
@@ -695,11 +703,32 @@ __device__ __forceinline__ void walk_start(OpticsWalk& W, const ds X[3], const d
     W.si = 0; W.dir = 1; W.bounces = 0; W.n_ghost = 0;
 }
 
-// The next surface of the walk; false once the ray has left it (R.flags then says lost, detected or handed off).
-__device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk& W, ds lam, int src, uint64_t ray,
+// A ray that a coating has turned round, with what its walk needs to go on (the glass index is computed again)
+struct __align__(16) DSGhost {
+    ds X[3], D[3], n_cur;
+    float lam, lam_lo;
+    unsigned long long idx;
+    int src, n_ghost;
+    short si, dir, bounces, pad;
+};
+// One round of ghosts: the rays with the same number of reflections behind them.  bins: rays by the coated surface
+// (its draw's slot) that turned them; placed: how many of each have their place in the order.
+constexpr int kGhostRounds = 4;
+struct GhostRound {
+    unsigned long long n, batch;
+    unsigned bins[8], placed[8];
+};
+
+// What a walk may meet: no reflecting coating (every ray is at the surface it is given), rays on their way
+// forward that end their part of the walk when a coating turns them round, or rays at surfaces of their own.
+enum WalkKind { kWalkPlain, kWalkForward, kWalkGhosts };
+
+// The next surface of the walk (si; a ray at a surface of its own gives W.si); false once the ray has left it
+// (R.flags then says lost, detected or handed off).
+template <WalkKind KIND>
+__device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk& W, int si, ds lam, int src, uint64_t ray,
                                                 PhotonOutS& R, const MemberDrawS* mb = nullptr,
                                                 DetectorHit* hand_off = nullptr) {
-    const int si = W.si;
     if (si < 0 || si >= P.n_surf) {
         R.flags = lost(PHOSIM_LOST_MISSED, si < 0 ? 0 : P.n_surf);
         return false;
@@ -712,7 +741,7 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
     ds l, Nv[3], hit[3];
     const uint32_t why = intersect_ds(E, flags, p, dl, l, Nv, hit);
     if (why) { R.flags = lost(why, si); return false; }
-    if (W.bounces > 0 && !(l.hi > 0.f)) { R.flags = lost(PHOSIM_LOST_MISSED, si); return false; }
+    if (KIND == kWalkGhosts && W.bounces > 0 && !(l.hi > 0.f)) { R.flags = lost(PHOSIM_LOST_MISSED, si); return false; }
     p[0] = hit[0]; p[1] = hit[1]; p[2] = hit[2];
     if (S.kind == PHOSIM_DETECTOR) {
         // the hit on the detector surface, its direction and the medium in front of it
@@ -752,10 +781,11 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
             it = it < 0 ? 0 : (it > C.nt - 1 ? C.nt - 1 : it);
         }
         const size_t ix = (size_t)coat_lambda_bin(C, lam) * C.nt + it;
-        const uint32_t w = W.bounces > 0 ? ghost_word_ds(P, src, ray, W.n_ghost++) : coat_word(P, src, ray, S.coat_slot);
+        const uint32_t w = KIND == kWalkGhosts && W.bounces > 0 ? ghost_word_ds(P, src, ray, W.n_ghost++)
+                                                                : coat_word(P, src, ray, S.coat_slot);
         if (!((unsigned long long)w < __ldg(C.T_thr + ix))) {
             // reflected backwards (a ghost) with probability R, absorbed otherwise
-            if ((P.flags & kGhostFlag) && S.kind != PHOSIM_MIRROR && C.TR_thr &&
+            if (KIND != kWalkPlain && (P.flags & kGhostFlag) && S.kind != PHOSIM_MIRROR && C.TR_thr &&
                 (unsigned long long)w < __ldg(C.TR_thr + ix)) {
                 const ds dn2 = dot3(dl, Nv) * -2.f;
                 {
@@ -784,7 +814,7 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
         dl[2] = dfma(dn2, Nv[2], dl[2]);
     } else {
         // the medium beyond the surface in the direction of travel (-1: vacuum)
-        const int mi = W.dir < 0 ? S.mat_before : S.material;
+        const int mi = KIND == kWalkGhosts && W.dir < 0 ? S.mat_before : S.material;
         ds n_next = ds_f(1.f), inv_next = ds_f(1.f);
         if (mi >= 0) {
             const DMaterial& m = P.mat[mi];
@@ -805,7 +835,7 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
         W.n_cur = n_next;
     }
     from_surface_ds(E, flags, p, dl, W.X, W.D);
-    W.si = si + W.dir;
+    if (KIND == kWalkGhosts) W.si = si + W.dir;
     return true;
 }
 
@@ -816,7 +846,7 @@ __device__ __forceinline__ void optics_ds(const TraceParams& P, const ds X[3], c
     OpticsWalk W;
     walk_start(W, X, D);
 #pragma unroll 1
-    while (surface_step_ds(P, W, lam, src, ray, R, mb, hand_off)) {
+    while (surface_step_ds<kWalkGhosts>(P, W, W.si, lam, src, ray, R, mb, hand_off)) {
     }
 }
 
