@@ -80,6 +80,13 @@ __device__ __forceinline__ ds operator*(ds a, float b) {
     return fast_two_sum(p, e);
 }
 
+// 1 - x for |x| <= 1: exact ordering of the operands, so Dekker's sum gives what Knuth's does (for x > 1 the sign
+// is right and the value is not used)
+__device__ __forceinline__ ds one_minus(ds x) {
+    const ds s = fast_two_sum(1.f, -x.hi);
+    return fast_two_sum(s.hi, __fsub_rn(s.lo, x.lo));
+}
+
 // a b + c with one normalisation
 __device__ __forceinline__ ds dfma(ds a, ds b, ds c) {
     const float p = __fmul_rn(a.hi, b.hi);
@@ -172,18 +179,22 @@ __device__ __forceinline__ ds2 dfma2(ds2 a, float b, ds2 c) {
     return fast_two_sum2(s.hi, e);
 }
 
+// a - b rounded to single precision where b.hi is within a factor of two of a.hi: the difference of the high words is
+// exact (Sterbenz), so no error term is needed
+__device__ __forceinline__ float near_difference(ds a, ds b) {
+    return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo));
+}
+
 // Quotient: a single-precision reciprocal estimate r, q1 = a r, then one correction from the remainder
 // a - q1 b evaluated in double-single; relative error about 2^-45.
 static __device__ PHOSIM_DS_HEAVY ds operator/(ds a, ds b) {
     const float r = __fdividef(1.f, b.hi);
     const float q1 = __fmul_rn(a.hi, r);
-    const ds rem = a - b * q1;
-    return fast_two_sum(q1, __fmul_rn(rem.hi, r));
+    return fast_two_sum(q1, __fmul_rn(near_difference(a, b * q1), r));
 }
 static __device__ PHOSIM_DS_HEAVY ds ds_rcp(ds b) {
     const float r = __fdividef(1.f, b.hi);
-    const ds rem = ds_f(1.f) - b * r;         // 1 - b r, small
-    return fast_two_sum(r, __fmul_rn(rem.hi, r));
+    return fast_two_sum(r, __fmul_rn(near_difference(ds_f(1.f), b * r), r));     // 1 - b r, small
 }
 
 // Square root: y = a rsqrt(a) in single precision, then the Newton correction (a - y^2) / (2 y) with the
@@ -192,8 +203,7 @@ static __device__ PHOSIM_DS_HEAVY ds ds_sqrt(ds a) {
     if (!(a.hi > 0.f)) return {0.f, 0.f};
     const float r = rsqrtf(a.hi);
     const float y = __fmul_rn(a.hi, r);
-    const ds rem = a - two_prod(y, y);
-    return fast_two_sum(y, __fmul_rn(rem.hi, __fmul_rn(0.5f, r)));
+    return fast_two_sum(y, __fmul_rn(near_difference(a, two_prod(y, y)), __fmul_rn(0.5f, r)));
 }
 
 // Reciprocal square root: r0 = rsqrt(a.hi), e = 1 - a r0^2 evaluated in double-single, then the second-

@@ -308,8 +308,10 @@ __global__ void __launch_bounds__(32 * kGradWarps) grad_kernel(const __grid_cons
                 const uint32_t k = base + lane;
                 bool go_on = k < count;
                 if (early && go_on) {
+                    const uint64_t ray = ray_of(s.bundle, s.first + off + k);
+                    const uint32_t w = philox(make_uint4((uint32_t)ray, (uint32_t)(ray >> 32), (uint32_t)src, 0u), P.k0, P.k1).z;
                     double lam;
-                    go_on = early_reject_surface<false>(P, s, src, s.first + off + k, lam) < 0;
+                    go_on = w - s.w_lo <= s.w_span && early_reject_surface<false>(P, s, src, s.first + off + k, lam) < 0;
                 }
                 const unsigned gmask = __ballot_sync(0xffffffffu, go_on);
                 if (go_on) queue[queued + __popc(gmask & lanes_below)] = k;

@@ -612,6 +612,7 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
         }
     }
     std::vector<void*> mem;
+    std::vector<std::vector<unsigned long long>> most((size_t)n_coat);     // each coating's accept thresholds, largest over angles
     bool ghosts = false;
     for (int k = 0; k < n_coat; ++k) {
         double *d, *dmax;
@@ -628,6 +629,7 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
         for (size_t i = 0; i < thr.size(); ++i) thr[i] = accept_threshold(coats[k].table[i]);
         for (size_t i = 0; i < tr.size(); ++i) tr_thr[i] = accept_threshold(tr[i]);
         for (int il = 0; il < nl; ++il) tmax_thr[il] = accept_threshold(tmax[il]);
+        most[(size_t)k] = tmax_thr;
         double* dtr = nullptr;
         unsigned long long* dtr_thr = nullptr;
         phosim_status st = upload(mem, coats[k].table, (size_t)nl * nt, &d);
@@ -653,6 +655,21 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
     }
     P.n_coat = n_coat;
     P.flags = ghosts ? (P.flags | kGhostFlag) : (P.flags & ~kGhostFlag);
+    // the wavelengths that the dynamic transmission test may let pass (with ghosts it tests the first coated surface)
+    P.pass_lo = -1e300; P.pass_hi = 1e300; P.pass_solid = 1;
+    for (int k = 0; k < (ghosts ? std::min(1, coated) : coated); ++k) {
+        const int c = surf[P.coated_surface[k]].coating, nl = coats[c].n_lambda;
+        const std::vector<unsigned long long>& thr = most[(size_t)c];
+        int i0 = 0, i1 = nl - 1;
+        while (i0 < nl && thr[(size_t)i0] == 0) ++i0;
+        while (i1 >= i0 && thr[(size_t)i1] == 0) --i1;
+        for (int i = i0; i <= i1; ++i) if (thr[(size_t)i] == 0) P.pass_solid = 0;
+        // the end bins extend to all wavelengths beyond them
+        const double lo = i0 > i1 ? 1e300 : i0 == 0 ? -1e300 : coats[c].lam0 + i0 * coats[c].dlam;
+        const double hi = i0 > i1 ? -1e300 : i1 == nl - 1 ? 1e300 : coats[c].lam0 + (i1 + 1) * coats[c].dlam;
+        P.pass_lo = std::max(P.pass_lo, lo);
+        P.pass_hi = std::min(P.pass_hi, hi);
+    }
     // the medium in front of each surface, for ghosts that refract on their way back
     {
         int m = -1;
@@ -1111,7 +1128,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     int n_src_arg = n_src;
     double* mom_arg = moments;
     void* chief_args[4] = {&P, &src_ptr, &n_src_arg, &mom_arg};
-    const dim3 chief_grid((unsigned)((n_src + 127) / 128)), chief_block(128);
+    const dim3 chief_grid((unsigned)((n_src + kChiefThreads - 1) / kChiefThreads)), chief_block(kChiefThreads);
     sc->timing_used = 0;
     // a launch between events of the scene's timing pool when per-kernel timing is on
     auto timed = [&](int kind, auto&& launch) -> phosim_status {

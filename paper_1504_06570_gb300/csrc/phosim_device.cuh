@@ -113,6 +113,9 @@ struct DSource {
     float ref_s[4];                           // ref_x, ref_y as double-single pairs (hi, lo, hi, lo)
     uint64_t first, count, rec_off;           // photons [first, first + count); record index of the first
     uint64_t ufirst, ucount;                  // work units of the two-kernel path: rays of a bundle, else photons
+    // Dynamic transmission: the wavelength-bin draws w that some coating may let pass have w - w_lo <= w_span
+    // (modulo 2^32); every other draw is a wavelength that a coating stops whatever its own draw (pass_draws)
+    uint32_t w_lo, w_span;
 };
 
 // counters: [0] traced, [1] detected, [1 + r] dropped for reason r
@@ -124,6 +127,10 @@ struct TraceParams {
     uint32_t flags;
     int n_surf, n_layers, n_coated, n_mat, n_coat;
     int coated_surface[PHOSIM_MAX_COATED];    // surface index of coated-surface draw k
+    // Dynamic transmission: outside [pass_lo, pass_hi) nm one of the coated surfaces it tests lets nothing pass; solid:
+    // inside none of them does
+    int pass_solid, pad_solid;
+    double pass_lo, pass_hi;
     double pr_in2, pr_dr2;                    // pupil annulus
     double h_top, z_ent;
     double lam_ref, kick0;                    // kick0 = lambda_ref [mm] / 2 pi

@@ -81,6 +81,9 @@ cudaError_t launch_chief_rays(const TraceParams& P, DSource* sources, int n_src,
 cudaError_t trace_occupancy(int mode, int threads, int* blocks_per_sm);
 const void* trace_kernel_ptr(int mode);
 const void* chief_kernel_ptr();
+// threads per block of the chief rays: one warp, so that few sources spread over many SMs (a warp alone on an SM
+// is bound by its FP64 latencies, four share the SM's FP64 pipe: 300 sources 53 us with 128 threads a block)
+constexpr int kChiefThreads = 32;
 size_t source_s_bytes();                       // sizeof(SourceS), which the host code does not see
 // the two-kernel double-single path (PHOSIM_MIXED_DS in phosim_trace)
 cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);

@@ -97,6 +97,7 @@ struct SourceS {
     ds zfac_s;
     int kind, sed, table;
     uint32_t bundle;
+    uint32_t w_lo, w_span;
 };
 
 __device__ __forceinline__ SourceS source_s(const DSource& s) {
@@ -106,6 +107,7 @@ __device__ __forceinline__ SourceS source_s(const DSource& s) {
     r.zfac = (float)s.zfac; r.zfac_s = ds_of(s.zfac); r.a = (float)s.a; r.b = (float)s.b; r.cpa = (float)s.cpa; r.spa = (float)s.spa;
     r.kind = s.kind; r.sed = s.sed; r.table = s.table;
     r.bundle = s.bundle; r.bsig = (float)s.bsig;
+    r.w_lo = s.w_lo; r.w_span = s.w_span;
     return r;
 }
 
@@ -285,11 +287,12 @@ __device__ __forceinline__ uint32_t newton_ds(const DSurfaceS& E, int flags, con
 // which vanishes at the intersection: it is already a unit vector (to the root's 1e-14) and needs no root.
 __device__ __forceinline__ void conic_normal_ds(const DSurfaceS& E, ds x, ds y, ds z, ds N[3]) {
     const ds2 cxy = mul2(E.c, ds2_of(x, y));
-    const ds vx = -ds2_x(cxy), vy = -ds2_y(cxy), vz = ds_f(1.f) - E.kc * z;
+    const ds vx = -ds2_x(cxy), vy = -ds2_y(cxy);
     if (E.kmc.hi == 0.f) {
-        N[0] = vx; N[1] = vy; N[2] = vz;
+        N[0] = vx; N[1] = vy; N[2] = one_minus(E.kc * z);
         return;
     }
+    const ds vz = ds_f(1.f) - E.kc * z;
     const ds inv = ds_rsqrt(dfma(vx, vx, dfma(vy, vy, vz * vz)));
     const ds2 nxy = mul2(ds2_of(vx, vy), inv);
     N[0] = ds2_x(nxy); N[1] = ds2_y(nxy);
@@ -397,20 +400,20 @@ static __device__ PHOSIM_DS_STEP uint32_t intersect_ds(const DSurfaceS& E, int f
 
 __device__ __forceinline__ ds dot3(const ds a[3], const ds b[3]) { return dfma(a[0], b[0], dfma(a[1], b[1], a[2] * b[2])); }
 
-// Snell's law in vector form (Sec. 2.4.2), mu = n1 / n2; false on total internal reflection
-static __device__ PHOSIM_DS_STEP bool refract_ds(ds d[3], ds N[3], ds mu) {
-    ds cosi = -dot3(d, N);
-    ds n0 = N[0], n1 = N[1], n2 = N[2];
-    if (cosi.hi < 0.f) { n0 = -n0; n1 = -n1; n2 = -n2; cosi = -cosi; }
-    const ds k = ds_f(1.f) - mu * mu * (ds_f(1.f) - cosi * cosi);
+// Snell's law in vector form (Sec. 2.4.2), mu = n1 / n2; false on total internal reflection.  flat: the normal is
+// (0, 0, 1), whose products are copies and zeros; leaving them out changes no bit of the result.
+static __device__ PHOSIM_DS_STEP bool refract_ds(ds d[3], ds N[3], ds mu, bool flat) {
+    ds cosi = flat ? -d[2] : -dot3(d, N);
+    const bool turn = cosi.hi < 0.f;
+    if (turn) cosi = -cosi;
+    const ds k = one_minus(mu * mu * one_minus(cosi * cosi));
     if (k.hi < 0.f) return false;
-    const ds a = mu * cosi - ds_sqrt(k);
-    {
-        const ds2 q = dfma2(mu, ds2_of(d[0], d[1]), mul2(a, ds2_of(n0, n1)));
-        d[0] = ds2_x(q);
-        d[1] = ds2_y(q);
-    }
-    d[2] = dfma(mu, d[2], a * n2);
+    const ds a = mu * cosi - ds_sqrt(k), s = turn ? -a : a;
+    const ds2 dxy = ds2_of(d[0], d[1]);
+    const ds2 q = flat ? mul2(mu, dxy) : dfma2(mu, dxy, mul2(s, ds2_of(N[0], N[1])));
+    d[0] = ds2_x(q);
+    d[1] = ds2_y(q);
+    d[2] = dfma(mu, d[2], flat ? s : s * N[2]);
     return true;
 }
 
@@ -637,7 +640,7 @@ __device__ __forceinline__ void detect_ds(const TraceParams& P, const DetectorHi
     if (P.flags & PHOSIM_SENSOR) {
         // refraction into the silicon, exponential conversion length (Sec. 2.4.2)
         const float n_si = silicon_index_f(lam);
-        if (!refract_ds(dl, Nv, H.n_cur / ds_f(n_si))) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
+        if (!refract_ds(dl, Nv, H.n_cur / ds_f(n_si), (P.surf[si].flags & SF_FLAT_ONLY) != 0)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
         const float ell = lerp_table_f(P.ell32, P.n_ell, (lam - P.ell_lam0f) * P.inv_ell_dlamf);
         const float L = ell * -logf(u32of(w_conv));
         const float rf = (n_si - 1.f) / (n_si + 1.f);
@@ -831,7 +834,7 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
                 inv_next = ds_rcp(n_next);
             }
         }
-        if (!refract_ds(dl, Nv, W.n_cur * inv_next)) { R.flags = lost(PHOSIM_LOST_TIR, si); return false; }
+        if (!refract_ds(dl, Nv, W.n_cur * inv_next, (flags & SF_FLAT_ONLY) != 0)) { R.flags = lost(PHOSIM_LOST_TIR, si); return false; }
         W.n_cur = n_next;
     }
     from_surface_ds(E, flags, p, dl, W.X, W.D);
@@ -850,9 +853,13 @@ __device__ __forceinline__ void optics_ds(const TraceParams& P, const ds X[3], c
     }
 }
 
+// 1 / |n_z| of a unit direction
+__device__ __forceinline__ ds inverse_nz(ds nx, ds ny) { return ds_rsqrt(one_minus(dfma(nx, nx, ny * ny))); }
+
 // Bilinear screen gradient (Sec. 2.3.2) at a double-single screen position; single-precision weights
-__device__ __forceinline__ void screen_gradient_ds(const DScale& S, ds sx, ds sy, float& gx, float& gy) {
-    const ds fx = sx * S.inv_pix_s, fy = sy * S.inv_pix_s;
+__device__ __forceinline__ void screen_gradient_ds(const DScale& S, ds2 at, float& gx, float& gy) {
+    const ds2 f2 = mul2(at, S.inv_pix_s);
+    const ds fx = ds2_x(f2), fy = ds2_y(f2);
     const float flx = ds_floor(fx), fly = ds_floor(fy);
     const int n = S.n;
     const int ix = (int)flx, iy = (int)fly;
@@ -866,7 +873,8 @@ __device__ __forceinline__ void screen_gradient_ds(const DScale& S, ds sx, ds sy
     }
     const size_t node = (size_t)j0 * n + i0;
     const float tx = ds_frac(fx, flx), ty = ds_frac(fy, fly);
-    const float4 A = __ldg(S.g32 + 2 * node), B = __ldg(S.g32 + 2 * node + 1);
+    float4 A, B;
+    load_block(S.g32 + 2 * node, A, B);
     const float w00 = (1.f - tx) * (1.f - ty), w10 = tx * (1.f - ty), w01 = (1.f - tx) * ty, w11 = tx * ty;
     gx += w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z;
     gy += w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w;
@@ -907,8 +915,7 @@ __device__ __forceinline__ bool photon_entry_ds(const TraceParams& P, const Sour
         nx = nx + s.a * g * cp;
         ny = ny + s.a * g * sp;
     }
-    ds w = ds_f(1.f) - dfma(nx, nx, ny * ny);
-    ds rinv = ds_rsqrt(w);
+    ds rinv = inverse_nz(nx, ny);
     w2 = philox_ds(make_uint4(clo, chi, (uint32_t)src, 2u), P.k0, P.k1);
     w3 = make_uint4(0u, 0u, 0u, 0u);
     if (P.n_coated > 2) w3 = philox_ds(make_uint4(clo, chi, (uint32_t)src, 3u), P.k0, P.k1);
@@ -936,22 +943,23 @@ __device__ __forceinline__ bool photon_entry_ds(const TraceParams& P, const Sour
     // frozen-flow layers top to bottom (Sec. 2.3)
     if (P.flags & PHOSIM_ATMOSPHERE) {
         const float kick = P.kick0f * exp2f(-0.2f * log2f(lam * P.inv_lam_ref_f));
+        // x and y as packed pairs (ds2)
+        ds2 X2 = ds2_of(x, y), N2 = ds2_of(nx, ny);
+        const ds minus_t = -t;
 #pragma unroll 1
         for (int k = 0; k < P.n_layers; ++k) {
             const DLayer& L = P.layer[k];
-            const ds ll = L.dzs * rinv;           // the drop from the plane above, z_above - z_k
-            x = dfma(nx, ll, x);
-            y = dfma(ny, ll, y);
-            z = L.zs;
-            const ds sx = x - L.vxs * t, sy = y - L.vys * t;
+            X2 = dfma2(L.dzs * rinv, N2, X2);     // the drop from the plane above, z_above - z_k
+            const ds2 at = dfma2(minus_t, ds2_of(L.vxs, L.vys), X2);
             float gx = 0.f, gy = 0.f;
 #pragma unroll 1
-            for (int q = 0; q < L.n_scales; ++q) screen_gradient_ds(L.s[q], sx, sy, gx, gy);
-            nx = nx + kick * gx;
-            ny = ny + kick * gy;
-            w = ds_f(1.f) - dfma(nx, nx, ny * ny);
-            rinv = ds_rsqrt(w);
+            for (int q = 0; q < L.n_scales; ++q) screen_gradient_ds(L.s[q], at, gx, gy);
+            N2 = add2(N2, make_float2(kick * gx, kick * gy));
+            rinv = inverse_nz(ds2_x(N2), ds2_y(N2));
+            z = L.zs;
         }
+        x = ds2_x(X2); y = ds2_y(X2);
+        nx = ds2_x(N2); ny = ds2_y(N2);
         // second kick (Sec. 2.3.2) from the long-exposure PSF of the screens above kappa_crit
         if (P.hf_K > 0) {
             const float ang = lerp_table_f(P.hf32, P.hf_K, u32of(w4.x) * (float)P.hf_K - 0.5f) * (kick / P.kick0f);
@@ -959,11 +967,10 @@ __device__ __forceinline__ bool photon_entry_ds(const TraceParams& P, const Sour
             sincospif(2.f * u32of(w4.y), &sa, &ca);
             nx = nx + ang * ca;
             ny = ny + ang * sa;
-            w = ds_f(1.f) - dfma(nx, nx, ny * ny);
-            rinv = ds_rsqrt(w);
+            rinv = inverse_nz(nx, ny);
         }
     }
-    const ds nz = -(w * rinv);
+    const ds nz = -(one_minus(dfma(nx, nx, ny * ny)) * rinv);
     {
         const ds l = (z - P.z_ent_s) * rinv;
         x = dfma(nx, l, x);

@@ -155,7 +155,18 @@ __global__ void __launch_bounds__(256, min_blocks(MODE)) trace_kernel(const __gr
                 const unsigned vmask = __ballot_sync(0xffffffffu, valid);
                 if (lane == 0) cnt[0] += __popc(vmask);
                 bool go_on = valid;
-                if (early) {
+                if (!DS && early && !P.records) {
+                    // stage 1: the wavelength draw, and for those that the coatings may let pass the coating draws
+                    const uint64_t ray = ray_of(s.bundle, first + k);
+                    const uint32_t w = philox(make_uint4((uint32_t)ray, (uint32_t)(ray >> 32), (uint32_t)src, 0u), P.k0, P.k1).z;
+                    go_on = valid && w - s.w_lo <= s.w_span;
+                    if (go_on) {
+                        double lam;
+                        go_on = early_reject_surface<MIXED>(P, s, src, first + k, lam) < 0;
+                    }
+                    const unsigned dropped = __popc(__ballot_sync(0xffffffffu, valid && !go_on));
+                    if (lane == 0) cnt[1 + PHOSIM_LOST_COATING] += dropped;
+                } else if (early) {
                     // stage 1: the early coating decision alone
                     Out R;
                     int rej = -1;
@@ -238,8 +249,15 @@ __global__ void __launch_bounds__(256, min_blocks(MODE)) trace_kernel(const __gr
 // The per-photon arithmetic and its order are those of trace_photon_ds, so both give the same results.  The
 // optics and bundle stages are in trace_optics.cu, compiled with the double-single quotient and roots inline.
 // ---------------------------------------------------------------------------------------------------------
+// The entry stage is bound by its fine screens' lookups: with 4096^2 screens nearly each is a read of its own from
+// memory, and this GPU serves 38e9 independent random reads a second from HBM whatever their size or the number in
+// flight (35e9 of 32 bytes by phosim_gather_rate); the stage does 42e9 a second (a few hit the L2).  With small
+// screens it is bound by issue (64 %).  Four blocks of 64 registers an SM hold the layer loop without spills: 1000
+// stars, 1e8 photons, 4096^2 screens 3.2 ms against 3.5 and 3.6 ms with 5 and 6 blocks and 3.6 ms with 3 (4.2 ms with
+// six blocks of 40 registers, before stage 1 became the interval test of the wavelength draw: its integer work had
+// filled the issue slots of two more blocks).
 #ifndef PHOSIM_DS_ENTRY_MIN_BLOCKS
-#define PHOSIM_DS_ENTRY_MIN_BLOCKS 6
+#define PHOSIM_DS_ENTRY_MIN_BLOCKS 4
 #endif
 
 // Accounting of photons the entry stage stops (the dynamic transmission test): record and loss counters.
@@ -301,16 +319,14 @@ __global__ void __launch_bounds__(256, PHOSIM_DS_ENTRY_MIN_BLOCKS) ds_entry_kern
         const SourceS& ss = src_mem[warp];
         const uint32_t nb = ss.bundle;          // the same for the whole warp (one source per tile)
         int queued = 0;
-        uint32_t base = 0;
+        uint32_t base = 0, passed = 0;
+        if (lane == 0 && nb <= 1) cnt[0] += count;
         for (;;) {
             if (base < count) {
                 const uint32_t k = base + lane;
                 const bool valid = k < count;
                 const uint64_t u = ufirst + k;
-                if (nb <= 1) {
-                    const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-                    if (lane == 0) cnt[0] += __popc(vmask);
-                } else {
+                if (nb > 1) {
                     uint64_t lo;
                     uint32_t nm;
                     unit_members(s, nb, u, lo, nm);
@@ -318,7 +334,23 @@ __global__ void __launch_bounds__(256, PHOSIM_DS_ENTRY_MIN_BLOCKS) ds_entry_kern
                     if (lane == 0) cnt[0] += traced;
                 }
                 bool go_on = valid;
-                if (early) {
+                if (early && !P.records) {
+                    // stage 1: whether the wavelength draw is one that the coatings may let pass; the photons it
+                    // passes take the full test at the start of their propagation
+                    const uint32_t w = philox(make_uint4((uint32_t)u, (uint32_t)(u >> 32), (uint32_t)src, 0u), P.k0, P.k1).z;
+                    go_on = valid && w - ss.w_lo <= ss.w_span;
+                    if (!P.pass_solid && go_on) {
+                        float lam;
+                        go_on = early_reject_certain_f(P, ss, src, u, lam) < 0;
+                    }
+                    if (nb > 1) {
+                        uint64_t lo;
+                        uint32_t nm;
+                        unit_members(s, nb, u, lo, nm);
+                        const unsigned dropped = __reduce_add_sync(0xffffffffu, valid && !go_on ? nm : 0u);
+                        if (lane == 0) cnt[1 + PHOSIM_LOST_COATING] += dropped;
+                    }
+                } else if (early) {
                     // stage 1: the early coating decision alone, for every photon of the unit
                     int rej = -1;
                     float lam = 0.f;
@@ -340,6 +372,7 @@ __global__ void __launch_bounds__(256, PHOSIM_DS_ENTRY_MIN_BLOCKS) ds_entry_kern
                 const unsigned gmask = __ballot_sync(0xffffffffu, go_on);
                 if (go_on) queue[queued + __popc(gmask & lanes_below)] = k;
                 queued += __popc(gmask);
+                passed += __popc(gmask);
                 base += 32;
                 __syncwarp();
             }
@@ -385,6 +418,7 @@ __global__ void __launch_bounds__(256, PHOSIM_DS_ENTRY_MIN_BLOCKS) ds_entry_kern
             }
             if (drained && queued == 0) break;
         }
+        if (lane == 0 && nb <= 1 && early && !P.records) cnt[1 + PHOSIM_LOST_COATING] += count - passed;
         __syncwarp();
     }
     __syncwarp();
@@ -409,6 +443,7 @@ __global__ void chief_ray_kernel(const __grid_constant__ TraceParams P, DSource*
     S.ref_y = ok ? R.y : 0.0;
     const ds rx = ds_of(S.ref_x), ry = ds_of(S.ref_y);
     S.ref_s[0] = rx.hi; S.ref_s[1] = rx.lo; S.ref_s[2] = ry.hi; S.ref_s[3] = ry.lo;
+    pass_draws(P, S, S.w_lo, S.w_span);
     // the double-single constants of the source, converted once here instead of once per tile (the conversions
     // from double run on the FP64 pipe)
     if (P.sources_s) P.sources_s[s] = source_s(S);
@@ -420,7 +455,7 @@ __global__ void chief_ray_kernel(const __grid_constant__ TraceParams P, DSource*
 
 cudaError_t launch_chief_rays(const TraceParams& P, DSource* sources, int n_src, double* moments, cudaStream_t st) {
     if (n_src <= 0) return cudaSuccess;
-    chief_ray_kernel<<<(n_src + 127) / 128, 128, 0, st>>>(P, sources, n_src, moments);
+    chief_ray_kernel<<<(n_src + kChiefThreads - 1) / kChiefThreads, kChiefThreads, 0, st>>>(P, sources, n_src, moments);
     return cudaGetLastError();
 }
 
