@@ -633,13 +633,13 @@ def main():
             "stage_ms": kt,
             "clocks": clock_rec,
             "fma_peaks_measured_tflops": {"fp64": fp64_rate, "fp32": fp32_rate}}
-    # kernels per step: chief rays, then per chunk of 2^27 photons the entry, optics and bundle stages, and
+    # kernels per step: the call preparation and the chief rays, then per chunk of 2^27 photons the entry, optics and bundle stages, and
     # the moment-stripe sum
     import math
     bundle = np.ones(n_src, np.uint64) if sc.sources.bundle is None else np.maximum(1, sc.sources.bundle).astype(np.uint64)
     units = int(np.sum((counts + bundle - np.uint64(1)) // bundle))
     chunks = max(1, math.ceil(units / (1 << 27)))
-    line["gpu_launches"] = (2 + 3 * chunks) * args.steps
+    line["gpu_launches"] = (3 + 3 * chunks) * args.steps
 
     if not args.no_oracle:
         work = algorithmic_work(sc, counts)

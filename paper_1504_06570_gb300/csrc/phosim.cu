@@ -58,6 +58,9 @@ constexpr int kCounterWords = kBatchWord + 1;
 constexpr uint64_t kStateChunk = 1ull << 27;
 // the same with reflecting coatings, whose turned rays take another 197 bytes a photon (3.3 GB)
 constexpr uint64_t kGhostChunk = 1ull << 24;
+// photons up to which the two-kernel path adds the moments without the striped copies (which take a kernel to clear and
+// one to add: 6 us of a 10^4-photon call)
+constexpr uint64_t kDirectMoments = 1ull << 16;
 
 // ----------------------------------------------------------------------------------------- Zernike figure
 // Noll index -> radial order n, |m| and whether the term is the cosine one (even j) or the sine one.
@@ -329,9 +332,12 @@ struct LaunchOp {
     void** args;
     void* dst;
     size_t bytes;
+    std::array<int, 2> after = {kPrevious, -1};   // the steps it follows (-1: none)
+    static constexpr int kPrevious = -2;
 };
 
-// Launch a trace call's sequence as one CUDA graph: built node by node (each depending on the one before) when
+// Launch a trace call's sequence as one CUDA graph: built node by node (each after the one before, or after the steps it
+// names) when
 // the sequence's shape (its kernels and memsets) differs from the scene's cached graph for this slot, then
 // replayed on the caller's stream with this call's kernel parameters and launch shapes.
 phosim_status launch_graph(phosim_scene* sc, int slot, const std::vector<LaunchOp>& ops, cudaStream_t st) {
@@ -339,15 +345,19 @@ phosim_status launch_graph(phosim_scene* sc, int slot, const std::vector<LaunchO
     const size_t n = ops.size();
     bool same = g.exec && g.func.size() == n;
     for (size_t i = 0; same && i < n; ++i)
-        same = g.func[i] == ops[i].func && g.memset_dst[i] == (ops[i].func ? nullptr : ops[i].dst) &&
+        same = g.func[i] == ops[i].func && g.after[i] == ops[i].after && g.memset_dst[i] == (ops[i].func ? nullptr : ops[i].dst) &&
                g.memset_bytes[i] == (ops[i].func ? 0 : ops[i].bytes);
     if (g.exec && !same) destroy_graph(g);
     if (!g.exec) {
         if (cudaGraphCreate(&g.graph, 0) != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_CUDA; }
-        cudaGraphNode_t prev = nullptr;
         for (size_t i = 0; i < n; ++i) {
             const LaunchOp& o = ops[i];
-            cudaGraphNode_t node = nullptr;
+            cudaGraphNode_t node = nullptr, deps[2];
+            size_t n_deps = 0;
+            for (int k : o.after) {
+                if (k == LaunchOp::kPrevious) k = (int)i - 1;
+                if (k >= 0) deps[n_deps++] = g.node[(size_t)k];
+            }
             cudaError_t e;
             if (o.func) {
                 cudaKernelNodeParams kp = {};
@@ -355,7 +365,7 @@ phosim_status launch_graph(phosim_scene* sc, int slot, const std::vector<LaunchO
                 kp.gridDim = o.grid;
                 kp.blockDim = o.block;
                 kp.kernelParams = o.args;
-                e = cudaGraphAddKernelNode(&node, g.graph, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
+                e = cudaGraphAddKernelNode(&node, g.graph, deps, n_deps, &kp);
             } else {
                 cudaMemsetParams mp = {};
                 mp.dst = o.dst;
@@ -364,14 +374,14 @@ phosim_status launch_graph(phosim_scene* sc, int slot, const std::vector<LaunchO
                 mp.width = o.bytes / 4;
                 mp.height = 1;
                 mp.pitch = 0;
-                e = cudaGraphAddMemsetNode(&node, g.graph, prev ? &prev : nullptr, prev ? 1 : 0, &mp);
+                e = cudaGraphAddMemsetNode(&node, g.graph, deps, n_deps, &mp);
             }
             if (e != cudaSuccess) { destroy_graph(g); (void)cudaGetLastError(); return PHOSIM_ERR_CUDA; }
             g.func.push_back(o.func);
             g.memset_dst.push_back(o.func ? nullptr : o.dst);
             g.memset_bytes.push_back(o.func ? 0 : o.bytes);
             g.node.push_back(node);
-            prev = node;
+            g.after.push_back(o.after);
         }
         if (cudaGraphInstantiate(&g.exec, g.graph, 0) != cudaSuccess) { destroy_graph(g); (void)cudaGetLastError(); return PHOSIM_ERR_CUDA; }
     } else {
@@ -539,7 +549,6 @@ void phosim_destroy_scene(phosim_scene* sc) {
     free_all(sc->hf_mem);
     cudaFree(sc->d_src);
     cudaFree(sc->d_src_s);
-    cudaFree(sc->d_prefix);
     cudaFree(sc->d_counters);
     cudaFree(sc->d_stage);
     cudaFree(sc->d_state);
@@ -980,12 +989,16 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     const int mode = sc->precision;
     const bool staged = mode == PHOSIM_MIXED_DS;        // the two-kernel double-single path
     // launch shape
-    int per_sm = 0, per_sm_optics = 0, per_sm_members = 0;
-    if (staged) CU(ds_stage_occupancy(sc->threads, &per_sm, &per_sm_optics, &per_sm_members));
-    else CU(trace_occupancy(mode, sc->threads, &per_sm));
-    per_sm = std::max(per_sm, 1);
-    per_sm_optics = std::max(per_sm_optics, 1);
-    per_sm_members = std::max(per_sm_members, 1);
+    auto& occ = sc->occupancy;
+    if (occ.mode != mode || occ.threads != sc->threads) {
+        occ.mode = -1;
+        if (staged) CU(ds_stage_occupancy(sc->threads, &occ.trace, &occ.optics, &occ.members));
+        else CU(trace_occupancy(mode, sc->threads, &occ.trace));
+        occ.mode = mode;
+        occ.threads = sc->threads;
+    }
+    const int per_sm = std::max(occ.trace, 1), per_sm_optics = std::max(occ.optics, 1);
+    const int per_sm_members = std::max(occ.members, 1);
     const int blocks = sc->sm_count * per_sm, blocks_optics = sc->sm_count * per_sm_optics;
     const int blocks_members = sc->sm_count * per_sm_members;
     const uint64_t warps = (uint64_t)blocks * (sc->threads / 32);
@@ -1035,11 +1048,10 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     if (sc->cap_src < (size_t)n_src) {
         cudaFree(sc->d_src);
         cudaFree(sc->d_src_s);
-        cudaFree(sc->d_prefix);
         sc->d_src = nullptr; sc->d_src_s = nullptr; sc->d_prefix = nullptr; sc->cap_src = 0;
-        CU(cudaMalloc(&sc->d_src, (size_t)n_src * sizeof(DSource)));
+        CU(cudaMalloc(&sc->d_src, (size_t)n_src * sizeof(DSource) + ((size_t)n_src + 1) * sizeof(unsigned long long)));
         CU(cudaMalloc(&sc->d_src_s, (size_t)n_src * source_s_bytes()));
-        CU(cudaMalloc(&sc->d_prefix, ((size_t)n_src + 1) * sizeof(unsigned long long)));
+        sc->d_prefix = (unsigned long long*)(sc->d_src + n_src);
         sc->cap_src = n_src;
     }
     // image: a pointer the device cannot use as device memory is staged through a scene buffer
@@ -1064,8 +1076,17 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         d_image = sc->d_stage;
         CU(cudaMemcpyAsync(d_image, image, img_bytes, cudaMemcpyHostToDevice, st));
     }
-    CU(cudaMemcpyAsync(sc->d_src, hs.data(), hs.size() * sizeof(DSource), cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(sc->d_prefix, prefix.data(), prefix.size() * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+    // a few sources go with the first kernel's parameters; more are copied
+    CallPrep C;
+    std::memset(&C, 0, sizeof(C));
+    if (n_src <= kInlineSources) {
+        C.n_inline = n_src;
+        std::memcpy(C.inline_sources, hs.data(), hs.size() * sizeof(DSource));
+        std::memcpy(C.inline_prefix, prefix.data(), prefix.size() * sizeof(unsigned long long));
+    } else {
+        CU(cudaMemcpyAsync(sc->d_src, hs.data(), hs.size() * sizeof(DSource), cudaMemcpyHostToDevice, st));
+        CU(cudaMemcpyAsync(sc->d_prefix, prefix.data(), prefix.size() * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+    }
     // two-kernel path: the entrance-plane states of one chunk of tiles at most (kStateChunk photons)
     const uint64_t n_tiles = prefix[n_src];
     const bool ghosts = staged && (sc->base.flags & kGhostFlag);
@@ -1093,12 +1114,15 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
                 sc->cap_ghost = need;
             }
             if (!sc->d_rounds) CU(cudaMalloc(&sc->d_rounds, kGhostRounds * sizeof(GhostRound)));
-            CU(cudaMemsetAsync(sc->d_rounds, 0, kGhostRounds * sizeof(GhostRound), st));
+            C.zero[1] = (uint32_t*)sc->d_rounds;
+            C.zero_words[1] = kGhostRounds * sizeof(GhostRound) / 4;
         }
     }
-    CU(cudaMemsetAsync(sc->d_counters, 0, kCounterWords * sizeof(unsigned long long), st));
-    // the two-kernel path's striped moment accumulators, added into the caller's sums after the last stage
-    const bool striped = staged && moments && n_src > 0;
+    C.zero[0] = (uint32_t*)sc->d_counters;
+    C.zero_words[0] = kCounterWords * sizeof(unsigned long long) / 4;
+    // the two-kernel path's striped moment accumulators, added into the caller's sums after the last stage; a small call's
+    // few atomics (at most 2048 an address of 65536 photons in runs of 32) go to the sums themselves
+    const bool striped = staged && moments && total > kDirectMoments;
     const size_t stripe_stride = (size_t)n_src * PHOSIM_MOMENT_WORDS;
     if (striped) {
         const size_t need = (size_t)kMomStripes * stripe_stride;
@@ -1108,7 +1132,8 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
             CU(cudaMalloc(&sc->d_mom_stripes, need * sizeof(double)));
             sc->cap_mom_stripes = need;
         }
-        CU(cudaMemsetAsync(sc->d_mom_stripes, 0, need * sizeof(double), st));
+        C.zero[2] = (uint32_t*)sc->d_mom_stripes;
+        C.zero_words[2] = need * 2;
     }
     TraceParams P = sc->base;
     P.mom_stripes = striped ? sc->d_mom_stripes : nullptr;
@@ -1124,6 +1149,16 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     P.image = d_image;
     P.moments = moments;
     P.records = records;
+    C.sources = sc->d_src;
+    C.sources_s = P.sources_s;
+    C.tile_prefix = sc->d_prefix;
+    C.n_src = n_src;
+    C.n_bins = P.n_bins;
+    C.pass_lo = P.pass_lo; C.pass_hi = P.pass_hi;
+    C.sed_lam0 = P.sed_lam0; C.sed_dlam = P.sed_dlam;
+    C.thr = P.thr;
+    void* prep_args[1] = {&C};
+    const LaunchOp prep = {call_prep_kernel_ptr(), dim3(call_prep_blocks(C)), dim3(kPrepThreads), prep_args, nullptr, 0};
     DSource* src_ptr = sc->d_src;
     int n_src_arg = n_src;
     double* mom_arg = moments;
@@ -1142,17 +1177,23 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         return PHOSIM_OK;
     };
     const bool use_graph = (P.flags & PHOSIM_GRAPH) && !sc->stage_timing;
+    // the rays start beside the chief rays (not between timing events, which stand between the kernels)
+    const bool beside = !sc->stage_timing;
     if (!staged) {
         void* trace_args[1] = {&P};
         if (use_graph) {
             const std::vector<LaunchOp> ops = {
+                prep,
                 {chief_kernel_ptr(), chief_grid, chief_block, chief_args, nullptr, 0},
                 {trace_kernel_ptr(mode), dim3((unsigned)blocks), dim3((unsigned)sc->threads), trace_args, nullptr, 0}};
             phosim_status gs = launch_graph(sc, mode, ops, st);
             if (gs != PHOSIM_OK) return gs;
         } else {
-            phosim_status ls = timed(0, [&] { return launch_chief_rays(P, sc->d_src, n_src, moments, st); });
-            if (ls == PHOSIM_OK) ls = timed(1, [&] { return launch_trace(P, mode, blocks, sc->threads, st); });
+            phosim_status ls = timed(0, [&] {
+                const cudaError_t e = launch_call_prep(C, st);
+                return e != cudaSuccess ? e : launch_chief_rays(P, sc->d_src, n_src, moments, st);
+            });
+            if (ls == PHOSIM_OK) ls = timed(1, [&] { return launch_trace(P, mode, blocks, sc->threads, st, beside); });
             if (ls != PHOSIM_OK) return ls;
         }
     } else {
@@ -1178,15 +1219,16 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         const LaunchOp reduce = {moment_stripes_kernel_ptr(), dim3((unsigned)((n_src * 6 + 255) / 256)), dim3(256),
                                  reduce_args, nullptr, 0};
         if (use_graph) {
-            // the whole call as one graph: chief rays; per chunk the counter resets (after the first), the entry,
-            // optics and bundle stages; the moment-stripe sum
+            // the whole call as one graph: the preparation; the chief rays, beside the first entry stage; per chunk the
+            // counter resets (after the first), the entry, optics and bundle stages; the moment-stripe sum
             const uint64_t n_chunks = (n_tiles + chunk_tiles - 1) / chunk_tiles;
             const uint64_t per_chunk = 1 + n_rounds;      // the chunk's stage, and one for each round of ghosts
             std::vector<DSStage> stages((size_t)(n_chunks * per_chunk), S);
             std::vector<std::array<void*, 2>> chunk_args((size_t)(n_chunks * per_chunk));
             std::vector<void*> order_args((size_t)(n_chunks * per_chunk));
             std::vector<LaunchOp> ops;
-            ops.reserve((size_t)n_chunks * (6 + 2 * n_rounds) + 2);
+            ops.reserve((size_t)n_chunks * (6 + 2 * n_rounds) + 3);
+            ops.push_back(prep);
             ops.push_back({chief_kernel_ptr(), chief_grid, chief_block, chief_args, nullptr, 0});
             for (uint64_t c = 0; c < n_chunks; ++c) {
                 for (uint64_t k = c * per_chunk; k < (c + 1) * per_chunk; ++k) {
@@ -1205,8 +1247,10 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
                     if (ghosts) ops.push_back({nullptr, dim3(), dim3(), nullptr, sc->d_rounds, kGhostRounds * sizeof(GhostRound)});
                 }
                 ops.push_back({ds_entry_kernel_ptr(), dim3((unsigned)blocks), block, a, nullptr, 0});
+                if (c == 0) ops.back().after = {0, -1};
                 const dim3 optics_grid((unsigned)blocks_optics), optics_block((unsigned)ds_optics_threads(sc->threads));
                 ops.push_back({ds_optics_kernel_ptr(walk), optics_grid, optics_block, a, nullptr, 0});
+                if (c == 0) ops.back().after = {LaunchOp::kPrevious, 1};
                 for (int r = 0; r < n_rounds; ++r) {
                     const size_t k = (size_t)(c * per_chunk + 1 + r);
                     ops.push_back({ghost_order_kernel_ptr(), optics_grid, dim3(256), &order_args[k], nullptr, 0});
@@ -1218,7 +1262,10 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
             phosim_status gs = launch_graph(sc, mode, ops, st);
             if (gs != PHOSIM_OK) return gs;
         } else {
-            phosim_status ls = timed(0, [&] { return launch_chief_rays(P, sc->d_src, n_src, moments, st); });
+            phosim_status ls = timed(0, [&] {
+                const cudaError_t e = launch_call_prep(C, st);
+                return e != cudaSuccess ? e : launch_chief_rays(P, sc->d_src, n_src, moments, st);
+            });
             if (ls != PHOSIM_OK) return ls;
             for (uint64_t t0 = 0; t0 < n_tiles; t0 += chunk_tiles) {
                 S.tile_begin = t0;
@@ -1228,7 +1275,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
                     CU(cudaMemsetAsync(sc->d_counters + kStateCountWord, 0, 3 * sizeof(unsigned long long), st));
                     if (ghosts) CU(cudaMemsetAsync(sc->d_rounds, 0, kGhostRounds * sizeof(GhostRound), st));
                 }
-                ls = timed(2, [&] { return launch_ds_entry(P, S, blocks, sc->threads, st); });
+                ls = timed(2, [&] { return launch_ds_entry(P, S, blocks, sc->threads, st, beside && t0 == 0); });
                 if (ls == PHOSIM_OK) ls = timed(3, [&] { return launch_ds_optics(P, S, walk, blocks_optics, sc->threads, st); });
                 for (int r = 0; ls == PHOSIM_OK && r < n_rounds; ++r)
                     ls = timed(3, [&] {

@@ -192,6 +192,30 @@ constexpr int kMomStripes = 16;
 // warps of the entry and bundle stages' blocks (the shared-memory queues and counters are sized for it)
 constexpr int kWarpsPerBlock = 8;
 
+// What a trace call does before its rays (call_prep_kernel): the source list and the tile prefix, given here when they
+// are few (no copy then), the sources' constants and passing wavelength draws, and zeroes for the call's scratch.
+constexpr int kInlineSources = 12;
+struct CallPrep {
+    DSource* sources;
+    SourceS* sources_s;                       // null outside the two-kernel path
+    unsigned long long* tile_prefix;
+    int n_src, n_inline;                      // n_inline: n_src when the lists are below, else 0 (they were copied)
+    int n_bins, pad;
+    double pass_lo, pass_hi, sed_lam0, sed_dlam;
+    const unsigned long long* thr;
+    uint32_t* zero[3];                        // words to clear
+    unsigned long long zero_words[3];
+    DSource inline_sources[kInlineSources];
+    unsigned long long inline_prefix[kInlineSources + 1];
+};
+
+// ------------------------------------------------------------------------------------------------------
+// Programmatic dependent launch: a kernel that lets the next one on the stream start beside it, and the next one's
+// wait for it (no effect on a kernel launched without that attribute).
+// ------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds, two 32x32 multiplications per round.
 // ------------------------------------------------------------------------------------------------------

@@ -1,6 +1,7 @@
 // Host-side scene object behind the phosim C ABI.
 #pragma once
 
+#include <array>
 #include <vector>
 
 #include "phosim_device.cuh"
@@ -16,6 +17,7 @@ struct TraceGraph {
     std::vector<const void*> func;              // per node: the kernel, or null for a memset
     std::vector<void*> memset_dst;              // per node: the memset's destination (null for a kernel)
     std::vector<size_t> memset_bytes;
+    std::vector<std::array<int, 2>> after;      // per node: the nodes it follows (-1: none)
     std::vector<cudaGraphNode_t> node;
 };
 
@@ -39,11 +41,10 @@ struct phosim_scene {
     std::vector<void*> sersic_mem;
     std::vector<void*> hf_mem;      // high-frequency kick quantiles
     // per-call scratch, grown on demand
-    phosim::DSource* d_src = nullptr;
+    phosim::DSource* d_src = nullptr;           // the sources, with the tile prefix behind them
     size_t cap_src = 0;
     void* d_src_s = nullptr;                    // the sources' double-single constants (phosim::SourceS, n_src)
-    unsigned long long* d_prefix = nullptr;
-    size_t cap_prefix = 0;
+    unsigned long long* d_prefix = nullptr;     // in d_src's memory, behind cap_src sources
     unsigned long long* d_counters = nullptr;   // [0] tile counter, [1..9] counters
     uint32_t* d_stage = nullptr;                // staging image for host image pointers
     phosim::DSState* d_state = nullptr;         // entrance-plane states of the two-kernel double-single path
@@ -66,8 +67,10 @@ struct phosim_scene {
     // CUDA graphs of the trace launch (PHOSIM_GRAPH), one per precision, captured on a private stream
     TraceGraph graphs[3];
     cudaStream_t capture_stream = nullptr;
+    // resident blocks an SM of the trace's kernels for a block size (asked of the driver once)
+    struct { int mode = -1, threads = 0, trace = 0, optics = 0, members = 0; } occupancy;
     // per-kernel timing (phosim_set_stage_timing): an event pair per launch of the last call, with the
-    // kernel kind (0 chief, 1 one-kernel trace, 2 entry stage, 3 optics stage)
+    // kernel kind (0 call preparation and chief, 1 one-kernel trace, 2 entry stage, 3 optics stage)
     bool stage_timing = false;
     std::vector<cudaEvent_t> timing_events;
     std::vector<int> timing_kind;
@@ -76,7 +79,12 @@ struct phosim_scene {
 
 namespace phosim {
 // mode: the scene's precision (PHOSIM_PLAIN_FP64, PHOSIM_MIXED, PHOSIM_MIXED_DS)
-cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads, cudaStream_t st);
+// beside: start beside the chief rays, the kernel before on the stream
+cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads, cudaStream_t st, bool beside = false);
+cudaError_t launch_call_prep(const CallPrep& C, cudaStream_t st);
+unsigned call_prep_blocks(const CallPrep& C);
+const void* call_prep_kernel_ptr();
+constexpr int kPrepThreads = 128;
 cudaError_t launch_chief_rays(const TraceParams& P, DSource* sources, int n_src, double* moments, cudaStream_t st);
 cudaError_t trace_occupancy(int mode, int threads, int* blocks_per_sm);
 const void* trace_kernel_ptr(int mode);
@@ -86,7 +94,7 @@ const void* chief_kernel_ptr();
 constexpr int kChiefThreads = 32;
 size_t source_s_bytes();                       // sizeof(SourceS), which the host code does not see
 // the two-kernel double-single path (PHOSIM_MIXED_DS in phosim_trace)
-cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
+cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st, bool beside);
 cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st);
 cudaError_t launch_ds_members(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
 const void* ds_members_kernel_ptr();

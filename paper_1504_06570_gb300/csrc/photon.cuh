@@ -391,7 +391,8 @@ __device__ __forceinline__ double sample_wavelength(const TraceParams& P, const 
 // 32-bit draw: the draws of the bins that reach into [pass_lo, pass_hi).  A bin whose last wavelength (its blur draw is
 // at most 1 - 2^-33) lies below pass_lo is left out, and so at the other end; delta is that distance in bins less the
 // rounding of the wavelengths the paths compute (a double-single wavelength is off by 2^-46 at most).
-__device__ __forceinline__ void pass_draws(const TraceParams& P, const DSource& s, uint32_t& w_lo, uint32_t& w_span) {
+template <class Params>
+__device__ __forceinline__ void pass_draws(const Params& P, const DSource& s, uint32_t& w_lo, uint32_t& w_span) {
     const double scale = P.sed_dlam * s.zfac;
     const double x = (P.pass_lo / s.zfac - P.sed_lam0) / P.sed_dlam, y = (P.pass_hi / s.zfac - P.sed_lam0) / P.sed_dlam;
     const double last = fabs(P.sed_lam0 + P.n_bins * P.sed_dlam) + fabs(P.sed_lam0);

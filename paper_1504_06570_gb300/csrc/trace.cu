@@ -204,11 +204,14 @@ __global__ void __launch_bounds__(256, min_blocks(MODE)) trace_kernel(const __gr
                 __syncwarp();
                 Out Q;
                 Q.flags = 0; Q.pix = -1;
+                // (the wait is for the chief rays beside this kernel, whose reference points the moments take)
                 if constexpr (DS) {
                     if (v) trace_photon_ds(P, ss, src, first + kk, Q);
+                    wait_for_previous();
                     consume<MIXED>(P, Q, v, rec_base + kk, ss.ref_x, ss.ref_y, lane, A, cnt);
                 } else {
                     if (v) trace_photon<MIXED>(P, s, src, first + kk, Q);
+                    wait_for_previous();
                     consume<MIXED>(P, Q, v, rec_base + kk, s.ref_x, s.ref_y, lane, A, cnt);
                 }
             }
@@ -423,11 +426,33 @@ __global__ void __launch_bounds__(256, PHOSIM_DS_ENTRY_MIN_BLOCKS) ds_entry_kern
     }
     __syncwarp();
     if (lane < kNumCounters && cnt[lane]) atomicAdd(P.counters + lane, cnt[lane]);
+    // the chief rays beside this kernel: done when it is, for the optics stage
+    wait_for_previous();
+}
+
+// The first kernel of a call: its lists, the sources' constants as the entry stage reads them (converted once here
+// instead of once per tile: the conversions from double run on the FP64 pipe), and its scratch cleared.
+// A small call is a chain of launches and copies: with it and the chief rays beside the next kernel, a star of 1e4 photons
+// (double-single) takes 43 us instead of 55 (two copies, two clears, chief rays, the stages and the moment copies in a row).
+__global__ void call_prep_kernel(const __grid_constant__ CallPrep C) {
+    const unsigned long long t = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        for (unsigned long long i = t; i < C.zero_words[k]; i += step) C.zero[k][i] = 0u;
+    if (C.n_inline && t <= (unsigned)C.n_inline) C.tile_prefix[t] = C.inline_prefix[t];
+    for (unsigned long long s = t; s < (unsigned)C.n_src; s += step) {
+        DSource S = C.n_inline ? C.inline_sources[s] : C.sources[s];
+        pass_draws(C, S, S.w_lo, S.w_span);
+        C.sources[s] = S;
+        if (C.sources_s) C.sources_s[s] = source_s(S);
+    }
 }
 
 // Chief ray of each source (pupil centre, source centre direction, lambda_ref, no apertures): the
-// reference point of the moment sums.
+// reference point of the moment sums.  A chain of some thousand dependent FP64 operations (10 us for two surfaces, 43
+// us for twelve); nothing needs it before the first moments, so the next kernel starts beside it.
 __global__ void chief_ray_kernel(const __grid_constant__ TraceParams P, DSource* sources, int n_src, double* moments) {
+    let_next_start();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n_src) return;
     DSource& S = sources[s];
@@ -443,14 +468,22 @@ __global__ void chief_ray_kernel(const __grid_constant__ TraceParams P, DSource*
     S.ref_y = ok ? R.y : 0.0;
     const ds rx = ds_of(S.ref_x), ry = ds_of(S.ref_y);
     S.ref_s[0] = rx.hi; S.ref_s[1] = rx.lo; S.ref_s[2] = ry.hi; S.ref_s[3] = ry.lo;
-    pass_draws(P, S, S.w_lo, S.w_span);
-    // the double-single constants of the source, converted once here instead of once per tile (the conversions
-    // from double run on the FP64 pipe)
-    if (P.sources_s) P.sources_s[s] = source_s(S);
     if (moments) {
         moments[(size_t)s * PHOSIM_MOMENT_WORDS + 6] = S.ref_x;
         moments[(size_t)s * PHOSIM_MOMENT_WORDS + 7] = S.ref_y;
     }
+}
+
+unsigned call_prep_blocks(const CallPrep& C) {
+    unsigned long long n = (unsigned long long)C.n_src;
+    for (int k = 0; k < 3; ++k) n = n > C.zero_words[k] ? n : C.zero_words[k];
+    n = (n + kPrepThreads - 1) / kPrepThreads;
+    return (unsigned)(n < 1024 ? n : 1024);
+}
+
+cudaError_t launch_call_prep(const CallPrep& C, cudaStream_t st) {
+    call_prep_kernel<<<call_prep_blocks(C), kPrepThreads, 0, st>>>(C);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_chief_rays(const TraceParams& P, DSource* sources, int n_src, double* moments, cudaStream_t st) {
@@ -459,7 +492,26 @@ cudaError_t launch_chief_rays(const TraceParams& P, DSource* sources, int n_src,
     return cudaGetLastError();
 }
 
-cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads, cudaStream_t st) {
+// a launch that starts beside the kernel before it on the stream, as soon as that one lets it
+template <class... Params, class... Args>
+static cudaError_t launch_beside(void (*kernel)(Params...), int blocks, int threads, cudaStream_t st, const Args&... args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config = {};
+    config.gridDim = dim3((unsigned)blocks);
+    config.blockDim = dim3((unsigned)threads);
+    config.stream = st;
+    config.attrs = &attr;
+    config.numAttrs = 1;
+    return cudaLaunchKernelEx(&config, kernel, args...);
+}
+
+cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads, cudaStream_t st, bool beside) {
+    if (beside && mode != kDS) {        // (the one-kernel double-single path reads the chief rays before its first photon)
+        if (mode == kMixed) return launch_beside(trace_kernel<kMixed>, blocks, threads, st, P);
+        return launch_beside(trace_kernel<kPlain>, blocks, threads, st, P);
+    }
     if (mode == kDS) trace_kernel<kDS><<<blocks, threads, 0, st>>>(P);
     else if (mode == kMixed) trace_kernel<kMixed><<<blocks, threads, 0, st>>>(P);
     else trace_kernel<kPlain><<<blocks, threads, 0, st>>>(P);
@@ -473,7 +525,9 @@ const void* trace_kernel_ptr(int mode) {
 const void* chief_kernel_ptr() { return (const void*)chief_ray_kernel; }
 size_t source_s_bytes() { return sizeof(SourceS); }
 const void* ds_entry_kernel_ptr() { return (const void*)ds_entry_kernel; }
-cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st) {
+const void* call_prep_kernel_ptr() { return (const void*)call_prep_kernel; }
+cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st, bool beside) {
+    if (beside) return launch_beside(ds_entry_kernel, blocks, threads, st, P, S);
     ds_entry_kernel<<<blocks, threads, 0, st>>>(P, S);
     return cudaGetLastError();
 }

@@ -139,7 +139,16 @@ extern "C" phosim_status phosim_trace_noalloc(phosim_scene* sc, const phosim_sou
     P.image = image;
     P.moments = moments;
     P.records = records;
-    if (launch_chief_rays(P, d_src, n_src, moments, s) != cudaSuccess ||
+    CallPrep C;
+    std::memset(&C, 0, sizeof(C));
+    C.sources = d_src;
+    C.tile_prefix = d_prefix;
+    C.n_src = n_src;
+    C.n_bins = P.n_bins;
+    C.pass_lo = P.pass_lo; C.pass_hi = P.pass_hi;
+    C.sed_lam0 = P.sed_lam0; C.sed_dlam = P.sed_dlam;
+    C.thr = P.thr;
+    if (launch_call_prep(C, s) != cudaSuccess || launch_chief_rays(P, d_src, n_src, moments, s) != cudaSuccess ||
         launch_trace(P, mode, blocks, sc->threads, s) != cudaSuccess) {
         (void)cudaGetLastError();
         return PHOSIM_ERR_CUDA;
