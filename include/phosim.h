@@ -278,7 +278,9 @@ phosim_status phosim_grad(phosim_scene* scene, const phosim_source* sources, int
 
 /* Launch shape of the trace kernel: threads per block and photons per warp tile (0 = keep current).  In the
    two-kernel double-single path it applies to the entry and bundle stages; the optics stage keeps blocks of
-   256 threads, whose warps take the surfaces together. */
+   256 threads, whose warps take the surfaces together.  In the FP64 paths with PHOSIM_EARLY_REJECT and coated
+   surfaces it applies to the kernel that tests the photons; the kernel that follows those that go on, in batches of
+   32, keeps blocks of one warp. */
 phosim_status phosim_set_schedule(phosim_scene* scene, int threads_per_block, int tile_photons);
 
 /* The launch shape phosim_trace uses now (after phosim_set_schedule or phosim_autotune): threads per block

@@ -10,8 +10,8 @@
 // What bounds it is the FP64 pipe, so the sweep recomputes nothing that the forward pass had, and the parameter
 // sums cost about one FP64 addition a value: all Zernike coefficients of a surface are linear in the sums of the 28
 // monomials of its figure, which a photon adds to whatever the number of coefficients, and the lanes' values
-// are summed by a transposed butterfly (31 additions for 32 values, the total of value k in lane k), which leaves
-// one accumulator a lane and group in shared memory.  A second kernel turns the sums into the parameters' gradients.
+// are summed by a transposed butterfly (31 additions for 32 values, the total of value k in lane k) and added to the
+// source's sums.  A second kernel turns the sums into the parameters' gradients.
 // Measured (GB300, 64 stars of 3e4 photons, 97 parameters of which 57 Zernike coefficients): a whole call 11.9 ms
 // with every coefficient's polynomial evaluated per photon, per-lane accumulators in local memory and the
 // intersections recomputed in the sweep, 5.6 ms in this form.
@@ -21,8 +21,6 @@
 #include "grad.hpp"
 
 namespace phosim {
-
-constexpr int kGradWarps = 4;
 
 // Second derivatives of the sag at the surface-frame point (x, y), without the Zernike figure's
 __device__ __forceinline__ void sag_hessian(const DSurface& S, double x, double y, double& zxx, double& zxy, double& zyy) {
@@ -82,41 +80,13 @@ __device__ __forceinline__ void refract_adjoint(const double d[3], const double 
     }
 }
 
-// v[k] of every lane to lane k's sum of v[k] over the warp: at each step a lane keeps half of its values and adds
-// its partner's copies of them
-__device__ __forceinline__ double transpose_sum32(double v[32], int lane) {
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        const bool up = (lane & s) != 0;
-#pragma unroll
-        for (int k = 0; k < s; ++k) {
-            const double keep = up ? v[k + s] : v[k], send = up ? v[k] : v[k + s];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-    return v[0];
-}
-// the same for eight values: lane k gets the sum of v[k % 8] over the lanes of its group of eight
-__device__ __forceinline__ double transpose_sum8(double v[8], int lane) {
-#pragma unroll
-    for (int s = 4; s >= 1; s >>= 1) {
-        const bool up = (lane & s) != 0;
-#pragma unroll
-        for (int k = 0; k < s; ++k) {
-            const double keep = up ? v[k + s] : v[k], send = up ? v[k] : v[k + s];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-    return v[0];
-}
-
 // Adjoint of one surface for a warp of photons (on: this lane's photon takes part).  For the detector, fb is the
 // adjoint of the final (x, y) in its frame and L the conversion length (the diffusion offset does not depend on the
 // optics); otherwise Xb / Db carry the adjoint of the telescope-frame state leaving the surface in and of the state
-// entering it out.  acc: the warp's accumulators of this surface, kGradWords.
+// entering it out.  sums: the source's sums of this surface, kGradWords.
 __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const GradParams& G, int si, const SurfaceRecord& q,
                                                 bool on, bool detector, const double fb[2], double L, double Xb[3],
-                                                double Db[3], double* acc, int lane) {
+                                                double Db[3], double* sums, int lane) {
     const DSurface& S = P.surf[si];
     const bool rotated = (S.flags & SF_ROTATED) != 0;
     const double h[3] = {q.h[0], q.h[1], q.h[2]}, d[3] = {q.d[0], q.d[1], q.d[2]}, N[3] = {q.N[0], q.N[1], q.N[2]};
@@ -218,7 +188,8 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
         }
 #pragma unroll
         for (int k = kZPoly; k < 32; ++k) g[k] = 0.0;
-        acc[lane] += transpose_sum32(g, lane);
+        const double sum = transpose_sum<32>(g, lane);
+        if (lane < kZPoly) atomicAdd(sums + lane, sum);
     }
     const bool shift = G.shift[si] != 0, tilt = G.tilt[si] != 0;
     // p = M (X - o), d = M D
@@ -273,85 +244,43 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
         }
 #pragma unroll
         for (int k = 0; k < 6; ++k) g[k] = on ? g[k] : 0.0;
-        acc[32 + lane] += transpose_sum8(g, lane);
+        const double sum = transpose_sum<8>(g, lane);
+        if ((lane & 7) < 6) atomicAdd(sums + 32 + lane, sum);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) { Xb[k] = Xn[k]; Db[k] = Dn[k]; }
 }
 
-__global__ void __launch_bounds__(32 * kGradWarps) grad_kernel(const __grid_constant__ TraceParams P,
-                                                                const __grid_constant__ GradParams G) {
-    // As in the trace kernel, photons the dynamic transmission test removes are dropped first and the
-    // survivors are queued per warp, so the recomputed forward pass and the reverse sweep run on full warps.
-    __shared__ uint32_t queue_mem[kGradWarps][64];
-    extern __shared__ double acc_mem[];                  // kGradWarps x n_surf x kGradWords
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t* queue = queue_mem[warp];
-    double* acc = acc_mem + (size_t)warp * P.n_surf * kGradWords;
-    const unsigned lanes_below = (1u << lane) - 1u;
-    const bool early = (P.flags & PHOSIM_EARLY_REJECT) != 0;
+__global__ void __launch_bounds__(32, 12) grad_kernel(const __grid_constant__ TraceParams P,
+                                                      const __grid_constant__ GradParams G,
+                                                      const __grid_constant__ BatchList L) {
+    // a warp a batch of photons of one source that go on past the dynamic transmission test, as in the trace
+    const int lane = threadIdx.x;
+    const unsigned long long n = *L.n;
     for (;;) {
-        unsigned long long t = 0;
-        if (lane == 0) t = atomicAdd(P.tile_counter, 1ull);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= P.n_tiles) break;
-        const int src = tile_source(P, t, lane);
+        unsigned long long b = 0;
+        if (lane == 0) b = atomicAdd(L.next, 1ull);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (b >= n) break;
+        const PhotonBatch& B = L.batch[b];
+        const int src = B.src;
+        const bool v = lane < (int)B.n;
         const DSource& s = P.sources[src];
-        const uint64_t off = (t - P.tile_prefix[src]) * P.tile_photons;
-        const uint32_t count = (uint32_t)min((uint64_t)P.tile_photons, s.count - off);
         const double* sd = G.seeds + (size_t)src * 8;
-        for (int k = lane; k < P.n_surf * kGradWords; k += 32) acc[k] = 0.0;
-        int queued = 0;
-        uint32_t base = 0;
-        for (;;) {
-            if (base < count) {
-                const uint32_t k = base + lane;
-                bool go_on = k < count;
-                if (early && go_on) {
-                    const uint64_t ray = ray_of(s.bundle, s.first + off + k);
-                    const uint32_t w = philox(make_uint4((uint32_t)ray, (uint32_t)(ray >> 32), (uint32_t)src, 0u), P.k0, P.k1).z;
-                    double lam;
-                    go_on = w - s.w_lo <= s.w_span && early_reject_surface<false>(P, s, src, s.first + off + k, lam) < 0;
-                }
-                const unsigned gmask = __ballot_sync(0xffffffffu, go_on);
-                if (go_on) queue[queued + __popc(gmask & lanes_below)] = k;
-                queued += __popc(gmask);
-                base += 32;
-                __syncwarp();
-            }
-            const bool drained = base >= count;
-            if (queued >= 32 || (drained && queued > 0)) {
-                const int take = queued < 32 ? queued : 32;
-                queued -= take;
-                const bool v = lane < take;
-                const uint32_t kk = v ? queue[queued + lane] : 0u;
-                __syncwarp();
-                ForwardRecord fr;
-                PhotonOut R;
-                R.flags = 0;
-                if (v) trace_photon<false, true>(P, s, src, s.first + off + kk, R, &fr);
-                const bool on = (R.flags & PHOSIM_F_DETECTED) != 0;
-                // the whole warp sweeps (the sums need every lane); the other lanes' values are dropped
-                if (__any_sync(0xffffffffu, on)) {
-                    const double dx = R.x - sd[5], dy = R.y - sd[6];
-                    const double fb[2] = {fma(sd[2], dx, fma(sd[3], dy, sd[0])), fma(sd[4], dy, fma(sd[3], dx, sd[1]))};
-                    double Xb[3] = {0.0, 0.0, 0.0}, Db[3] = {0.0, 0.0, 0.0};
-#pragma unroll 1
-                    for (int si = P.n_surf - 1; si >= G.first_surface; --si)
-                        surface_adjoint(P, G, si, fr.s[si], on, si == P.n_surf - 1, fb, fr.L, Xb, Db,
-                                        acc + si * kGradWords, lane);
-                }
-            }
-            if (drained && queued == 0) break;
-        }
+        ForwardRecord fr;
+        PhotonOut R;
+        R.flags = 0;
+        if (v) trace_photon<false, true, true>(P, s, src, B.first + B.k[lane], R, &fr);
+        const bool on = (R.flags & PHOSIM_F_DETECTED) != 0;
+        // the whole warp sweeps (the sums need every lane); the other lanes' values are dropped
+        if (!__any_sync(0xffffffffu, on)) continue;
+        const double dx = R.x - sd[5], dy = R.y - sd[6];
+        const double fb[2] = {fma(sd[2], dx, fma(sd[3], dy, sd[0])), fma(sd[4], dy, fma(sd[3], dx, sd[1]))};
+        double Xb[3] = {0.0, 0.0, 0.0}, Db[3] = {0.0, 0.0, 0.0};
         double* out = G.sums + (size_t)src * P.n_surf * kGradWords;
 #pragma unroll 1
-        for (int si = G.first_surface; si < P.n_surf; ++si) {
-            if (G.figure[si] && lane < kZPoly) atomicAdd(out + si * kGradWords + lane, acc[si * kGradWords + lane]);
-            if ((G.shift[si] || G.tilt[si]) && (lane & 7) < 6)
-                atomicAdd(out + si * kGradWords + 32 + lane, acc[si * kGradWords + 32 + lane]);
-        }
-        __syncwarp();
+        for (int si = P.n_surf - 1; si >= G.first_surface; --si)
+            surface_adjoint(P, G, si, fr.s[si], on, si == P.n_surf - 1, fb, fr.L, Xb, Db, out + si * kGradWords, lane);
     }
 }
 
@@ -373,10 +302,8 @@ __global__ void grad_finish_kernel(const __grid_constant__ GradParams G, int n_s
     G.grad[i] = s;
 }
 
-static size_t grad_shared_bytes(int n_surf) { return (size_t)kGradWarps * n_surf * kGradWords * sizeof(double); }
-
-cudaError_t launch_grad(const TraceParams& P, const GradParams& G, int blocks, cudaStream_t st) {
-    grad_kernel<<<blocks, 32 * kGradWarps, grad_shared_bytes(P.n_surf), st>>>(P, G);
+cudaError_t launch_grad(const TraceParams& P, const GradParams& G, const BatchList& L, int blocks, cudaStream_t st) {
+    grad_kernel<<<blocks, 32, 0, st>>>(P, G, L);
     return cudaGetLastError();
 }
 
@@ -387,9 +314,7 @@ cudaError_t launch_grad_finish(const TraceParams& P, const GradParams& G, cudaSt
 }
 
 cudaError_t grad_occupancy(int* blocks_per_sm) {
-    // sized for the most surfaces a scene may have (32 KB of accumulators a block)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, grad_kernel, 32 * kGradWarps,
-                                                         grad_shared_bytes(PHOSIM_MAX_SURFACES));
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, grad_kernel, 32, 0);
 }
 
 }  // namespace phosim

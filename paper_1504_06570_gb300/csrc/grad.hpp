@@ -24,7 +24,7 @@ struct GradParams {
     double* grad;                                        // n_src x n_params, written by launch_grad_finish
 };
 
-cudaError_t launch_grad(const TraceParams& P, const GradParams& G, int blocks, cudaStream_t st);
+cudaError_t launch_grad(const TraceParams& P, const GradParams& G, const BatchList& L, int blocks, cudaStream_t st);
 cudaError_t launch_grad_finish(const TraceParams& P, const GradParams& G, cudaStream_t st);
 cudaError_t grad_occupancy(int* blocks_per_sm);
 

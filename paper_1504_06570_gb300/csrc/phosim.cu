@@ -553,6 +553,7 @@ void phosim_destroy_scene(phosim_scene* sc) {
     cudaFree(sc->d_stage);
     cudaFree(sc->d_state);
     cudaFree(sc->d_hits);
+    cudaFree(sc->d_batches);
     cudaFree(sc->d_ghost);
     cudaFree(sc->d_rounds);
     cudaFree(sc->d_mom_stripes);
@@ -989,13 +990,17 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     const int mode = sc->precision;
     const bool staged = mode == PHOSIM_MIXED_DS;        // the two-kernel double-single path
     // launch shape
+    // an FP64 path whose photons the dynamic transmission test may stop: batches of those that go on, then their trace
+    const bool listed = !staged && (sc->base.flags & PHOSIM_EARLY_REJECT) && sc->base.n_coated > 0;
     auto& occ = sc->occupancy;
-    if (occ.mode != mode || occ.threads != sc->threads) {
+    if (occ.mode != mode || occ.threads != sc->threads || occ.listed != (int)listed) {
         occ.mode = -1;
         if (staged) CU(ds_stage_occupancy(sc->threads, &occ.trace, &occ.optics, &occ.members));
+        else if (listed) CU(batch_occupancy(mode, sc->threads, &occ.trace, &occ.optics));
         else CU(trace_occupancy(mode, sc->threads, &occ.trace));
         occ.mode = mode;
         occ.threads = sc->threads;
+        occ.listed = listed;
     }
     const int per_sm = std::max(occ.trace, 1), per_sm_optics = std::max(occ.optics, 1);
     const int per_sm_members = std::max(occ.members, 1);
@@ -1005,7 +1010,11 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     uint64_t total = 0;
     for (int s = 0; s < n_src; ++s) total += n_photons[s];
     uint64_t T = sc->tile_photons;
-    if (!T) {
+    if (!T && listed) {
+        // long tiles leave few batches half full; a few hundred tiles are enough for the test
+        T = total / ((uint64_t)sc->sm_count * 8);
+        T = std::min<uint64_t>(4096, std::max<uint64_t>(128, (T + 31) / 32 * 32));
+    } else if (!T) {
         T = total / (warps * 8);
         T = std::min<uint64_t>(1024, std::max<uint64_t>(32, (T + 31) / 32 * 32));
     }
@@ -1044,6 +1053,8 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         }
         prefix[s + 1] = prefix[s] + (d.ucount + T - 1) / T;
     }
+    sc->batches_whole = false;
+    sc->last_tiles = 0;
     if (n_src == 0 || total == 0) return PHOSIM_OK;
     if (sc->cap_src < (size_t)n_src) {
         cudaFree(sc->d_src);
@@ -1090,7 +1101,20 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     // two-kernel path: the entrance-plane states of one chunk of tiles at most (kStateChunk photons)
     const uint64_t n_tiles = prefix[n_src];
     const bool ghosts = staged && (sc->base.flags & kGhostFlag);
-    const uint64_t chunk_tiles = staged ? std::max<uint64_t>(1, (ghosts ? kGhostChunk : kStateChunk) / T) : n_tiles;
+    const uint64_t chunk_tiles = staged || listed ? std::max<uint64_t>(1, (ghosts ? kGhostChunk : kStateChunk) / T) : n_tiles;
+    if (listed) {
+        // a tile leaves at most one batch more than its photons fill
+        const size_t need = (size_t)(std::min<uint64_t>(total, chunk_tiles * T) / 32 + std::min(n_tiles, chunk_tiles));
+        if (sc->cap_batches < need) {
+            cudaFree(sc->d_batches);
+            sc->d_batches = nullptr; sc->cap_batches = 0;
+            CU(cudaMalloc(&sc->d_batches, need * sizeof(PhotonBatch)));
+            sc->cap_batches = need;
+        }
+    }
+    sc->batches_whole = listed && n_tiles <= chunk_tiles;
+    sc->last_tile = (uint32_t)T;
+    sc->last_tiles = n_tiles;
     if (staged) {
         const size_t need = (size_t)std::min<uint64_t>(total, chunk_tiles * T);
         if (sc->cap_state < need) {
@@ -1179,7 +1203,53 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     const bool use_graph = (P.flags & PHOSIM_GRAPH) && !sc->stage_timing;
     // the rays start beside the chief rays (not between timing events, which stand between the kernels)
     const bool beside = !sc->stage_timing;
-    if (!staged) {
+    if (listed) {
+        BatchList B;
+        B.batch = sc->d_batches;
+        B.n = sc->d_counters + kStateCountWord;
+        B.next = sc->d_counters + kBatchWord;
+        const uint64_t n_chunks = (n_tiles + chunk_tiles - 1) / chunk_tiles;
+        std::vector<BatchList> lists((size_t)n_chunks, B);
+        for (uint64_t c = 0; c < n_chunks; ++c) {
+            lists[(size_t)c].tile_begin = c * chunk_tiles;
+            lists[(size_t)c].tile_end = std::min(n_tiles, (c + 1) * chunk_tiles);
+        }
+        if (use_graph) {
+            // the preparation; the chief rays beside the first chunk's test; per chunk the counter resets (after the
+            // first), the batches and their trace
+            std::vector<std::array<void*, 2>> args((size_t)n_chunks);
+            std::vector<LaunchOp> ops = {prep, {chief_kernel_ptr(), chief_grid, chief_block, chief_args, nullptr, 0}};
+            for (uint64_t c = 0; c < n_chunks; ++c) {
+                args[(size_t)c] = {&P, &lists[(size_t)c]};
+                void** a = args[(size_t)c].data();
+                if (c > 0) {
+                    ops.push_back({nullptr, dim3(), dim3(), nullptr, sc->d_counters, sizeof(unsigned long long)});
+                    ops.push_back({nullptr, dim3(), dim3(), nullptr, sc->d_counters + kStateCountWord,
+                                   3 * sizeof(unsigned long long)});
+                }
+                ops.push_back({batch_kernel_ptr(mode), dim3((unsigned)blocks), dim3((unsigned)sc->threads), a, nullptr, 0});
+                if (c == 0) ops.back().after = {0, -1};
+                ops.push_back({trace_batch_kernel_ptr(mode), dim3((unsigned)blocks_optics), dim3(32), a, nullptr, 0});
+                if (c == 0) ops.back().after = {LaunchOp::kPrevious, 1};
+            }
+            phosim_status gs = launch_graph(sc, mode, ops, st);
+            if (gs != PHOSIM_OK) return gs;
+        } else {
+            phosim_status ls = timed(0, [&] { return launch_call_prep(C, st); });
+            for (uint64_t c = 0; ls == PHOSIM_OK && c < n_chunks; ++c) {
+                if (c > 0) {
+                    CU(cudaMemsetAsync(sc->d_counters, 0, sizeof(unsigned long long), st));
+                    CU(cudaMemsetAsync(sc->d_counters + kStateCountWord, 0, 3 * sizeof(unsigned long long), st));
+                }
+                const BatchList& Lc = lists[(size_t)c];
+                ls = timed(1, [&] { return launch_batches(P, Lc, mode, blocks, sc->threads, st); });
+                if (ls == PHOSIM_OK && c == 0) ls = timed(0, [&] { return launch_chief_rays(P, sc->d_src, n_src, moments, st); });
+                if (ls == PHOSIM_OK)
+                    ls = timed(1, [&] { return launch_trace_batches(P, Lc, mode, blocks_optics, st, beside && c == 0); });
+            }
+            if (ls != PHOSIM_OK) return ls;
+        }
+    } else if (!staged) {
         void* trace_args[1] = {&P};
         if (use_graph) {
             const std::vector<LaunchOp> ops = {
@@ -1396,35 +1466,55 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     double* d_grad = d_sums + sum_words;
     CU(cudaMemcpyAsync(d_seeds, seeds.data(), seeds.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     CU(cudaMemsetAsync(d_sums, 0, sum_words * sizeof(double), st));
-    CU(cudaMemsetAsync(sc->d_counters, 0, sizeof(unsigned long long), st));
     G.seeds = d_seeds;
     G.sums = d_sums;
     G.grad = d_grad;
-    // the trace left its source list (with chief-ray references) and tile prefix in the scene's scratch
+    // the trace left its source list (with chief-ray references), tile prefix and, where one chunk held them all, the
+    // batches of photons that go on; otherwise they are made again, chunk by chunk
     TraceParams P = sc->base;
     P.flags |= PHOSIM_EARLY_REJECT;
     P.sources = sc->d_src;
     P.tile_prefix = sc->d_prefix;
     P.n_src = n_src;
-    uint64_t total = 0;
-    for (int s = 0; s < n_src; ++s) total += n_photons[s];
-    int per_sm = 0;
-    CU(grad_occupancy(&per_sm));
-    per_sm = std::max(per_sm, 1);
-    const int blocks = sc->sm_count * per_sm;
-    uint64_t T = total / ((uint64_t)blocks * 4 * 8);
-    T = std::min<uint64_t>(1024, std::max<uint64_t>(32, (T + 31) / 32 * 32));
-    std::vector<unsigned long long> prefix((size_t)n_src + 1, 0);
-    for (int s = 0; s < n_src; ++s) prefix[s + 1] = prefix[s] + (n_photons[s] + T - 1) / T;
-    CU(cudaMemcpyAsync(sc->d_prefix, prefix.data(), prefix.size() * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
-    P.tile_photons = (uint32_t)T;
-    P.n_tiles = prefix[n_src];
+    P.tile_photons = sc->last_tile;
+    P.n_tiles = sc->last_tiles;
     P.tile_counter = sc->d_counters;
     P.counters = sc->d_counters + 1;
     P.image = nullptr;
     P.moments = nullptr;
     P.records = nullptr;
-    CU(launch_grad(P, G, blocks, st));
+    int per_sm = 0, batch_per_sm = 0, unused = 0;
+    CU(grad_occupancy(&per_sm));
+    CU(batch_occupancy(PHOSIM_PLAIN_FP64, sc->threads, &batch_per_sm, &unused));
+    const int blocks = sc->sm_count * std::max(per_sm, 1), blocks_batch = sc->sm_count * std::max(batch_per_sm, 1);
+    BatchList L;
+    L.n = sc->d_counters + kStateCountWord;
+    L.next = sc->d_counters + kBatchWord;
+    const bool whole = sc->batches_whole;
+    const uint64_t tile = sc->last_tile, n_tiles = sc->last_tiles;
+    const uint64_t chunk_tiles = std::max<uint64_t>(1, kStateChunk / std::max<uint64_t>(tile, 1));
+    if (!whole) {
+        const size_t need = (size_t)(std::min(n_tiles, chunk_tiles) * (tile / 32 + 1));
+        if (sc->cap_batches < need) {
+            cudaFree(sc->d_batches);
+            sc->d_batches = nullptr; sc->cap_batches = 0;
+            CU(cudaMalloc(&sc->d_batches, need * sizeof(PhotonBatch)));
+            sc->cap_batches = need;
+        }
+    }
+    L.batch = sc->d_batches;
+    for (uint64_t t0 = 0; t0 < n_tiles; t0 += chunk_tiles) {
+        L.tile_begin = t0;
+        L.tile_end = std::min(n_tiles, t0 + chunk_tiles);
+        if (whole) {
+            CU(cudaMemsetAsync(L.next, 0, sizeof(unsigned long long), st));
+        } else {
+            CU(cudaMemsetAsync(sc->d_counters, 0, sizeof(unsigned long long), st));
+            CU(cudaMemsetAsync(L.n, 0, 3 * sizeof(unsigned long long), st));
+            CU(launch_batches(P, L, PHOSIM_PLAIN_FP64, blocks_batch, sc->threads, st));
+        }
+        CU(launch_grad(P, G, L, blocks, st));
+    }
     CU(launch_grad_finish(P, G, st));
     CU(cudaMemcpyAsync(grad, d_grad, (size_t)n_src * n_params * sizeof(double), cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));

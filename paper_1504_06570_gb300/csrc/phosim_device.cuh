@@ -192,6 +192,20 @@ constexpr int kMomStripes = 16;
 // warps of the entry and bundle stages' blocks (the shared-memory queues and counters are sized for it)
 constexpr int kWarpsPerBlock = 8;
 
+// Up to 32 photons of one source that go on past the dynamic transmission test, for one warp: photons first + k
+struct __align__(16) PhotonBatch {
+    int src;
+    uint32_t n;
+    unsigned long long first;
+    uint32_t k[32];
+};
+// The batches of tiles [tile_begin, tile_end): their number, and the next one to be taken
+struct BatchList {
+    PhotonBatch* batch;
+    unsigned long long *n, *next;
+    uint64_t tile_begin, tile_end;
+};
+
 // What a trace call does before its rays (call_prep_kernel): the source list and the tile prefix, given here when they
 // are few (no copy then), the sources' constants and passing wavelength draws, and zeroes for the call's scratch.
 constexpr int kInlineSources = 12;

@@ -68,7 +68,13 @@ struct phosim_scene {
     TraceGraph graphs[3];
     cudaStream_t capture_stream = nullptr;
     // resident blocks an SM of the trace's kernels for a block size (asked of the driver once)
-    struct { int mode = -1, threads = 0, trace = 0, optics = 0, members = 0; } occupancy;
+    struct { int mode = -1, threads = 0, trace = 0, optics = 0, members = 0, listed = 0; } occupancy;
+    // the last FP64 call's photon batches: whether they are all there (one chunk), for the adjoint that follows it
+    phosim::PhotonBatch* d_batches = nullptr;
+    size_t cap_batches = 0;
+    bool batches_whole = false;
+    uint32_t last_tile = 0;                     // its photons per tile, tiles and batch kernel's blocks
+    uint64_t last_tiles = 0;
     // per-kernel timing (phosim_set_stage_timing): an event pair per launch of the last call, with the
     // kernel kind (0 call preparation and chief, 1 one-kernel trace, 2 entry stage, 3 optics stage)
     bool stage_timing = false;
@@ -81,6 +87,12 @@ namespace phosim {
 // mode: the scene's precision (PHOSIM_PLAIN_FP64, PHOSIM_MIXED, PHOSIM_MIXED_DS)
 // beside: start beside the chief rays, the kernel before on the stream
 cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads, cudaStream_t st, bool beside = false);
+// the FP64 paths with the dynamic transmission test: batches of photons that go on, then a warp a batch
+cudaError_t launch_batches(const TraceParams& P, const BatchList& L, int mode, int blocks, int threads, cudaStream_t st);
+cudaError_t launch_trace_batches(const TraceParams& P, const BatchList& L, int mode, int blocks, cudaStream_t st, bool beside);
+const void* batch_kernel_ptr(int mode);
+const void* trace_batch_kernel_ptr(int mode);
+cudaError_t batch_occupancy(int mode, int threads, int* batch_per_sm, int* trace_per_sm);
 cudaError_t launch_call_prep(const CallPrep& C, cudaStream_t st);
 unsigned call_prep_blocks(const CallPrep& C);
 const void* call_prep_kernel_ptr();

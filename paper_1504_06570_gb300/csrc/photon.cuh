@@ -441,7 +441,8 @@ __device__ __forceinline__ int early_reject_surface(const TraceParams& P, const 
     return early_coating_reject(P, lam, w2, w3);
 }
 
-template <bool MIXED, bool RECORD = false>
+// TESTED: the photon has passed the dynamic transmission test (or is not subject to it)
+template <bool MIXED, bool RECORD = false, bool TESTED = false>
 __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource& s, int src, uint64_t photon,
                                              PhotonOut& R, ForwardRecord* fr = nullptr) {
     const uint64_t i = ray_of(s.bundle, photon);
@@ -494,7 +495,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
     const uint4 w2 = philox(make_uint4(clo, chi, (uint32_t)src, 2u), P.k0, P.k1);
     uint4 w3 = make_uint4(0u, 0u, 0u, 0u);
     if (P.n_coated > 2) w3 = philox(make_uint4(clo, chi, (uint32_t)src, 3u), P.k0, P.k1);
-    if (P.flags & PHOSIM_EARLY_REJECT) {
+    if (!TESTED && (P.flags & PHOSIM_EARLY_REJECT)) {
         const int si = early_coating_reject(P, lam, w2, w3);
         if (si >= 0) { R.flags = lost(PHOSIM_LOST_COATING, si); return; }
     }
@@ -579,6 +580,23 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
     optics<MIXED, true, RECORD>(P, X, D, lam, w1, w2, w3, w4, R, fr, bundled ? &mb : nullptr, src, i);
 }
 
+
+// v[k] of every lane to lane k's sum of v[k] over the warp: at each step a lane keeps half of its values and adds
+// its partner's copies of them, so that N values cost N - 1 additions a lane (and log2(32 / N) more, below, where N is
+// less than 32: lane k holds the sum of v[k % N] over the lanes of its group of N)
+template <int N>
+__device__ __forceinline__ double transpose_sum(double v[N], int lane) {
+#pragma unroll
+    for (int s = N / 2; s >= 1; s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int k = 0; k < s; ++k) {
+            const double keep = up ? v[k + s] : v[k], send = up ? v[k] : v[k + s];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+    }
+    return v[0];
+}
 
 // Which source owns launch tile t: binary search over the per-source tile prefix (lane 0, then broadcast).
 __device__ __forceinline__ int tile_source(const TraceParams& P, uint64_t t, int lane) {

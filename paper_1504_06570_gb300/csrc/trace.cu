@@ -240,6 +240,162 @@ __global__ void __launch_bounds__(256, min_blocks(MODE)) trace_kernel(const __gr
 }
 
 // ---------------------------------------------------------------------------------------------------------
+// The FP64 paths with the dynamic transmission test, in two kernels.  The FP64 pipe takes a warp's instruction in the
+// same time for one lane as for 32, so a warp that follows the few photons left at the end of its tile wastes it: in
+// one kernel (trace_kernel) 21 of 32 lanes were active with tiles of 160 photons (6 batches' worth of photons a warp)
+// and 7 with the shortest tiles that small calls are cut into.  batch_kernel tests every photon, a cheap integer pass
+// whose tiles can be long, and packs those that go on into batches of 32; trace_batch_kernel follows a batch a warp,
+// each warp claiming the next batch when it is done, in blocks of one warp so that few batches spread over all SMs (a
+// warp alone on an SM does not wait for the FP64 pipe).
+// Measured (GB300): 300 stars, 2e7 photons, all FP64 10.4 ms in one kernel and 8.7 ms in two, mixed 6.8 and 5.6 ms; the
+// adjoint's call for 64 stars of 3e4 photons, which takes the same batches, 5.5 and 3.8 ms.
+// ---------------------------------------------------------------------------------------------------------
+template <bool MIXED>
+__global__ void __launch_bounds__(256, 4) batch_kernel(const __grid_constant__ TraceParams P, const __grid_constant__ BatchList L) {
+    __shared__ uint32_t first_mem[kWarpsPerBlock][64], passed_mem[kWarpsPerBlock][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lanes_below = (1u << lane) - 1u;
+    uint32_t *q1 = first_mem[warp], *q2 = passed_mem[warp];
+    const bool early = (P.flags & PHOSIM_EARLY_REJECT) && P.n_coated > 0;
+    unsigned long long traced = 0, stopped = 0;
+    for (;;) {
+        unsigned long long t = 0;
+        if (lane == 0) t = L.tile_begin + atomicAdd(P.tile_counter, 1ull);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= L.tile_end) break;
+        const int src = tile_source(P, t, lane);
+        const DSource& s = P.sources[src];
+        const uint64_t off = (t - P.tile_prefix[src]) * P.tile_photons;
+        const uint32_t count = (uint32_t)min((uint64_t)P.tile_photons, s.count - off);
+        const uint64_t first = s.first + off;
+        const uint32_t w_lo = s.w_lo, w_span = s.w_span, bundle = s.bundle;
+        uint32_t base = 0, went_on = 0;
+        int n1 = 0, n2 = 0;                   // photons whose wavelength may pass; photons past the test
+        for (;;) {
+            if (base < count) {
+                const uint32_t k = base + lane;
+                bool go = k < count;
+                if (early && go && !P.records) {
+                    const uint64_t ray = ray_of(bundle, first + k);
+                    const uint32_t w = philox(make_uint4((uint32_t)ray, (uint32_t)(ray >> 32), (uint32_t)src, 0u), P.k0, P.k1).z;
+                    go = w - w_lo <= w_span;
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, go);
+                if (go) q1[n1 + __popc(mask & lanes_below)] = k;
+                n1 += __popc(mask);
+                base += 32;
+                __syncwarp();
+            }
+            const bool read = base >= count;
+            if (n1 >= 32 || (read && n1 > 0)) {
+                const int take = min(n1, 32);
+                n1 -= take;
+                const bool v = lane < take;
+                const uint32_t k = v ? q1[n1 + lane] : 0u;
+                bool go = v;
+                if (early && v) {
+                    double lam;
+                    const int si = early_reject_surface<MIXED>(P, s, src, first + k, lam);
+                    go = si < 0;
+                    if (!go && P.records) {
+                        phosim_photon_record rec;
+                        rec.x = rec.y = rec.xc = rec.yc = 0.0;
+                        rec.lambda = lam;
+                        rec.flags = lost(PHOSIM_LOST_COATING, si); rec.pix = -1;
+                        P.records[s.rec_off + off + k] = rec;
+                    }
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, go);
+                if (go) q2[n2 + __popc(mask & lanes_below)] = k;
+                n2 += __popc(mask);
+                went_on += __popc(mask);
+                __syncwarp();
+            }
+            const bool tested = read && n1 == 0;
+            if (n2 >= 32 || (tested && n2 > 0)) {
+                const int take = min(n2, 32);
+                n2 -= take;
+                unsigned long long b = 0;
+                if (lane == 0) b = atomicAdd(L.n, 1ull);
+                PhotonBatch& B = L.batch[__shfl_sync(0xffffffffu, b, 0)];
+                if (lane == 0) { B.src = src; B.n = (uint32_t)take; B.first = first; }
+                B.k[lane] = lane < take ? q2[n2 + lane] : 0u;
+                __syncwarp();
+            }
+            if (tested && n2 == 0) break;
+        }
+        traced += count;
+        stopped += count - went_on;
+    }
+    if (lane == 0 && traced) {
+        atomicAdd(P.counters, traced);
+        if (stopped) atomicAdd(P.counters + 1 + PHOSIM_LOST_COATING, stopped);
+    }
+}
+
+template <bool MIXED>
+__global__ void __launch_bounds__(32, 16) trace_batch_kernel(const __grid_constant__ TraceParams P,
+                                                             const __grid_constant__ BatchList L) {
+    const int lane = threadIdx.x;
+    const unsigned long long n = *L.n;
+    unsigned detected = 0, lost_for[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (;;) {
+        unsigned long long b = 0;
+        if (lane == 0) b = atomicAdd(L.next, 1ull);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (b >= n) break;
+        const PhotonBatch& B = L.batch[b];
+        const int src = B.src;
+        const bool v = lane < (int)B.n;
+        const uint64_t photon = B.first + B.k[lane];
+        const DSource& s = P.sources[src];
+        PhotonOut R;
+        R.flags = 0; R.pix = -1;
+        if (v) trace_photon<MIXED, false, true>(P, s, src, photon, R);
+        // the chief rays beside this kernel, whose reference points the moments take
+        wait_for_previous();
+        if (v && P.records) {
+            phosim_photon_record rec;
+            rec.x = R.x; rec.y = R.y; rec.xc = R.xc; rec.yc = R.yc; rec.lambda = R.lam;
+            rec.flags = R.flags; rec.pix = R.pix;
+            P.records[s.rec_off + (photon - s.first)] = rec;
+        }
+        const bool det = v && (R.flags & PHOSIM_F_DETECTED);
+        const unsigned dmask = __ballot_sync(0xffffffffu, det);
+        detected += __popc(dmask);
+        if (det) {
+            const unsigned same = __match_any_sync(dmask, R.pix);
+            if (lane == __ffs(same) - 1) atomicAdd(P.image + R.pix, (unsigned)__popc(same));
+        }
+        const uint32_t reason = v ? ((R.flags >> 8) & 0xffu) : 0u;
+        if (__any_sync(0xffffffffu, reason != 0u)) {
+#pragma unroll
+            for (int q = 1; q <= 8; ++q) lost_for[q - 1] += __popc(__ballot_sync(0xffffffffu, reason == (uint32_t)q));
+        }
+        if (P.moments && dmask) {
+            const double dx = det ? R.x - s.ref_x : 0.0, dy = det ? R.y - s.ref_y : 0.0;
+            double m[8] = {det ? 1.0 : 0.0, dx, dy, 0.0, 0.0, 0.0, 0.0, 0.0};
+            if constexpr (MIXED) {            // the mixed path's terms are single precision (its one-kernel form's too)
+                const float fx = (float)dx, fy = (float)dy;
+                m[1] = f64_exact(fx); m[2] = f64_exact(fy);
+                m[3] = f64_exact(fx * fx); m[4] = f64_exact(fx * fy); m[5] = f64_exact(fy * fy);
+            } else {
+                m[3] = dx * dx; m[4] = dx * dy; m[5] = dy * dy;
+            }
+            double sum = transpose_sum<8>(m, lane);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+            if (lane < 6) atomicAdd(P.moments + (size_t)src * PHOSIM_MOMENT_WORDS + lane, sum);
+        }
+    }
+    wait_for_previous();
+    if (lane == 0 && detected) atomicAdd(P.counters + 1, (unsigned long long)detected);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (lane == 0 && lost_for[q]) atomicAdd(P.counters + 2 + q, (unsigned long long)lost_for[q]);
+}
+
+// ---------------------------------------------------------------------------------------------------------
 // The double-single path in two kernels.  One megakernel that samples, crosses the atmosphere and traces
 // the optics keeps the whole path's code and live state at once; on this GPU its FP32 instruction stream
 // outruns the instruction cache and its registers spill.  Split at the entrance plane of the telescope
@@ -518,6 +674,25 @@ cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads
     return cudaGetLastError();
 }
 
+cudaError_t launch_batches(const TraceParams& P, const BatchList& L, int mode, int blocks, int threads, cudaStream_t st) {
+    if (mode == kMixed) batch_kernel<true><<<blocks, threads, 0, st>>>(P, L);
+    else batch_kernel<false><<<blocks, threads, 0, st>>>(P, L);
+    return cudaGetLastError();
+}
+cudaError_t launch_trace_batches(const TraceParams& P, const BatchList& L, int mode, int blocks, cudaStream_t st, bool beside) {
+    if (beside) return mode == kMixed ? launch_beside(trace_batch_kernel<true>, blocks, 32, st, P, L)
+                                      : launch_beside(trace_batch_kernel<false>, blocks, 32, st, P, L);
+    if (mode == kMixed) trace_batch_kernel<true><<<blocks, 32, 0, st>>>(P, L);
+    else trace_batch_kernel<false><<<blocks, 32, 0, st>>>(P, L);
+    return cudaGetLastError();
+}
+const void* batch_kernel_ptr(int mode) {
+    return mode == kMixed ? (const void*)batch_kernel<true> : (const void*)batch_kernel<false>;
+}
+const void* trace_batch_kernel_ptr(int mode) {
+    return mode == kMixed ? (const void*)trace_batch_kernel<true> : (const void*)trace_batch_kernel<false>;
+}
+
 const void* trace_kernel_ptr(int mode) {
     if (mode == kDS) return (const void*)trace_kernel<kDS>;
     return mode == kMixed ? (const void*)trace_kernel<kMixed> : (const void*)trace_kernel<kPlain>;
@@ -530,6 +705,12 @@ cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, 
     if (beside) return launch_beside(ds_entry_kernel, blocks, threads, st, P, S);
     ds_entry_kernel<<<blocks, threads, 0, st>>>(P, S);
     return cudaGetLastError();
+}
+
+cudaError_t batch_occupancy(int mode, int threads, int* batch_per_sm, int* trace_per_sm) {
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(batch_per_sm, batch_kernel_ptr(mode), threads, 0);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(trace_per_sm, trace_batch_kernel_ptr(mode), 32, 0);
 }
 
 cudaError_t trace_occupancy(int mode, int threads, int* blocks_per_sm) {
