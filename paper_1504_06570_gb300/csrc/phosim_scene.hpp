@@ -27,6 +27,7 @@ struct phosim_scene {
     int device = 0;                 // the CUDA device current at creation; every call must run with it current
     bool optics_loaded = false, seds_loaded = false;
     int sm_count = 0;
+    int host_atomics = 0;           // whether the GPU's atomics on host memory are native
     int threads = 256;
     int tile_photons = 0;           // 0 = chosen per call from the workload
     int n_sed = 0;
@@ -47,6 +48,9 @@ struct phosim_scene {
     unsigned long long* d_prefix = nullptr;     // in d_src's memory, behind cap_src sources
     unsigned long long* d_counters = nullptr;   // [0] tile counter, [1..9] counters
     uint32_t* d_stage = nullptr;                // staging image for host image pointers
+    uint32_t* d_delta = nullptr;                // a short exposure's counts before they are added to a pinned image
+    size_t cap_delta = 0;
+    bool delta_clean = false;                   // all zeroes (no call has left counts behind)
     phosim::DSState* d_state = nullptr;         // entrance-plane states of the two-kernel double-single path
     size_t cap_state = 0;
     phosim::DSHit* d_hits = nullptr;            // detector hits of its bundle rays
