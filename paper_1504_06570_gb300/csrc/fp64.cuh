@@ -67,13 +67,14 @@ __device__ __forceinline__ double f64_exact(float f) {
 // (double)n of a non-negative n, exact: 2^52 + n by its bits, then 2^52 off
 __device__ __forceinline__ double f64_of_count(uint32_t n) { return __hiloint2double(0x43300000, (int)n) - 4503599627370496.0; }
 
-// floor(f) for |f| < 2^31 (floor_in_range) as a double and an integer: adding 1.5 2^52 rounded down leaves the
-// integer in the low word
-__device__ __forceinline__ bool floor_in_range(double f) { return (__double2hiint(f) & 0x7fffffff) < 0x41e00000; }
-__device__ __forceinline__ double floor64(double f, int& i) {
-    const double t = __dadd_rd(f, 6755399441055744.0);
+// floor(s k) as a double and an integer: the product added to 1.5 2^52 and rounded down in one operation leaves the
+// integer in the low word.  False where the floor is not within 32 bits (nothing is set then).
+__device__ __forceinline__ bool floor_product64(double s, double k, double& fl, int& i) {
+    const double t = __fma_rd(s, k, 6755399441055744.0);
+    if ((unsigned)(__double2hiint(t) - 0x4337ffff) > 1u) return false;
+    fl = t - 6755399441055744.0;
     i = __double2loint(t);
-    return t - 6755399441055744.0;
+    return true;
 }
 
 }  // namespace phosim

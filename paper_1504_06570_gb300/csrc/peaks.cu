@@ -283,6 +283,7 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n) {
     if (i >= n) return;
     const double x = a[i];
     int k = 0;
+    double f = 0.0;
     switch (op) {
         case 0: out[i] = rcp64(x); break;
         case 1: out[i] = rsqrt64(x); break;
@@ -290,8 +291,8 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n) {
         case 3: out[i] = (double)f32_trunc(x); break;
         case 4: out[i] = (double)f32_rn_pos(x); break;
         case 5: out[i] = f64_exact((float)x); break;
-        case 6: out[i] = floor64(x, k); break;
-        case 7: floor64(x, k); out[i] = (double)k; break;
+        case 6: out[i] = floor_product64(x, 1.0, f, k) ? f : 0.5; break;
+        case 7: out[i] = floor_product64(x, 1.0, f, k) ? (double)k : 0.5; break;
         case 8: out[i] = u64of((uint32_t)x); break;
         default: break;
     }

@@ -98,6 +98,7 @@ struct DLayer {
     double z, vx, vy;
     ds zs, vxs, vys;
     ds dzs;                                   // height of the plane above (the previous layer or the top) over z
+    double dz;                                // the same
     int n_scales, pad;
     DScale s[PHOSIM_MAX_SCALES];
 };
@@ -324,27 +325,14 @@ __device__ __forceinline__ void zern_hess_f(const float* __restrict__ zp, float 
     zuu = wuu; zuv = wuv; zvv = 2.f * hv;
 }
 
-// Sag and its partial derivatives in the surface frame; false outside the conic's domain.  With E (the
-// single-precision constants of the surface) also the second derivatives H = (S_xx, S_xy, S_yy) in single
-// precision, from g = (1/r) dS/dr and its derivative in r^2: S_xx = g + 2 x^2 g1 and so on.
-template <bool CURV>
-__device__ __forceinline__ bool sag(const DSurface& S, const DSurfaceS* E, double x, double y, double& z, double& zx,
-                                    double& zy, float H[3]) {
-    const double r2 = fma(x, x, y * y);
+// The aspheric and Zernike part of the sag, its slopes, and its second derivatives H = (xx, xy, yy) in single
+// precision (from g = (1/r) dS/dr and its derivative in r^2: S_xx = g + 2 x^2 g1 and so on).  E: the single-precision
+// constants of the surface.
+__device__ __forceinline__ void aspheric(const DSurface& S, const DSurfaceS& E, double x, double y, double r2, double& z,
+                                         double& zx, double& zy, float H[3]) {
     double g = 0.0;
     float g1 = 0.f;
     z = 0.0;
-    if (S.flags & SF_CONIC) {
-        const double arg = fma(-S.k1c2, r2, 1.0);
-        if (negative64(arg)) return false;
-        const double rs = rsqrt64(arg);
-        z = S.c * r2 * rcp64(fma(arg, rs, 1.0));
-        g = S.c * rs;
-        if constexpr (CURV) {
-            const float rf = f32_trunc(rs);
-            g1 = 0.5f * E->k1c2.hi * E->c.hi * rf * rf * rf;
-        }
-    }
     // Horner from the last nonzero coefficient: the zero terms above it would add exact zeros
     if (S.flags & SF_EVEN) {
         int k = S.ne - 1;
@@ -354,16 +342,14 @@ __device__ __forceinline__ bool sag(const DSurface& S, const DSurfaceS* E, doubl
             pe = fma(r2, pe, S.ae[k]);
             pd = fma(r2, pd, S.aed[k]);
         }
-        z = fma(r2 * r2, pe, z);
-        g = fma(r2, pd, g);
-        if constexpr (CURV) {
-            const float u = f32_trunc(r2) * E->inv_rn2.hi;
-            k = E->ne - 1;
-            float q = E->ae2[k];
+        z = r2 * r2 * pe;
+        g = r2 * pd;
+        const float u = f32_trunc(r2) * E.inv_rn2.hi;
+        k = E.ne - 1;
+        float q = E.ae2[k];
 #pragma unroll 1
-            while (--k >= 0) q = fmaf(q, u, E->ae2[k]);
-            g1 += q;
-        }
+        while (--k >= 0) q = fmaf(q, u, E.ae2[k]);
+        g1 += q;
     }
     if (S.flags & SF_ODD) {
         const double r = sqrt64(r2);
@@ -376,38 +362,56 @@ __device__ __forceinline__ bool sag(const DSurface& S, const DSurfaceS* E, doubl
         }
         z = fma(r2 * r, po, z);
         g = fma(r, pd, g);
-        if constexpr (CURV) {
-            // with rho = r / rn the odd part of g is rho sum_k aod[k] rho^(2k) / rn^2
-            const float rho = f32_trunc(r) * E->inv_rn.hi, u = rho * rho;
-            k = E->no - 1;
-            float q = ((float)k + 0.5f) * E->aod[k].hi;
+        // with rho = r / rn the odd part of g is rho sum_k aod[k] rho^(2k) / rn^2
+        const float rho = f32_trunc(r) * E.inv_rn.hi, u = rho * rho;
+        k = E.no - 1;
+        float q = ((float)k + 0.5f) * E.aod[k].hi;
 #pragma unroll 1
-            while (--k >= 0) q = fmaf(q, u, ((float)k + 0.5f) * E->aod[k].hi);
-            if (rho > 1e-12f) g1 += q / rho * (E->inv_rn2.hi * E->inv_rn2.hi);
-        }
+        while (--k >= 0) q = fmaf(q, u, ((float)k + 0.5f) * E.aod[k].hi);
+        if (rho > 1e-12f) g1 += q / rho * (E.inv_rn2.hi * E.inv_rn2.hi);
     }
     zx = x * g;
     zy = y * g;
-    if constexpr (CURV) {
-        const float xf = f32_trunc(x), yf = f32_trunc(y), gf = f32_trunc(g);
-        H[0] = fmaf(2.f * xf * xf, g1, gf);
-        H[1] = 2.f * xf * yf * g1;
-        H[2] = fmaf(2.f * yf * yf, g1, gf);
-    }
+    const float xf = f32_trunc(x), yf = f32_trunc(y), gf = f32_trunc(g);
+    H[0] = fmaf(2.f * xf * xf, g1, gf);
+    H[1] = 2.f * xf * yf * g1;
+    H[2] = fmaf(2.f * yf * yf, g1, gf);
     if (S.flags & SF_ZERN) {
         double zz, zu, zv;
         zern_eval(S.zp, x * S.zinv, y * S.zinv, zz, zu, zv);
         z += zz;
         zx = fma(zu, S.zinv, zx);
         zy = fma(zv, S.zinv, zy);
-        if constexpr (CURV) {
-            float huu, huv, hvv;
-            zern_hess_f(E->zp, f32_trunc(x) * E->zinv, f32_trunc(y) * E->zinv, huu, huv, hvv);
-            const float k = E->zinv * E->zinv;
-            H[0] = fmaf(huu, k, H[0]); H[1] = fmaf(huv, k, H[1]); H[2] = fmaf(hvv, k, H[2]);
-        }
+        float huu, huv, hvv;
+        zern_hess_f(E.zp, xf * E.zinv, yf * E.zinv, huu, huv, hvv);
+        const float k = E.zinv * E.zinv;
+        H[0] = fmaf(huu, k, H[0]); H[1] = fmaf(huv, k, H[1]); H[2] = fmaf(hvv, k, H[2]);
     }
-    return true;
+}
+
+// Sag of the conic, even and odd terms at squared radius r2 (the pupil is sampled on the nominal first surface)
+__device__ __forceinline__ double sag(const DSurface& S, double r2) {
+    double z = 0.0;
+    if (S.flags & SF_CONIC) {
+        const double arg = fma(-S.k1c2, r2, 1.0);
+        if (negative64(arg)) return 0.0;          // outside the conic's domain
+        z = S.c * r2 * rcp64(1.0 + sqrt64(arg));
+    }
+    if (S.flags & SF_EVEN) {
+        int k = S.ne - 1;
+        double pe = S.ae[k];
+#pragma unroll 1
+        while (--k >= 0) pe = fma(r2, pe, S.ae[k]);
+        z = fma(r2 * r2, pe, z);
+    }
+    if (S.flags & SF_ODD) {
+        int k = S.no - 1;
+        double po = S.ao[k];
+#pragma unroll 1
+        while (--k >= 0) po = fma(r2, po, S.ao[k]);
+        z = fma(r2 * sqrt64(r2), po, z);
+    }
+    return z;
 }
 
 __device__ __forceinline__ void zern_eval_f(const float* __restrict__ zp, float u, float v, float& z, float& zu,
@@ -504,18 +508,17 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
 }
 
 // Intersection (Sec. 2.4.2): the paper's first guess is the root of a quadric approximating the surface; here the
-// quadric is the conic itself, and Newton's method then solves F(l) = p_z + l d_z - S(p_x + l d_x, p_y + l d_y) = 0
-// for the aspheric and Zernike terms.  Any start near the root leads to it, so the ray moves in FP64 to the plane
-// of the vertex and the start is found from there on the idle FP32 pipe: the conic's root, and for the aspheric
-// and Zernike surfaces Newton steps, which leave about 1e-4 mm.  One FP64 evaluation finishes: the Newton step
-// s = F / F' with the second-order term of Chebyshev's method, s - F'' s^2 / (2 F'), leaves an error near
-// (F'' / F')^2 s^3, and the slopes move to the root with the second derivatives H; both corrections are so small
-// that single precision carries them below the FP64 rounding of the results.  A step that is not that small is
-// taken and followed by another.  For a plain conic the same is done on the quadric, whose gradient
-// (-c x, -c y, 1 - kc z) is along the normal; for a sphere (kappa = 0) it has unit length on the surface.  A ray that
-// grazes the conic takes the FP64 root.
-// Measured (GB300, 300 stars, 2e7 photons, all FP64): 17.6 ms with the conic's FP64 root (a root and a quotient)
-// and two to three FP64 Newton steps a mirror, 10.3 ms with this start and the savings of fp64.cuh; on steep and
+// quadric is the conic itself.  With the aspheric and Zernike part a(x, y) of the sag and t = z - a the surface is
+// Q = c (x^2 + y^2) / 2 + (1 + kappa) c t^2 / 2 - t = 0, which needs no root: Newton's method on Q along the ray solves
+// it.  Any start near the root leads to it, so the ray moves in FP64 to the plane of the vertex and the start is found
+// from there on the idle FP32 pipe: the conic's root, and for the aspheric and Zernike surfaces Newton steps on the
+// sag, which leave about 1e-4 mm.  One FP64 evaluation finishes: the step s = Q / Q' with the second-order term of
+// Chebyshev's method, s + Q'' s^2 / (2 Q'), leaves an error near (Q'' / Q')^2 s^3, and the gradient of Q, which is
+// along the normal, moves to the root with its derivative; both corrections are so small that single precision
+// carries them below the FP64 rounding of the results.  A step that is not that small is taken and followed by
+// another.  For a sphere the gradient has unit length on the surface.  A ray that grazes the conic takes the FP64 root.
+// Measured (GB300, 300 stars, 2e7 photons, all FP64): 17.6 ms with the conic's FP64 root (a root and a quotient) and two
+// to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; on steep and
 // aspheric lenses the position error against the oracle fell from up to 9e-10 mm to 8e-13 mm.
 // On success h is the point and N the unit normal (along (-S_x, -S_y, 1)); ahead says whether the distance is positive.
 __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS& E, const double p[3], const double d[3],
@@ -565,57 +568,63 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
             }
         }
     }
-    double l0 = f64_exact(lf), x, y, z;
-#pragma unroll 1
-    for (;;) {
+    double x, y, z;
+    {
+        double l0 = f64_exact(lf);
         if (!started) {
             l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2]);
             if (!(fabs(l0) < 1e300)) return PHOSIM_LOST_MISSED;
         }
         x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
-        if (newton) break;
-        // half the quadric and half its slope along the ray
-        const double kz = S.kc * z;
-        const double Q = fma(0.5 * S.c, fma(x, x, y * y), z * fma(0.5, kz, -1.0));
-        const double b = fma(S.c, fma(x, d[0], y * d[1]), (kz - 1.0) * d[2]);
-        const double inv = rcp64(b), s = Q * inv;
-        const float sf = f32_trunc(s), k = A * sf * f32_trunc(inv);
-        if (started && !(fabsf(k * k * sf) < 1e-13f)) { started = false; continue; }
-        const double step = s + f64_exact(0.5f * k * sf);
-        h[0] = fma(-step, d[0], x); h[1] = fma(-step, d[1], y); h[2] = fma(-step, d[2], z);
-        N[0] = -S.c * h[0]; N[1] = -S.c * h[1]; N[2] = fma(-S.kc, h[2], 1.0);
-        if (E.kmc.hi != 0.f) {
-            const double n = rsqrt64(fma(N[0], N[0], fma(N[1], N[1], N[2] * N[2])));
-            N[0] *= n; N[1] *= n; N[2] *= n;
-        }
         ahead = lp + f32_trunc(l0) > 0.f;
-        return 0;
     }
-    ahead = lp + f32_trunc(l0) > 0.f;
+    const float c = E.c.hi, kc = E.kc.hi;
 #pragma unroll 1
     for (int it = 0; it < 20; ++it) {
-        double zs, zx, zy;
-        float H[3];
-        if (!sag<true>(S, &E, x, y, zs, zx, zy, H)) return PHOSIM_LOST_MISSED;
-        const double dF = fma(-zy, d[1], fma(-zx, d[0], d[2]));
-        if ((__double2hiint(dF) & 0x7fffffff) < 0x00100000) return PHOSIM_LOST_NEWTON;
-        const double inv = rcp64(dF), s = (z - zs) * inv;
-        const float sf = f32_trunc(s), hx = fmaf(H[0], dx, H[1] * dy), hy = fmaf(H[1], dx, H[2] * dy);
-        const float k = fmaf(hx, dx, hy * dy) * f32_trunc(inv) * sf;       // -F'' s / F'
-        // s - (k / 2) s; the terms left out are of order k^2 s
-        const float more = 0.5f * k * sf;
-        const bool last = fabsf(sf) < 1e-3f && fabsf(more * k) < 1e-14f;
-        const double step = s - f64_exact(more);
+        const double r2 = fma(x, x, y * y);
+        double a = 0.0, ax = 0.0, ay = 0.0;
+        float H[3] = {0.f, 0.f, 0.f};
+        if (newton) aspheric(S, E, x, y, r2, a, ax, ay, H);
+        const double t = newton ? z - a : z, kt = S.kc * t, u = 1.0 - kt;
+        const double Q = fma(0.5 * S.c, r2, t * fma(0.5, kt, -1.0));
+        const double tl = newton ? fma(-ay, d[1], fma(-ax, d[0], d[2])) : d[2];          // dt / dl
+        const double Ql = fma(S.c, fma(x, d[0], y * d[1]), -(u * tl));
+        if ((__double2hiint(Ql) & 0x7fffffff) < 0x00100000) return newton ? PHOSIM_LOST_NEWTON : PHOSIM_LOST_MISSED;
+        const double inv = rcp64(Ql), s = Q * inv;
+        const float sf = f32_trunc(s), invf = f32_trunc(inv), uf = f32_trunc(u), tlf = newton ? f32_trunc(tl) : dz;
+        const float hx = fmaf(H[0], dx, H[1] * dy), hy = fmaf(H[1], dx, H[2] * dy);
+        // Q'' along the ray, and the step with its second-order term
+        const float Qll = fmaf(c, fmaf(dx, dx, dy * dy), fmaf(kc * tlf, tlf, uf * fmaf(hx, dx, hy * dy)));
+        const float k = Qll * invf * sf, more = 0.5f * k * sf;
+        const bool last = (!newton || fabsf(sf) < 1e-3f) && fabsf(more * k) < 1e-14f;
+        const double step = s + f64_exact(more);
         x = fma(-step, d[0], x); y = fma(-step, d[1], y); z = fma(-step, d[2], z);
         if (last || fabsf(sf) < 1e-8f) {
-            zx -= f64_exact(sf * hx);
-            zy -= f64_exact(sf * hy);
-            const double n = rsqrt64(fma(zx, zx, fma(zy, zy, 1.0)));
-            N[0] = -zx * n; N[1] = -zy * n; N[2] = n;
             h[0] = x; h[1] = y; h[2] = z;
+            if (!newton) {
+                N[0] = -S.c * x; N[1] = -S.c * y; N[2] = fma(-S.kc, z, 1.0);
+                if (E.kmc.hi == 0.f) return 0;
+            } else {
+                // outside the conic's domain the sag has no value (decided in single precision away from its edge)
+                if (fmaf(-E.k1c2.hi, f32_trunc(r2), 1.f) < 1e-4f && fma(-S.k1c2, fma(x, x, y * y), 1.0) < 0.0)
+                    return PHOSIM_LOST_MISSED;
+                // minus the gradient of Q at the evaluated point, moved to the root: it changes by -s times its derivative
+                const float ul = -kc * tlf;
+                N[0] = fma(-S.c, x, fma(-u, ax, f64_exact(sf * fmaf(ul, f32_trunc(ax), uf * hx))));
+                N[1] = fma(-S.c, y, fma(-u, ay, f64_exact(sf * fmaf(ul, f32_trunc(ay), uf * hy))));
+                N[2] = u - f64_exact(sf * ul);
+            }
+            const double n = rsqrt64(fma(N[0], N[0], fma(N[1], N[1], N[2] * N[2])));
+            N[0] *= n; N[1] *= n; N[2] *= n;
             return 0;
         }
         if (!(fabsf(sf) < 1e37f)) return PHOSIM_LOST_NEWTON;
+        // the start was too far off (a ray that grazes the conic): the conic's FP64 root
+        if (!newton && started && it == 0) {
+            const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2]);
+            if (!(fabs(l0) < 1e300)) return PHOSIM_LOST_MISSED;
+            x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
+        }
     }
     return PHOSIM_LOST_NEWTON;
 }
@@ -709,6 +718,11 @@ __device__ __forceinline__ bool refract(double d[3], double Nx, double Ny, doubl
 
 __device__ __forceinline__ void to_surface(const DSurface& S, const double x[3], const double d[3], double p[3],
                                            double dl[3]) {
+    if (!(S.flags & (SF_ROTATED | SF_DECENTERED))) {     // a vertex on the axis: x - 0 is x
+        p[0] = x[0]; p[1] = x[1]; p[2] = x[2] - S.o[2];
+        dl[0] = d[0]; dl[1] = d[1]; dl[2] = d[2];
+        return;
+    }
     const double rx = x[0] - S.o[0], ry = x[1] - S.o[1], rz = x[2] - S.o[2];
     if (!(S.flags & SF_ROTATED)) {        // the identity rotation: the products below would be exact copies
         p[0] = rx; p[1] = ry; p[2] = rz;
@@ -724,6 +738,11 @@ __device__ __forceinline__ void to_surface(const DSurface& S, const double x[3],
 
 __device__ __forceinline__ void from_surface(const DSurface& S, const double p[3], const double dl[3], double x[3],
                                              double d[3]) {
+    if (!(S.flags & (SF_ROTATED | SF_DECENTERED))) {
+        x[0] = p[0]; x[1] = p[1]; x[2] = p[2] + S.o[2];
+        d[0] = dl[0]; d[1] = dl[1]; d[2] = dl[2];
+        return;
+    }
     if (!(S.flags & SF_ROTATED)) {
         x[0] = p[0] + S.o[0]; x[1] = p[1] + S.o[1]; x[2] = p[2] + S.o[2];
         d[0] = dl[0]; d[1] = dl[1]; d[2] = dl[2];

@@ -67,39 +67,52 @@ __device__ __forceinline__ int near_index(int i, int n) {
     return m < 0 ? m + n : m;
 }
 
-// Gradient of the phase at screen position (sx, sy), bilinear between central-difference nodes (Sec. 2.3.2)
-template <bool MIXED>
-__device__ __forceinline__ void screen_gradient(const DScale& S, double sx, double sy, double& gx, double& gy) {
-    const double fx = sx * S.inv_pix, fy = sy * S.inv_pix;
-    const int n = S.n;
-    double flx, fly;
-    int i0, j0;
-    if (floor_in_range(fx) && floor_in_range(fy)) {
-        flx = floor64(fx, i0);
-        fly = floor64(fy, j0);
-        i0 = near_index(i0, n);
-        j0 = near_index(j0, n);
+// a screen coordinate's node and the distance from it (s inv less its floor, in one rounding)
+__device__ __forceinline__ int node_of(double s, double inv, int n, double& frac) {
+    double fl;
+    int i;
+    if (floor_product64(s, inv, fl, i)) {
+        i = near_index(i, n);
     } else {
-        flx = floor(fx);
-        fly = floor(fy);
-        i0 = far_index(flx, n);
-        j0 = far_index(fly, n);
+        fl = floor(s * inv);
+        i = far_index(fl, n);
     }
+    frac = fma(s, inv, -fl);
+    return i;
+}
+
+// Gradient of the phase at screen position (sx, sy), bilinear between central-difference nodes (Sec. 2.3.2), added to
+// (gx, gy) or, for the first scale, in their place
+template <bool MIXED, bool FIRST>
+__device__ __forceinline__ void screen_gradient(const DScale& S, double sx, double sy, double& gx, double& gy) {
+    const int n = S.n;
+    double tx, ty;
+    const int i0 = node_of(sx, S.inv_pix, n, tx), j0 = node_of(sy, S.inv_pix, n, ty);
     const size_t node = (size_t)j0 * n + i0;
     if constexpr (MIXED) {
-        const float tx = f32_rn_pos(fx - flx), ty = f32_rn_pos(fy - fly);
+        const float fx = f32_rn_pos(tx), fy = f32_rn_pos(ty);
         float4 A, B;
         load_block(S.g32 + 2 * node, A, B);
-        const float w00 = (1.f - tx) * (1.f - ty), w10 = tx * (1.f - ty), w01 = (1.f - tx) * ty, w11 = tx * ty;
-        gx += f64_exact(w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z);
-        gy += f64_exact(w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w);
+        const float w00 = (1.f - fx) * (1.f - fy), w10 = fx * (1.f - fy), w01 = (1.f - fx) * fy, w11 = fx * fy;
+        const double ax = f64_exact(w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z);
+        const double ay = f64_exact(w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w);
+        gx = FIRST ? ax : gx + ax;
+        gy = FIRST ? ay : gy + ay;
     } else {
-        const double tx = fx - flx, ty = fy - fly;
         double2 a, b, c, d;
         load_block(S.g64 + 4 * node, a, b, c, d);
-        gx += fma(ty, fma(tx, d.x, c.x), fma(tx, b.x, a.x));
-        gy += fma(ty, fma(tx, d.y, c.y), fma(tx, b.y, a.y));
+        const double ax = fma(ty, fma(tx, d.x, c.x), fma(tx, b.x, a.x)), ay = fma(ty, fma(tx, d.y, c.y), fma(tx, b.y, a.y));
+        gx = FIRST ? ax : gx + ax;
+        gy = FIRST ? ay : gy + ay;
     }
+}
+
+// 1 / |n_z| = (1 - q)^(-1/2) of a unit direction, q = n_x^2 + n_y^2: within half a degree of the axis (q < 1e-4) the
+// series to q^3, which leaves 35 q^4 / 128 < 3e-17
+__device__ __forceinline__ double inverse_nz(double nx, double ny) {
+    const double q = fma(nx, nx, ny * ny);
+    if (__double2hiint(q) < 0x3f1a36e2) return fma(q, fma(q, fma(q, 0.3125, 0.375), 0.5), 1.0);
+    return rsqrt64(1.0 - q);
 }
 
 __device__ __forceinline__ double lerp_table(const double* __restrict__ t, int n, double f) {
@@ -490,8 +503,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
         }
     }
     // 1 / |n_z| = rsqrt(1 - n_x^2 - n_y^2): layer-to-layer distances are height differences times it
-    double w = fma(-nx, nx, fma(-ny, ny, 1.0));
-    double rinv = rsqrt64(w);
+    double rinv = inverse_nz(nx, ny);
     const uint4 w2 = philox(make_uint4(clo, chi, (uint32_t)src, 2u), P.k0, P.k1);
     uint4 w3 = make_uint4(0u, 0u, 0u, 0u);
     if (P.n_coated > 2) w3 = philox(make_uint4(clo, chi, (uint32_t)src, 3u), P.k0, P.k1);
@@ -504,9 +516,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
     double sp, cp;
     sincospi(2.0 * u64of(w0.y), &sp, &cp);
     double x = r * cp, y = r * sp;
-    double zs = 0.0, zx, zy;
-    sag<false>(P.pupil_surf, nullptr, x, y, zs, zx, zy, nullptr);
-    double z = P.pupil_z + zs;
+    double z = P.pupil_z + sag(P.pupil_surf, fma(x, x, y * y));
     {
         const double l = (P.h_top - z) * rinv;
         x = fma(-nx, l, x);
@@ -532,18 +542,18 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
 #pragma unroll 1
         for (int k = 0; k < P.n_layers; ++k) {
             const DLayer& L = P.layer[k];
-            const double ll = (z - L.z) * rinv;
+            const double ll = L.dz * rinv;            // the drop from the plane above
             x = fma(nx, ll, x);
             y = fma(ny, ll, y);
             z = L.z;
             const double sx = fma(-L.vx, t, x), sy = fma(-L.vy, t, y);
-            double gx = 0.0, gy = 0.0;
+            double gx, gy;
+            screen_gradient<MIXED, true>(L.s[0], sx, sy, gx, gy);
 #pragma unroll 1
-            for (int q = 0; q < L.n_scales; ++q) screen_gradient<MIXED>(L.s[q], sx, sy, gx, gy);
+            for (int q = 1; q < L.n_scales; ++q) screen_gradient<MIXED, false>(L.s[q], sx, sy, gx, gy);
             nx = fma(kick, gx, nx);
             ny = fma(kick, gy, ny);
-            w = fma(-nx, nx, fma(-ny, ny, 1.0));
-            rinv = rsqrt64(w);
+            rinv = inverse_nz(nx, ny);
         }
         // second kick (Sec. 2.3.2): a draw from the long-exposure PSF of the screens above kappa_crit,
         // scaled like the refractive kick by (lambda / lambda_ref)^(-1/5)
@@ -562,11 +572,10 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
                 nx = fma(ang, cp, nx);
                 ny = fma(ang, sp, ny);
             }
-            w = fma(-nx, nx, fma(-ny, ny, 1.0));
-            rinv = rsqrt64(w);
+            rinv = inverse_nz(nx, ny);
         }
     }
-    const double nz = -w * rinv;
+    const double nz = -fma(-nx, nx, fma(-ny, ny, 1.0)) * rinv;
     {
         const double l = (z - P.z_ent) * rinv;
         x = fma(nx, l, x);
