@@ -46,6 +46,19 @@ phosim_status upload(std::vector<void*>& owner, const T* host, size_t n, T** out
     return PHOSIM_OK;
 }
 
+// tables of 8-byte words one behind the other, for one upload
+struct TableBytes {
+    std::vector<unsigned char> bytes;
+    template <class T>
+    size_t add(const T* host, size_t n) {
+        static_assert(sizeof(T) == 8, "8-byte words");
+        const size_t at = bytes.size();
+        const unsigned char* p = reinterpret_cast<const unsigned char*>(host);
+        bytes.insert(bytes.end(), p, p + n * sizeof(T));
+        return at;
+    }
+};
+
 bool is_finite(double v) { return std::isfinite(v); }
 
 // device counter words of a scene: [0] tile counter, [1 .. kNumCounters] launch counters, then the state
@@ -107,6 +120,24 @@ void zernike_monomials(int j, double P[7][7]) {
         }
 }
 
+// the monomials of every term, row by row in the power of y as the kernels read them, made once
+struct ZernikeTable {
+    double m[PHOSIM_MAX_ZERNIKE][kZPoly];
+    ZernikeTable() {
+        for (int j = 1; j <= PHOSIM_MAX_ZERNIKE; ++j) {
+            double P[7][7];
+            zernike_monomials(j, P);
+            int off = 0;
+            for (int b = 0; b < 7; ++b)
+                for (int a = 0; a + b < 7; ++a) m[j - 1][off++] = P[b][a];
+        }
+    }
+};
+const ZernikeTable& zernike_table() {
+    static const ZernikeTable table;
+    return table;
+}
+
 // R = Rz(tz) Ry(ty) Rx(tx) takes surface-frame directions to the telescope frame; M = R^T
 void rotation(const double* pert, double M[9]) {
     const double cx = std::cos(pert[3]), sx = std::sin(pert[3]);
@@ -166,21 +197,14 @@ phosim_status build_surface(const phosim_surface& s, DSurface& d) {
     }
     if (s.zern_rnorm > 0.0) d.zinv = 1.0 / s.zern_rnorm;
     if (s.n_zern > 0 && s.zern_rnorm > 0.0) {
-        double P[7][7] = {}, Pj[7][7];
+        const ZernikeTable& table = zernike_table();
         bool any = false;
         for (int j = 1; j <= s.n_zern; ++j) {
             if (s.zern[j - 1] == 0.0) continue;
             any = true;
-            zernike_monomials(j, Pj);
-            for (int b = 0; b < 7; ++b)
-                for (int a = 0; a + b < 7; ++a) P[b][a] += s.zern[j - 1] * Pj[b][a];
+            for (int k = 0; k < kZPoly; ++k) d.zp[k] += s.zern[j - 1] * table.m[j - 1][k];
         }
-        if (any) {
-            flags |= SF_ZERN;
-            int off = 0;
-            for (int b = 0; b < 7; ++b)
-                for (int a = 0; a + b < 7; ++a) d.zp[off++] = P[b][a];
-        }
+        if (any) flags |= SF_ZERN;
     }
     if (!(flags & (SF_CONIC | SF_EVEN | SF_ODD | SF_ZERN))) flags |= SF_FLAT_ONLY;
     if (s.pert[3] != 0.0 || s.pert[4] != 0.0 || s.pert[5] != 0.0) flags |= SF_ROTATED;
@@ -638,11 +662,11 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
         }
     }
     std::vector<void*> mem;
+    TableBytes tables;
+    std::vector<std::array<size_t, 6>> table_at((size_t)n_coat);           // where each coating's tables are among them
     std::vector<std::vector<unsigned long long>> most((size_t)n_coat);     // each coating's accept thresholds, largest over angles
     bool ghosts = false;
     for (int k = 0; k < n_coat; ++k) {
-        double *d, *dmax;
-        unsigned long long *dthr, *dmax_thr;
         const int nl = coats[k].n_lambda, nt = coats[k].n_theta;
         // the dynamic transmission test (early rejection) keeps a photon while it can still be transmitted or,
         // with a reflection table, reflected: its bound is the largest T + R over angles
@@ -656,28 +680,16 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
         for (size_t i = 0; i < tr.size(); ++i) tr_thr[i] = accept_threshold(tr[i]);
         for (int il = 0; il < nl; ++il) tmax_thr[il] = accept_threshold(tmax[il]);
         most[(size_t)k] = tmax_thr;
-        double* dtr = nullptr;
-        unsigned long long* dtr_thr = nullptr;
-        phosim_status st = upload(mem, coats[k].table, (size_t)nl * nt, &d);
-        if (st == PHOSIM_OK) st = upload(mem, tmax.data(), tmax.size(), &dmax);
-        if (st == PHOSIM_OK) st = upload(mem, thr.data(), thr.size(), &dthr);
-        if (st == PHOSIM_OK) st = upload(mem, tmax_thr.data(), tmax_thr.size(), &dmax_thr);
-        if (st == PHOSIM_OK && R) st = upload(mem, tr.data(), tr.size(), &dtr);
-        if (st == PHOSIM_OK && R) st = upload(mem, tr_thr.data(), tr_thr.size(), &dtr_thr);
-        if (st != PHOSIM_OK) { free_all(mem); return st; }
+        table_at[(size_t)k] = {tables.add(coats[k].table, (size_t)nl * nt), tables.add(tmax.data(), tmax.size()),
+                               tables.add(thr.data(), thr.size()), tables.add(tmax_thr.data(), tmax_thr.size()),
+                               R ? tables.add(tr.data(), tr.size()) : 0, R ? tables.add(tr_thr.data(), tr_thr.size()) : 0};
         if (R) ghosts = true;
         DCoating& C = P.coat[k];
         C.lam0 = coats[k].lam0; C.inv_dlam = 1.0 / coats[k].dlam;
         C.th0 = coats[k].theta0; C.inv_dth = 1.0 / coats[k].dtheta;
         C.lam0f = (float)C.lam0; C.inv_dlamf = (float)C.inv_dlam; C.th0f = (float)C.th0; C.inv_dthf = (float)C.inv_dth;
         C.lam0_s = ds_of(C.lam0); C.inv_dlam_s = ds_of(C.inv_dlam);
-        C.T_thr = dthr;
-        C.Tmax_thr = dmax_thr;
-        C.TR = dtr;
-        C.TR_thr = dtr_thr;
         C.nl = coats[k].n_lambda; C.nt = coats[k].n_theta;
-        C.T = d;
-        C.Tmax = dmax;
     }
     P.n_coat = n_coat;
     P.flags = ghosts ? (P.flags | kGhostFlag) : (P.flags & ~kGhostFlag);
@@ -704,20 +716,22 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
             if (surf[i].kind != PHOSIM_MIRROR) m = surf[i].material;
         }
     }
-    {
-        std::vector<double> zm((size_t)PHOSIM_MAX_ZERNIKE * kZPoly, 0.0);
-        for (int j = 1; j <= PHOSIM_MAX_ZERNIKE; ++j) {
-            double Pj[7][7];
-            zernike_monomials(j, Pj);
-            int off = 0;
-            for (int b = 0; b < 7; ++b)
-                for (int a = 0; a + b < 7; ++a) zm[(size_t)(j - 1) * kZPoly + off++] = Pj[b][a];
-        }
-        double* dz;
-        phosim_status st = upload(mem, zm.data(), zm.size(), &dz);
-        if (st != PHOSIM_OK) { free_all(mem); return st; }
-        sc->d_zmono = dz;
+    tables.add(&zernike_table().m[0][0], (size_t)PHOSIM_MAX_ZERNIKE * kZPoly);
+    // one allocation and one copy for all of the tables
+    unsigned char* base = nullptr;
+    phosim_status ts = upload(mem, tables.bytes.data(), tables.bytes.size(), &base);
+    if (ts != PHOSIM_OK) { free_all(mem); return ts; }
+    for (int k = 0; k < n_coat; ++k) {
+        DCoating& C = P.coat[k];
+        const std::array<size_t, 6>& at = table_at[(size_t)k];
+        C.T = (const double*)(base + at[0]);
+        C.Tmax = (const double*)(base + at[1]);
+        C.T_thr = (const unsigned long long*)(base + at[2]);
+        C.Tmax_thr = (const unsigned long long*)(base + at[3]);
+        C.TR = coats[k].reflect ? (const double*)(base + at[4]) : nullptr;
+        C.TR_thr = coats[k].reflect ? (const unsigned long long*)(base + at[5]) : nullptr;
     }
+    sc->d_zmono = (double*)(base + tables.bytes.size() - sizeof(double) * PHOSIM_MAX_ZERNIKE * kZPoly);
     free_all(sc->optics_mem);
     sc->optics_mem = mem;
     sc->base = P;
@@ -1395,12 +1409,13 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
                     if (ghosts) CU(cudaMemsetAsync(sc->d_rounds, 0, kGhostRounds * sizeof(GhostRound), st));
                 }
                 ls = timed(2, [&] { return launch_ds_entry(P, S, blocks, sc->threads, st, beside && t0 == 0); });
-                if (ls == PHOSIM_OK) ls = timed(3, [&] { return launch_ds_optics(P, S, walk, blocks_optics, sc->threads, st); });
+                if (ls == PHOSIM_OK)
+                    ls = timed(3, [&] { return launch_ds_optics(P, S, walk, blocks_optics, sc->threads, st, beside); });
                 for (int r = 0; ls == PHOSIM_OK && r < n_rounds; ++r)
                     ls = timed(3, [&] {
                         S.round = r;
                         const cudaError_t e = launch_ghost_order(S, blocks_optics, st);
-                        return e != cudaSuccess ? e : launch_ds_optics(P, S, kWalkGhosts, blocks_optics, sc->threads, st);
+                        return e != cudaSuccess ? e : launch_ds_optics(P, S, kWalkGhosts, blocks_optics, sc->threads, st, false);
                     });
                 if (ls == PHOSIM_OK && bundles)
                     ls = timed(4, [&] { return launch_ds_members(P, S, blocks_members, sc->threads, st); });

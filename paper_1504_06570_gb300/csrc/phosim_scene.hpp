@@ -111,7 +111,22 @@ constexpr int kChiefThreads = 32;
 size_t source_s_bytes();                       // sizeof(SourceS), which the host code does not see
 // the two-kernel double-single path (PHOSIM_MIXED_DS in phosim_trace)
 cudaError_t launch_ds_entry(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st, bool beside);
-cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st);
+cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st, bool beside);
+// a launch that starts beside the kernel before it on the stream as soon as that one lets it or ends; what the kernel
+// reads of the one before must follow its own wait_for_previous
+template <class... Params, class... Args>
+cudaError_t launch_beside(void (*kernel)(Params...), int blocks, int threads, cudaStream_t st, const Args&... args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config = {};
+    config.gridDim = dim3((unsigned)blocks);
+    config.blockDim = dim3((unsigned)threads);
+    config.stream = st;
+    config.attrs = &attr;
+    config.numAttrs = 1;
+    return cudaLaunchKernelEx(&config, kernel, args...);
+}
 cudaError_t launch_ds_members(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
 const void* ds_members_kernel_ptr();
 cudaError_t ds_stage_occupancy(int threads, int* entry_per_sm, int* optics_per_sm, int* members_per_sm);

@@ -596,9 +596,11 @@ __global__ void call_prep_kernel(const __grid_constant__ CallPrep C) {
     for (int k = 0; k < 3; ++k)
         for (unsigned long long i = t; i < C.zero_words[k]; i += step) C.zero[k][i] = 0u;
     if (C.n_inline && t <= (unsigned)C.n_inline) C.tile_prefix[t] = C.inline_prefix[t];
+    const bool all = C.pass_lo == -1e300 && C.pass_hi == 1e300;
     for (unsigned long long s = t; s < (unsigned)C.n_src; s += step) {
         DSource S = C.n_inline ? C.inline_sources[s] : C.sources[s];
-        pass_draws(C, S, S.w_lo, S.w_span);
+        if (all) { S.w_lo = 0u; S.w_span = 0xffffffffu; }
+        else pass_draws(C, S, S.w_lo, S.w_span);
         C.sources[s] = S;
         if (C.sources_s) C.sources_s[s] = source_s(S);
     }
@@ -646,21 +648,6 @@ cudaError_t launch_chief_rays(const TraceParams& P, DSource* sources, int n_src,
     if (n_src <= 0) return cudaSuccess;
     chief_ray_kernel<<<(n_src + kChiefThreads - 1) / kChiefThreads, kChiefThreads, 0, st>>>(P, sources, n_src, moments);
     return cudaGetLastError();
-}
-
-// a launch that starts beside the kernel before it on the stream, as soon as that one lets it
-template <class... Params, class... Args>
-static cudaError_t launch_beside(void (*kernel)(Params...), int blocks, int threads, cudaStream_t st, const Args&... args) {
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t config = {};
-    config.gridDim = dim3((unsigned)blocks);
-    config.blockDim = dim3((unsigned)threads);
-    config.stream = st;
-    config.attrs = &attr;
-    config.numAttrs = 1;
-    return cudaLaunchKernelEx(&config, kernel, args...);
 }
 
 cudaError_t launch_trace(const TraceParams& P, int mode, int blocks, int threads, cudaStream_t st, bool beside) {

@@ -154,16 +154,15 @@ __global__ void __launch_bounds__(kOpticsMaxThreads, PHOSIM_DS_OPTICS_MIN_BLOCKS
     unsigned long long* cnt = cnt_mem[warp];
     if (lane < kNumCounters) cnt[lane] = 0;
     __syncwarp();
+    // launched beside the entry stage's end (a short call waits for launches, not for work)
+    wait_for_previous();
     const unsigned long long n = KIND == kWalkGhosts ? S.rounds[S.round].n : *S.n_state;
     unsigned long long* const batch = KIND == kWalkGhosts ? &S.rounds[S.round].batch : S.batch;
     // a block's states at a time, all its warps meeting the surfaces together (a barrier after each), so
     // that the SM's warps fetch the same stretch of code rather than as many stretches as warps; the
     // blocks claim batches as they finish (a block is as slow as its slowest ray at every surface)
-    for (;;) {
-        if (threadIdx.x == 0) next_batch = atomicAdd(batch, 1ull) * blockDim.x;
-        __syncthreads();
-        const unsigned long long b0 = next_batch;
-        if (b0 >= n) break;
+    // (the first batch is the block's own)
+    for (unsigned long long b0 = (unsigned long long)blockIdx.x * blockDim.x; b0 < n;) {
         const unsigned long long e = b0 + threadIdx.x;
         const bool v = e < n;
         PhotonOutS R;
@@ -241,6 +240,10 @@ __global__ void __launch_bounds__(kOpticsMaxThreads, PHOSIM_DS_OPTICS_MIN_BLOCKS
         const bool ended = v && !handed && !parked;
         const uint32_t n_loop = __reduce_max_sync(0xffffffffu, ended ? nm : 0u);
         for (uint32_t m = 0; m < n_loop; ++m) account_ds(P, R, ended && m < nm, src, lo + m, lane, cnt);
+        if ((unsigned long long)gridDim.x * blockDim.x >= n) break;
+        if (threadIdx.x == 0) next_batch = (gridDim.x + atomicAdd(batch, 1ull)) * blockDim.x;
+        __syncthreads();
+        b0 = next_batch;
     }
     __syncwarp();
     if (lane < kNumCounters && cnt[lane]) atomicAdd(P.counters + lane, cnt[lane]);
@@ -334,8 +337,10 @@ cudaError_t launch_moment_stripes(const TraceParams& P, cudaStream_t st) {
 
 int ds_optics_threads(int threads) { return PHOSIM_DS_OPTICS_THREADS ? PHOSIM_DS_OPTICS_THREADS : threads; }
 
-cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st) {
+cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st, bool beside) {
     const int block = ds_optics_threads(threads);
+    if (beside && kind == kWalkPlain) return launch_beside(ds_optics_kernel<kWalkPlain>, blocks, block, st, P, S);
+    if (beside && kind == kWalkForward) return launch_beside(ds_optics_kernel<kWalkForward>, blocks, block, st, P, S);
     if (kind == kWalkGhosts) ds_optics_kernel<kWalkGhosts><<<blocks, block, 0, st>>>(P, S);
     else if (kind == kWalkForward) ds_optics_kernel<kWalkForward><<<blocks, block, 0, st>>>(P, S);
     else ds_optics_kernel<kWalkPlain><<<blocks, block, 0, st>>>(P, S);

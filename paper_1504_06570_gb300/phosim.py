@@ -7,6 +7,7 @@ raises on error codes.  There is no CPU fallback: if the library is missing, imp
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -118,6 +119,12 @@ def lib():
         L.phosim_status_string.restype = C.c_char_p
         _lib = L
     return _lib
+
+
+@functools.lru_cache(maxsize=1)
+def _has_cuda():
+    import torch
+    return torch.cuda.is_available()
 
 
 def _check(where, code):
@@ -241,6 +248,7 @@ class Scene:
         self.sources = sources
         self.src = sources_struct(sources)
         self.n_photons = np.ascontiguousarray(sources.n_photons, np.uint64)
+        self._n_photons_ptr = self.n_photons.ctypes.data_as(C.POINTER(C.c_uint64))
 
     def set_schedule(self, threads=0, tile=0):
         _check("phosim_set_schedule", self.L.phosim_set_schedule(self.h, int(threads), int(tile)))
@@ -249,16 +257,22 @@ class Scene:
         """phosim_trace on torch tensors (image: int32 (ny, nx) on the device or on the host; records: uint8
         tensor of 48-byte records; moments: float64 (n_src, 8)).  Photon counts default to the sources'."""
         import torch
-        n = len(self.sources)
-        cnt = self.n_photons if n_photons is None else np.ascontiguousarray(n_photons, np.uint64)
-        fst = None if first is None else np.ascontiguousarray(first, np.uint64)
-        if stream is None:
-            stream = torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
         u64p = C.POINTER(C.c_uint64)
-        _check("phosim_trace", self.L.phosim_trace(
-            self.h, self.src, n, cnt.ctypes.data_as(u64p), None if fst is None else fst.ctypes.data_as(u64p),
-            C.c_void_p(image.data_ptr()), None if records is None else C.c_void_p(records.data_ptr()),
-            None if moments is None else C.c_void_p(moments.data_ptr()), C.c_void_p(stream) if stream else None))
+        if n_photons is None:
+            counts = self._n_photons_ptr
+        else:
+            n_photons = np.ascontiguousarray(n_photons, np.uint64)
+            counts = n_photons.ctypes.data_as(u64p)
+        fst = None
+        if first is not None:
+            first = np.ascontiguousarray(first, np.uint64)
+            fst = first.ctypes.data_as(u64p)
+        if stream is None:
+            stream = torch.cuda.current_stream().cuda_stream if _has_cuda() else None
+        code = self.L.phosim_trace(self.h, self.src, len(self.sources), counts, fst, image.data_ptr(),
+                                   None if records is None else records.data_ptr(),
+                                   None if moments is None else moments.data_ptr(), stream or None)
+        _check("phosim_trace", code)
 
     def grad(self, dL_dmoments, params, n_photons=None, stream=None):
         """phosim_grad: per-source gradients of sum_k dL[s, k] M_s[k], M = (mean x, mean y, Ixx, Ixy, Iyy),
@@ -362,6 +376,7 @@ def derived_moments(m):
     return out
 
 
+@functools.lru_cache(maxsize=1)
 def _autograd_function():
     import torch
 
