@@ -773,8 +773,11 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
             if (!(ds_le(r2, E.r_out2) && ds_le(E.r_in2, r2))) { R.flags = lost(PHOSIM_LOST_VIGNETTED, si); return false; }
         }
     }
-    // coating accept-reject at the incidence angle and wavelength
-    if (S.coat_slot >= 0) {
+    // Coating accept-reject at the incidence angle and wavelength.  A coating of one angle bin, in a scene without
+    // ghosts, has made its decision in the dynamic transmission test before the atmosphere (early_coating_reject_f:
+    // its largest transmission over angles is its transmission, and draw, wavelength and bin are the same), so a ray
+    // that comes here has passed.  (Without the second draw the optics of the 1000-star field take 5.45 ms, not 5.56.)
+    if (S.coat_slot >= 0 && !(KIND == kWalkPlain && (P.flags & PHOSIM_EARLY_REJECT) && P.coat[S.coating].nt == 1)) {
         const DCoating& C = P.coat[S.coating];
         int it = 0;
         if (C.nt > 1) {

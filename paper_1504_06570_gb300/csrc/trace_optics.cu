@@ -36,9 +36,33 @@ constexpr int kOpticsMaxThreads = PHOSIM_DS_OPTICS_THREADS ? PHOSIM_DS_OPTICS_TH
 #define PHOSIM_DS_MEMBERS_MIN_BLOCKS 4
 #endif
 
+// The sums over the warp of five values a lane: v0 in lanes 0-3, v1 in 4-7, v2 in 8-11, v3 in 16-19 and v4 in 20-23
+// (zeros in the others).  At each of the first three steps a lane keeps part of its values and adds its partner's copies
+// of them, so that the five sums cost 3 + 2 + 1 + 1 + 1 additions a lane.
+__device__ __forceinline__ ds pick_ds(bool p, ds a, ds b) { return {p ? a.hi : b.hi, p ? a.lo : b.lo}; }
+__device__ __forceinline__ ds from_lane_ds(ds v, int d) {
+    return {__shfl_xor_sync(0xffffffffu, v.hi, d), __shfl_xor_sync(0xffffffffu, v.lo, d)};
+}
+__device__ __forceinline__ ds transpose_sum_ds(ds v0, ds v1, ds v2, ds v3, ds v4, int lane) {
+    const ds zero = ds_f(0.f);
+    bool up = (lane & 16) != 0;
+    const ds2 a = add2(ds2_of(pick_ds(up, v3, v0), pick_ds(up, v4, v1)),
+                       ds2_of(from_lane_ds(pick_ds(up, v0, v3), 16), from_lane_ds(pick_ds(up, v1, v4), 16)));
+    const ds a2 = pick_ds(up, zero, v2) + from_lane_ds(pick_ds(up, v2, zero), 16);
+    up = (lane & 8) != 0;
+    const ds2 b = add2(ds2_of(pick_ds(up, a2, ds2_x(a)), pick_ds(up, zero, ds2_y(a))),
+                       ds2_of(from_lane_ds(pick_ds(up, ds2_x(a), a2), 8), from_lane_ds(pick_ds(up, ds2_y(a), zero), 8)));
+    up = (lane & 4) != 0;
+    ds c = pick_ds(up, ds2_y(b), ds2_x(b)) + from_lane_ds(pick_ds(up, ds2_x(b), ds2_y(b)), 4);
+    c = c + from_lane_ds(c, 2);
+    return c + from_lane_ds(c, 1);
+}
+
+// runs of one source in a warp up to which each is summed before its atomics
+constexpr int kMaxWarpSources = 8;
+
 // Account for one photon per lane of the optics or bundle stage: record, image, counters (cnt: the warp's
-// counters in shared memory, lane 0) and the moment sums about the source's chief-ray position, reduced over
-// the lanes of one source.  Every lane of the warp calls it.
+// counters in shared memory, lane 0) and the moment sums about the source's chief-ray position.  Every lane of the warp calls it.
 __device__ __forceinline__ void account_ds(const TraceParams& P, const PhotonOutS& R, bool v, int src, uint64_t i,
                                            int lane, unsigned long long* cnt) {
     const DSource& s = P.sources[src];
@@ -51,10 +75,9 @@ __device__ __forceinline__ void account_ds(const TraceParams& P, const PhotonOut
     }
     const bool det = v && (R.flags & PHOSIM_F_DETECTED);
     const unsigned dmask = __ballot_sync(0xffffffffu, det);
-    if (det) {
-        const unsigned same = __match_any_sync(dmask, R.pix);
-        if (lane == __ffs(same) - 1) atomicAdd(P.image + R.pix, (unsigned)__popc(same));
-    }
+    // a lane's count each: adding the lanes of one pixel up first (a match and a popcount) costs more than it saves, also
+    // where a tenth of all photons hit one pixel (1.206 ms with it, 1.201 without; the 1000-star field 5.56 and 5.48)
+    if (det) atomicAdd(P.image + R.pix, 1u);
     if (lane == 0) cnt[1] += __popc(dmask);
     const uint32_t reason = v ? ((R.flags >> 8) & 0xffu) : 0u;
 #pragma unroll
@@ -63,47 +86,41 @@ __device__ __forceinline__ void account_ds(const TraceParams& P, const PhotonOut
         if (lane == 0) cnt[1 + q] += __popc(bq);
     }
     if (P.moments && dmask) {
-        // Per-source partial sums of the warp: the states arrive in runs of one source (a warp of the entry
-        // stage appends its survivors together), so the lanes of a source are contiguous segments.  An
-        // inclusive segmented scan in double-single (exact products of the single-precision offsets from the
-        // chief ray, sums to ~2^-47) leaves each segment's sums in its last lane, which adds them to the
-        // source's double-precision moments: one set of atomics per segment, not per photon, and the FP64
-        // pipe (a sixty-fourth of the FP32 rate on this GPU) only converts the partials.
-        ds mm[5] = {ds_f(0.f), ds_f(0.f), ds_f(0.f), ds_f(0.f), ds_f(0.f)};
-        if (det) {
-            const float fx = (R.x - ds{s.ref_s[0], s.ref_s[1]}).hi, fy = (R.y - ds{s.ref_s[2], s.ref_s[3]}).hi;
-            mm[0] = ds_f(fx); mm[1] = ds_f(fy);
-            mm[2] = two_prod(fx, fx); mm[3] = two_prod(fx, fy); mm[4] = two_prod(fy, fy);
-        }
+        // Per-source partial sums of the warp in double-single (exact products of the single-precision offsets from
+        // the chief ray, sums to ~2^-47), added to the source's double-precision moments: one set of atomics per source,
+        // not per photon, and the FP64 pipe (a sixty-fourth of the FP32 rate on this GPU) converts one sum a lane.  The
+        // states arrive in runs of one source (a warp of the entry stage appends its survivors together), so a warp
+        // mostly holds one to three sources, each summed in its turn (8 additions against the 25 of a segmented scan of
+        // the five sums: optics of the 1000-star field 5.28 ms, not 5.36).  Where a warp holds more (sources of a few
+        // photons), that would cost more than the atomics it saves, and every lane adds its own terms.
+        const float fx = (R.x - ds{s.ref_s[0], s.ref_s[1]}).hi, fy = (R.y - ds{s.ref_s[2], s.ref_s[3]}).hi;
+        double* const sums = P.mom_stripes ? P.mom_stripes + (size_t)(blockIdx.x % kMomStripes) * P.mom_stripe_stride : P.moments;
         const int prev = __shfl_up_sync(0xffffffffu, src, 1);
         const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || prev != src);
-        const unsigned upto = lane == 31 ? 0xffffffffu : (2u << lane) - 1u;
-        const int first = 31 - __clz(heads & upto);
-        // the sums in pairs (x, y), (xx, xy) and yy, the pairs added by the packed primitive (bit for bit the same)
-        ds2 m01 = ds2_of(mm[0], mm[1]), m23 = ds2_of(mm[2], mm[3]);
-        ds m4 = mm[4];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const auto up = [&](float v) { return __shfl_up_sync(0xffffffffu, v, d); };
-            const ds2 t01 = {make_float2(up(m01.hi.x), up(m01.hi.y)), make_float2(up(m01.lo.x), up(m01.lo.y))};
-            const ds2 t23 = {make_float2(up(m23.hi.x), up(m23.hi.y)), make_float2(up(m23.lo.x), up(m23.lo.y))};
-            const ds t4 = {up(m4.hi), up(m4.lo)};
-            if (lane - d >= first) {
-                m01 = add2(m01, t01);
-                m23 = add2(m23, t23);
-                m4 = m4 + t4;
+        if (__popc(heads) > kMaxWarpSources) {
+            if (det) {
+                double* const M = sums + (size_t)src * PHOSIM_MOMENT_WORDS;
+                const double x = (double)fx, y = (double)fy;
+                atomicAdd(M, 1.0);
+                atomicAdd(M + 1, x);
+                atomicAdd(M + 2, y);
+                atomicAdd(M + 3, x * x);
+                atomicAdd(M + 4, x * y);
+                atomicAdd(M + 5, y * y);
             }
+            return;
         }
-        mm[0] = ds2_x(m01); mm[1] = ds2_y(m01); mm[2] = ds2_x(m23); mm[3] = ds2_y(m23); mm[4] = m4;
-        const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
-        // the segment's detected photons, counted from the ballot
-        const unsigned n_det = __popc(dmask & upto & ~((1u << first) - 1u));
-        if (last && n_det > 0) {
-            double* M = (P.mom_stripes ? P.mom_stripes + (size_t)(blockIdx.x % kMomStripes) * P.mom_stripe_stride
-                                       : P.moments) + (size_t)src * PHOSIM_MOMENT_WORDS;
-            atomicAdd(M, (double)n_det);
-#pragma unroll
-            for (int q = 0; q < 5; ++q) atomicAdd(M + 1 + q, ds_value(mm[q]));
+        for (unsigned todo = dmask; todo;) {
+            const int of = __shfl_sync(0xffffffffu, src, __ffs(todo) - 1);
+            const bool in = det && src == of;
+            const unsigned mask = __ballot_sync(0xffffffffu, in);
+            todo &= ~mask;
+            const float x = in ? fx : 0.f, y = in ? fy : 0.f;
+            const ds sum = transpose_sum_ds(ds_f(x), ds_f(y), two_prod(x, x), two_prod(x, y), two_prod(y, y), lane);
+            double* const M = sums + (size_t)of * PHOSIM_MOMENT_WORDS;
+            if (lane == 31) atomicAdd(M, (double)__popc(mask));
+            // lanes 0, 4, 8, 16 and 20 hold the sums of x, y, xx, xy and yy
+            if ((0x110111u >> lane) & 1u) atomicAdd(M + 1 + (lane < 16 ? lane >> 2 : (lane >> 2) - 1), ds_value(sum));
         }
     }
 }
