@@ -138,6 +138,17 @@ __device__ __forceinline__ ds2 dfma2(ds a, ds2 b, ds2 c) {
     e = __fadd2_rn(e, __fadd2_rn(s.lo, c.lo));
     return fast_two_sum2(s.hi, e);
 }
+// dfma(a, b, c) in each half, b shared
+__device__ __forceinline__ ds2 dfma2(ds2 a, ds b, ds2 c) {
+    const float2 bh = make_float2(b.hi, b.hi), bl = make_float2(b.lo, b.lo);
+    const float2 p = __fmul2_rn(a.hi, bh);
+    float2 e = __ffma2_rn(a.hi, bh, f2_neg(p));
+    const ds2 s = two_sum2(p, c.hi);
+    e = __ffma2_rn(a.hi, bl, e);
+    e = __ffma2_rn(a.lo, bh, e);
+    e = __fadd2_rn(e, __fadd2_rn(s.lo, c.lo));
+    return fast_two_sum2(s.hi, e);
+}
 // a * b in each half with a shared (the scalar operator*(a, b))
 __device__ __forceinline__ ds2 mul2(ds a, ds2 b) {
     const float2 ah = make_float2(a.hi, a.hi), al = make_float2(a.lo, a.lo);

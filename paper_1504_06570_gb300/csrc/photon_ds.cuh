@@ -946,14 +946,14 @@ __device__ __forceinline__ bool photon_entry_ds(const TraceParams& P, const Sour
     // frozen-flow layers top to bottom (Sec. 2.3)
     if (P.flags & PHOSIM_ATMOSPHERE) {
         const float kick = P.kick0f * exp2f(-0.2f * log2f(lam * P.inv_lam_ref_f));
-        // x and y as packed pairs (ds2)
+        // x and y as packed pairs (ds2), in the operations and the order of the scalar expressions: a position another
+        // rounding away would move a photon in some 1e9 to the next pixel
         ds2 X2 = ds2_of(x, y), N2 = ds2_of(nx, ny);
-        const ds minus_t = -t;
 #pragma unroll 1
         for (int k = 0; k < P.n_layers; ++k) {
             const DLayer& L = P.layer[k];
-            X2 = dfma2(L.dzs * rinv, N2, X2);     // the drop from the plane above, z_above - z_k
-            const ds2 at = dfma2(minus_t, ds2_of(L.vxs, L.vys), X2);
+            X2 = dfma2(N2, L.dzs * rinv, X2);     // the drop from the plane above, z_above - z_k
+            const ds2 at = add2(X2, neg2(mul2(ds2_of(L.vxs, L.vys), t)));
             float gx = 0.f, gy = 0.f;
 #pragma unroll 1
             for (int q = 0; q < L.n_scales; ++q) screen_gradient_ds(L.s[q], at, gx, gy);
