@@ -72,7 +72,7 @@ struct phosim_scene {
     TraceGraph graphs[3];
     cudaStream_t capture_stream = nullptr;
     // resident blocks an SM of the trace's kernels for a block size (asked of the driver once)
-    struct { int mode = -1, threads = 0, trace = 0, optics = 0, members = 0, listed = 0; } occupancy;
+    struct { int mode = -1, threads = 0, walk = 0, trace = 0, optics = 0, members = 0, listed = 0; } occupancy;
     // the last FP64 call's photon batches: whether they are all there (one chunk), for the adjoint that follows it
     phosim::PhotonBatch* d_batches = nullptr;
     size_t cap_batches = 0;
@@ -129,9 +129,9 @@ cudaError_t launch_beside(void (*kernel)(Params...), int blocks, int threads, cu
 }
 cudaError_t launch_ds_members(const TraceParams& P, const DSStage& S, int blocks, int threads, cudaStream_t st);
 const void* ds_members_kernel_ptr();
-cudaError_t ds_stage_occupancy(int threads, int* entry_per_sm, int* optics_per_sm, int* members_per_sm);
+cudaError_t ds_stage_occupancy(int kind, int threads, int* entry_per_sm, int* optics_per_sm, int* members_per_sm);
 const void* ds_entry_kernel_ptr();
-// kind of walk (WalkKind): 0 no reflecting coating, 1 forward with ghosts leaving, 2 a round of ghosts
+// kind of walk (WalkKind): 0 no reflecting coating, 1 forward with ghosts leaving, 2 a round of ghosts, 3 as 0 for simple surfaces
 const void* ds_optics_kernel_ptr(int kind);
 const void* ghost_order_kernel_ptr();
 cudaError_t launch_ghost_order(const DSStage& S, int blocks, cudaStream_t st);

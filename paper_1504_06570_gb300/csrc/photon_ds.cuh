@@ -307,6 +307,24 @@ __device__ __forceinline__ void ray_point_ds(ds l, const ds p[3], const ds d[3],
     out[2] = dfma(l, d[2], p[2]);
 }
 
+// the conic's root in double-single, kNoRoot where the ray misses it.  Out of line: few rays take it, and inline its
+// registers and its place among the instructions would cost every ray
+constexpr float kNoRoot = 3e38f;
+static __device__ __noinline__ ds conic_root_ds(const DSurfaceS& E, ds px, ds py, ds pz, ds dx, ds dy, ds dz) {
+    // the quadric's l^2 coefficient c (d_x^2 + d_y^2) + kc d_z^2, which for the unit direction is c + (kc - c) d_z^2
+    const ds A = dfma(E.kmc * dz, dz, E.c);
+    const ds b = dfma(E.kc * pz, dz, E.c * dfma(px, dx, py * dy)) - dz;
+    const ds C = dfma(E.kc * pz, pz, E.c * dfma(px, px, py * py)) - pz * 2.f;
+    const ds disc = dfma(b, b, -(A * C));
+    if (disc.hi < 0.f) return ds_f(kNoRoot);
+    const ds sq = ds_sqrt(disc);
+    const ds q = b.hi >= 0.f ? -(b + sq) : sq - b;
+    if (q.hi == 0.f) return ds_f(kNoRoot);
+    ds l = C / q;
+    if (A.hi != 0.f && (ds_f(1.f) - E.kc * dfma(l, dz, pz)).hi < 0.f) l = q / A;
+    return l;
+}
+
 // Intersection (Sec. 2.4.2), the steps of intersect() in phosim_device.cuh: the conic's exact root on the
 // vertex branch, then Newton's method for the aspheric and Zernike terms until the step is below 1e-8 mm.
 // Newton converges to the same root from any start close enough to it, so the start is computed in single
@@ -327,7 +345,8 @@ static __device__ PHOSIM_DS_STEP uint32_t intersect_ds(const DSurfaceS& E, int f
         return 0;
     }
     const bool newton = (flags & (SF_EVEN | SF_ODD | SF_ZERN)) != 0;
-    if (newton) {
+    bool started = false;
+    {
         const float c = E.c.hi, kc = E.kc.hi;
         const float Af = fmaf(E.kmc.hi * d[2].hi, d[2].hi, c);
         const float bf = fmaf(kc * p[2].hi, d[2].hi, c * fmaf(p[0].hi, d[0].hi, p[1].hi * d[1].hi)) - d[2].hi;
@@ -338,60 +357,36 @@ static __device__ PHOSIM_DS_STEP uint32_t intersect_ds(const DSurfaceS& E, int f
             const float qf = bf >= 0.f ? -(bf + sq) : sq - bf;
             float lf = Cf / qf;
             if (Af != 0.f && fmaf(-kc, fmaf(lf, d[2].hi, p[2].hi), 1.f) < 0.f) lf = qf / Af;
+            if (newton) {
 #pragma unroll 1
-            for (int it = 0; it < 4; ++it) {
-                const float x = fmaf(lf, d[0].hi, p[0].hi), y = fmaf(lf, d[1].hi, p[1].hi);
-                float zs, zxf, zyf;
-                if (!sag_f(E, flags, x, y, zs, zxf, zyf)) break;
-                const float dF = d[2].hi - zxf * d[0].hi - zyf * d[1].hi;
-                const float step = (fmaf(lf, d[2].hi, p[2].hi) - zs) / dF;
-                if (!(fabsf(step) < 1e30f)) break;
-                lf -= step;
-                if (fabsf(step) < 1e-2f) break;
-            }
-            if (fabsf(lf) < 1e30f) {
-                l = ds_f(lf);
-                return newton_ds(E, flags, p, d, l, N, hit);
-            }
-        }
-    } else {
-        const float c = E.c.hi, kc = E.kc.hi;
-        const float Af = fmaf(E.kmc.hi * d[2].hi, d[2].hi, c);
-        const float bf = fmaf(kc * p[2].hi, d[2].hi, c * fmaf(p[0].hi, d[0].hi, p[1].hi * d[1].hi)) - d[2].hi;
-        const float Cf = fmaf(kc * p[2].hi, p[2].hi, c * fmaf(p[0].hi, p[0].hi, p[1].hi * p[1].hi)) - 2.f * p[2].hi;
-        const float disc = fmaf(bf, bf, -(Af * Cf));
-        if (disc > 1e-6f * bf * bf) {
-            const float sq = sqrtf(disc);
-            const float qf = bf >= 0.f ? -(bf + sq) : sq - bf;
-            float lf = Cf / qf;
-            if (Af != 0.f && fmaf(-kc, fmaf(lf, d[2].hi, p[2].hi), 1.f) < 0.f) lf = qf / Af;
-            if (fabsf(lf) < 1e30f) {
-                l = ds_f(lf);
-                ds q0[3];
-                ray_point_ds(l, p, d, q0);
-                const ds x = q0[0], y = q0[1], z = q0[2];
-                const ds Q = dfma(E.c, dfma(x, x, y * y), dfma(E.kc * z, z, z * -2.f));
-                const float dQ = 2.f * (fmaf(c, fmaf(x.hi, d[0].hi, y.hi * d[1].hi), kc * z.hi * d[2].hi) - d[2].hi);
-                if (dQ != 0.f) {
-                    l = l - Q.hi / dQ;
-                    ray_point_ds(l, p, d, hit);
-                    conic_normal_ds(E, hit[0], hit[1], hit[2], N);
-                    return 0;
+                for (int it = 0; it < 4; ++it) {
+                    const float x = fmaf(lf, d[0].hi, p[0].hi), y = fmaf(lf, d[1].hi, p[1].hi);
+                    float zs, zxf, zyf;
+                    if (!sag_f(E, flags, x, y, zs, zxf, zyf)) break;
+                    const float dF = d[2].hi - zxf * d[0].hi - zyf * d[1].hi;
+                    const float step = (fmaf(lf, d[2].hi, p[2].hi) - zs) / dF;
+                    if (!(fabsf(step) < 1e30f)) break;
+                    lf -= step;
+                    if (fabsf(step) < 1e-2f) break;
                 }
             }
+            started = fabsf(lf) < 1e30f;
+            if (started) l = ds_f(lf);
         }
     }
-    // the quadric's l^2 coefficient c (d_x^2 + d_y^2) + kc d_z^2, which for the unit direction is c + (kc - c) d_z^2
-    const ds A = dfma(E.kmc * d[2], d[2], E.c);
-    const ds b = dfma(E.kc * p[2], d[2], E.c * dfma(p[0], d[0], p[1] * d[1])) - d[2];
-    const ds C = dfma(E.kc * p[2], p[2], E.c * dfma(p[0], p[0], p[1] * p[1])) - p[2] * 2.f;
-    const ds disc = dfma(b, b, -(A * C));
-    if (disc.hi < 0.f) return PHOSIM_LOST_MISSED;
-    const ds sq = ds_sqrt(disc);
-    const ds q = b.hi >= 0.f ? -(b + sq) : sq - b;
-    if (q.hi == 0.f) return PHOSIM_LOST_MISSED;
-    l = C / q;
-    if (A.hi != 0.f && (ds_f(1.f) - E.kc * dfma(l, d[2], p[2])).hi < 0.f) l = q / A;
+    if (started && !newton) {
+        ds q0[3];
+        ray_point_ds(l, p, d, q0);
+        const ds x = q0[0], y = q0[1], z = q0[2];
+        const ds Q = dfma(E.c, dfma(x, x, y * y), dfma(E.kc * z, z, z * -2.f));
+        const float dQ = 2.f * (fmaf(E.c.hi, fmaf(x.hi, d[0].hi, y.hi * d[1].hi), E.kc.hi * z.hi * d[2].hi) - d[2].hi);
+        started = dQ != 0.f;
+        if (started) l = l - Q.hi / dQ;
+    }
+    if (!started) {
+        l = conic_root_ds(E, p[0], p[1], p[2], d[0], d[1], d[2]);
+        if (l.hi == kNoRoot) return PHOSIM_LOST_MISSED;
+    }
     if (newton) return newton_ds(E, flags, p, d, l, N, hit);
     ray_point_ds(l, p, d, hit);
     conic_normal_ds(E, hit[0], hit[1], hit[2], N);
@@ -688,20 +683,19 @@ __device__ __forceinline__ void detect_ds(const TraceParams& P, const DetectorHi
 constexpr uint32_t kHandedOff = 0x80000000u;
 
 // where a ray is in its walk through the surfaces: position and direction in the telescope frame, the surface
-// it meets next and the way it travels (backwards after a ghost reflection), the index of the medium it is in
-// and the last glass index computed
+// it meets next and the way it travels (backwards after a ghost reflection), and the media: their indices are met a few
+// times a walk and have their places in shared memory in the kernels that keep their registers for the surfaces
+enum { kHere, kGlass, kGlassInverse, kMedia };     // the medium the ray is in; the last glass computed and its reciprocal
 struct OpticsWalk {
     ds X[3], D[3];
-    ds n_cur, glass_n, glass_inv;
+    ds* media;                    // kMedia
     int glass_mat, si, dir, bounces, n_ghost;
 };
 
 __device__ __forceinline__ void walk_start(OpticsWalk& W, const ds X[3], const ds D[3]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) { W.X[k] = X[k]; W.D[k] = D[k]; }
-    W.n_cur = ds_f(1.f);
-    W.glass_n = ds_f(1.f);
-    W.glass_inv = ds_f(1.f);
+    W.media[kHere] = ds_f(1.f);
     W.glass_mat = -1;
     W.si = 0; W.dir = 1; W.bounces = 0; W.n_ghost = 0;
 }
@@ -723,13 +717,31 @@ struct GhostRound {
 };
 
 // What a walk may meet: no reflecting coating (every ray is at the surface it is given), rays on their way
-// forward that end their part of the walk when a coating turns them round, or rays at surfaces of their own.
-enum WalkKind { kWalkPlain, kWalkForward, kWalkGhosts };
+// forward that end their part of the walk when a coating turns them round, or rays at surfaces of their own; kWalkSimple
+// as kWalkPlain, with no surface rotated or with odd or Zernike terms (kSimpleAbsent), whose code it leaves out.
+enum WalkKind { kWalkPlain, kWalkForward, kWalkGhosts, kWalkSimple };
+constexpr int kSimpleAbsent = SF_ROTATED | SF_ODD | SF_ZERN;
+
+// what a walk needs to know of its ray now and then: held, or read again where the entry stage left it
+struct RayHeld {
+    ds lam_;
+    int src_;
+    uint64_t idx_;
+    __device__ __forceinline__ ds lam() const { return lam_; }
+    __device__ __forceinline__ int src() const { return src_; }
+    __device__ __forceinline__ uint64_t idx() const { return idx_; }
+};
+struct RayInState {
+    const DSState* st;
+    __device__ __forceinline__ ds lam() const { return ds{st->lam, st->lam_lo}; }
+    __device__ __forceinline__ int src() const { return st->src; }
+    __device__ __forceinline__ uint64_t idx() const { return st->idx; }
+};
 
 // The next surface of the walk (si; a ray at a surface of its own gives W.si); false once the ray has left it
 // (R.flags then says lost, detected or handed off).
-template <WalkKind KIND>
-__device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk& W, int si, ds lam, int src, uint64_t ray,
+template <WalkKind KIND, class Ray>
+__device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk& W, int si, const Ray& ray,
                                                 PhotonOutS& R, const MemberDrawS* mb = nullptr,
                                                 DetectorHit* hand_off = nullptr) {
     if (si < 0 || si >= P.n_surf) {
@@ -738,7 +750,7 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
     }
     const DSurface& S = P.surf[si];
     const DSurfaceS& E = P.surf_s[si];
-    const int flags = S.flags;
+    const int flags = KIND == kWalkSimple ? S.flags & ~kSimpleAbsent : S.flags;
     ds p[3], dl[3];
     to_surface_ds(E, flags, W.X, W.D, p, dl);
     ds l, Nv[3], hit[3];
@@ -752,14 +764,14 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
         H.px = p[0]; H.py = p[1];
         H.dl[0] = dl[0]; H.dl[1] = dl[1]; H.dl[2] = dl[2];
         H.N[0] = Nv[0]; H.N[1] = Nv[1]; H.N[2] = Nv[2];
-        H.n_cur = W.n_cur;
+        H.n_cur = W.media[kHere];
         H.si = si;
         if (hand_off) {
             *hand_off = H;
             R.flags = kHandedOff;
             return false;
         }
-        detect_ds(P, H, lam, src, ray, R, mb);
+        detect_ds(P, H, ray.lam(), ray.src(), ray.idx(), R, mb);
         return false;
     }
     // clear aperture
@@ -777,7 +789,7 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
     // ghosts, has made its decision in the dynamic transmission test before the atmosphere (early_coating_reject_f:
     // its largest transmission over angles is its transmission, and draw, wavelength and bin are the same), so a ray
     // that comes here has passed.  (Without the second draw the optics of the 1000-star field take 5.45 ms, not 5.56.)
-    if (S.coat_slot >= 0 && !(KIND == kWalkPlain && (P.flags & PHOSIM_EARLY_REJECT) && P.coat[S.coating].nt == 1)) {
+    if (S.coat_slot >= 0 && !((KIND == kWalkPlain || KIND == kWalkSimple) && (P.flags & PHOSIM_EARLY_REJECT) && P.coat[S.coating].nt == 1)) {
         const DCoating& C = P.coat[S.coating];
         int it = 0;
         if (C.nt > 1) {
@@ -786,12 +798,12 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
             it = (int)floorf((th - C.th0f) * C.inv_dthf);
             it = it < 0 ? 0 : (it > C.nt - 1 ? C.nt - 1 : it);
         }
-        const size_t ix = (size_t)coat_lambda_bin(C, lam) * C.nt + it;
-        const uint32_t w = KIND == kWalkGhosts && W.bounces > 0 ? ghost_word_ds(P, src, ray, W.n_ghost++)
-                                                                : coat_word(P, src, ray, S.coat_slot);
+        const size_t ix = (size_t)coat_lambda_bin(C, ray.lam()) * C.nt + it;
+        const uint32_t w = KIND == kWalkGhosts && W.bounces > 0 ? ghost_word_ds(P, ray.src(), ray.idx(), W.n_ghost++)
+                                                                : coat_word(P, ray.src(), ray.idx(), S.coat_slot);
         if (!((unsigned long long)w < __ldg(C.T_thr + ix))) {
             // reflected backwards (a ghost) with probability R, absorbed otherwise
-            if (KIND != kWalkPlain && (P.flags & kGhostFlag) && S.kind != PHOSIM_MIRROR && C.TR_thr &&
+            if (KIND != kWalkPlain && KIND != kWalkSimple && (P.flags & kGhostFlag) && S.kind != PHOSIM_MIRROR && C.TR_thr &&
                 (unsigned long long)w < __ldg(C.TR_thr + ix)) {
                 const ds dn2 = dot3(dl, Nv) * -2.f;
                 {
@@ -826,19 +838,19 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
             const DMaterial& m = P.mat[mi];
             if (m.kind == PHOSIM_SELLMEIER) {
                 if (W.glass_mat != mi) {
-                    W.glass_n = sellmeier_ds(m, lam.hi);
-                    W.glass_inv = ds_rcp(W.glass_n);
+                    W.media[kGlass] = sellmeier_ds(m, ray.lam().hi);
+                    W.media[kGlassInverse] = ds_rcp(W.media[kGlass]);
                     W.glass_mat = mi;
                 }
-                n_next = W.glass_n;
-                inv_next = W.glass_inv;
+                n_next = W.media[kGlass];
+                inv_next = W.media[kGlassInverse];
             } else if (m.kind == PHOSIM_SILICON) {
-                n_next = ds_f(silicon_index_f(lam.hi));
+                n_next = ds_f(silicon_index_f(ray.lam().hi));
                 inv_next = ds_rcp(n_next);
             }
         }
-        if (!refract_ds(dl, Nv, W.n_cur * inv_next, (flags & SF_FLAT_ONLY) != 0)) { R.flags = lost(PHOSIM_LOST_TIR, si); return false; }
-        W.n_cur = n_next;
+        if (!refract_ds(dl, Nv, W.media[kHere] * inv_next, (flags & SF_FLAT_ONLY) != 0)) { R.flags = lost(PHOSIM_LOST_TIR, si); return false; }
+        W.media[kHere] = n_next;
     }
     from_surface_ds(E, flags, p, dl, W.X, W.D);
     if (KIND == kWalkGhosts) W.si = si + W.dir;
@@ -847,12 +859,13 @@ __device__ __forceinline__ bool surface_step_ds(const TraceParams& P, OpticsWalk
 
 // the whole walk of one ray
 __device__ __forceinline__ void optics_ds(const TraceParams& P, const ds X[3], const ds D[3], ds lam, int src,
-                                          uint64_t ray, PhotonOutS& R, const MemberDrawS* mb = nullptr,
-                                          DetectorHit* hand_off = nullptr) {
+                                          uint64_t ray, PhotonOutS& R, const MemberDrawS* mb = nullptr) {
     OpticsWalk W;
+    ds media[kMedia];
+    W.media = media;
     walk_start(W, X, D);
 #pragma unroll 1
-    while (surface_step_ds<kWalkGhosts>(P, W, W.si, lam, src, ray, R, mb, hand_off)) {
+    while (surface_step_ds<kWalkGhosts>(P, W, W.si, RayHeld{lam, src, ray}, R, mb)) {
     }
 }
 

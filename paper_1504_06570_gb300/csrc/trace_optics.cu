@@ -20,9 +20,14 @@
 
 namespace phosim {
 
-// blocks per SM the optics stage is compiled for: 3 of 80 registers (fewer spills) measured faster than 4 of 64
+// blocks per SM the optics stage is compiled for: 3 of 80 registers (the ghost walks: 3.56 ms for 4e6 photons, 3.70 with 4
+// of 64, 3.91 with 2 of 128); for simple surfaces 4 of 64, which hold that walk with few spills (the 1000-star field of
+// 1e8 photons: 4.62 ms, 4.92 with 3 and 4.99 with 5)
 #ifndef PHOSIM_DS_OPTICS_MIN_BLOCKS
 #define PHOSIM_DS_OPTICS_MIN_BLOCKS 3
+#endif
+#ifndef PHOSIM_DS_SIMPLE_MIN_BLOCKS
+#define PHOSIM_DS_SIMPLE_MIN_BLOCKS 4
 #endif
 // threads per block of the optics stage (0: the schedule's block size).  Fixed at 256: the lockstep wants
 // blocks of 8 warps (128- and 64-thread blocks measured 17 % and 28 % slower), whatever the schedule chosen
@@ -141,7 +146,7 @@ __device__ __forceinline__ void park_ghosts(const DSStage& S, bool parked, const
     DSGhost g;
 #pragma unroll
     for (int k = 0; k < 3; ++k) { g.X[k] = W.X[k]; g.D[k] = W.D[k]; }
-    g.n_cur = W.n_cur;
+    g.n_cur = W.media[kHere];
     g.lam = lam.hi; g.lam_lo = lam.lo;
     g.idx = ray; g.src = src; g.n_ghost = W.n_ghost;
     g.si = (short)W.si; g.dir = (short)W.dir; g.bounces = (short)W.bounces; g.pad = 0;
@@ -149,8 +154,15 @@ __device__ __forceinline__ void park_ghosts(const DSStage& S, bool parked, const
     S.ghost_bin[slot] = (uint8_t)bin;
 }
 
-// The optics stage.  KIND: the scene has no reflecting coating (kWalkPlain), the states of the entry stage with
-// rays that a coating may turn round (kWalkForward), or a round of such rays (kWalkGhosts, S.round).
+// The optics stage.  KIND: the scene has no reflecting coating (kWalkPlain; kWalkSimple where its surfaces are simple too),
+// the states of the entry stage with rays that a coating may turn round (kWalkForward), or a round of such rays
+// (kWalkGhosts, S.round).
+//
+// Bound by instruction issue (7 of 10 cycles issue): what its registers hold decides how many warps fill the others.
+// So they hold the ray and little else: wavelength, source and index are read again from the entry stage's state where a
+// surface or the accounting asks for them, the media's indices wait in shared memory, the double-single root of the rays
+// that the single-precision one does not serve is out of line, and a scene of simple surfaces has a kernel without the
+// code of the others (together 5.27 -> 4.62 ms for the 1000-star field, and 3.81 -> 3.56 with ghosts).
 //
 // Without ghosts every ray of a block is at the same surface, so the surface's constants are read at a uniform
 // index, and nothing of the ghosts is in the code.  (One kernel for all scenes, its surface index a ray's own,
@@ -162,10 +174,11 @@ __device__ __forceinline__ void park_ghosts(const DSStage& S, bool parked, const
 // goes on in place (few are left).  (Every ray in place: 16 of 32 lanes active and 9.05 ms for 4e6 photons of which
 // three in four are turned by a filter that reflects what it does not pass; 3.8 ms in rounds.)
 template <WalkKind KIND>
-__global__ void __launch_bounds__(kOpticsMaxThreads, PHOSIM_DS_OPTICS_MIN_BLOCKS)
+__global__ void __launch_bounds__(kOpticsMaxThreads, KIND == kWalkSimple ? PHOSIM_DS_SIMPLE_MIN_BLOCKS : PHOSIM_DS_OPTICS_MIN_BLOCKS)
     ds_optics_kernel(const __grid_constant__ TraceParams P, const __grid_constant__ DSStage S) {
     __shared__ unsigned long long cnt_mem[kOpticsMaxThreads / 32][kNumCounters];
     __shared__ unsigned long long next_batch;
+    __shared__ ds media[kOpticsMaxThreads][kMedia];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lanes_below = (1u << lane) - 1u;
     unsigned long long* cnt = cnt_mem[warp];
@@ -189,49 +202,60 @@ __global__ void __launch_bounds__(kOpticsMaxThreads, PHOSIM_DS_OPTICS_MIN_BLOCKS
         uint64_t u = 0;
         DetectorHit H;
         OpticsWalk W;
+        W.media = media[threadIdx.x];
         ds lam = ds_f(0.f);
         bool go = false, bundled = false, parked = false;
         if (v) {
             if constexpr (KIND == kWalkGhosts) {
                 const DSGhost& g = S.ghost[S.round & 1][S.ghost_order[e]];
                 src = g.src;
+                bundled = P.sources[src].bundle > 1;
                 u = g.idx;
                 lam = ds{g.lam, g.lam_lo};
                 walk_start(W, g.X, g.D);
-                W.n_cur = g.n_cur;
+                W.media[kHere] = g.n_cur;
                 W.si = g.si; W.dir = g.dir; W.bounces = g.bounces; W.n_ghost = g.n_ghost;
             } else {
-                const DSState st = S.state[e];
-                src = st.src;
-                u = st.idx;
-                lam = ds{st.lam, st.lam_lo};
+                const DSState& st = S.state[e];
                 const ds X[3] = {st.x, st.y, P.z_ent_s}, D[3] = {st.nx, st.ny, st.nz};
                 walk_start(W, X, D);
+                bundled = P.sources[st.src].bundle > 1;
             }
-            R.lam = lam.hi;
-            bundled = P.sources[src].bundle > 1;
             go = true;
         }
         int bin = 0;
-        if constexpr (KIND == kWalkPlain) {
+        if constexpr (KIND == kWalkGhosts) {
 #pragma unroll 1
-            for (int si = 0; __syncthreads_or(go); ++si) {
-                if (go) go = surface_step_ds<KIND>(P, W, si, lam, src, u, R, nullptr, bundled ? &H : nullptr);
-            }
-        } else {
-#pragma unroll 1
-            for (int s0 = 0; __syncthreads_or(go); ++s0) {
+            while (__syncthreads_or(go)) {
                 if (!go) continue;
-                const int si = KIND == kWalkForward ? s0 : W.si, before = W.bounces;
-                go = surface_step_ds<KIND>(P, W, si, lam, src, u, R, nullptr, bundled ? &H : nullptr);
+                const int si = W.si, before = W.bounces;
+                go = surface_step_ds<KIND>(P, W, si, RayHeld{lam, src, u}, R, nullptr, bundled ? &H : nullptr);
                 if (go && W.bounces > before && W.bounces <= kGhostRounds) {
                     parked = true;
                     go = false;
                     bin = P.surf[si].coat_slot;
                 }
             }
-            park_ghosts(S, parked, W, lam, src, u, bin, lane);
+        } else {
+            const RayInState ray = {S.state + (v ? e : 0)};
+#pragma unroll 1
+            for (int si = 0; __syncthreads_or(go); ++si) {
+                if (!go) continue;
+                go = surface_step_ds<KIND>(P, W, si, ray, R, nullptr, bundled ? &H : nullptr);
+                if (KIND == kWalkForward && go && W.bounces > 0) {
+                    parked = true;
+                    go = false;
+                    bin = P.surf[si].coat_slot;
+                }
+            }
+            if (v) {
+                src = ray.src();
+                u = ray.idx();
+                lam = ray.lam();
+            }
         }
+        if constexpr (KIND == kWalkForward || KIND == kWalkGhosts) park_ghosts(S, parked, W, lam, src, u, bin, lane);
+        R.lam = lam.hi;
         // a bundle's ray that reached the detector surface hands its hit over to the bundle stage
         const bool handed = v && R.flags == kHandedOff;
         const unsigned hmask = __ballot_sync(0xffffffffu, handed);
@@ -340,6 +364,7 @@ __global__ void moment_stripes_kernel(const __grid_constant__ TraceParams P) {
 const void* ds_optics_kernel_ptr(int kind) {
     return kind == kWalkGhosts ? (const void*)ds_optics_kernel<kWalkGhosts>
                                : kind == kWalkForward ? (const void*)ds_optics_kernel<kWalkForward>
+                               : kind == kWalkSimple  ? (const void*)ds_optics_kernel<kWalkSimple>
                                                       : (const void*)ds_optics_kernel<kWalkPlain>;
 }
 const void* ghost_order_kernel_ptr() { return (const void*)ghost_order_kernel; }
@@ -356,10 +381,12 @@ int ds_optics_threads(int threads) { return PHOSIM_DS_OPTICS_THREADS ? PHOSIM_DS
 
 cudaError_t launch_ds_optics(const TraceParams& P, const DSStage& S, int kind, int blocks, int threads, cudaStream_t st, bool beside) {
     const int block = ds_optics_threads(threads);
+    if (beside && kind == kWalkSimple) return launch_beside(ds_optics_kernel<kWalkSimple>, blocks, block, st, P, S);
     if (beside && kind == kWalkPlain) return launch_beside(ds_optics_kernel<kWalkPlain>, blocks, block, st, P, S);
     if (beside && kind == kWalkForward) return launch_beside(ds_optics_kernel<kWalkForward>, blocks, block, st, P, S);
     if (kind == kWalkGhosts) ds_optics_kernel<kWalkGhosts><<<blocks, block, 0, st>>>(P, S);
     else if (kind == kWalkForward) ds_optics_kernel<kWalkForward><<<blocks, block, 0, st>>>(P, S);
+    else if (kind == kWalkSimple) ds_optics_kernel<kWalkSimple><<<blocks, block, 0, st>>>(P, S);
     else ds_optics_kernel<kWalkPlain><<<blocks, block, 0, st>>>(P, S);
     return cudaGetLastError();
 }
@@ -376,10 +403,10 @@ cudaError_t launch_ds_members(const TraceParams& P, const DSStage& S, int blocks
 
 const void* ds_members_kernel_ptr() { return (const void*)ds_members_kernel; }
 
-cudaError_t ds_stage_occupancy(int threads, int* entry_per_sm, int* optics_per_sm, int* members_per_sm) {
+cudaError_t ds_stage_occupancy(int kind, int threads, int* entry_per_sm, int* optics_per_sm, int* members_per_sm) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(entry_per_sm, ds_entry_kernel_ptr(), threads, 0);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(optics_per_sm, ds_optics_kernel<kWalkPlain>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(optics_per_sm, ds_optics_kernel_ptr(kind),
                                                           ds_optics_threads(threads), 0);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(members_per_sm, ds_members_kernel, threads, 0);
