@@ -11,10 +11,13 @@
 // sums cost about one FP64 addition a value: all Zernike coefficients of a surface are linear in the sums of the 28
 // monomials of its figure, which a photon adds to whatever the number of coefficients, and the lanes' values
 // are summed by a transposed butterfly (31 additions for 32 values, the total of value k in lane k) and added to the
-// source's sums.  A second kernel turns the sums into the parameters' gradients.
-// Measured (GB300, 64 stars of 3e4 photons, 97 parameters of which 57 Zernike coefficients): a whole call 11.9 ms
+// source's sums.  A surface's misalignments take the force and the torque on it, six sums.  A second kernel turns the
+// sums into the parameters' gradients.
+// Measured (GB300, 64 stars of 3e4 photons, 97 parameters of which 57 Zernike coefficients), a whole call: 11.9 ms
 // with every coefficient's polynomial evaluated per photon, per-lane accumulators in local memory and the
-// intersections recomputed in the sweep, 5.6 ms in this form.
+// intersections recomputed in the sweep; 5.6 ms without; 3.8 ms with the photons in batches; 3.2 ms with force and
+// torque for the nine elements of each matrix's adjoint, and the figure's second derivatives from their own
+// coefficients.
 #include "phosim_device.cuh"
 #include "phosim_scene.hpp"
 #include "photon.cuh"
@@ -59,14 +62,12 @@ __device__ __forceinline__ void sag_hessian(const DSurface& S, double x, double 
     zyy = fma(y * y, G2, g);
 }
 
-// Snell refraction's adjoint, with the forward direction d, normal Nin and index ratio mu: given
+// Snell refraction's adjoint, with the forward direction d, normal Nin, dn = d . Nin and index ratio mu: given
 // ob = d(L)/d(out), db = d(L)/d(d) and Nb = d(L)/d(Nin).
-__device__ __forceinline__ void refract_adjoint(const double d[3], const double Nin[3], double mu, const double ob[3],
-                                                double db[3], double Nb[3]) {
-    double cosi = -fma(d[0], Nin[0], fma(d[1], Nin[1], d[2] * Nin[2]));
-    const bool turn = negative64(cosi);       // the normal on the side the ray comes from is s N, s = +-1
-    const double s = turn ? -1.0 : 1.0;
-    cosi = turn ? -cosi : cosi;
+__device__ __forceinline__ void refract_adjoint(const double d[3], const double Nin[3], double dn, double mu,
+                                                const double ob[3], double db[3], double Nb[3]) {
+    const bool turn = !negative64(dn);        // the normal on the side the ray comes from is s N, s = +-1
+    const double s = turn ? -1.0 : 1.0, cosi = turn ? dn : -dn;
     const double k = fma(-(mu * mu), fma(-cosi, cosi, 1.0), 1.0);
     const double ik = rsqrt64(k), sk = k * ik;
     const double a = fma(mu, cosi, -sk);
@@ -91,14 +92,14 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
     const bool rotated = (S.flags & SF_ROTATED) != 0;
     const double h[3] = {q.h[0], q.h[1], q.h[2]}, d[3] = {q.d[0], q.d[1], q.d[2]}, N[3] = {q.N[0], q.N[1], q.N[2]};
     const double dn = fma(d[0], N[0], fma(d[1], N[1], d[2] * N[2]));
-    double hb[3] = {0.0, 0.0, 0.0}, ob[3] = {0.0, 0.0, 0.0}, db[3] = {0.0, 0.0, 0.0}, Nb[3] = {0.0, 0.0, 0.0};
+    double hb[3] = {0.0, 0.0, 0.0}, c[3] = {0.0, 0.0, 0.0}, ob[3] = {0.0, 0.0, 0.0}, db[3] = {0.0, 0.0, 0.0}, Nb[3] = {0.0, 0.0, 0.0};
     if (detector) {
         hb[0] = fb[0];
         hb[1] = fb[1];
         if (P.flags & PHOSIM_SENSOR) {
             ob[0] = L * fb[0];
             ob[1] = L * fb[1];
-            refract_adjoint(d, N, q.mu, ob, db, Nb);
+            refract_adjoint(d, N, dn, q.mu, ob, db, Nb);
         }
     } else {
         // X' = M^T h + o, D' = M^T out: adjoints into h and out
@@ -115,7 +116,7 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
                 Nb[i] = fma(d2, ob[i], n2 * d[i]);
             }
         } else {
-            refract_adjoint(d, N, q.mu, ob, db, Nb);
+            refract_adjoint(d, N, dn, q.mu, ob, db, Nb);
         }
     }
     // normal N = (-S_x, -S_y, 1) / |.|: adjoint into the slopes; slopes at the hit: into h by the second derivatives
@@ -144,24 +145,23 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
         double sxx, sxy, syy;
         sag_hessian(S, h[0], h[1], sxx, sxy, syy);
         if (zernike) {
-            double zuu = 0.0, zuv = 0.0, zvv = 0.0;
-            int off = 0, down = 0, down2 = 0;            // the rows b, b - 1 and b - 2
+            const ZernikeHessian& Z = G.hessian[si];
+            int off = 0, k = 0;
 #pragma unroll
-            for (int b = 0; b <= 6; ++b) {
+            for (int b = 0; b <= 4; ++b) {
 #pragma unroll
-                for (int a = 0; a + b <= 6; ++a) {
-                    const double c = S.zp[off + a];
-                    if (a >= 2) zuu = fma(c, (a * (a - 1)) * m[off + a - 2], zuu);
-                    if (a >= 1 && b >= 1) zuv = fma(c, (a * b) * m[down + a - 1], zuv);
-                    if (b >= 2) zvv = fma(c, (b * (b - 1)) * m[down2 + a], zvv);
+                for (int a = 0; a + b <= 4; ++a, ++k) {
+                    sxx = fma(Z.xx[k], m[off + a], sxx);
+                    sxy = fma(Z.xy[k], m[off + a], sxy);
+                    syy = fma(Z.yy[k], m[off + a], syy);
                 }
-                down2 = down; down = off; off += 7 - b;
+                off += 7 - b;
             }
-            const double k2 = S.zinv * S.zinv;
-            sxx = fma(zuu, k2, sxx); sxy = fma(zuv, k2, sxy); syy = fma(zvv, k2, syy);
         }
-        hb[0] = fma(sxx, zxb, fma(sxy, zyb, hb[0]));
-        hb[1] = fma(sxy, zxb, fma(syy, zyb, hb[1]));
+        c[0] = fma(sxx, zxb, sxy * zyb);
+        c[1] = fma(sxy, zxb, syy * zyb);
+        hb[0] += c[0];
+        hb[1] += c[1];
     }
     // h = p + l d with the implicit intersection F(l; p, d, c) = p_z + l d_z - S(p_xy + l d_xy; c) = 0:
     // F_l = d . N / N_z, so l's adjoint enters p along the normal with weight W
@@ -202,44 +202,26 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
         Dn[k] = rotated ? fma(S.M[k], dt[0], fma(S.M[3 + k], dt[1], S.M[6 + k] * dt[2])) : dt[k];
     }
     if (shift || tilt) {
+        // The surface as a rigid body, in its frame: the force F on its vertex and the torque T on its axes, from which
+        // grad_finish_kernel takes the parameters' gradients.  M enters p + l d = M (X + l D - o), d = M D and past the
+        // surface X' = M^T h + o, D' = M^T out; with dM = [w] M its terms are w . (h x (pb - hb0) + d x db - out x ob),
+        // where pb - hb0 is c, the part of the hit's adjoint that the surface put in, and d x db - out x ob is Nb x N for
+        // a reflection as for a refraction (both commute with a rotation of d, N and out together).
         double g[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) g[k] = 0.0;
-        if (shift) {                                     // vertex o = (dx, dy, z + dz): X' and p
 #pragma unroll
-            for (int k = 0; k < 3; ++k) g[k] = (detector ? 0.0 : Xb[k]) - Xn[k];
+        for (int i = 0; i < 3; ++i) c[i] = detector ? pb[i] : fma(W, N[i], c[i]);
+        if (shift) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) g[k] = -c[k];
         }
         if (tilt) {
-            // M enters p + l d = M (X + l D - o), with pb, and d = M D, with db; and, past the surface, h and out
-            double Mb[9], rh[3], D[3], out[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                rh[k] = rotated ? fma(S.M[k], h[0], fma(S.M[3 + k], h[1], S.M[6 + k] * h[2])) : h[k];
-                D[k] = rotated ? fma(S.M[k], d[0], fma(S.M[3 + k], d[1], S.M[6 + k] * d[2])) : d[k];
-                out[k] = d[k];
-            }
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) Mb[3 * i + k] = fma(pb[i], rh[k], db[i] * D[k]);
-            if (!detector) {
-                if (S.kind == PHOSIM_MIRROR) {
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) out[k] = fma(-2.0 * dn, N[k], d[k]);
-                } else {
-                    refract(out, N[0], N[1], N[2], q.mu);
-                }
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) Mb[3 * i + k] = fma(h[i], Xb[k], fma(out[i], Db[k], Mb[3 * i + k]));
-            }
-#pragma unroll
-            for (int f = 0; f < 3; ++f) {
-                double s = 0.0;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) s = fma(Mb[k], G.dM[si][f][k], s);
-                g[3 + f] = s;
+                const int i = (k + 1) % 3, j = (k + 2) % 3;
+                const double hc = fma(h[i], c[j], -(h[j] * c[i]));
+                g[3 + k] = detector ? fma(d[i], db[j], fma(-d[j], db[i], hc)) : fma(Nb[i], N[j], fma(-Nb[j], N[i], hc));
             }
         }
 #pragma unroll
@@ -297,7 +279,12 @@ __global__ void grad_finish_kernel(const __grid_constant__ GradParams G, int n_s
         for (int k = 0; k < kZPoly; ++k) s = fma(z[k], a[k], s);
     } else {
 #pragma unroll
-        for (int g = 0; g < 4; ++g) s += a[32 + f + 8 * g];
+        for (int i = 0; i < 3; ++i) {
+            double sum = 0.0;                            // of the force (f < 3) or the torque
+#pragma unroll
+            for (int g = 0; g < 4; ++g) sum += a[32 + (f < 3 ? 0 : 3) + i + 8 * g];
+            s = fma(G.axis[G.param_surface[p]][f][i], sum, s);
+        }
     }
     G.grad[i] = s;
 }

@@ -1481,7 +1481,34 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
         G.param_field[p] = f;
         G.first_surface = std::min(G.first_surface, s);
     }
-    for (int s = 0; s < B.n_surf; ++s) rotation_derivatives(sc->surfaces[s].pert, G.dM[s]);
+    for (int s = 0; s < B.n_surf; ++s) {
+        const DSurface& S = B.surf[s];
+        double dM[3][9];
+        rotation_derivatives(sc->surfaces[s].pert, dM);
+        for (int f = 0; f < 3; ++f) {
+            // a shift along telescope axis f is M's column f in the surface's frame; dM_f = [w] M, w of dM_f M^T
+            double A[9];
+            for (int i = 0; i < 3; ++i) {
+                G.axis[s][f][i] = S.M[3 * i + f];
+                for (int j = 0; j < 3; ++j) {
+                    A[3 * i + j] = 0.0;
+                    for (int k = 0; k < 3; ++k) A[3 * i + j] += dM[f][3 * i + k] * S.M[3 * j + k];
+                }
+            }
+            G.axis[s][3 + f][0] = 0.5 * (A[7] - A[5]);
+            G.axis[s][3 + f][1] = 0.5 * (A[2] - A[6]);
+            G.axis[s][3 + f][2] = 0.5 * (A[3] - A[1]);
+        }
+        if (!(S.flags & SF_ZERN)) continue;
+        const double k2 = S.zinv * S.zinv;
+        const auto row = [](int b) { return 7 * b - b * (b - 1) / 2; };       // where u^0 v^b stands
+        for (int b = 0, k = 0; b <= 4; ++b)
+            for (int a = 0; a + b <= 4; ++a, ++k) {
+                G.hessian[s].xx[k] = k2 * (a + 2) * (a + 1) * S.zp[row(b) + a + 2];
+                G.hessian[s].xy[k] = k2 * (a + 1) * (b + 1) * S.zp[row(b + 1) + a + 1];
+                G.hessian[s].yy[k] = k2 * (b + 2) * (b + 1) * S.zp[row(b + 2) + a];
+            }
+    }
     G.zmono = sc->d_zmono;
     cudaStream_t st = (cudaStream_t)stream;
     // forward pass in FP64: moment sums about each source's chief ray
