@@ -1,9 +1,10 @@
 // Adjoint raytrace: pathwise gradients of per-source PSF moments with respect to surface misalignments and
 // Zernike figure coefficients (the optics of Peterson et al. 2015, Sec. 2.4.1-2.4.2, differentiated).
 //
-// Per photon the forward path is recomputed with the trace's own code (same random numbers, same accept
-// decisions), keeping at each surface the hit point, the direction, the distance, the normal and the index
-// ratio in its frame.  The reverse sweep then walks the surfaces backwards and applies the hand-derived
+// The forward path is the trace's (same random numbers, same accept decisions), which keeps at each surface the hit
+// point, the direction, the distance, the normal and the index ratio in its frame: the forward pass that gives the
+// moments does so for the batches of photons that find room on the tape (512 MB), the others are traced again here.  The
+// reverse sweep then walks the surfaces backwards and applies the hand-derived
 // vector-Jacobian products of: the frame transform, the implicit intersection (dl = -F_theta / F_l at the
 // root), the normal from the sag slopes, and reflection or Snell refraction.
 //
@@ -17,7 +18,8 @@
 // with every coefficient's polynomial evaluated per photon, per-lane accumulators in local memory and the
 // intersections recomputed in the sweep; 5.6 ms without; 3.8 ms with the photons in batches; 3.2 ms with force and
 // torque for the nine elements of each matrix's adjoint, and the figure's second derivatives from their own
-// coefficients.
+// coefficients; 2.5 ms with the forward states kept (a photon's 1.1 KB written and read once, against 40 % of the sweep's
+// FP64 operations).
 #include "phosim_device.cuh"
 #include "phosim_scene.hpp"
 #include "photon.cuh"
@@ -85,12 +87,19 @@ __device__ __forceinline__ void refract_adjoint(const double d[3], const double 
 // adjoint of the final (x, y) in its frame and L the conversion length (the diffusion offset does not depend on the
 // optics); otherwise Xb / Db carry the adjoint of the telescope-frame state leaving the surface in and of the state
 // entering it out.  sums: the source's sums of this surface, kGradWords.
-__device__ __forceinline__ void surface_adjoint(const TraceParams& P, const GradParams& G, int si, const SurfaceRecord& q,
+__device__ __forceinline__ void surface_adjoint(const TraceParams& P, const GradParams& G, int si, const double* q,
                                                 bool on, bool detector, const double fb[2], double L, double Xb[3],
                                                 double Db[3], double* sums, int lane) {
     const DSurface& S = P.surf[si];
     const bool rotated = (S.flags & SF_ROTATED) != 0;
-    const double h[3] = {q.h[0], q.h[1], q.h[2]}, d[3] = {q.d[0], q.d[1], q.d[2]}, N[3] = {q.N[0], q.N[1], q.N[2]};
+    double h[3], d[3], N[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        h[k] = on ? q[32 * (kTapeH + k)] : 0.0;
+        d[k] = on ? q[32 * (kTapeD + k)] : 0.0;
+        N[k] = on ? q[32 * (kTapeN + k)] : 0.0;
+    }
+    const double q_l = on ? q[32 * kTapeL] : 0.0, mu = on && S.kind != PHOSIM_MIRROR ? q[32 * kTapeMu] : 0.0;
     const double dn = fma(d[0], N[0], fma(d[1], N[1], d[2] * N[2]));
     double hb[3] = {0.0, 0.0, 0.0}, c[3] = {0.0, 0.0, 0.0}, ob[3] = {0.0, 0.0, 0.0}, db[3] = {0.0, 0.0, 0.0}, Nb[3] = {0.0, 0.0, 0.0};
     if (detector) {
@@ -99,7 +108,7 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
         if (P.flags & PHOSIM_SENSOR) {
             ob[0] = L * fb[0];
             ob[1] = L * fb[1];
-            refract_adjoint(d, N, dn, q.mu, ob, db, Nb);
+            refract_adjoint(d, N, dn, mu, ob, db, Nb);
         }
     } else {
         // X' = M^T h + o, D' = M^T out: adjoints into h and out
@@ -116,7 +125,7 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
                 Nb[i] = fma(d2, ob[i], n2 * d[i]);
             }
         } else {
-            refract_adjoint(d, N, dn, q.mu, ob, db, Nb);
+            refract_adjoint(d, N, dn, mu, ob, db, Nb);
         }
     }
     // normal N = (-S_x, -S_y, 1) / |.|: adjoint into the slopes; slopes at the hit: into h by the second derivatives
@@ -195,7 +204,7 @@ __device__ __forceinline__ void surface_adjoint(const TraceParams& P, const Grad
     // p = M (X - o), d = M D
     double dt[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) dt[i] = fma(q.l, pb[i], db[i]);
+    for (int i = 0; i < 3; ++i) dt[i] = fma(q_l, pb[i], db[i]);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         Xn[k] = rotated ? fma(S.M[k], pb[0], fma(S.M[3 + k], pb[1], S.M[6 + k] * pb[2])) : pb[k];
@@ -249,20 +258,32 @@ __global__ void __launch_bounds__(32, 12) grad_kernel(const __grid_constant__ Tr
         const bool v = lane < (int)B.n;
         const DSource& s = P.sources[src];
         const double* sd = G.seeds + (size_t)src * 8;
-        ForwardRecord fr;
-        PhotonOut R;
-        R.flags = 0;
-        if (v) trace_photon<false, true, true>(P, s, src, B.first + B.k[lane], R, &fr);
-        const bool on = (R.flags & PHOSIM_F_DETECTED) != 0;
+        // what the trace kept, or the photons once more
+        const bool taped = b < L.tape_batches;
+        ForwardRecord fr = forward_record(P, L, taped ? b : L.tape_batches + blockIdx.x, lane);
+        const double* end = fr.end();
+        bool on = false;
+        if (taped) {
+            on = v && end[32 * kTapeOn] != 0.0;
+        } else if (v) {
+            PhotonOut R;
+            R.flags = 0;
+            trace_photon<false, true, true>(P, s, src, B.first + B.k[lane], R, &fr);
+            on = (R.flags & PHOSIM_F_DETECTED) != 0;
+            double* q = fr.end();
+            q[32 * kTapeX] = R.x;
+            q[32 * kTapeY] = R.y;
+        }
         // the whole warp sweeps (the sums need every lane); the other lanes' values are dropped
         if (!__any_sync(0xffffffffu, on)) continue;
-        const double dx = R.x - sd[5], dy = R.y - sd[6];
+        const double dx = on ? end[32 * kTapeX] - sd[5] : 0.0, dy = on ? end[32 * kTapeY] - sd[6] : 0.0;
+        const double depth = on && (P.flags & PHOSIM_SENSOR) ? end[32 * kTapeDepth] : 0.0;
         const double fb[2] = {fma(sd[2], dx, fma(sd[3], dy, sd[0])), fma(sd[4], dy, fma(sd[3], dx, sd[1]))};
         double Xb[3] = {0.0, 0.0, 0.0}, Db[3] = {0.0, 0.0, 0.0};
         double* out = G.sums + (size_t)src * P.n_surf * kGradWords;
 #pragma unroll 1
         for (int si = P.n_surf - 1; si >= G.first_surface; --si)
-            surface_adjoint(P, G, si, fr.s[si], on, si == P.n_surf - 1, fb, fr.L, Xb, Db, out + si * kGradWords, lane);
+            surface_adjoint(P, G, si, fr.surface(si), on, si == P.n_surf - 1, fb, depth, Xb, Db, out + si * kGradWords, lane);
     }
 }
 

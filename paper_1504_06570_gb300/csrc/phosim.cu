@@ -74,6 +74,9 @@ constexpr uint64_t kGhostChunk = 1ull << 24;
 // photons up to which the two-kernel path adds the moments without the striped copies (which take a kernel to clear and
 // one to add: 6 us of a 10^4-photon call)
 constexpr uint64_t kDirectMoments = 1ull << 16;
+// the adjoint's tape, at most: batches past it are traced again (a telescope of 12 surfaces takes 35 KB a batch of 32
+// photons, so 4.9e5 photons past the dynamic transmission test)
+constexpr size_t kTapeBytes = 512ull << 20;
 
 // ----------------------------------------------------------------------------------------- Zernike figure
 // Noll index -> radial order n, |m| and whether the term is the cosine one (even j) or the sine one.
@@ -598,6 +601,7 @@ void phosim_destroy_scene(phosim_scene* sc) {
     cudaFree(sc->d_rounds);
     cudaFree(sc->d_mom_stripes);
     cudaFree(sc->d_grad_scratch);
+    cudaFree(sc->d_tape);
     cudaFree(sc->d_mom_scratch);
     for (TraceGraph& g : sc->graphs) destroy_graph(g);
     for (cudaEvent_t e : sc->timing_events) cudaEventDestroy(e);
@@ -1277,6 +1281,16 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         B.batch = sc->d_batches;
         B.n = sc->d_counters + kStateCountWord;
         B.next = sc->d_counters + kBatchWord;
+        B.tape = nullptr;
+        B.tape_batches = B.tape_stride = 0;
+        B.tape_first = 0;
+        if (sc->tape_wanted && sc->batches_whole) {
+            B.tape = sc->d_tape;
+            B.tape_batches = sc->tape_batches;
+            B.tape_stride = sc->tape_stride;
+            B.tape_first = sc->tape_first;
+            sc->tape_written = true;
+        }
         const uint64_t n_chunks = (n_tiles + chunk_tiles - 1) / chunk_tiles;
         std::vector<BatchList> lists((size_t)n_chunks, B);
         for (uint64_t c = 0; c < n_chunks; ++c) {
@@ -1528,11 +1542,36 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     }
     CU(cudaMemsetAsync(sc->d_mom_scratch, 0, mom_bytes, st));
     // FP64 and the dynamic transmission test (it leaves the detected photons unchanged) for both passes
+    int per_sm = 0, batch_per_sm = 0, trace_per_sm = 0;
+    CU(grad_occupancy(&per_sm));
+    CU(batch_occupancy(PHOSIM_PLAIN_FP64, sc->threads, &batch_per_sm, &trace_per_sm));
+    const int blocks = sc->sm_count * std::max(per_sm, 1), blocks_batch = sc->sm_count * std::max(batch_per_sm, 1);
+    // the tape: a slot for each batch there can be, 512 MB of them at most, and one a block
+    uint64_t total = 0;
+    for (int s = 0; s < n_src; ++s) total += n_photons[s];
+    sc->tape_first = G.first_surface;
+    sc->tape_stride = (size_t)(kTapeSurface * (B.n_surf - G.first_surface) + kTapeEnd) * 32;
+    const size_t slot_bytes = sc->tape_stride * sizeof(double);
+    const size_t block_slots = (size_t)std::max(blocks, sc->sm_count * std::max(trace_per_sm, 1));
+    sc->tape_batches = std::min<uint64_t>(kTapeBytes / slot_bytes, total / 32 + n_src);
+    if (sc->cap_tape < (sc->tape_batches + block_slots) * slot_bytes) {
+        cudaFree(sc->d_tape);
+        sc->d_tape = nullptr; sc->cap_tape = 0;
+        if (cudaMalloc(&sc->d_tape, (sc->tape_batches + block_slots) * slot_bytes) != cudaSuccess) {
+            (void)cudaGetLastError();                    // no room: every photon is traced again
+            sc->tape_batches = 0;
+            CU(cudaMalloc(&sc->d_tape, block_slots * slot_bytes));
+        }
+        sc->cap_tape = (sc->tape_batches + block_slots) * slot_bytes;
+    }
     const int saved_precision = sc->precision;
     const uint32_t saved_flags = sc->base.flags;
     sc->precision = PHOSIM_PLAIN_FP64;
     sc->base.flags = (saved_flags | PHOSIM_EARLY_REJECT) & ~PHOSIM_GRAPH;
+    sc->tape_wanted = sc->tape_batches > 0;
+    sc->tape_written = false;
     phosim_status rs = phosim_trace(sc, src, n_src, n_photons, nullptr, sc->d_stage, nullptr, sc->d_mom_scratch, stream);
+    sc->tape_wanted = false;
     sc->precision = saved_precision;
     sc->base.flags = saved_flags;
     if (rs != PHOSIM_OK) return rs;
@@ -1588,11 +1627,11 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     P.image = nullptr;
     P.moments = nullptr;
     P.records = nullptr;
-    int per_sm = 0, batch_per_sm = 0, unused = 0;
-    CU(grad_occupancy(&per_sm));
-    CU(batch_occupancy(PHOSIM_PLAIN_FP64, sc->threads, &batch_per_sm, &unused));
-    const int blocks = sc->sm_count * std::max(per_sm, 1), blocks_batch = sc->sm_count * std::max(batch_per_sm, 1);
     BatchList L;
+    L.tape = sc->d_tape;
+    L.tape_batches = sc->tape_written ? sc->tape_batches : 0;
+    L.tape_stride = sc->tape_stride;
+    L.tape_first = sc->tape_first;
     L.n = sc->d_counters + kStateCountWord;
     L.next = sc->d_counters + kBatchWord;
     const bool whole = sc->batches_whole;

@@ -200,11 +200,19 @@ struct __align__(16) PhotonBatch {
     unsigned long long first;
     uint32_t k[32];
 };
+// the words of a photon's forward state: of each surface, and after the surfaces
+enum { kTapeH = 0, kTapeD = 3, kTapeL = 6, kTapeN = 7, kTapeMu = 10, kTapeSurface = 11 };       // words of a surface
+enum { kTapeDepth = 0, kTapeX = 1, kTapeY = 2, kTapeOn = 3, kTapeEnd = 4 };                     // words after the surfaces
 // The batches of tiles [tile_begin, tile_end): their number, and the next one to be taken
 struct BatchList {
     PhotonBatch* batch;
     unsigned long long *n, *next;
     uint64_t tile_begin, tile_end;
+    // For the adjoint, the photons' forward state (ForwardRecord in photon.cuh): the first tape_batches batches' in a slot
+    // each of tape_stride words, and after those a slot for each block that works on a batch without one
+    double* tape;
+    unsigned long long tape_batches, tape_stride;
+    int tape_first;               // the first surface recorded
 };
 
 // What a trace call does before its rays (call_prep_kernel): the source list and the tile prefix, given here when they

@@ -77,6 +77,12 @@ struct phosim_scene {
     phosim::PhotonBatch* d_batches = nullptr;
     size_t cap_batches = 0;
     bool batches_whole = false;
+    // the adjoint's tape (BatchList): asked for while phosim_grad runs its forward pass, and whether that pass wrote it
+    double* d_tape = nullptr;
+    size_t cap_tape = 0;
+    unsigned long long tape_batches = 0, tape_stride = 0;
+    int tape_first = 0;
+    bool tape_wanted = false, tape_written = false;
     uint32_t last_tile = 0;                     // its photons per tile, tiles and batch kernel's blocks
     uint64_t last_tiles = 0;
     // per-kernel timing (phosim_set_stage_timing): an event pair per launch of the last call, with the

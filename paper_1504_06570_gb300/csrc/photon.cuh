@@ -131,16 +131,19 @@ __device__ __forceinline__ float lerp_table_f(const float* __restrict__ t, int n
 
 // Surfaces in order (Sec. 2.4.2).  FULL = apertures, coatings and the sensor; otherwise the bare rays that
 // give each source's chief-ray reference.
-// Forward state kept for the adjoint sweep (RECORD): at each surface, in its frame, the hit point, the direction
-// before it, the distance travelled to it, the normal and (refracting surfaces, the sensor) the index ratio n1 / n2;
-// and the conversion length of the sensor.
-struct SurfaceRecord {
-    double h[3], d[3], l, N[3], mu;
-};
+// Forward state kept for the adjoint sweep (RECORD): at each surface from the tape's first on, in its frame, the hit point,
+// the direction before it, the distance travelled to it, the normal and (refracting surfaces, the sensor) the index ratio
+// n1 / n2; and the conversion length of the sensor, the final position and whether the photon was detected.  A warp's
+// records are words of its 32 lanes side by side (BatchList).
 struct ForwardRecord {
-    SurfaceRecord s[PHOSIM_MAX_SURFACES];
-    double L;
+    double* w;                    // this lane's first word
+    int first, n_surf;
+    __device__ __forceinline__ double* surface(int si) const { return w + (size_t)(kTapeSurface * (si - first)) * 32; }
+    __device__ __forceinline__ double* end() const { return surface(n_surf); }
 };
+__device__ __forceinline__ ForwardRecord forward_record(const TraceParams& P, const BatchList& L, unsigned long long slot, int lane) {
+    return {L.tape + slot * L.tape_stride + lane, L.tape_first, P.n_surf};
+}
 
 // A photon of a bundle (Sec. 3.2 background optimisation): it follows its ray (the photon index divided by
 // the bundle size) to the detector surface, lands at a Gaussian offset of the source's spread sigma from the
@@ -208,10 +211,16 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
         if (why) { R.flags = lost(why, si); return; }
         if (GHOSTS && bounces > 0 && !ahead) { R.flags = lost(PHOSIM_LOST_MISSED, si); return; }
         if constexpr (RECORD) {
-            SurfaceRecord& q = fr->s[si];
+            if (si >= fr->first) {
+                double* q = fr->surface(si);
 #pragma unroll
-            for (int k = 0; k < 3; ++k) { q.h[k] = h[k]; q.d[k] = dl[k]; q.N[k] = Nv[k]; }
-            q.l = fma(h[0] - p[0], dl[0], fma(h[1] - p[1], dl[1], (h[2] - p[2]) * dl[2]));
+                for (int k = 0; k < 3; ++k) {
+                    q[32 * (kTapeH + k)] = h[k];
+                    q[32 * (kTapeD + k)] = dl[k];
+                    q[32 * (kTapeN + k)] = Nv[k];
+                }
+                q[32 * kTapeL] = fma(h[0] - p[0], dl[0], fma(h[1] - p[1], dl[1], (h[2] - p[2]) * dl[2]));
+            }
         }
         p[0] = h[0]; p[1] = h[1]; p[2] = h[2];
         const bool flat = (S.flags & SF_FLAT_ONLY) != 0;
@@ -243,7 +252,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     r_back = (double)(rf * rf);
                 } else {
                     const double n_si = silicon_index(lam), mu = n_cur * rcp64(n_si);
-                    if constexpr (RECORD) fr->s[si].mu = mu;
+                    if constexpr (RECORD) fr->surface(si)[32 * kTapeMu] = mu;
                     if (!refract(dl, Nx, Ny, Nz, mu, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
                     const double ell = lerp_table(P.ell, P.n_ell, (lam - P.ell_lam0) * P.inv_ell_dlam);
                     L = ell * -log(u64of(w_conv));
@@ -290,7 +299,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 }
                 fx = fma(sigma, gxd, fx);
                 fy = fma(sigma, gyd, fy);
-                if constexpr (RECORD) fr->L = L;
+                if constexpr (RECORD) fr->end()[32 * kTapeDepth] = L;
             }
             R.x = fx; R.y = fy;
             if (FULL) {
@@ -380,7 +389,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 }
             }
             const double mu = n_cur * inv_next;
-            if constexpr (RECORD) fr->s[si].mu = mu;
+            if constexpr (RECORD) {
+                if (si >= fr->first) fr->surface(si)[32 * kTapeMu] = mu;
+            }
             if (!refract(dl, Nx, Ny, Nz, mu, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
             n_cur = n_next;
         }

@@ -333,7 +333,8 @@ __global__ void __launch_bounds__(256, 4) batch_kernel(const __grid_constant__ T
     }
 }
 
-template <bool MIXED>
+// TAPE: the forward state of every photon is kept for the adjoint
+template <bool MIXED, bool TAPE = false>
 __global__ void __launch_bounds__(32, 16) trace_batch_kernel(const __grid_constant__ TraceParams P,
                                                              const __grid_constant__ BatchList L) {
     const int lane = threadIdx.x;
@@ -351,7 +352,18 @@ __global__ void __launch_bounds__(32, 16) trace_batch_kernel(const __grid_consta
         const DSource& s = P.sources[src];
         PhotonOut R;
         R.flags = 0; R.pix = -1;
-        if (v) trace_photon<MIXED, false, true>(P, s, src, photon, R);
+        if constexpr (TAPE) {
+            ForwardRecord fr = forward_record(P, L, b < L.tape_batches ? b : L.tape_batches + blockIdx.x, lane);
+            if (v) {
+                trace_photon<MIXED, true, true>(P, s, src, photon, R, &fr);
+                double* q = fr.end();
+                q[32 * kTapeX] = R.x;
+                q[32 * kTapeY] = R.y;
+                q[32 * kTapeOn] = (R.flags & PHOSIM_F_DETECTED) ? 1.0 : 0.0;
+            }
+        } else {
+            if (v) trace_photon<MIXED, false, true>(P, s, src, photon, R);
+        }
         // the chief rays beside this kernel, whose reference points the moments take
         wait_for_previous();
         if (v && P.records) {
@@ -667,6 +679,8 @@ cudaError_t launch_batches(const TraceParams& P, const BatchList& L, int mode, i
     return cudaGetLastError();
 }
 cudaError_t launch_trace_batches(const TraceParams& P, const BatchList& L, int mode, int blocks, cudaStream_t st, bool beside) {
+    if (L.tape) return beside ? launch_beside(trace_batch_kernel<false, true>, blocks, 32, st, P, L)
+                              : (trace_batch_kernel<false, true><<<blocks, 32, 0, st>>>(P, L), cudaGetLastError());
     if (beside) return mode == kMixed ? launch_beside(trace_batch_kernel<true>, blocks, 32, st, P, L)
                                       : launch_beside(trace_batch_kernel<false>, blocks, 32, st, P, L);
     if (mode == kMixed) trace_batch_kernel<true><<<blocks, 32, 0, st>>>(P, L);
