@@ -520,14 +520,15 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
 // Q = c (x^2 + y^2) / 2 + (1 + kappa) c t^2 / 2 - t = 0, which needs no root: Newton's method on Q along the ray solves
 // it.  Any start near the root leads to it, so the ray moves in FP64 to the plane of the vertex and the start is found
 // from there on the idle FP32 pipe: the conic's root, and for the aspheric and Zernike surfaces Newton steps on the
-// sag, which leave about 1e-4 mm.  One FP64 evaluation finishes: the step s = Q / Q' with the second-order term of
+// sag, which leave about 1e-4 mm.  One FP64 evaluation of Q finishes: the step s = Q / Q' with the second-order term of
 // Chebyshev's method, s + Q'' s^2 / (2 Q'), leaves an error near (Q'' / Q')^2 s^3, and the gradient of Q, which is
-// along the normal, moves to the root with its derivative; both corrections are so small that single precision
-// carries them below the FP64 rounding of the results.  A step that is not that small is taken and followed by
-// another.  For a sphere the gradient has unit length on the surface.  A ray that grazes the conic takes the FP64 root.
+// along the normal, moves to the root with its derivative; the slope Q', which only scales the step, and both
+// corrections are taken in single precision, whose 1e-7 of the step stays below the FP64 rounding of the results.  A step
+// that is not that small is taken and followed by another.  For a sphere the gradient has unit length on the surface.  A ray that grazes the conic takes the FP64 root.
 // Measured (GB300, 300 stars, 2e7 photons, all FP64): 17.6 ms with the conic's FP64 root (a root and a quotient) and two
-// to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; on steep and
-// aspheric lenses the position error against the oracle fell from up to 9e-10 mm to 8e-13 mm.
+// to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; with the slope in
+// single precision 7.7 ms, 8.1 with an FP64 slope and its reciprocal.  On steep and aspheric lenses the position error
+// against the oracle fell from up to 9e-10 mm to 9e-13 mm, with either slope.
 // On success h is the point and N the unit normal (along (-S_x, -S_y, 1)); ahead says whether the distance is positive.
 __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS& E, const double p[3], const double d[3],
                                               double h[3], double N[3], bool& ahead) {
@@ -544,12 +545,12 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     // the ray from the plane of the vertex (rays nearly parallel to it stay where they are)
     const float lp = fabsf(dz) > 1e-3f ? -f32_trunc(p[2]) / dz : 0.f;
     const double lpd = f64_exact(lp);
-    const double q[3] = {fma(lpd, d[0], p[0]), fma(lpd, d[1], p[1]), fma(lpd, d[2], p[2])};
     const float A = fmaf(E.kmc.hi * dz, dz, E.c.hi);      // the quadric's l^2 coefficient for a unit direction
     bool started = false;
     float lf = 0.f;
     {
-        const float px = f32_trunc(q[0]), py = f32_trunc(q[1]), pz = f32_trunc(q[2]);
+        const float px = fmaf(lp, dx, f32_trunc(p[0])), py = fmaf(lp, dy, f32_trunc(p[1]));
+        const float pz = f32_trunc(fma(lpd, d[2], p[2]));
         const float c = E.c.hi, kc = E.kc.hi;
         const float bf = fmaf(kc * pz, dz, c * fmaf(px, dx, py * dy)) - dz;
         const float Cf = fmaf(kc * pz, pz, c * fmaf(px, px, py * py)) - 2.f * pz;
@@ -577,15 +578,21 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         }
     }
     double x, y, z;
-    {
-        double l0 = f64_exact(lf);
-        if (!started) {
-            l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2]);
-            if (!(fabs(l0) < 1e300)) return PHOSIM_LOST_MISSED;
-        }
+    const auto to_conic = [&] {
+        const double q[3] = {fma(lpd, d[0], p[0]), fma(lpd, d[1], p[1]), fma(lpd, d[2], p[2])};
+        const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2]);
+        if (!(fabs(l0) < 1e300)) return false;
         x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
-        ahead = lp + f32_trunc(l0) > 0.f;
+        lf = f32_trunc(l0);
+        return true;
+    };
+    if (started) {
+        const double l0 = lpd + f64_exact(lf);
+        x = fma(l0, d[0], p[0]); y = fma(l0, d[1], p[1]); z = fma(l0, d[2], p[2]);
+    } else if (!to_conic()) {
+        return PHOSIM_LOST_MISSED;
     }
+    ahead = lp + lf > 0.f;
     const float c = E.c.hi, kc = E.kc.hi;
 #pragma unroll 1
     for (int it = 0; it < 20; ++it) {
@@ -593,19 +600,26 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         double a = 0.0, ax = 0.0, ay = 0.0;
         float H[3] = {0.f, 0.f, 0.f};
         if (newton) aspheric(S, E, x, y, r2, a, ax, ay, H);
-        const double t = newton ? z - a : z, kt = S.kc * t, u = 1.0 - kt;
+        const double t = newton ? z - a : z, kt = S.kc * t;
         const double Q = fma(0.5 * S.c, r2, t * fma(0.5, kt, -1.0));
-        const double tl = newton ? fma(-ay, d[1], fma(-ax, d[0], d[2])) : d[2];          // dt / dl
-        const double Ql = fma(S.c, fma(x, d[0], y * d[1]), -(u * tl));
-        if ((__double2hiint(Ql) & 0x7fffffff) < 0x00100000) return newton ? PHOSIM_LOST_NEWTON : PHOSIM_LOST_MISSED;
-        const double inv = rcp64(Ql), s = Q * inv;
-        const float sf = f32_trunc(s), invf = f32_trunc(inv), uf = f32_trunc(u), tlf = newton ? f32_trunc(tl) : dz;
+        // the slope Q' along the ray only scales the step: in single precision unless it is small (t' = dt / dl)
+        const float uf = fmaf(-kc, f32_trunc(t), 1.f);
+        const float tlf = newton ? fmaf(-f32_trunc(ay), dy, fmaf(-f32_trunc(ax), dx, dz)) : dz;
+        const float Qlf = fmaf(c, fmaf(f32_trunc(x), dx, f32_trunc(y) * dy), -(uf * tlf));
+        float invf = 1.f / Qlf, sf = f32_trunc(Q) * invf;
+        if (!(fabsf(Qlf) > 0.01f)) {
+            const double tl = newton ? fma(-ay, d[1], fma(-ax, d[0], d[2])) : d[2];
+            const double Ql = fma(S.c, fma(x, d[0], y * d[1]), -((1.0 - kt) * tl));
+            if ((__double2hiint(Ql) & 0x7fffffff) < 0x00100000) return newton ? PHOSIM_LOST_NEWTON : PHOSIM_LOST_MISSED;
+            invf = f32_trunc(rcp64(Ql));
+            sf = f32_trunc(Q * rcp64(Ql));
+        }
         const float hx = fmaf(H[0], dx, H[1] * dy), hy = fmaf(H[1], dx, H[2] * dy);
         // Q'' along the ray, and the step with its second-order term
         const float Qll = fmaf(c, fmaf(dx, dx, dy * dy), fmaf(kc * tlf, tlf, uf * fmaf(hx, dx, hy * dy)));
         const float k = Qll * invf * sf, more = 0.5f * k * sf;
-        const bool last = (!newton || fabsf(sf) < 1e-3f) && fabsf(more * k) < 1e-14f;
-        const double step = s + f64_exact(more);
+        const bool last = fabsf(sf) < 1e-3f && fabsf(more * k) < 1e-14f;
+        const double step = f64_exact(sf + more);
         x = fma(-step, d[0], x); y = fma(-step, d[1], y); z = fma(-step, d[2], z);
         if (last || fabsf(sf) < 1e-8f) {
             h[0] = x; h[1] = y; h[2] = z;
@@ -618,6 +632,7 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
                     return PHOSIM_LOST_MISSED;
                 // minus the gradient of Q at the evaluated point, moved to the root: it changes by -s times its derivative
                 const float ul = -kc * tlf;
+                const double u = 1.0 - kt;
                 N[0] = fma(-S.c, x, fma(-u, ax, f64_exact(sf * fmaf(ul, f32_trunc(ax), uf * hx))));
                 N[1] = fma(-S.c, y, fma(-u, ay, f64_exact(sf * fmaf(ul, f32_trunc(ay), uf * hy))));
                 N[2] = u - f64_exact(sf * ul);
@@ -628,11 +643,7 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         }
         if (!(fabsf(sf) < 1e37f)) return PHOSIM_LOST_NEWTON;
         // the start was too far off (a ray that grazes the conic): the conic's FP64 root
-        if (!newton && started && it == 0) {
-            const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2]);
-            if (!(fabs(l0) < 1e300)) return PHOSIM_LOST_MISSED;
-            x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
-        }
+        if (!newton && started && it == 0 && !(fabsf(more * k) < 1e-14f) && !to_conic()) return PHOSIM_LOST_MISSED;
     }
     return PHOSIM_LOST_NEWTON;
 }
