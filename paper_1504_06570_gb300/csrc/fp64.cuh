@@ -9,6 +9,7 @@
 // Arguments are finite, non-zero and far from the ends of the exponent range where not said otherwise.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -75,6 +76,41 @@ __device__ __forceinline__ bool floor_product64(double s, double k, double& fl, 
     fl = t - 6755399441055744.0;
     i = __double2loint(t);
     return true;
+}
+
+// s k for a factor k = m 2^(E - 63) (m its significand in the top 53 bits, factor64) by integers: the floor, and the first
+// 52 bits after it.  s is taken to 2^-40 (finer than the rounding of a position in millimetres beyond 4 m) and below 2^22;
+// false beyond, or where the factor has no integer form (shift 0).
+__device__ __forceinline__ bool split_product64(double s, unsigned long long m, int shift, int& i, unsigned long long& frac) {
+    const uint32_t hi = (uint32_t)__double2hiint(s), lo = (uint32_t)__double2loint(s), e = (hi >> 20) & 0x7ffu;
+    if (e >= 1023u + 22u || shift == 0) return false;
+    // |s| = norm 2^(e - 1023 - 63), and in units of 2^-40
+    const unsigned long long norm = ((unsigned long long)(((hi & 0xfffffu) | 0x100000u) << 11 | lo >> 21) << 32) | (unsigned long long)(lo << 11);
+    const unsigned long long fixed = norm >> min(1023u + 23u - e, 63u);
+    unsigned long long ph = __umul64hi(fixed, m), pl = fixed * m;
+    if ((int)hi < 0) { pl = 0ull - pl; ph = ~ph + (pl == 0ull); }
+    i = (int)((long long)ph >> (shift - 12));
+    frac = shift < 64 ? (ph << (64 - shift)) | (pl >> shift) : (unsigned long long)((long long)ph >> (shift - 64));
+    frac &= 0xfffffffffffffull;
+    return true;
+}
+// 1 + the fraction of 52 bits, exact
+__device__ __forceinline__ double one_and_fraction64(unsigned long long frac) {
+    return __longlong_as_double((long long)(frac | 0x3ff0000000000000ull));
+}
+// the fraction in single precision, rounded to nearest (above 2^-21): its first 23 bits, and the next 23 with a last one
+// that says whether any is left, which are exact, in one sum
+__device__ __forceinline__ float fraction_f32(unsigned long long frac) {
+    const uint32_t head = (uint32_t)(frac >> 29), tail = (uint32_t)frac & 0x1fffffffu;
+    return fmaf((float)(tail >> 5 | (uint32_t)((tail & 31u) != 0u)), 0x1p-47f, (float)head * 0x1p-23f);
+}
+// m and shift of a factor k > 0 for split_product64; shift 0: it has none
+inline void factor64(double k, unsigned long long& m, int& shift) {
+    int x = 0;
+    const double f = std::frexp(k, &x);                  // k = f 2^x, f in [1/2, 1)
+    m = (unsigned long long)std::ldexp(f, 53) << 11;
+    shift = 51 - (x - 1);
+    if (!(k > 0.0) || shift < 43 || shift > 75) { m = 0; shift = 0; }
 }
 
 }  // namespace phosim

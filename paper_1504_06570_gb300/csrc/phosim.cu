@@ -282,10 +282,12 @@ __global__ void gradient_screen_kernel(const double* __restrict__ ph, int n, dou
     const double2 a = central_gradient(ph, n, two_pix, i, j), b = central_gradient(ph, n, two_pix, i1, j);
     const double2 c = central_gradient(ph, n, two_pix, i, j1), d = central_gradient(ph, n, two_pix, i1, j1);
     const size_t node = (size_t)j * n + i;
-    g64[4 * node] = a;
-    g64[4 * node + 1] = make_double2(b.x - a.x, b.y - a.y);
-    g64[4 * node + 2] = make_double2(c.x - a.x, c.y - a.y);
-    g64[4 * node + 3] = make_double2((a.x - b.x) + (d.x - c.x), (a.y - b.y) + (d.y - c.y));
+    const double2 p = make_double2(b.x - a.x, b.y - a.y), q = make_double2(c.x - a.x, c.y - a.y);
+    const double2 r = make_double2((d.x - c.x) - p.x, (d.y - c.y) - p.y);
+    g64[4 * node] = make_double2(a.x - p.x - (q.x - r.x), a.y - p.y - (q.y - r.y));
+    g64[4 * node + 1] = make_double2(p.x - r.x, p.y - r.y);
+    g64[4 * node + 2] = make_double2(q.x - r.x, q.y - r.y);
+    g64[4 * node + 3] = r;
     g32[2 * node] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
     g32[2 * node + 1] = make_float4((float)c.x, (float)c.y, (float)d.x, (float)d.y);
 }
@@ -788,6 +790,7 @@ phosim_status phosim_load_screens(phosim_scene* sc, const phosim_layer* layers, 
             D.s[q].n = S.n;
             D.s[q].inv_pix = 1.0 / S.pixel;
             D.s[q].inv_pix_s = ds_of(1.0 / S.pixel);
+            factor64(1.0 / S.pixel, D.s[q].inv_m, D.s[q].inv_shift);
             D.s[q].g64 = (const double2*)g64;
             D.s[q].g32 = (const float4*)g32;
         }

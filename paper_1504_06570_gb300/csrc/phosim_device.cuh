@@ -86,11 +86,12 @@ constexpr int kMaxGhostBounces = PHOSIM_MAX_GHOST_BOUNCES;
 // nodes the bilinear interpolation needs, (i, j), (i+1, j), (i, j+1), (i+1, j+1) (periodic): one lookup is
 // one aligned 32-byte (FP32) or 64-byte (FP64) read instead of two rows of scattered 8- or 16-byte taps.
 struct DScale {
-    int n, pad;
+    int n, inv_shift;
     double inv_pix;
+    unsigned long long inv_m;                 // inv_pix as a factor of integers (factor64), with inv_shift
     ds inv_pix_s;
-    const double2* g64;                       // 4 double2 per node, n x n nodes: g00, g10 - g00, g01 - g00 and
-                                              // g00 - g10 - g01 + g11, the bilinear form's coefficients
+    const double2* g64;                       // 4 double2 per node, n x n nodes: the bilinear form's coefficients of 1, X, Y
+                                              // and X Y, where X and Y are 1 + the distance from the node in pixels
     const float4* g32;                        // 2 float4 per node: (g00, g10), (g01, g11)
 };
 
