@@ -535,7 +535,7 @@ phosim_status phosim_create_scene(const phosim_scene_desc* d, phosim_scene** out
     P.ell_lam0 = d->ell_lam0; P.inv_ell_dlam = 1.0 / d->ell_dlam;
     P.n_ell = d->n_ell; P.n_sig = d->n_sigma;
     P.sig_scale = (d->n_sigma - 1) / d->t_si;
-    P.dead_layer = d->dead_layer;
+    P.dead_layer = d->dead_layer + 0.0;      // (-0 is 0)
     // fringing: optical thickness t_si + gx (x - x0) + gy (y - y0) = fr_t0 + gx x + gy y
     P.fr_gx = d->t_si_gx; P.fr_gy = d->t_si_gy;
     P.fr_t0 = d->t_si - d->t_si_gx * d->x0 - d->t_si_gy * d->y0;
@@ -543,7 +543,8 @@ phosim_status phosim_create_scene(const phosim_scene_desc* d, phosim_scene** out
     P.pr_in2_s = ds_of(P.pr_in2); P.pr_dr2_s = ds_of(P.pr_dr2);
     P.h_top_s = ds_of(P.h_top); P.z_ent_s = ds_of(P.z_ent);
     P.xlo_s = ds_of(P.xlo); P.ylo_s = ds_of(P.ylo); P.inv_pixel_s = ds_of(P.inv_pixel);
-    P.chip_w_s = ds_of(P.nx * P.pixel); P.chip_h_s = ds_of(P.ny * P.pixel);
+    P.chip_w = P.nx * P.pixel; P.chip_h = P.ny * P.pixel;
+    P.chip_w_s = ds_of(P.chip_w); P.chip_h_s = ds_of(P.chip_h);
     P.kick0f = (float)P.kick0; P.inv_lam_ref_f = (float)(1.0 / P.lam_ref);
     P.t_sif = (float)P.t_si; P.dead_layerf = (float)P.dead_layer;
     P.ell_lam0f = (float)P.ell_lam0; P.inv_ell_dlamf = (float)P.inv_ell_dlam; P.sig_scalef = (float)P.sig_scale;

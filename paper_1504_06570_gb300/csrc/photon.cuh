@@ -124,9 +124,16 @@ __device__ __forceinline__ double inverse_nz(double nx, double ny) {
 }
 
 __device__ __forceinline__ double lerp_table(const double* __restrict__ t, int n, double f) {
-    int k = __double2int_rd(f);
-    k = k < 0 ? 0 : (k > n - 2 ? n - 2 : k);
-    const double w = fmin(fmax(f - (double)k, 0.0), 1.0), a = __ldg(t + k);
+    int k = 0;
+    double fl = 0.0;
+    const bool found = floor_product64(f, 1.0, fl, k);
+    double w = f - fl;
+    if (!found || k < 0 || k > n - 2) {              // off the table: its first or last value
+        const bool last = found ? k > 0 : f > 0.0;
+        k = last ? n - 2 : 0;
+        w = last ? 1.0 : 0.0;
+    }
+    const double a = __ldg(t + k);
     return fma(w, __ldg(t + k + 1) - a, a);
 }
 __device__ __forceinline__ float lerp_table_f(const float* __restrict__ t, int n, float f) {
@@ -241,7 +248,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 w_conv = mb->conv; w_diff_a = mb->diff_a; w_diff_b = mb->diff_b; w_back = mb->back;
             }
             const double hx = p[0] - P.xlo, hy = p[1] - P.ylo;
-            if (FULL && !(hx >= 0.0 && hy >= 0.0 && hx < P.nx * P.pixel && hy < P.ny * P.pixel)) {
+            if (FULL && !(within64(hx, P.chip_w) && within64(hy, P.chip_h))) {
                 R.flags = lost(PHOSIM_LOST_OFF_CHIP, si);
                 return;
             }
@@ -268,7 +275,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     r_back = rf * rf;
                 }
                 double depth = L * fabs(dl[2]);
-                if (!(depth <= P.t_si)) {
+                if (!(within64(depth, P.t_si) || depth == P.t_si)) {
                     // back-side reflection: the photon turns round at the back and converts on its way back
                     bool back = false;
                     if (P.flags & PHOSIM_BACK_REFLECT) {
@@ -287,7 +294,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     if (!back) { R.flags = lost(PHOSIM_LOST_NOT_CONVERTED, si); return; }
                 }
                 // field-free dead layer at the entrance: the charge is not collected
-                if (depth < P.dead_layer) { R.flags = lost(PHOSIM_LOST_DEAD_LAYER, si); return; }
+                if (within64(depth, P.dead_layer)) { R.flags = lost(PHOSIM_LOST_DEAD_LAYER, si); return; }
                 fx = fma(L, dl[0], fx);
                 fy = fma(L, dl[1], fy);
                 R.xc = fx; R.yc = fy;
@@ -300,7 +307,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     sigma = 1.0; gxd = (double)(sg * g * cs); gyd = (double)(sg * g * sn);
                 } else {
                     sigma = lerp_table(P.sig, P.n_sig, depth * P.sig_scale);
-                    const double g = sqrt(-2.0 * log(u64of(w_diff_a)));
+                    const double g = sqrt64_pos(-2.0 * log(u64of(w_diff_a)));
                     double sn, cs;
                     sincospi(2.0 * u64of(w_diff_b), &sn, &cs);
                     gxd = g * cs; gyd = g * sn;
@@ -312,8 +319,10 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
             R.x = fx; R.y = fy;
             if (FULL) {
                 const double ux = fx - P.xlo, uy = fy - P.ylo;
-                // (conversions saturate; a NaN becomes the most negative integer)
-                const int px = __double2int_rd(ux * P.inv_pixel), py = __double2int_rd(uy * P.inv_pixel);
+                int px = -1, py = -1;
+                double fl;
+                floor_product64(ux, P.inv_pixel, fl, px);
+                floor_product64(uy, P.inv_pixel, fl, py);
                 if (!(px >= 0 && py >= 0 && px < P.nx && py < P.ny)) {
                     R.flags = lost(PHOSIM_LOST_OFF_CHIP, si);
                     return;
@@ -334,8 +343,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 clear = r2 <= S.r_out2 && r2 >= S.r_in2;
             }
             if (!clear) { R.flags = lost(PHOSIM_LOST_VIGNETTED, si); return; }
-            // coating accept-reject at the incidence angle and wavelength
-            if (S.coat_slot >= 0) {
+            // coating accept-reject at the incidence angle and wavelength.  A coating of one angle bin, without ghosts, has
+            // decided in the dynamic transmission test (early_coating_reject: the same draw, bin and threshold).
+            if (S.coat_slot >= 0 && !((P.flags & PHOSIM_EARLY_REJECT) && !ghosts && P.coat[S.coating].nt == 1)) {
                 const DCoating& C = P.coat[S.coating];
                 int it = 0;
                 if (C.nt > 1) {
