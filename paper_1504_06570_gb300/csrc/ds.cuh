@@ -80,6 +80,18 @@ __device__ __forceinline__ ds operator*(ds a, float b) {
     return fast_two_sum(p, e);
 }
 
+// a / b and sqrt(a) (a > 0) in single precision for operands whose quotient, reciprocal and root are far from the ends of
+// the exponent range: the hardware's approximation and one correction by the exact remainder (Markstein 1990), which
+// gives the correctly rounded value but for about one operand in 1e6.  Without the range checks and their branch a
+// quotient is 4 instructions.
+__device__ __forceinline__ float quotient_f(float a, float b) {
+    const float r = __fdividef(1.f, b), q = __fmul_rn(a, r);
+    return __fmaf_rn(__fmaf_rn(-q, b, a), r, q);
+}
+__device__ __forceinline__ float root_f(float a) {
+    const float y = rsqrtf(a), s = __fmul_rn(a, y);
+    return __fmaf_rn(__fmaf_rn(-s, s, a), __fmul_rn(0.5f, y), s);
+}
 // 1 - x for |x| <= 1: exact ordering of the operands, so Dekker's sum gives what Knuth's does (for x > 1 the sign
 // is right and the value is not used)
 __device__ __forceinline__ ds one_minus(ds x) {

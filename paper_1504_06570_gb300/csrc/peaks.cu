@@ -277,7 +277,7 @@ extern "C" phosim_status phosim_ds_eval(int op, const double* a, const double* b
 }
 
 namespace {
-__global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, unsigned long long m, int shift) {
+__global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, double factor, unsigned long long m, int shift) {
     using namespace phosim;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -294,6 +294,8 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, un
         case 6: out[i] = floor_product64(x, 1.0, f, k) ? f : 0.5; break;
         case 7: out[i] = floor_product64(x, 1.0, f, k) ? (double)k : 0.5; break;
         case 8: out[i] = u64of((uint32_t)x); break;
+        case 12: out[i] = (double)quotient_f((float)x, (float)factor); break;
+        case 13: out[i] = (double)root_f((float)x); break;
         default: {
             unsigned long long frac = 0;
             if (!split_product64(x, m, shift, k, frac)) out[i] = -1.0;
@@ -304,7 +306,7 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, un
 }  // namespace
 
 extern "C" phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n) {
-    if (op < 0 || op > 11 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
+    if (op < 0 || op > 13 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
     const size_t bytes = (size_t)n * sizeof(double);
     double* d = nullptr;
     if (cudaMalloc(&d, bytes) != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_OUT_OF_MEMORY; }
@@ -312,8 +314,8 @@ extern "C" phosim_status phosim_fp64_eval(int op, const double* a, double* out, 
     if (e == cudaSuccess) {
         unsigned long long m = 0;
         int shift = 0;
-        if (op >= 9) phosim::factor64(out[0], m, shift);
-        fp64_eval_kernel<<<(n + 127) / 128, 128>>>(op, d, d, n, m, shift);
+        if (op >= 9 && op <= 11) phosim::factor64(out[0], m, shift);
+        fp64_eval_kernel<<<(n + 127) / 128, 128>>>(op, d, d, n, out[0], m, shift);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(out, d, bytes, cudaMemcpyDeviceToHost);

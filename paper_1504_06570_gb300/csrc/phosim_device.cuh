@@ -459,7 +459,7 @@ __device__ __forceinline__ bool sag_f(const DSurfaceS& E, int flags, float x, fl
         const float arg = fmaf(-E.k1c2.hi, r2, 1.f);
         if (arg < 0.f) return false;
         const float rs = rsqrtf(arg);
-        z = E.c.hi * r2 / fmaf(arg, rs, 1.f);
+        z = quotient_f(E.c.hi * r2, fmaf(arg, rs, 1.f));
         g = E.c.hi * rs;
     }
     if (flags & SF_EVEN) {
@@ -663,7 +663,7 @@ __device__ __forceinline__ double silicon_index(double lam_nm) {
     return fma(2.79, exp((E - 3.30) * (1.0 / 0.398)), fma(0.211, E, 3.36));
 }
 __device__ __forceinline__ float silicon_index_f(float lam_nm) {
-    const float E = 1239.841984f / lam_nm;
+    const float E = quotient_f(1239.841984f, lam_nm);
     return 3.36f + 0.211f * E + 2.79f * expf((E - 3.30f) * (1.0f / 0.398f));
 }
 

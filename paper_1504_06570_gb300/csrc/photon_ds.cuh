@@ -353,10 +353,10 @@ static __device__ PHOSIM_DS_STEP uint32_t intersect_ds(const DSurfaceS& E, int f
         const float Cf = fmaf(kc * p[2].hi, p[2].hi, c * fmaf(p[0].hi, p[0].hi, p[1].hi * p[1].hi)) - 2.f * p[2].hi;
         const float disc = fmaf(bf, bf, -(Af * Cf));
         if (disc > 1e-6f * bf * bf) {
-            const float sq = sqrtf(disc);
+            const float sq = root_f(disc);
             const float qf = bf >= 0.f ? -(bf + sq) : sq - bf;
-            float lf = Cf / qf;
-            if (Af != 0.f && fmaf(-kc, fmaf(lf, d[2].hi, p[2].hi), 1.f) < 0.f) lf = qf / Af;
+            float lf = quotient_f(Cf, qf);
+            if (Af != 0.f && fmaf(-kc, fmaf(lf, d[2].hi, p[2].hi), 1.f) < 0.f) lf = quotient_f(qf, Af);
             if (newton) {
 #pragma unroll 1
                 for (int it = 0; it < 4; ++it) {
@@ -364,7 +364,7 @@ static __device__ PHOSIM_DS_STEP uint32_t intersect_ds(const DSurfaceS& E, int f
                     float zs, zxf, zyf;
                     if (!sag_f(E, flags, x, y, zs, zxf, zyf)) break;
                     const float dF = d[2].hi - zxf * d[0].hi - zyf * d[1].hi;
-                    const float step = (fmaf(lf, d[2].hi, p[2].hi) - zs) / dF;
+                    const float step = quotient_f(fmaf(lf, d[2].hi, p[2].hi) - zs, dF);
                     if (!(fabsf(step) < 1e30f)) break;
                     lf -= step;
                     if (fabsf(step) < 1e-2f) break;
@@ -381,7 +381,7 @@ static __device__ PHOSIM_DS_STEP uint32_t intersect_ds(const DSurfaceS& E, int f
         const ds Q = dfma(E.c, dfma(x, x, y * y), dfma(E.kc * z, z, z * -2.f));
         const float dQ = 2.f * (fmaf(E.c.hi, fmaf(x.hi, d[0].hi, y.hi * d[1].hi), E.kc.hi * z.hi * d[2].hi) - d[2].hi);
         started = dQ != 0.f;
-        if (started) l = l - Q.hi / dQ;
+        if (started) l = l - quotient_f(Q.hi, dQ);
     }
     if (!started) {
         l = conic_root_ds(E, p[0], p[1], p[2], d[0], d[1], d[2]);
