@@ -38,11 +38,12 @@ __device__ __forceinline__ double sqrt64_pos(double a) {
     const double y = rsqrt_seed64(a), s = a * y, e = fma(-s, y, 1.0);
     return fma(s * e, fma(0.375, e, 0.5), s);
 }
-// sign tests on the high word, and 0 <= a < b by the order of the words (a double comparison takes the FP64 pipe; a NaN
-// is not below, and -0 not above 0)
+// sign tests on the high word, and 0 <= a < b for b > 0 by the order of the words (a double comparison takes the FP64
+// pipe); -0 is 0, and a NaN is not below
 __device__ __forceinline__ bool negative64(double a) { return __double2hiint(a) < 0; }
 __device__ __forceinline__ bool within64(double a, double b) {
-    return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
+    const unsigned long long u = (unsigned long long)__double_as_longlong(a);
+    return u < (unsigned long long)__double_as_longlong(b) || u == 1ull << 63;
 }
 // sqrt(a) for a >= 0; numbers below 1e-290 give 0
 __device__ __forceinline__ double sqrt64(double a) { return __double2hiint(a) > 0x03c00000 ? sqrt64_pos(a) : 0.0; }

@@ -535,7 +535,7 @@ phosim_status phosim_create_scene(const phosim_scene_desc* d, phosim_scene** out
     P.ell_lam0 = d->ell_lam0; P.inv_ell_dlam = 1.0 / d->ell_dlam;
     P.n_ell = d->n_ell; P.n_sig = d->n_sigma;
     P.sig_scale = (d->n_sigma - 1) / d->t_si;
-    P.dead_layer = d->dead_layer + 0.0;      // (-0 is 0)
+    P.dead_layer = d->dead_layer;
     // fringing: optical thickness t_si + gx (x - x0) + gy (y - y0) = fr_t0 + gx x + gy y
     P.fr_gx = d->t_si_gx; P.fr_gy = d->t_si_gy;
     P.fr_t0 = d->t_si - d->t_si_gx * d->x0 - d->t_si_gy * d->y0;

@@ -275,7 +275,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     r_back = rf * rf;
                 }
                 double depth = L * fabs(dl[2]);
-                if (!(within64(depth, P.t_si) || depth == P.t_si)) {
+                if (!(depth <= P.t_si)) {
                     // back-side reflection: the photon turns round at the back and converts on its way back
                     bool back = false;
                     if (P.flags & PHOSIM_BACK_REFLECT) {
@@ -294,7 +294,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     if (!back) { R.flags = lost(PHOSIM_LOST_NOT_CONVERTED, si); return; }
                 }
                 // field-free dead layer at the entrance: the charge is not collected
-                if (within64(depth, P.dead_layer)) { R.flags = lost(PHOSIM_LOST_DEAD_LAYER, si); return; }
+                if (depth < P.dead_layer) { R.flags = lost(PHOSIM_LOST_DEAD_LAYER, si); return; }
                 fx = fma(L, dl[0], fx);
                 fy = fma(L, dl[1], fy);
                 R.xc = fx; R.yc = fy;
