@@ -1,5 +1,6 @@
 // FMA issue-rate probe (the denominator of the arithmetic roofline of the photon kernels) and the check
 // entries of phosim_bench.h: the device Philox and the double-single primitives.
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "phosim_bench.h"
@@ -277,7 +278,7 @@ extern "C" phosim_status phosim_ds_eval(int op, const double* a, const double* b
 }
 
 namespace {
-__global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, double factor, unsigned long long m, int shift) {
+__global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, double factor, unsigned long long m, int shift, const double* table) {
     using namespace phosim;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -296,6 +297,7 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, do
         case 8: out[i] = u64of((uint32_t)x); break;
         case 12: out[i] = (double)quotient_f((float)x, (float)factor); break;
         case 13: out[i] = (double)root_f((float)x); break;
+        case 14: out[i] = log_draw64(table, (uint32_t)x); break;
         default: {
             unsigned long long frac = 0;
             if (!split_product64(x, m, shift, k, frac)) out[i] = -1.0;
@@ -306,16 +308,20 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, do
 }  // namespace
 
 extern "C" phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n) {
-    if (op < 0 || op > 13 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
+    if (op < 0 || op > 14 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
     const size_t bytes = (size_t)n * sizeof(double);
+    std::vector<double> table(phosim::kLogTable + 34);
+    phosim::log_table(table.data());
     double* d = nullptr;
-    if (cudaMalloc(&d, bytes) != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_OUT_OF_MEMORY; }
+    if (cudaMalloc(&d, bytes + (table.size() + 1) * sizeof(double)) != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_OUT_OF_MEMORY; }
+    double* const dt = d + n + (n & 1);          // its pairs on 16 bytes
     cudaError_t e = cudaMemcpy(d, a, bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(dt, table.data(), table.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         unsigned long long m = 0;
         int shift = 0;
         if (op >= 9 && op <= 11) phosim::factor64(out[0], m, shift);
-        fp64_eval_kernel<<<(n + 127) / 128, 128>>>(op, d, d, n, out[0], m, shift);
+        fp64_eval_kernel<<<(n + 127) / 128, 128>>>(op, d, d, n, out[0], m, shift, dt);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(out, d, bytes, cudaMemcpyDeviceToHost);

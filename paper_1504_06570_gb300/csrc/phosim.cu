@@ -566,6 +566,12 @@ phosim_status phosim_create_scene(const phosim_scene_desc* d, phosim_scene** out
     P.ell = pd;
     if ((st = upload(sc->table_mem, f.data(), f.size(), &pf)) != PHOSIM_OK) goto fail;
     P.ell32 = pf;
+    {
+        std::vector<double> table(kLogTable + 34);
+        log_table(table.data());
+        if ((st = upload(sc->table_mem, table.data(), table.size(), &pd)) != PHOSIM_OK) goto fail;
+        P.log_table = pd;
+    }
     if ((st = upload(sc->table_mem, d->sigma, (size_t)d->n_sigma, &pd)) != PHOSIM_OK) goto fail;
     P.sig = pd;
     if ((st = upload(sc->table_mem, g.data(), g.size(), &pf)) != PHOSIM_OK) goto fail;

@@ -181,7 +181,7 @@ __device__ __forceinline__ MemberDraw member_draw(const TraceParams& P, double b
         m.sx = (double)((float)bsig * g * cs);
         m.sy = (double)((float)bsig * g * sn);
     } else {
-        const double g = sqrt(-2.0 * log(u64of(m5.x)));
+        const double g = sqrt64_pos(-2.0 * log_draw64(P.log_table, m5.x));
         double sn, cs;
         sincospi(2.0 * u64of(m5.y), &sn, &cs);
         m.sx = bsig * g * cs;
@@ -270,7 +270,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     if constexpr (RECORD) fr->surface(si)[32 * kTapeMu] = mu;
                     if (!refract(dl, Nx, Ny, Nz, mu, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
                     const double ell = lerp_table(P.ell, P.n_ell, (lam - P.ell_lam0) * P.inv_ell_dlam);
-                    L = ell * -log(u64of(w_conv));
+                    L = ell * -log_draw64(P.log_table, w_conv);
                     const double rf = (n_si - 1.0) / (n_si + 1.0);
                     r_back = rf * rf;
                 }
@@ -307,7 +307,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     sigma = 1.0; gxd = (double)(sg * g * cs); gyd = (double)(sg * g * sn);
                 } else {
                     sigma = lerp_table(P.sig, P.n_sig, depth * P.sig_scale);
-                    const double g = sqrt64_pos(-2.0 * log(u64of(w_diff_a)));
+                    const double g = sqrt64_pos(-2.0 * log_draw64(P.log_table, w_diff_a));
                     double sn, cs;
                     sincospi(2.0 * u64of(w_diff_b), &sn, &cs);
                     gxd = g * cs; gyd = g * sn;
@@ -524,7 +524,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
             nx += (double)((float)s.a * g * cp);
             ny += (double)((float)s.a * g * sp);
         } else {
-            const double g = sqrt(-2.0 * log(u64of(w1.y)));
+            const double g = sqrt64_pos(-2.0 * log_draw64(P.log_table, w1.y));
             double sp, cp;
             sincospi(2.0 * u64of(w1.z), &sp, &cp);
             nx += s.a * g * cp;
