@@ -59,7 +59,7 @@ phosim_status phosim_ds_eval(int op, const double* a, const double* b, double* o
    single precision, 5 the single-precision a as a double, 6 floor(a), 7 the integer floor(a), 8 (a + 1/2) 2^-32 of
    the 32-bit integer a; and of a k with the factor k = out[0] as the caller leaves it: 9 the floor, 10 the fraction,
    11 the fraction in single precision (-1: beyond the form's range); 12 a / k and 13 sqrt(a) in single precision;
-   14 log of 8.  a, out: host, n values.  Errors: INVALID_ARGUMENT (unknown op, null pointer, n < 1),
+   14 log of 8, 15 and 16 sin and cos of 2 pi times it.  a, out: host, n values.  Errors: INVALID_ARGUMENT (unknown op, null pointer, n < 1),
    OUT_OF_MEMORY, CUDA. */
 phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n);
 

@@ -126,7 +126,21 @@ __device__ __forceinline__ double log_draw64(const double* __restrict__ table, u
     const double p = fma(r, fma(r, f64_exact(q), 1.0 / 3.0), -0.5);
     return (te + t.y) + fma(r * r, p, r);
 }
-inline void log_table(double* table) {
+// sin and cos of 2 pi (w + 1/2) 2^-32: the nearest of 256 tabulated angles and the rest a, |a| < 0.0123, by the series of
+// sin a and cos a - 1 (tails in single precision) and the addition theorems.  Fourteen operations on the FP64 pipe.
+constexpr int kSinTable = kLogTable + 34, kDrawTable = kSinTable + 512;     // 256 (sin, cos) pairs after the logarithm's
+__device__ __forceinline__ void sincos_draw64(const double* __restrict__ table, uint32_t w, double& sn, double& cs) {
+    const double2 t = __ldg((const double2*)(table + kSinTable) + ((w + 0x800000u) >> 24));
+    const int d = (int)(w << 8) >> 8;                                       // w less the tabulated angle's draw
+    const double turn = __hiloint2double(0x41300000, d + 0x800000) - (1048576.0 + 0x1p-9);     // d 2^-32
+    const double a = fma(turn, 6.283185307179586477, 7.314590396335798e-10), a2 = a * a;
+    const float f = f32_trunc(a2);
+    const double s = fma(a * a2, fma(a2, f64_exact(fmaf(f, -1.f / 5040.f, 1.f / 120.f)), -1.0 / 6.0), a);
+    const double c = a2 * fma(a2, f64_exact(fmaf(f, -1.f / 720.f, 1.f / 24.f)), -0.5);
+    sn = t.x + fma(t.y, s, t.x * c);
+    cs = t.y + fma(-t.x, s, t.y * c);
+}
+inline void draw_table(double* table) {
     for (int i = 0; i < 1 << kLogBits; ++i) {
         const bool half = i >= kLogHalf;
         const double mid = 1.0 + (i + 0.5) / (1 << kLogBits), c = i + 1 == 1 << kLogBits ? 0.5 : std::rint(4096.0 / mid) / 4096.0;
@@ -134,6 +148,16 @@ inline void log_table(double* table) {
         table[2 * i + 1] = -std::log(half ? 2.0 * c : c);
     }
     for (int e = 0; e < 34; ++e) table[kLogTable + e] = -e * 0.69314718055994530942;
+    // the first octant's values, and the others by symmetry (exact zeros and ones on the axes)
+    for (int j = 0; j < 256; ++j) {
+        const int quarter = j >> 6, k = j & 63, o = k > 32 ? 64 - k : k;
+        const double angle = o * (3.14159265358979323846 / 128.0), so = std::sin(angle), co = std::cos(angle);
+        const double sk = k > 32 ? co : so, ck = k > 32 ? so : co;
+        const double sv = quarter == 0 ? sk : quarter == 1 ? ck : quarter == 2 ? -sk : -ck;
+        const double cv = quarter == 0 ? ck : quarter == 1 ? -sk : quarter == 2 ? -ck : sk;
+        table[kSinTable + 2 * j] = sv;
+        table[kSinTable + 2 * j + 1] = cv;
+    }
 }
 
 // m and shift of a factor k > 0 for split_product64; shift 0: it has none

@@ -19,7 +19,7 @@
 // intersections recomputed in the sweep; 5.6 ms without; 3.8 ms with the photons in batches; 3.2 ms with force and
 // torque for the nine elements of each matrix's adjoint, and the figure's second derivatives from their own
 // coefficients; 2.5 ms with the forward states kept (a photon's 1.1 KB written and read once, against 40 % of the sweep's
-// FP64 operations).
+// FP64 operations); 2.3 ms with the forward pass as it is now.
 #include "phosim_device.cuh"
 #include "phosim_scene.hpp"
 #include "photon.cuh"

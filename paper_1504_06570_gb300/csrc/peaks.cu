@@ -298,6 +298,8 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, do
         case 12: out[i] = (double)quotient_f((float)x, (float)factor); break;
         case 13: out[i] = (double)root_f((float)x); break;
         case 14: out[i] = log_draw64(table, (uint32_t)x); break;
+        case 15: sincos_draw64(table, (uint32_t)x, out[i], f); break;
+        case 16: sincos_draw64(table, (uint32_t)x, f, out[i]); break;
         default: {
             unsigned long long frac = 0;
             if (!split_product64(x, m, shift, k, frac)) out[i] = -1.0;
@@ -308,10 +310,10 @@ __global__ void fp64_eval_kernel(int op, const double* a, double* out, int n, do
 }  // namespace
 
 extern "C" phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n) {
-    if (op < 0 || op > 14 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
+    if (op < 0 || op > 16 || !a || !out || n < 1) return PHOSIM_ERR_INVALID_ARGUMENT;
     const size_t bytes = (size_t)n * sizeof(double);
-    std::vector<double> table(phosim::kLogTable + 34);
-    phosim::log_table(table.data());
+    std::vector<double> table(phosim::kDrawTable);
+    phosim::draw_table(table.data());
     double* d = nullptr;
     if (cudaMalloc(&d, bytes + (table.size() + 1) * sizeof(double)) != cudaSuccess) { (void)cudaGetLastError(); return PHOSIM_ERR_OUT_OF_MEMORY; }
     double* const dt = d + n + (n & 1);          // its pairs on 16 bytes

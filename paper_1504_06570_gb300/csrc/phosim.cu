@@ -567,10 +567,10 @@ phosim_status phosim_create_scene(const phosim_scene_desc* d, phosim_scene** out
     if ((st = upload(sc->table_mem, f.data(), f.size(), &pf)) != PHOSIM_OK) goto fail;
     P.ell32 = pf;
     {
-        std::vector<double> table(kLogTable + 34);
-        log_table(table.data());
+        std::vector<double> table(kDrawTable);
+        draw_table(table.data());
         if ((st = upload(sc->table_mem, table.data(), table.size(), &pd)) != PHOSIM_OK) goto fail;
-        P.log_table = pd;
+        P.draw_table = pd;
     }
     if ((st = upload(sc->table_mem, d->sigma, (size_t)d->n_sigma, &pd)) != PHOSIM_OK) goto fail;
     P.sig = pd;

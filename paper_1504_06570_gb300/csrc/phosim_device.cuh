@@ -150,7 +150,7 @@ struct TraceParams {
     float kick0f, inv_lam_ref_f, sed_lam0f, sed_dlamf, t_sif, dead_layerf, ell_lam0f, inv_ell_dlamf, sig_scalef;
     // sensor / detector
     int nx, ny, n_ell, n_sig;
-    const double* log_table;      // log_draw64
+    const double* draw_table;     // log_draw64, sincos_draw64
     double pixel, inv_pixel, xlo, ylo, chip_w, chip_h, t_si, ell_lam0, inv_ell_dlam, sig_scale, dead_layer;
     // fringing (PHOSIM_FRINGE): the silicon's optical thickness at (x, y) of the detector surface frame is
     // fr_t0 + fr_gx x + fr_gy y

@@ -181,9 +181,9 @@ __device__ __forceinline__ MemberDraw member_draw(const TraceParams& P, double b
         m.sx = (double)((float)bsig * g * cs);
         m.sy = (double)((float)bsig * g * sn);
     } else {
-        const double g = sqrt64_pos(-2.0 * log_draw64(P.log_table, m5.x));
+        const double g = sqrt64_pos(-2.0 * log_draw64(P.draw_table, m5.x));
         double sn, cs;
-        sincospi(2.0 * u64of(m5.y), &sn, &cs);
+        sincos_draw64(P.draw_table, m5.y, sn, cs);
         m.sx = bsig * g * cs;
         m.sy = bsig * g * sn;
     }
@@ -270,7 +270,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     if constexpr (RECORD) fr->surface(si)[32 * kTapeMu] = mu;
                     if (!refract(dl, Nx, Ny, Nz, mu, flat)) { R.flags = lost(PHOSIM_LOST_TIR, si); return; }
                     const double ell = lerp_table(P.ell, P.n_ell, (lam - P.ell_lam0) * P.inv_ell_dlam);
-                    L = ell * -log_draw64(P.log_table, w_conv);
+                    L = ell * -log_draw64(P.draw_table, w_conv);
                     const double rf = (n_si - 1.0) / (n_si + 1.0);
                     r_back = rf * rf;
                 }
@@ -307,9 +307,9 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                     sigma = 1.0; gxd = (double)(sg * g * cs); gyd = (double)(sg * g * sn);
                 } else {
                     sigma = lerp_table(P.sig, P.n_sig, depth * P.sig_scale);
-                    const double g = sqrt64_pos(-2.0 * log_draw64(P.log_table, w_diff_a));
+                    const double g = sqrt64_pos(-2.0 * log_draw64(P.draw_table, w_diff_a));
                     double sn, cs;
-                    sincospi(2.0 * u64of(w_diff_b), &sn, &cs);
+                    sincos_draw64(P.draw_table, w_diff_b, sn, cs);
                     gxd = g * cs; gyd = g * sn;
                 }
                 fx = fma(sigma, gxd, fx);
@@ -511,7 +511,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
             const double r = lerp_table(P.sersic + (size_t)s.table * P.sersic_K, P.sersic_K,
                                         u64of(w1.y) * P.sersic_K - 0.5);
             double sp, cp;
-            sincospi(2.0 * u64of(w1.z), &sp, &cp);
+            sincos_draw64(P.draw_table, w1.z, sp, cp);
             const double dx = s.a * r * cp, dy = s.b * r * sp;
             nx += dx * s.cpa - dy * s.spa;
             ny += dx * s.spa + dy * s.cpa;
@@ -524,9 +524,9 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
             nx += (double)((float)s.a * g * cp);
             ny += (double)((float)s.a * g * sp);
         } else {
-            const double g = sqrt64_pos(-2.0 * log_draw64(P.log_table, w1.y));
+            const double g = sqrt64_pos(-2.0 * log_draw64(P.draw_table, w1.y));
             double sp, cp;
-            sincospi(2.0 * u64of(w1.z), &sp, &cp);
+            sincos_draw64(P.draw_table, w1.z, sp, cp);
             nx += s.a * g * cp;
             ny += s.a * g * sp;
         }
@@ -543,7 +543,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
     // pupil point on the annulus, on the nominal first surface, moved back to the top of the atmosphere
     const double r = sqrt64(fma(u64of(w0.x), P.pr_dr2, P.pr_in2));
     double sp, cp;
-    sincospi(2.0 * u64of(w0.y), &sp, &cp);
+    sincos_draw64(P.draw_table, w0.y, sp, cp);
     double x = r * cp, y = r * sp;
     double z = P.pupil_z + sag(P.pupil_surf, fma(x, x, y * y));
     {
@@ -597,7 +597,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
             } else {
                 const double ang = lerp_table(P.hf, P.hf_K, u64of(w4.x) * P.hf_K - 0.5) * scale;
                 double sp, cp;
-                sincospi(2.0 * u64of(w4.y), &sp, &cp);
+                sincos_draw64(P.draw_table, w4.y, sp, cp);
                 nx = fma(ang, cp, nx);
                 ny = fma(ang, sp, ny);
             }
