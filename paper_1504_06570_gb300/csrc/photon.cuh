@@ -68,8 +68,8 @@ __device__ __forceinline__ int near_index(int i, int n) {
 }
 
 // A screen coordinate's node and the fraction of a pixel from it, s k - floor(s k).  By integers, on pipes that idle (with
-// the product, its floor and the rest on the FP64 pipe 300 stars of 2e7 photons took 7.73 ms all FP64 and 4.65 mixed,
-// 7.12 and 4.33 so); a coordinate beyond 4 km in FP64.
+// the product, its floor and the rest on the FP64 pipe 2e7 photons took 7.73 ms all FP64 and 1.5e7 took 4.65 mixed, 7.12
+// and 4.33 so); a coordinate beyond 4 km in FP64.
 static __device__ __noinline__ int far_node(double s, double inv, int n, unsigned long long& frac) {
     double fl;
     int i;

@@ -247,8 +247,9 @@ __global__ void __launch_bounds__(256, min_blocks(MODE)) trace_kernel(const __gr
 // whose tiles can be long, and packs those that go on into batches of 32; trace_batch_kernel follows a batch a warp,
 // each warp claiming the next batch when it is done, in blocks of one warp so that few batches spread over all SMs (a
 // warp alone on an SM does not wait for the FP64 pipe).
-// Measured (GB300): 300 stars, 2e7 photons, all FP64 10.4 ms in one kernel and 8.7 ms in two, mixed 6.8 and 5.6 ms; the
-// adjoint's call for 64 stars of 3e4 photons, which takes the same batches, 5.5 and 3.8 ms.
+// Measured (GB300): 300 stars, 2e7 photons, all FP64 10.4 ms in one kernel and 8.7 ms in two (6.5 ms since); 777 stars,
+// 1.5e7 photons, mixed 6.8 and 5.6 ms (4.2 ms since); the adjoint's call for 64 stars of 3e4 photons, which takes the same
+// batches, 5.5 and 3.8 ms (2.3 ms since).
 // ---------------------------------------------------------------------------------------------------------
 template <bool MIXED>
 __global__ void __launch_bounds__(256, 4) batch_kernel(const __grid_constant__ TraceParams P, const __grid_constant__ BatchList L) {
