@@ -74,12 +74,14 @@ __device__ __forceinline__ double f64_exact(float f) {
 __device__ __forceinline__ double f64_of_count(uint32_t n) { return __hiloint2double(0x43300000, (int)n) - 4503599627370496.0; }
 
 // floor(s k) as a double and an integer: the product added to 1.5 2^52 and rounded down in one operation leaves the
-// integer in the low word.  False where the floor is not within 32 bits (nothing is set then).
+// integer in the low word.  False where the floor is not a signed 32-bit integer (nothing is set then): the high word
+// holds all that is above the low one, so it is 0x43380000 less the low word's sign.
 __device__ __forceinline__ bool floor_product64(double s, double k, double& fl, int& i) {
     const double t = __fma_rd(s, k, 6755399441055744.0);
-    if ((unsigned)(__double2hiint(t) - 0x4337ffff) > 1u) return false;
+    const int low = __double2loint(t);
+    if (__double2hiint(t) != 0x43380000 + (low >> 31)) return false;
     fl = t - 6755399441055744.0;
-    i = __double2loint(t);
+    i = low;
     return true;
 }
 
