@@ -501,10 +501,10 @@ __device__ __forceinline__ bool sag_f(const DSurfaceS& E, int flags, float x, fl
 }
 
 // Exact root of the conic's quadric c (x^2 + y^2) + kc z^2 - 2 z = 0 (kc = (1 + kappa) c) along the ray p + l d on
-// the vertex branch (1 - kc z >= 0); NaN when the ray misses it.  Out of line: only rays that graze the conic,
-// where the single-precision root says too little, come here.
+// the vertex branch (1 - kc z >= 0), of two such the one nearer to the ray's own start at l = -from; NaN when the ray
+// misses it.  Out of line: only rays that graze the conic, where the single-precision root says too little, come here.
 static __device__ __noinline__ double conic_root(double c, double kc, double p0, double p1, double p2, double d0, double d1,
-                                                 double d2) {
+                                                 double d2, double from) {
     const double A = c * fma(d0, d0, d1 * d1) + kc * d2 * d2;
     const double b = c * fma(p0, d0, p1 * d1) + fma(kc * p2, d2, -d2);
     const double C = c * fma(p0, p0, p1 * p1) + fma(kc * p2, p2, -2.0 * p2);
@@ -512,8 +512,10 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
     if (!(disc >= 0.0)) return nan("");
     const double q = -(b + copysign(sqrt(disc), b));
     if (q == 0.0) return nan("");
-    double l = C / q;
-    if (A != 0.0 && fma(-kc, fma(l, d2, p2), 1.0) < 0.0) l = q / A;   // the other root is the vertex branch
+    const double near = C / q;                                        // the root nearer to p; the other is q / A
+    const bool second = fabs((from + near) * A) > fabs(fma(from, A, q));
+    const double l = second ? q / A : near;
+    if (A != 0.0 && fma(-kc, fma(l, d2, p2), 1.0) < 0.0) return second ? near : q / A;   // the other is the vertex branch
     return l;
 }
 
@@ -560,9 +562,13 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         if (disc > 1e-3f * bf * bf) {
             const float sq = sqrtf(disc);
             const float qf = bf >= 0.f ? -(bf + sq) : sq - bf;
-            lf = Cf / qf;
+            // of the roots Cf / qf and qf / A the one nearer to where the ray comes from (-lp from here), which a ray far off
+            // the axis may not have nearer to the vertex's plane; the other where that one is not on the vertex branch
+            const float near = Cf / qf;
+            const bool second = fabsf((lp + near) * A) > fabsf(fmaf(lp, A, qf));
+            lf = second ? qf / A : near;
             const float branch = fmaf(-kc, fmaf(lf, dz, pz), 1.f);
-            if (A != 0.f && branch < 0.f) lf = qf / A;
+            if (A != 0.f && branch < 0.f) lf = second ? near : qf / A;
             started = fabsf(branch) > 1e-3f && fabsf(lf) < 1e30f;
             if (started && newton) {
 #pragma unroll 1
@@ -582,7 +588,7 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     double x, y, z;
     const auto to_conic = [&] {
         const double q[3] = {fma(lpd, d[0], p[0]), fma(lpd, d[1], p[1]), fma(lpd, d[2], p[2])};
-        const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2]);
+        const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2], lpd);
         if (!(fabs(l0) < 1e300)) return false;
         x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
         lf = f32_trunc(l0);
