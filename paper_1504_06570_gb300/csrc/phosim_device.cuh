@@ -533,15 +533,14 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
 // to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; with the slope in
 // single precision 7.7 ms, 8.1 with an FP64 slope and its reciprocal.  On steep and aspheric lenses the position error
 // against the oracle fell from up to 9e-10 mm to 9e-13 mm, with either slope.
-// On success h is the point and N the unit normal (along (-S_x, -S_y, 1)); ahead says whether the distance is positive.
+// On success h is the point and N the unit normal (along (-S_x, -S_y, 1)).
 __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS& E, const double p[3], const double d[3],
-                                              double h[3], double N[3], bool& ahead) {
+                                              double h[3], double N[3]) {
     if (S.flags & SF_FLAT_ONLY) {
         if ((__double2hiint(d[2]) & 0x7fffffff) < 0x00100000) return PHOSIM_LOST_MISSED;
         const double l = -p[2] * rcp64(d[2]);
         h[0] = fma(l, d[0], p[0]); h[1] = fma(l, d[1], p[1]); h[2] = 0.0;
         N[0] = 0.0; N[1] = 0.0; N[2] = 1.0;
-        ahead = __double2hiint(l) > 0;
         return 0;
     }
     const bool newton = (S.flags & (SF_EVEN | SF_ODD | SF_ZERN)) != 0;
@@ -591,7 +590,6 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2], lpd);
         if (!(fabs(l0) < 1e300)) return false;
         x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
-        lf = f32_trunc(l0);
         return true;
     };
     if (started) {
@@ -600,7 +598,6 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     } else if (!to_conic()) {
         return PHOSIM_LOST_MISSED;
     }
-    ahead = lp + lf > 0.f;
     const float c = E.c.hi, kc = E.kc.hi;
 #pragma unroll 1
     for (int it = 0; it < 20; ++it) {
