@@ -1633,7 +1633,7 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     P.tile_photons = sc->last_tile;
     P.n_tiles = sc->last_tiles;
     P.tile_counter = sc->d_counters;
-    P.counters = sc->d_counters + 1;
+    P.counters = nullptr;                                // the forward pass has counted the photons
     P.image = nullptr;
     P.moments = nullptr;
     P.records = nullptr;

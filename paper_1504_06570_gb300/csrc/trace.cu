@@ -328,7 +328,8 @@ __global__ void __launch_bounds__(256, 4) batch_kernel(const __grid_constant__ T
         traced += count;
         stopped += count - went_on;
     }
-    if (lane == 0 && traced) {
+    // (no counters: the adjoint makes the batches of a trace again, whose photons are counted)
+    if (lane == 0 && traced && P.counters) {
         atomicAdd(P.counters, traced);
         if (stopped) atomicAdd(P.counters + 1 + PHOSIM_LOST_COATING, stopped);
     }
