@@ -248,7 +248,16 @@ class Scene:
         self.sources = sources
         self.src = sources_struct(sources)
         self.n_photons = np.ascontiguousarray(sources.n_photons, np.uint64)
-        self._n_photons_ptr = self.n_photons.ctypes.data_as(C.POINTER(C.c_uint64))
+
+    # the sources' photon counts, with the pointer that each trace passes on (making one costs a short call a microsecond)
+    @property
+    def n_photons(self):
+        return self._n_photons
+
+    @n_photons.setter
+    def n_photons(self, counts):
+        self._n_photons = counts
+        self._n_photons_ptr = counts.ctypes.data_as(C.POINTER(C.c_uint64))
 
     def set_schedule(self, threads=0, tile=0):
         _check("phosim_set_schedule", self.L.phosim_set_schedule(self.h, int(threads), int(tile)))
