@@ -251,9 +251,11 @@ phosim_status phosim_load_hf_kick(phosim_scene* scene, const double* quantiles, 
 /* Trace photons first[s] .. first[s] + n_photons[s] - 1 of every source s (first = NULL: from 0).
    sources, n_photons and first are host arrays.  Photon i of source s always draws the same random
    numbers (counter = (i, s, block), key = seed), whatever the batching.
-   image: nx * ny uint32 counts, ADDED to (device or host pointer; a host pointer is staged through a
-          scene-owned device buffer and the call returns after the copy back; another device's memory is
-          INVALID_ARGUMENT).
+   image: nx * ny uint32 counts, ADDED to (device or host pointer; another device's memory is INVALID_ARGUMENT).
+          A host pointer's call returns once the counts are in the host's memory: the image is staged through a
+          scene-owned device buffer and copied back whole, or, for a short exposure into page-locked memory that
+          the GPU adds to natively, counted in a device image of the scene's whose pixels with counts are added
+          to the host's, one atomic addition each (the others are not touched).
    records: NULL or a device array of sum(n_photons) records in source order.
    moments: NULL or a device array of n_src * PHOSIM_MOMENT_WORDS doubles; sums are added.
    records and moments must be device (or managed) memory of the scene's device: a host pointer returns

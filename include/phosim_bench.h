@@ -73,6 +73,12 @@ phosim_status phosim_fp64_eval(int op, const double* a, double* out, int n);
 phosim_status phosim_set_stage_timing(phosim_scene* scene, int on);
 phosim_status phosim_stage_times(phosim_scene* scene, double* ms, int n);
 
+/* How a phosim_trace call of n_photons photons in all would count into this image: 0 in place (device or managed
+   memory), 1 in a scene buffer copied from and to the host, 2 in a scene buffer whose pixels with counts are added to
+   the mapped host memory.  Nothing is launched.  Errors: INVALID_ARGUMENT (a null pointer, another device's memory),
+   NOT_READY. */
+phosim_status phosim_image_route(const phosim_scene* scene, const uint32_t* image, uint64_t n_photons, int* route);
+
 #ifdef __cplusplus
 }
 #endif

@@ -11,6 +11,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "phosim_bench.h"
 #include "phosim_device.cuh"
 #include "phosim_scene.hpp"
@@ -344,6 +346,57 @@ __global__ void add_counts_kernel(uint4* __restrict__ counts, size_t quads, uint
         if (v.w) atomicAdd(image + 4 * i + 3, v.w);
         counts[i] = make_uint4(0u, 0u, 0u, 0u);
     }
+}
+
+// Whether the page-locked allocation or registration that p lies in holds the `bytes` from p on.  (The runtime's pointer
+// attributes tell of the one address only, the driver's of its range as well.)
+bool host_range_holds(const void* p, size_t bytes) {
+    using GetAttributes = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    void* entry = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &entry, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned long long start = 0;
+    size_t size = 0;
+    void* out[2] = {&start, &size};
+    const unsigned long long at = (unsigned long long)(uintptr_t)p;
+    if (((GetAttributes)entry)(2, what, out, (CUdeviceptr)at) != CUDA_SUCCESS) return false;
+    return at >= start && at - start <= size && bytes <= size - (at - start);
+}
+
+// How a call counts into its image: in place, in a scene buffer that is copied from and to host memory, or in one whose
+// pixels with counts are added to mapped host memory
+enum ImageRoute { kImageDevice, kImageStaged, kImageAdded };
+phosim_status image_route(const phosim_scene* sc, const uint32_t* image, uint64_t photons, ImageRoute* route, uint32_t** mapped) {
+    cudaPointerAttributes attr;
+    *route = kImageStaged;
+    if (cudaPointerGetAttributes(&attr, image) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return PHOSIM_OK;
+    }
+    if (attr.type == cudaMemoryTypeDevice && attr.device != sc->device) return PHOSIM_ERR_INVALID_ARGUMENT;
+    if (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged) *route = kImageDevice;
+    // Where the GPU adds to host memory natively (the link to the host's memory carries atomics), a short exposure is
+    // counted in a device image of its own and only its pixels with counts are added to a pinned image.  Staging moves
+    // every pixel twice whatever the photons (0.71 ms for 4096^2); a pixel added over the link takes 0.35 ns, so the
+    // two cost the same where every eighth pixel has counts.  Up to a photon for every twelfth pixel, by the share
+    // of the spectrum's range that the coatings may pass, the pixels are added.  (3e6 photons of 100 stars, a sixth of
+    // them within the filter, with the host's clearing of the image: 1.35 ms staged, 0.86 ms with every photon's count
+    // over the link, 0.65 ms so.)  The image has to lie within one mapping, which an address alone does not tell.
+    if (attr.type == cudaMemoryTypeHost && sc->host_atomics && attr.devicePointer) {
+        const TraceParams& B = sc->base;
+        const double lo = B.sed_lam0, hi = B.sed_lam0 + B.n_bins * B.sed_dlam, pixels = (double)B.nx * B.ny;
+        const double share = std::max(0.0, std::min(hi, B.pass_hi) - std::max(lo, B.pass_lo)) / (hi - lo);
+        if (share * (double)photons <= pixels / 12.0 && host_range_holds(image, (size_t)B.nx * B.ny * sizeof(uint32_t))) {
+            *route = kImageAdded;
+            *mapped = (uint32_t*)attr.devicePointer;
+        }
+    }
+    return PHOSIM_OK;
 }
 
 void destroy_graph(TraceGraph& g) {
@@ -1020,6 +1073,16 @@ phosim_status phosim_get_counters(phosim_scene* sc, uint64_t* out, int n) {
     return PHOSIM_OK;
 }
 
+phosim_status phosim_image_route(const phosim_scene* sc, const uint32_t* image, uint64_t n_photons, int* out) {
+    if (!sc || !image || !out) return PHOSIM_ERR_INVALID_ARGUMENT;
+    if (!sc->optics_loaded || !sc->seds_loaded) return PHOSIM_ERR_NOT_READY;
+    ImageRoute route;
+    uint32_t* mapped = nullptr;
+    const phosim_status st = image_route(sc, image, n_photons, &route, &mapped);
+    if (st == PHOSIM_OK) *out = (int)route;
+    return st;
+}
+
 phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src, const uint64_t* n_photons,
                            const uint64_t* first, uint32_t* image, phosim_photon_record* records, double* moments,
                            void* stream) {
@@ -1122,30 +1185,15 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         sc->d_prefix = (unsigned long long*)(sc->d_src + n_src);
         sc->cap_src = n_src;
     }
-    // image: a pointer the device cannot use as device memory is staged through a scene buffer
-    cudaPointerAttributes attr;
-    bool host_image = false, added = false;
-    uint32_t* d_image = image;
-    if (cudaPointerGetAttributes(&attr, image) != cudaSuccess) {
-        (void)cudaGetLastError();
-        host_image = true;
-    } else {
-        host_image = attr.type != cudaMemoryTypeDevice && attr.type != cudaMemoryTypeManaged;
-        if (attr.type == cudaMemoryTypeDevice && attr.device != sc->device) return PHOSIM_ERR_INVALID_ARGUMENT;
-        // Where the GPU adds to host memory natively (the link to the host's memory carries atomics), a short exposure is
-        // counted in a device image of its own and only its pixels with counts are added to a pinned image.  Staging moves
-        // every pixel twice whatever the photons (0.71 ms for 4096^2); a pixel added over the link takes 0.35 ns, so the
-        // two cost the same where every eighth pixel has counts.  Up to a photon for every twelfth pixel, by the share
-        // of the spectrum's range that the coatings may pass, the pixels are added.  (3e6 photons of 100 stars, a sixth of
-        // them within the filter, with the host's clearing of the image: 1.35 ms staged, 0.86 ms with every photon's count
-        // over the link, 0.65 ms so.)
-        if (host_image && sc->host_atomics && attr.type == cudaMemoryTypeHost && attr.devicePointer) {
-            const TraceParams& B = sc->base;
-            const double lo = B.sed_lam0, hi = B.sed_lam0 + B.n_bins * B.sed_dlam;
-            const double share = std::max(0.0, std::min(hi, B.pass_hi) - std::max(lo, B.pass_lo)) / (hi - lo);
-            added = share * (double)total <= (double)B.nx * B.ny / 12.0;
-        }
+    // image: a pointer the device cannot use as device memory is staged through a scene buffer, or its pixels are added
+    ImageRoute route;
+    uint32_t* mapped = nullptr;
+    {
+        const phosim_status vs = image_route(sc, image, total, &route, &mapped);
+        if (vs != PHOSIM_OK) return vs;
     }
+    const bool host_image = route != kImageDevice, added = route == kImageAdded;
+    uint32_t* d_image = image;
     const size_t img_bytes = (size_t)sc->base.nx * sc->base.ny * sizeof(uint32_t);
     if (added) {
         // this image is all zeroes between calls: the pixels are cleared as they are added
@@ -1462,7 +1510,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         if (added) {
             const size_t quads = (img_bytes + 15) / 16;
             add_counts_kernel<<<(unsigned)std::min<size_t>((quads + 255) / 256, (size_t)sc->sm_count * 16), 256, 0, st>>>(
-                (uint4*)d_image, quads, (uint32_t*)attr.devicePointer);
+                (uint4*)d_image, quads, mapped);
             CU(cudaGetLastError());
         } else {
             CU(cudaMemcpyAsync(image, d_image, img_bytes, cudaMemcpyDeviceToHost, st));
