@@ -261,6 +261,10 @@ phosim_status phosim_load_hf_kick(phosim_scene* scene, const double* quantiles, 
    records and moments must be device (or managed) memory of the scene's device: a host pointer returns
    INVALID_ARGUMENT before anything is launched.
    stream: a cudaStream_t (NULL = legacy default stream); all device work is ordered on it.
+   Scratch that the scene keeps, grown to the largest call: of PHOSIM_MIXED_DS 64 bytes a photon (of 2^27 at most, 8.6 GB),
+   with reflecting coatings 261 (of 2^24 at most, 4.4 GB); of the FP64 precisions with PHOSIM_EARLY_REJECT and a coated
+   surface some 4.5 (of 2^27 at most, 0.6 GB), and none otherwise.  Where the device has less room, a call with batches
+   or reflecting coatings goes through its photons in smaller chunks.
    Errors: INVALID_ARGUMENT, NOT_READY, LIMIT, OUT_OF_MEMORY, CUDA. */
 phosim_status phosim_trace(phosim_scene* scene, const phosim_source* sources, int n_src,
                            const uint64_t* n_photons, const uint64_t* first, uint32_t* image,
@@ -272,6 +276,9 @@ phosim_status phosim_trace(phosim_scene* scene, const phosim_source* sources, in
    param_surface[p], param_field[p]: field 0..5 = pert[0..5], field 100 + j = zern[j].
    dL_dmoments: host, n_src x 5.  grad: host, n_src x n_params, written (per-source contributions).
    moments_out: NULL or host n_src x 6 (count, mean x, mean y, Ixx, Ixy, Iyy).
+   Scratch that the scene keeps beside phosim_trace's: the forward states of the photons that go on past the coatings' test,
+   some 1.1 KB a photon of 12 surfaces and 512 MB at most, where the device has room for them (they give way to any other
+   scratch of the scene); one state a resident warp (85 MB of 12 surfaces); 512 bytes a source and surface.
    Errors: INVALID_ARGUMENT, NOT_READY, LIMIT, OUT_OF_MEMORY, CUDA. */
 phosim_status phosim_grad(phosim_scene* scene, const phosim_source* sources, int n_src,
                           const uint64_t* n_photons, const double* dL_dmoments, const int32_t* param_surface,

@@ -79,6 +79,9 @@ constexpr uint64_t kDirectMoments = 1ull << 16;
 // the adjoint's tape, at most: batches past it are traced again (a telescope of 12 surfaces takes 35 KB a batch of 32
 // photons, so 4.9e5 photons past the dynamic transmission test)
 constexpr size_t kTapeBytes = 512ull << 20;
+// photons that a chunk is not cut below where the device has little room, and what is left to the call's other scratch
+constexpr uint64_t kLeastChunk = 1ull << 16;
+constexpr size_t kRoomLeft = 32ull << 20;
 
 // ----------------------------------------------------------------------------------------- Zernike figure
 // Noll index -> radial order n, |m| and whether the term is the cosine one (even j) or the sine one.
@@ -346,6 +349,62 @@ __global__ void add_counts_kernel(uint4* __restrict__ counts, size_t quads, uint
         if (v.w) atomicAdd(image + 4 * i + 3, v.w);
         counts[i] = make_uint4(0u, 0u, 0u, 0u);
     }
+}
+
+// The adjoint's tape gives way to any other scratch: without it the adjoint traces its photons again.
+void drop_tape(phosim_scene* sc) {
+    cudaFree(sc->d_tape);
+    sc->d_tape = nullptr;
+    sc->cap_tape = 0;
+    sc->tape_batches = 0;
+    sc->tape_written = false;
+}
+
+template <class T>
+cudaError_t scratch_alloc(phosim_scene* sc, T** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && sc->d_tape) {
+        (void)cudaGetLastError();
+        drop_tape(sc);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
+// what a buffer of held elements has to grow by to hold need of them
+size_t growth(size_t need, size_t held, size_t element) { return need > held ? (need - held) * element : 0; }
+
+// Halves a chunk (tiles of T photons) until the device has room for the bytes that the scene's scratch has to grow by for
+// it (bytes_of); a chunk that needs none asks nothing of the device.
+template <class BytesOf>
+phosim_status fit_chunk(phosim_scene* sc, uint64_t T, const BytesOf& bytes_of, uint64_t* tiles) {
+    while (bytes_of(*tiles) > 0) {
+        size_t free_bytes = 0, all = 0;
+        CU(cudaMemGetInfo(&free_bytes, &all));
+        if (bytes_of(*tiles) + kRoomLeft <= free_bytes) break;
+        if (sc->d_tape) drop_tape(sc);
+        else if (*tiles > 1 && *tiles * T > kLeastChunk) *tiles = (*tiles + 1) / 2;
+        else break;                                      // the allocation will say
+    }
+    return PHOSIM_OK;
+}
+
+// The photon batches' memory for the chunks of a call of total photons in n_tiles tiles of T, and the tiles of a chunk
+phosim_status batch_room(phosim_scene* sc, uint64_t total, uint64_t n_tiles, uint64_t T, uint64_t* chunk_tiles) {
+    // a tile leaves at most one batch more than its photons fill
+    const auto batches = [&](uint64_t tiles) { return (size_t)(std::min<uint64_t>(total, tiles * T) / 32 + std::min(n_tiles, tiles)); };
+    uint64_t tiles = std::max<uint64_t>(1, std::min(n_tiles, kStateChunk / T));
+    const phosim_status st = fit_chunk(sc, T, [&](uint64_t t) { return growth(batches(t), sc->cap_batches, sizeof(PhotonBatch)); }, &tiles);
+    if (st != PHOSIM_OK) return st;
+    const size_t need = batches(tiles);
+    if (sc->cap_batches < need) {
+        cudaFree(sc->d_batches);
+        sc->d_batches = nullptr; sc->cap_batches = 0;
+        CU(scratch_alloc(sc, &sc->d_batches, need * sizeof(PhotonBatch)));
+        sc->cap_batches = need;
+    }
+    *chunk_tiles = tiles;
+    return PHOSIM_OK;
 }
 
 // Whether the page-locked allocation or registration that p lies in holds the `bytes` from p on.  (The runtime's pointer
@@ -1006,7 +1065,7 @@ phosim_status phosim_autotune(phosim_scene* sc, const phosim_source* src, int n_
     if (sc->cap_stage < img_bytes) {
         cudaFree(sc->d_stage);
         sc->d_stage = nullptr; sc->cap_stage = 0;
-        CU(cudaMalloc(&sc->d_stage, img_bytes));
+        CU(scratch_alloc(sc, &sc->d_stage, img_bytes));
         sc->cap_stage = img_bytes;
     }
     cudaStream_t st = (cudaStream_t)stream;
@@ -1180,8 +1239,8 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         cudaFree(sc->d_src);
         cudaFree(sc->d_src_s);
         sc->d_src = nullptr; sc->d_src_s = nullptr; sc->d_prefix = nullptr; sc->cap_src = 0;
-        CU(cudaMalloc(&sc->d_src, (size_t)n_src * sizeof(DSource) + ((size_t)n_src + 1) * sizeof(unsigned long long)));
-        CU(cudaMalloc(&sc->d_src_s, (size_t)n_src * source_s_bytes()));
+        CU(scratch_alloc(sc, &sc->d_src, (size_t)n_src * sizeof(DSource) + ((size_t)n_src + 1) * sizeof(unsigned long long)));
+        CU(scratch_alloc(sc, &sc->d_src_s, (size_t)n_src * source_s_bytes()));
         sc->d_prefix = (unsigned long long*)(sc->d_src + n_src);
         sc->cap_src = n_src;
     }
@@ -1201,7 +1260,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         if (sc->cap_delta < need) {
             cudaFree(sc->d_delta);
             sc->d_delta = nullptr; sc->cap_delta = 0;
-            CU(cudaMalloc(&sc->d_delta, need));
+            CU(scratch_alloc(sc, &sc->d_delta, need));
             sc->cap_delta = need;
             sc->delta_clean = false;
         }
@@ -1212,7 +1271,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         if (sc->cap_stage < img_bytes) {
             cudaFree(sc->d_stage);
             sc->d_stage = nullptr; sc->cap_stage = 0;
-            CU(cudaMalloc(&sc->d_stage, img_bytes));
+            CU(scratch_alloc(sc, &sc->d_stage, img_bytes));
             sc->cap_stage = img_bytes;
         }
         d_image = sc->d_stage;
@@ -1232,17 +1291,18 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
     // two-kernel path: the entrance-plane states of one chunk of tiles at most (kStateChunk photons)
     const uint64_t n_tiles = prefix[n_src];
     const bool ghosts = staged && (sc->base.flags & kGhostFlag);
-    const uint64_t chunk_tiles = staged || listed ? std::max<uint64_t>(1, (ghosts ? kGhostChunk : kStateChunk) / T) : n_tiles;
-    if (listed) {
-        // a tile leaves at most one batch more than its photons fill
-        const size_t need = (size_t)(std::min<uint64_t>(total, chunk_tiles * T) / 32 + std::min(n_tiles, chunk_tiles));
-        if (sc->cap_batches < need) {
-            cudaFree(sc->d_batches);
-            sc->d_batches = nullptr; sc->cap_batches = 0;
-            CU(cudaMalloc(&sc->d_batches, need * sizeof(PhotonBatch)));
-            sc->cap_batches = need;
-        }
+    uint64_t chunk_tiles = staged ? std::max<uint64_t>(1, (ghosts ? kGhostChunk : kStateChunk) / T) : n_tiles;
+    constexpr size_t kGhostBytes = 2 * sizeof(DSGhost) + sizeof(uint32_t) + 1;
+    phosim_status room = PHOSIM_OK;
+    if (listed) room = batch_room(sc, total, n_tiles, T, &chunk_tiles);
+    if (ghosts) {
+        chunk_tiles = std::min(chunk_tiles, n_tiles);
+        room = fit_chunk(sc, T, [&](uint64_t t) {
+            const size_t n = (size_t)std::min<uint64_t>(total, t * T);
+            return growth(n, sc->cap_state, sizeof(DSState)) + growth(n, sc->cap_ghost, kGhostBytes);
+        }, &chunk_tiles);
     }
+    if (room != PHOSIM_OK) return room;
     sc->batches_whole = listed && n_tiles <= chunk_tiles;
     sc->last_tile = (uint32_t)T;
     sc->last_tiles = n_tiles;
@@ -1251,24 +1311,24 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         if (sc->cap_state < need) {
             cudaFree(sc->d_state);
             sc->d_state = nullptr; sc->cap_state = 0;
-            CU(cudaMalloc(&sc->d_state, need * sizeof(DSState)));
+            CU(scratch_alloc(sc, &sc->d_state, need * sizeof(DSState)));
             sc->cap_state = need;
         }
         const size_t need_hits = (size_t)std::min<uint64_t>(bundled_units, chunk_tiles * T);
         if (sc->cap_hits < need_hits) {
             cudaFree(sc->d_hits);
             sc->d_hits = nullptr; sc->cap_hits = 0;
-            CU(cudaMalloc(&sc->d_hits, need_hits * sizeof(DSHit)));
+            CU(scratch_alloc(sc, &sc->d_hits, need_hits * sizeof(DSHit)));
             sc->cap_hits = need_hits;
         }
         if (ghosts) {
             if (sc->cap_ghost < need) {
                 cudaFree(sc->d_ghost);
                 sc->d_ghost = nullptr; sc->cap_ghost = 0;
-                CU(cudaMalloc(&sc->d_ghost, need * (2 * sizeof(DSGhost) + sizeof(uint32_t) + 1)));
+                CU(scratch_alloc(sc, &sc->d_ghost, need * kGhostBytes));
                 sc->cap_ghost = need;
             }
-            if (!sc->d_rounds) CU(cudaMalloc(&sc->d_rounds, kGhostRounds * sizeof(GhostRound)));
+            if (!sc->d_rounds) CU(scratch_alloc(sc, &sc->d_rounds, kGhostRounds * sizeof(GhostRound)));
             C.zero[1] = (uint32_t*)sc->d_rounds;
             C.zero_words[1] = kGhostRounds * sizeof(GhostRound) / 4;
         }
@@ -1284,7 +1344,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         if (sc->cap_mom_stripes < need) {
             cudaFree(sc->d_mom_stripes);
             sc->d_mom_stripes = nullptr; sc->cap_mom_stripes = 0;
-            CU(cudaMalloc(&sc->d_mom_stripes, need * sizeof(double)));
+            CU(scratch_alloc(sc, &sc->d_mom_stripes, need * sizeof(double)));
             sc->cap_mom_stripes = need;
         }
         C.zero[2] = (uint32_t*)sc->d_mom_stripes;
@@ -1342,7 +1402,7 @@ phosim_status phosim_trace(phosim_scene* sc, const phosim_source* src, int n_src
         B.tape = nullptr;
         B.tape_batches = B.tape_stride = 0;
         B.tape_first = 0;
-        if (sc->tape_wanted && sc->batches_whole) {
+        if (sc->tape_wanted && sc->d_tape && sc->batches_whole) {
             B.tape = sc->d_tape;
             B.tape_batches = sc->tape_batches;
             B.tape_stride = sc->tape_stride;
@@ -1588,14 +1648,14 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     if (sc->cap_mom < mom_bytes) {
         cudaFree(sc->d_mom_scratch);
         sc->d_mom_scratch = nullptr; sc->cap_mom = 0;
-        CU(cudaMalloc(&sc->d_mom_scratch, mom_bytes));
+        CU(scratch_alloc(sc, &sc->d_mom_scratch, mom_bytes));
         sc->cap_mom = mom_bytes;
     }
     const size_t img_bytes = (size_t)B.nx * B.ny * sizeof(uint32_t);
     if (sc->cap_stage < img_bytes) {
         cudaFree(sc->d_stage);
         sc->d_stage = nullptr; sc->cap_stage = 0;
-        CU(cudaMalloc(&sc->d_stage, img_bytes));
+        CU(scratch_alloc(sc, &sc->d_stage, img_bytes));
         sc->cap_stage = img_bytes;
     }
     CU(cudaMemsetAsync(sc->d_mom_scratch, 0, mom_bytes, st));
@@ -1611,16 +1671,22 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     sc->tape_stride = (size_t)(kTapeSurface * (B.n_surf - G.first_surface) + kTapeEnd) * 32;
     const size_t slot_bytes = sc->tape_stride * sizeof(double);
     const size_t block_slots = (size_t)std::max(blocks, sc->sm_count * std::max(trace_per_sm, 1));
-    sc->tape_batches = std::min<uint64_t>(kTapeBytes / slot_bytes, total / 32 + n_src);
-    if (sc->cap_tape < (sc->tape_batches + block_slots) * slot_bytes) {
-        cudaFree(sc->d_tape);
-        sc->d_tape = nullptr; sc->cap_tape = 0;
-        if (cudaMalloc(&sc->d_tape, (sc->tape_batches + block_slots) * slot_bytes) != cudaSuccess) {
-            (void)cudaGetLastError();                    // no room: every photon is traced again
-            sc->tape_batches = 0;
-            CU(cudaMalloc(&sc->d_tape, block_slots * slot_bytes));
+    // (without a coated surface the forward pass makes no batches.)  Where the device has no room for it, what there is of
+    // it serves; and scratch that finds no room later takes the tape's (drop_tape).
+    const size_t least_tape = block_slots * slot_bytes;
+    sc->tape_batches = B.n_coated > 0 ? std::min<uint64_t>(kTapeBytes / slot_bytes, total / 32 + n_src) : 0;
+    const size_t want_tape = sc->tape_batches * slot_bytes + least_tape;
+    if (sc->cap_tape < want_tape) {
+        size_t free_bytes = 0, all = 0;
+        CU(cudaMemGetInfo(&free_bytes, &all));
+        if (want_tape + kRoomLeft <= free_bytes + sc->cap_tape) {
+            cudaFree(sc->d_tape);
+            sc->d_tape = nullptr; sc->cap_tape = 0;
+            if (cudaMalloc(&sc->d_tape, want_tape) == cudaSuccess) sc->cap_tape = want_tape;
+            else (void)cudaGetLastError();
         }
-        sc->cap_tape = (sc->tape_batches + block_slots) * slot_bytes;
+        const size_t slots = sc->cap_tape / slot_bytes;
+        sc->tape_batches = std::min<uint64_t>(sc->tape_batches, slots > block_slots ? slots - block_slots : 0);
     }
     const int saved_precision = sc->precision;
     const uint32_t saved_flags = sc->base.flags;
@@ -1660,8 +1726,18 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     if (sc->cap_grad < gbytes) {
         cudaFree(sc->d_grad_scratch);
         sc->d_grad_scratch = nullptr; sc->cap_grad = 0;
-        CU(cudaMalloc(&sc->d_grad_scratch, gbytes));
+        CU(scratch_alloc(sc, &sc->d_grad_scratch, gbytes));
         sc->cap_grad = gbytes;
+    }
+    uint64_t chunk_tiles = 0;
+    if (!sc->batches_whole && sc->last_tiles) {
+        const phosim_status vs = batch_room(sc, total, sc->last_tiles, sc->last_tile, &chunk_tiles);
+        if (vs != PHOSIM_OK) return vs;
+    }
+    if (sc->cap_tape < least_tape) {
+        drop_tape(sc);
+        CU(cudaMalloc(&sc->d_tape, least_tape));
+        sc->cap_tape = least_tape;
     }
     double* d_seeds = sc->d_grad_scratch;
     double* d_sums = d_seeds + (size_t)n_src * 8;
@@ -1693,17 +1769,8 @@ phosim_status phosim_grad(phosim_scene* sc, const phosim_source* src, int n_src,
     L.n = sc->d_counters + kStateCountWord;
     L.next = sc->d_counters + kBatchWord;
     const bool whole = sc->batches_whole;
-    const uint64_t tile = sc->last_tile, n_tiles = sc->last_tiles;
-    const uint64_t chunk_tiles = std::max<uint64_t>(1, kStateChunk / std::max<uint64_t>(tile, 1));
-    if (!whole) {
-        const size_t need = (size_t)(std::min(n_tiles, chunk_tiles) * (tile / 32 + 1));
-        if (sc->cap_batches < need) {
-            cudaFree(sc->d_batches);
-            sc->d_batches = nullptr; sc->cap_batches = 0;
-            CU(cudaMalloc(&sc->d_batches, need * sizeof(PhotonBatch)));
-            sc->cap_batches = need;
-        }
-    }
+    const uint64_t n_tiles = sc->last_tiles;
+    if (whole) chunk_tiles = n_tiles;
     L.batch = sc->d_batches;
     for (uint64_t t0 = 0; t0 < n_tiles; t0 += chunk_tiles) {
         L.tile_begin = t0;

@@ -83,8 +83,8 @@ struct phosim_scene {
     unsigned long long tape_batches = 0, tape_stride = 0;
     int tape_first = 0;
     bool tape_wanted = false, tape_written = false;
-    uint32_t last_tile = 0;                     // its photons per tile, tiles and batch kernel's blocks
-    uint64_t last_tiles = 0;
+    uint32_t last_tile = 0;                     // the last call's photons per tile
+    uint64_t last_tiles = 0;                    // and its tiles
     // per-kernel timing (phosim_set_stage_timing): an event pair per launch of the last call, with the
     // kernel kind (0 call preparation and chief, 1 one-kernel trace, 2 entry stage, 3 optics stage)
     bool stage_timing = false;
