@@ -788,7 +788,7 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
     }
     std::vector<void*> mem;
     TableBytes tables;
-    std::vector<std::array<size_t, 6>> table_at((size_t)n_coat);           // where each coating's tables are among them
+    std::vector<std::array<size_t, 3>> table_at((size_t)n_coat);           // where each coating's tables are among them
     std::vector<std::vector<unsigned long long>> most((size_t)n_coat);     // each coating's accept thresholds, largest over angles
     bool ghosts = false;
     for (int k = 0; k < n_coat; ++k) {
@@ -805,9 +805,8 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
         for (size_t i = 0; i < tr.size(); ++i) tr_thr[i] = accept_threshold(tr[i]);
         for (int il = 0; il < nl; ++il) tmax_thr[il] = accept_threshold(tmax[il]);
         most[(size_t)k] = tmax_thr;
-        table_at[(size_t)k] = {tables.add(coats[k].table, (size_t)nl * nt), tables.add(tmax.data(), tmax.size()),
-                               tables.add(thr.data(), thr.size()), tables.add(tmax_thr.data(), tmax_thr.size()),
-                               R ? tables.add(tr.data(), tr.size()) : 0, R ? tables.add(tr_thr.data(), tr_thr.size()) : 0};
+        table_at[(size_t)k] = {tables.add(thr.data(), thr.size()), tables.add(tmax_thr.data(), tmax_thr.size()),
+                               R ? tables.add(tr_thr.data(), tr_thr.size()) : 0};
         if (R) ghosts = true;
         DCoating& C = P.coat[k];
         C.lam0 = coats[k].lam0; C.inv_dlam = 1.0 / coats[k].dlam;
@@ -848,13 +847,10 @@ phosim_status phosim_load_optics(phosim_scene* sc, const phosim_surface* surf, i
     if (ts != PHOSIM_OK) { free_all(mem); return ts; }
     for (int k = 0; k < n_coat; ++k) {
         DCoating& C = P.coat[k];
-        const std::array<size_t, 6>& at = table_at[(size_t)k];
-        C.T = (const double*)(base + at[0]);
-        C.Tmax = (const double*)(base + at[1]);
-        C.T_thr = (const unsigned long long*)(base + at[2]);
-        C.Tmax_thr = (const unsigned long long*)(base + at[3]);
-        C.TR = coats[k].reflect ? (const double*)(base + at[4]) : nullptr;
-        C.TR_thr = coats[k].reflect ? (const unsigned long long*)(base + at[5]) : nullptr;
+        const std::array<size_t, 3>& at = table_at[(size_t)k];
+        C.T_thr = (const unsigned long long*)(base + at[0]);
+        C.Tmax_thr = (const unsigned long long*)(base + at[1]);
+        C.TR_thr = coats[k].reflect ? (const unsigned long long*)(base + at[2]) : nullptr;
     }
     sc->d_zmono = (double*)(base + tables.bytes.size() - sizeof(double) * PHOSIM_MAX_ZERNIKE * kZPoly);
     free_all(sc->optics_mem);

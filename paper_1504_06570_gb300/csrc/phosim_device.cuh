@@ -70,11 +70,10 @@ struct DCoating {
     float lam0f, inv_dlamf, th0f, inv_dthf;
     ds lam0_s, inv_dlam_s;                    // the wavelength grid as double-single pairs (its bins)
     int nl, nt, pad0, pad1;
-    const double* T;                          // nl x nt
-    const double* Tmax;                       // nl: the largest transmission over angles at each wavelength
-    const unsigned long long* T_thr;          // the same as integer thresholds ceil(T 2^32 - 1/2) on the draw
-    const unsigned long long* Tmax_thr;
-    const double* TR;                         // T + R (ghosts), or null when the coating does not reflect
+    // transmissions as integer thresholds ceil(T 2^32 - 1/2) on the draw
+    const unsigned long long* T_thr;          // nl x nt
+    const unsigned long long* Tmax_thr;       // nl: the largest over angles at each wavelength
+    // of T + R (ghosts), or null when the coating does not reflect
     const unsigned long long* TR_thr;
 };
 

@@ -369,7 +369,7 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
                 }
                 if (!((unsigned long long)w < __ldg(C.T_thr + ix))) {    // (w + 1/2) 2^-32 < T
                     // reflected backwards (a ghost) with probability R, absorbed otherwise
-                    if (ghosts && S.kind != PHOSIM_MIRROR && C.TR && (unsigned long long)w < __ldg(C.TR_thr + ix)) {
+                    if (ghosts && S.kind != PHOSIM_MIRROR && C.TR_thr && (unsigned long long)w < __ldg(C.TR_thr + ix)) {
                         const double dn = dl[0] * Nx + dl[1] * Ny + dl[2] * Nz;
                         dl[0] = fma(-2.0 * dn, Nx, dl[0]);
                         dl[1] = fma(-2.0 * dn, Ny, dl[1]);
