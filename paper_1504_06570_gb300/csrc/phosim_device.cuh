@@ -518,6 +518,44 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
     return l;
 }
 
+// An aspheric or Zernike surface where the single-precision start below does not come near it: Newton's method on the sag
+// in FP64 from the conic's root along p + l d (the ray's own start is at l = -from), until the step is below 1e-8 mm.  Whether it gets there within 20 steps, and
+// whether it leaves the conic's domain on its way, is what says that a ray meets such a surface or how it is lost: steep
+// terms have roots of their own beyond the aperture, which a method with larger steps finds where this one ends.  Out of
+// line: rays that come in within the aperture of a lens or a mirror do not get here.
+static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, const DSurfaceS& E, double3 p, double3 d, double from,
+                                                      double* h, double* N) {
+    double l = conic_root(S.c, S.kc, p.x, p.y, p.z, d.x, d.y, d.z, from);
+    if (!(fabs(l) < 1e300)) return PHOSIM_LOST_MISSED;
+    bool done = false;
+    for (int it = 0; it < 21; ++it) {
+        const double x = fma(l, d.x, p.x), y = fma(l, d.y, p.y), z = fma(l, d.z, p.z), r2 = fma(x, x, y * y);
+        double zs, zx, zy;
+        float H[3];
+        aspheric(S, E, x, y, r2, zs, zx, zy, H);
+        if (S.flags & SF_CONIC) {
+            const double arg = fma(-S.k1c2, r2, 1.0);
+            if (arg < 0.0) return PHOSIM_LOST_MISSED;
+            const double root = sqrt(arg), g = S.c / root;
+            zs += S.c * r2 / (1.0 + root);
+            zx = fma(x, g, zx);
+            zy = fma(y, g, zy);
+        }
+        if (done) {
+            const double n = rsqrt(fma(zx, zx, fma(zy, zy, 1.0)));
+            h[0] = x; h[1] = y; h[2] = z;
+            N[0] = -zx * n; N[1] = -zy * n; N[2] = n;
+            return 0;
+        }
+        const double slope = d.z - zx * d.x - zy * d.y;
+        if (slope == 0.0) return PHOSIM_LOST_NEWTON;
+        const double step = (z - zs) / slope;
+        l -= step;
+        done = fabs(step) < 1e-8;
+    }
+    return PHOSIM_LOST_NEWTON;
+}
+
 // Intersection (Sec. 2.4.2): the paper's first guess is the root of a quadric approximating the surface; here the
 // quadric is the conic itself.  With the aspheric and Zernike part a(x, y) of the sag and t = z - a the surface is
 // Q = c (x^2 + y^2) / 2 + (1 + kappa) c t^2 / 2 - t = 0, which needs no root: Newton's method on Q along the ray solves
@@ -527,7 +565,9 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
 // Chebyshev's method, s + Q'' s^2 / (2 Q'), leaves an error near (Q'' / Q')^2 s^3, and the gradient of Q, which is
 // along the normal, moves to the root with its derivative; the slope Q', which only scales the step, and both
 // corrections are taken in single precision, whose 1e-7 of the step stays below the FP64 rounding of the results.  A step
-// that is not that small is taken and followed by another.  For a sphere the gradient has unit length on the surface.  A ray that grazes the conic takes the FP64 root.
+// that is not that small is taken and followed by another.  For a sphere the gradient has unit length on the surface.  A ray
+// that grazes the conic takes the FP64 root; where the start of an aspheric surface does not settle, or the first FP64 step
+// is not that of a start near the surface, Newton's method on the sag decides (intersect_far).
 // Measured (GB300, 300 stars, 2e7 photons, all FP64): 17.6 ms with the conic's FP64 root (a root and a quotient) and two
 // to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; with the slope in
 // single precision 7.7 ms, 8.1 with an FP64 slope and its reciprocal.  On steep and aspheric lenses the position error
@@ -549,7 +589,7 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     const double lpd = f64_exact(lp);
     const float A = fmaf(E.kmc.hi * dz, dz, E.c.hi);      // the quadric's l^2 coefficient for a unit direction
     bool started = false;
-    float lf = 0.f;
+    float lf = 0.f;                                       // from there to the surface
     {
         const float px = fmaf(lp, dx, f32_trunc(p[0])), py = fmaf(lp, dy, f32_trunc(p[1]));
         const float pz = f32_trunc(fma(lpd, d[2], p[2]));
@@ -569,17 +609,17 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
             if (A != 0.f && branch < 0.f) lf = second ? near : qf / A;
             started = fabsf(branch) > 1e-3f && fabsf(lf) < 1e30f;
             if (started && newton) {
+                started = false;
 #pragma unroll 1
-                for (int it = 0; it < 4; ++it) {
+                for (int it = 0; it < 4 && !started; ++it) {
                     const float x = fmaf(lf, dx, px), y = fmaf(lf, dy, py);
                     float zs, zxf, zyf;
                     if (!sag_f(E, S.flags, x, y, zs, zxf, zyf)) break;
                     const float step = (fmaf(lf, dz, pz) - zs) / (dz - zxf * dx - zyf * dy);
                     if (!(fabsf(step) < 1e30f)) break;
                     lf -= step;
-                    if (fabsf(step) < 1e-2f) break;
+                    started = fabsf(step) < 1e-2f;
                 }
-                started = fabsf(lf) < 1e30f;
             }
         }
     }
@@ -591,15 +631,17 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
         return true;
     };
-    if (started) {
-        const double l0 = lpd + f64_exact(lf);
+    if (!started) lf = 0.f;
+    const double l0 = lpd + f64_exact(lf);
+    if (started || newton) {
         x = fma(l0, d[0], p[0]); y = fma(l0, d[1], p[1]); z = fma(l0, d[2], p[2]);
     } else if (!to_conic()) {
         return PHOSIM_LOST_MISSED;
     }
+    bool far = newton && !started;
     const float c = E.c.hi, kc = E.kc.hi;
 #pragma unroll 1
-    for (int it = 0; it < 20; ++it) {
+    for (int it = 0; it < 20 && !far; ++it) {
         const double r2 = fma(x, x, y * y);
         double a = 0.0, ax = 0.0, ay = 0.0;
         float H[3] = {0.f, 0.f, 0.f};
@@ -618,6 +660,8 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
             invf = f32_trunc(rcp64(Ql));
             sf = f32_trunc(Q * rcp64(Ql));
         }
+        far = newton && it == 0 && !(fabsf(sf) < 0.1f);
+        if (far) break;
         const float hx = fmaf(H[0], dx, H[1] * dy), hy = fmaf(H[1], dx, H[2] * dy);
         // Q'' along the ray, and the step with its second-order term
         const float Qll = fmaf(c, fmaf(dx, dx, dy * dy), fmaf(kc * tlf, tlf, uf * fmaf(hx, dx, hy * dy)));
@@ -649,7 +693,12 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         // the start was too far off (a ray that grazes the conic): the conic's FP64 root
         if (!newton && started && it == 0 && !(fabsf(more * k) < 1e-14f) && !to_conic()) return PHOSIM_LOST_MISSED;
     }
-    return PHOSIM_LOST_NEWTON;
+    if (!far) return PHOSIM_LOST_NEWTON;
+    double at[3], normal[3];
+    const uint32_t why = intersect_far(S, E, make_double3(x, y, z), make_double3(d[0], d[1], d[2]), lpd + f64_exact(lf), at, normal);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { h[k] = at[k]; N[k] = normal[k]; }
+    return why;
 }
 
 // Sellmeier index, its three fractions over one denominator
