@@ -174,7 +174,7 @@ struct TraceParams {
     // work and outputs: tile t of the launch is tile t - tile_prefix[s] of the source s with
     // tile_prefix[s] <= t < tile_prefix[s + 1]; a tile holds tile_photons consecutive photons
     const DSource* sources;
-    SourceS* sources_s;                       // the same sources converted once by the chief-ray kernel (two-kernel path)
+    SourceS* sources_s;                       // the same sources converted once by call_prep_kernel (two-kernel path)
     const unsigned long long* tile_prefix;
     int n_src;
     uint32_t tile_photons;
@@ -522,7 +522,8 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
 // in FP64 from the conic's root along p + l d (the ray's own start is at l = -from), until the step is below 1e-8 mm.  Whether it gets there within 20 steps, and
 // whether it leaves the conic's domain on its way, is what says that a ray meets such a surface or how it is lost: steep
 // terms have roots of their own beyond the aperture, which a method with larger steps finds where this one ends.  Out of
-// line: rays that come in within the aperture of a lens or a mirror do not get here.
+// line, for the rays that come in far off the aperture: those that a lens or a mirror is made for do not get here (2e7 photons
+// all FP64 6.24 ms with it, 6.33 where every ray went on from whatever start it had).
 static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, const DSurfaceS& E, double3 p, double3 d, double from,
                                                       double* h, double* N) {
     double l = conic_root(S.c, S.kc, p.x, p.y, p.z, d.x, d.y, d.z, from);

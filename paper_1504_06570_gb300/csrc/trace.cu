@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(256, min_blocks(MODE)) trace_kernel(const __gr
 // whose tiles can be long, and packs those that go on into batches of 32; trace_batch_kernel follows a batch a warp,
 // each warp claiming the next batch when it is done, in blocks of one warp so that few batches spread over all SMs (a
 // warp alone on an SM does not wait for the FP64 pipe).
-// Measured (GB300): 300 stars, 2e7 photons, all FP64 10.4 ms in one kernel and 8.7 ms in two (6.5 ms since); 777 stars,
-// 1.5e7 photons, mixed 6.8 and 5.6 ms (4.2 ms since); the adjoint's call for 64 stars of 3e4 photons, which takes the same
+// Measured (GB300): 300 stars, 2e7 photons, all FP64 10.4 ms in one kernel and 8.7 ms in two (6.3 ms since); 777 stars,
+// 1.5e7 photons, mixed 6.8 and 5.6 ms (4.1 ms since); the adjoint's call for 64 stars of 3e4 photons, which takes the same
 // batches, 5.5 and 3.8 ms (2.3 ms since).
 // ---------------------------------------------------------------------------------------------------------
 template <bool MIXED>
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(256, PHOSIM_DS_ENTRY_MIN_BLOCKS) ds_entry_kern
         const uint64_t off = j * P.tile_photons;
         const uint32_t count = (uint32_t)min((uint64_t)P.tile_photons, s.ucount - off);
         const uint64_t ufirst = s.ufirst + off;
-        {   // the source's constants, converted by the chief-ray kernel: one word a lane
+        {   // the source's constants, converted by the call's preparation: one word a lane
             static_assert(sizeof(SourceS) % 4 == 0 && sizeof(SourceS) <= 128, "SourceS copy");
             const uint32_t* from = reinterpret_cast<const uint32_t*>(P.sources_s + src);
             uint32_t* to = reinterpret_cast<uint32_t*>(&src_mem[warp]);
