@@ -518,30 +518,80 @@ static __device__ __noinline__ double conic_root(double c, double kc, double p0,
     return l;
 }
 
+// The sag and its slopes in FP64, term by term in rolled loops, which take few registers from the caller; false outside the
+// conic's domain.
+static __device__ __forceinline__ bool far_sag(const DSurface& S, double x, double y, double& z, double& zx, double& zy) {
+    const double r2 = fma(x, x, y * y);
+    double g = 0.0;                       // (1/r) dz/dr of the terms of the radius
+    z = 0.0;
+    if (S.flags & SF_CONIC) {
+        const double arg = fma(-S.k1c2, r2, 1.0);
+        if (arg < 0.0) return false;
+        const double root = sqrt(arg);
+        z = S.c * r2 / (1.0 + root);
+        g = S.c / root;
+    }
+    double p = 0.0, q = 0.0;
+    if (S.flags & SF_EVEN) {
+#pragma unroll 1
+        for (int k = S.ne - 1; k >= 0; --k) {
+            p = fma(r2, p, S.ae[k]);
+            q = fma(r2, q, S.aed[k]);
+        }
+        z = fma(r2 * r2, p, z);
+        g = fma(r2, q, g);
+    }
+    if (S.flags & SF_ODD) {
+        const double r = sqrt(r2);
+        p = q = 0.0;
+#pragma unroll 1
+        for (int k = S.no - 1; k >= 0; --k) {
+            p = fma(r2, p, S.ao[k]);
+            q = fma(r2, q, S.aod[k]);
+        }
+        z = fma(r2 * r, p, z);
+        g = fma(r, q, g);
+    }
+    zx = x * g;
+    zy = y * g;
+    if (S.flags & SF_ZERN) {
+        const double u = x * S.zinv, v = y * S.zinv;
+        double zz = 0.0, zu = 0.0, zv = 0.0;
+        const double* row = S.zp + kZPoly - 1;           // the rows of powers of v, each of the powers of u, from the last
+#pragma unroll 1
+        for (int n = 1; n <= 7; ++n) {
+            double a = 0.0, da = 0.0;
+#pragma unroll 1
+            for (int k = 0; k < n; ++k, --row) {
+                da = fma(da, u, a);
+                a = fma(a, u, *row);
+            }
+            zv = fma(zv, v, zz);
+            zz = fma(zz, v, a);
+            zu = fma(zu, v, da);
+        }
+        z += zz;
+        zx = fma(zu, S.zinv, zx);
+        zy = fma(zv, S.zinv, zy);
+    }
+    return true;
+}
+
 // An aspheric or Zernike surface where the single-precision start below does not come near it: Newton's method on the sag
 // in FP64 from the conic's root along p + l d (the ray's own start is at l = -from), until the step is below 1e-8 mm.  Whether it gets there within 20 steps, and
 // whether it leaves the conic's domain on its way, is what says that a ray meets such a surface or how it is lost: steep
 // terms have roots of their own beyond the aperture, which a method with larger steps finds where this one ends.  Out of
 // line, for the rays that come in far off the aperture: those that a lens or a mirror is made for do not get here (2e7 photons
 // all FP64 6.24 ms with it, 6.33 where every ray went on from whatever start it had).
-static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, const DSurfaceS& E, double3 p, double3 d, double from,
+static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, double3 p, double3 d, double from,
                                                       double* h, double* N) {
     double l = conic_root(S.c, S.kc, p.x, p.y, p.z, d.x, d.y, d.z, from);
     if (!(fabs(l) < 1e300)) return PHOSIM_LOST_MISSED;
     bool done = false;
     for (int it = 0; it < 21; ++it) {
-        const double x = fma(l, d.x, p.x), y = fma(l, d.y, p.y), z = fma(l, d.z, p.z), r2 = fma(x, x, y * y);
+        const double x = fma(l, d.x, p.x), y = fma(l, d.y, p.y), z = fma(l, d.z, p.z);
         double zs, zx, zy;
-        float H[3];
-        aspheric(S, E, x, y, r2, zs, zx, zy, H);
-        if (S.flags & SF_CONIC) {
-            const double arg = fma(-S.k1c2, r2, 1.0);
-            if (arg < 0.0) return PHOSIM_LOST_MISSED;
-            const double root = sqrt(arg), g = S.c / root;
-            zs += S.c * r2 / (1.0 + root);
-            zx = fma(x, g, zx);
-            zy = fma(y, g, zy);
-        }
+        if (!far_sag(S, x, y, zs, zx, zy)) return PHOSIM_LOST_MISSED;
         if (done) {
             const double n = rsqrt(fma(zx, zx, fma(zy, zy, 1.0)));
             h[0] = x; h[1] = y; h[2] = z;
@@ -573,14 +623,16 @@ static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, const D
 // to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; with the slope in
 // single precision 7.7 ms, 8.1 with an FP64 slope and its reciprocal.  On steep and aspheric lenses the position error
 // against the oracle fell from up to 9e-10 mm to 9e-13 mm, with either slope.
-// On success h is the point and N the unit normal (along (-S_x, -S_y, 1)).
+// On success h is the point and N the unit normal (along (-S_x, -S_y, 1)); way has the sign of the distance, or is 0 where
+// the single-precision start does not say it for certain (a start within 0.1 mm of the surface does beyond 1 mm).
 __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS& E, const double p[3], const double d[3],
-                                              double h[3], double N[3]) {
+                                              double h[3], double N[3], float& way) {
     if (S.flags & SF_FLAT_ONLY) {
         if ((__double2hiint(d[2]) & 0x7fffffff) < 0x00100000) return PHOSIM_LOST_MISSED;
         const double l = -p[2] * rcp64(d[2]);
         h[0] = fma(l, d[0], p[0]); h[1] = fma(l, d[1], p[1]); h[2] = 0.0;
         N[0] = 0.0; N[1] = 0.0; N[2] = 1.0;
+        way = __double2hiint(l) > 0 ? 1.f : -1.f;
         return 0;
     }
     const bool newton = (S.flags & (SF_EVEN | SF_ODD | SF_ZERN)) != 0;
@@ -639,6 +691,8 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     } else if (!to_conic()) {
         return PHOSIM_LOST_MISSED;
     }
+    way = lp + lf;
+    if (!(started && fabsf(way) > 1.f + 1e-4f * fabsf(lp))) way = 0.f;
     bool far = newton && !started;
     const float c = E.c.hi, kc = E.kc.hi;
 #pragma unroll 1
@@ -661,8 +715,11 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
             invf = f32_trunc(rcp64(Ql));
             sf = f32_trunc(Q * rcp64(Ql));
         }
-        far = newton && it == 0 && !(fabsf(sf) < 0.1f);
-        if (far) break;
+        if (it == 0 && !(fabsf(sf) < 0.1f)) {
+            way = 0.f;
+            far = newton;
+            if (far) break;
+        }
         const float hx = fmaf(H[0], dx, H[1] * dy), hy = fmaf(H[1], dx, H[2] * dy);
         // Q'' along the ray, and the step with its second-order term
         const float Qll = fmaf(c, fmaf(dx, dx, dy * dy), fmaf(kc * tlf, tlf, uf * fmaf(hx, dx, hy * dy)));
@@ -696,7 +753,7 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     }
     if (!far) return PHOSIM_LOST_NEWTON;
     double at[3], normal[3];
-    const uint32_t why = intersect_far(S, E, make_double3(x, y, z), make_double3(d[0], d[1], d[2]), lpd + f64_exact(lf), at, normal);
+    const uint32_t why = intersect_far(S, make_double3(x, y, z), make_double3(d[0], d[1], d[2]), lpd + f64_exact(lf), at, normal);
 #pragma unroll
     for (int k = 0; k < 3; ++k) { h[k] = at[k]; N[k] = normal[k]; }
     return why;

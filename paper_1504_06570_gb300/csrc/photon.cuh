@@ -221,10 +221,13 @@ __device__ __forceinline__ void optics(const TraceParams& P, double X[3], double
         double p[3], dl[3];
         to_surface(S, X, D, p, dl);
         double h[3], Nv[3];
-        const uint32_t why = intersect(S, P.surf_s[si], p, dl, h, Nv);
+        float way;
+        const uint32_t why = intersect(S, P.surf_s[si], p, dl, h, Nv, way);
         if (why) { R.flags = lost(why, si); return; }
-        // a ghost only meets surfaces ahead of it: the distance from the points, to their FP64 rounding
-        if (GHOSTS && bounces > 0 && !(fma(h[0] - p[0], dl[0], fma(h[1] - p[1], dl[1], (h[2] - p[2]) * dl[2])) > 0.0)) {
+        // a ghost only meets surfaces ahead of it: a distance near 0 from the points, to their FP64 rounding (for every
+        // distance that took 2 % of 2.8e6 photons with ghosts, mixed: 21.0 ms)
+        if (GHOSTS && bounces > 0 &&
+            !(way != 0.f ? way > 0.f : fma(h[0] - p[0], dl[0], fma(h[1] - p[1], dl[1], (h[2] - p[2]) * dl[2])) > 0.0)) {
             R.flags = lost(PHOSIM_LOST_MISSED, si);
             return;
         }
