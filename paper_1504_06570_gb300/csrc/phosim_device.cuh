@@ -500,17 +500,17 @@ __device__ __forceinline__ bool sag_f(const DSurfaceS& E, int flags, float x, fl
 }
 
 // Exact root of the conic's quadric c (x^2 + y^2) + kc z^2 - 2 z = 0 (kc = (1 + kappa) c) along the ray p + l d on
-// the vertex branch (1 - kc z >= 0), of two such the one nearer to the ray's own start at l = -from; NaN when the ray
-// misses it.  Out of line: only rays that graze the conic, where the single-precision root says too little, come here.
+// the vertex branch (1 - kc z >= 0), of two such the one nearer to the ray's own start at l = -from; infinity when the ray
+// misses it, and NaN for a ray without a place or a direction.  Out of line: only rays that graze the conic, where the single-precision root says too little, come here.
 static __device__ __noinline__ double conic_root(double c, double kc, double p0, double p1, double p2, double d0, double d1,
                                                  double d2, double from) {
     const double A = c * fma(d0, d0, d1 * d1) + kc * d2 * d2;
     const double b = c * fma(p0, d0, p1 * d1) + fma(kc * p2, d2, -d2);
     const double C = c * fma(p0, p0, p1 * p1) + fma(kc * p2, p2, -2.0 * p2);
     const double disc = fma(b, b, -A * C);
-    if (!(disc >= 0.0)) return nan("");
+    if (disc < 0.0) return INFINITY;
     const double q = -(b + copysign(sqrt(disc), b));
-    if (q == 0.0) return nan("");
+    if (q == 0.0) return INFINITY;
     const double near = C / q;                                        // the root nearer to p; the other is q / A
     const bool second = fabs((from + near) * A) > fabs(fma(from, A, q));
     const double l = second ? q / A : near;
@@ -586,7 +586,7 @@ static __device__ __forceinline__ bool far_sag(const DSurface& S, double x, doub
 static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, double3 p, double3 d, double from,
                                                       double* h, double* N) {
     double l = conic_root(S.c, S.kc, p.x, p.y, p.z, d.x, d.y, d.z, from);
-    if (!(fabs(l) < 1e300)) return PHOSIM_LOST_MISSED;
+    if (fabs(l) >= 1e300) return PHOSIM_LOST_MISSED;
     bool done = false;
     for (int it = 0; it < 21; ++it) {
         const double x = fma(l, d.x, p.x), y = fma(l, d.y, p.y), z = fma(l, d.z, p.z);
@@ -680,16 +680,23 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     const auto to_conic = [&] {
         const double q[3] = {fma(lpd, d[0], p[0]), fma(lpd, d[1], p[1]), fma(lpd, d[2], p[2])};
         const double l0 = conic_root(S.c, S.kc, q[0], q[1], q[2], d[0], d[1], d[2], lpd);
-        if (!(fabs(l0) < 1e300)) return false;
         x = fma(l0, d[0], q[0]); y = fma(l0, d[1], q[1]); z = fma(l0, d[2], q[2]);
-        return true;
+        return l0;
+    };
+    // a ray without a place or a direction meets the conic nowhere: the aperture drops it
+    const auto nowhere = [&](double l0) {
+        if (fabs(l0) >= 1e300) return (uint32_t)PHOSIM_LOST_MISSED;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) h[k] = N[k] = l0;
+        return 0u;
     };
     if (!started) lf = 0.f;
     const double l0 = lpd + f64_exact(lf);
     if (started || newton) {
         x = fma(l0, d[0], p[0]); y = fma(l0, d[1], p[1]); z = fma(l0, d[2], p[2]);
-    } else if (!to_conic()) {
-        return PHOSIM_LOST_MISSED;
+    } else if (const double l1 = to_conic(); !(fabs(l1) < 1e300)) {
+        way = 0.f;
+        return nowhere(l1);
     }
     way = lp + lf;
     if (!(started && fabsf(way) > 1.f + 1e-4f * fabsf(lp))) way = 0.f;
@@ -749,7 +756,8 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
         }
         if (!(fabsf(sf) < 1e37f)) return PHOSIM_LOST_NEWTON;
         // the start was too far off (a ray that grazes the conic): the conic's FP64 root
-        if (!newton && started && it == 0 && !(fabsf(more * k) < 1e-14f) && !to_conic()) return PHOSIM_LOST_MISSED;
+        if (!newton && started && it == 0 && !(fabsf(more * k) < 1e-14f))
+            if (const double l1 = to_conic(); !(fabs(l1) < 1e300)) return nowhere(l1);
     }
     if (!far) return PHOSIM_LOST_NEWTON;
     double at[3], normal[3];

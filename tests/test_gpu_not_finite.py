@@ -1,0 +1,47 @@
+"""Values that are no numbers, or beyond single precision, on the FP64 and mixed paths: a photon without a direction or a
+place is lost where Newton's method does not settle (an aspheric surface, as the oracle has it) or at the aperture (a
+conic), and never detected; the others of its scene are as they are without it."""
+import numpy as np
+import pytest
+
+from paper_1504_06570_gb300 import inputs as I
+from paper_1504_06570_gb300 import phosim as P
+from tests import gpu_helpers as G
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
+
+VIGNETTED, MISSED, NEWTON = 1, 2, 3
+BOTH = pytest.mark.parametrize("precision", [P.PLAIN_FP64, P.MIXED])
+
+
+def scene():
+    return G.test_system_scene(sources=G.mixed_sources([4000, 3000, 2000], seed=4))
+
+
+def reasons(rec):
+    """(reason, surface) of every photon; (0, .) of a detected one."""
+    return np.where(rec["flags"] & 1, 0, rec["flags"] >> 8 & 0xff), rec["flags"] >> 16
+
+
+@BOTH
+@pytest.mark.parametrize("width", [np.nan, np.inf, 3.0])
+@pytest.mark.parametrize("figure", [True, False])
+def test_photons_without_a_direction(precision, width, figure):
+    # the second and third source's offsets: no numbers, or most of them beyond 1 rad
+    sc = scene()
+    sc.sources.a = np.full(3, width)
+    if not figure:
+        sc.surfaces[0].zern = ()
+    rec = G.run_gpu(sc, precision, moments=False)["rec"]
+    plain = scene()
+    if not figure:
+        plain.surfaces[0].zern = ()
+    points = G.run_gpu(plain, precision, moments=False)["rec"]
+    assert np.array_equal(rec[:4000], points[:4000])
+    why, surface = reasons(rec[4000:])
+    assert not np.any(why == 0)
+    at_first = (why == (NEWTON if figure else VIGNETTED)) & (surface == 0)
+    assert np.mean(at_first) > (0.5 if width == 3.0 else 0.999)
+    assert not np.any((why == MISSED) & (surface == 0)) or width == 3.0
+
