@@ -101,7 +101,8 @@ __device__ __forceinline__ bool split_product64(double s, unsigned long long m, 
     frac &= 0xfffffffffffffull;
     return true;
 }
-// 1 + the fraction of 52 bits, exact
+// 1 + the fraction of 52 bits, exact; kNoFraction gives a NaN, here and in single precision
+constexpr unsigned long long kNoFraction = ~0ull;
 __device__ __forceinline__ double one_and_fraction64(unsigned long long frac) {
     return __longlong_as_double((long long)(frac | 0x3ff0000000000000ull));
 }
@@ -109,7 +110,8 @@ __device__ __forceinline__ double one_and_fraction64(unsigned long long frac) {
 // that says whether any is left, which are exact, in one sum
 __device__ __forceinline__ float fraction_f32(unsigned long long frac) {
     const uint32_t head = (uint32_t)(frac >> 29), tail = (uint32_t)frac & 0x1fffffffu;
-    return fmaf((float)(tail >> 5 | (uint32_t)((tail & 31u) != 0u)), 0x1p-47f, (float)head * 0x1p-23f);
+    const float f = fmaf((float)(tail >> 5 | (uint32_t)((tail & 31u) != 0u)), 0x1p-47f, (float)head * 0x1p-23f);
+    return head >> 23 ? __uint_as_float(0x7fffffffu) : f;
 }
 // log((w + 1/2) 2^-32) by a table (Tang 1990): with (w + 1/2) 2^-32 = 2^-e m, m in [1, 2), c near 1 / m from the first 8
 // bits after m's leading one and r = m c - 1, exact, it is -e log 2 - log c + log(1 + r); from m = sqrt 2 on the table

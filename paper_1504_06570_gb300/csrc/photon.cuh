@@ -59,8 +59,6 @@ __device__ __forceinline__ void load_block(const double2* p, double2& a, double2
         : "=d"(c.x), "=d"(c.y), "=d"(d.x), "=d"(d.y) : "l"(p + 2));
 }
 
-// node index of a floor beyond the integer range (a screen that many pixels from the origin)
-static __device__ __noinline__ int far_index(double fl, int n) { return wrap_index((long long)fl, n); }
 __device__ __forceinline__ int near_index(int i, int n) {
     if ((n & (n - 1)) == 0) return i & (n - 1);
     const int m = i % n;
@@ -69,18 +67,12 @@ __device__ __forceinline__ int near_index(int i, int n) {
 
 // A screen coordinate's node and the fraction of a pixel from it, s k - floor(s k).  By integers, on pipes that idle (with
 // the product, its floor and the rest on the FP64 pipe 2e7 photons took 7.73 ms all FP64 and 1.5e7 took 4.65 mixed, 7.12
-// and 4.33 so); a coordinate beyond 4 km in FP64.
+// and 4.33 so); a coordinate beyond 4 km in FP64, from the rounded product, whose last places are all that is left of the
+// fraction far out; one that is no number has no fraction (kNoFraction).
 static __device__ __noinline__ int far_node(double s, double inv, int n, unsigned long long& frac) {
-    double fl;
-    int i;
-    if (floor_product64(s, inv, fl, i)) {
-        i = near_index(i, n);
-    } else {
-        fl = floor(s * inv);
-        i = far_index(fl, n);
-    }
-    frac = (unsigned long long)fmin(fmax(fma(s, inv, -fl) * 4503599627370496.0, 0.0), 4503599627370495.0);
-    return i;
+    const double f = s * inv, fl = floor(f), rest = f - fl;
+    frac = isnan(rest) ? kNoFraction : (unsigned long long)fmin(rest * 4503599627370496.0, 4503599627370495.0);
+    return wrap_index((long long)fl, n);
 }
 __device__ __forceinline__ int node_of(const DScale& S, double s, unsigned long long& frac) {
     int i;

@@ -45,3 +45,26 @@ def test_photons_without_a_direction(precision, width, figure):
     assert np.mean(at_first) > (0.5 if width == 3.0 else 0.999)
     assert not np.any((why == MISSED) & (surface == 0)) or width == 3.0
 
+
+
+@BOTH
+@pytest.mark.parametrize("t0, t_exp", [(np.nan, 15.0), (np.inf, 15.0), (-np.inf, 0.0), (0.0, np.inf), (0.0, np.nan)])
+def test_photons_without_a_time(oracle_mod, precision, t0, t_exp):
+    # no place on the drifting screens, so no kick and no direction
+    sc = scene()
+    sc.sources.t0, sc.sources.t_exp = np.full(3, t0), np.full(3, t_exp)
+    rec = G.run_gpu(sc, precision, moments=False)["rec"]
+    assert np.array_equal(rec["flags"], G.oracle_trace(oracle_mod, sc)["flags"]) and not np.any(rec["flags"] & 1)
+
+
+@BOTH
+@pytest.mark.parametrize("v", [1280.0, -1280.0])
+def test_screen_too_far_for_a_fraction(oracle_mod, precision, v):
+    # 2^60 s at 1280 mm/s: the coordinate is -+1280 2^60 mm whatever the photon's place, a node of the 256 of 40 mm
+    sc = scene()
+    sc.sources.t0, sc.sources.t_exp = np.full(3, 2.0 ** 60), np.zeros(3)
+    for layer in sc.layers:
+        layer.vx, layer.vy = v, -v
+    gpu, ora = G.run_gpu(sc, precision, moments=False), G.oracle_trace(oracle_mod, sc)
+    assert np.sum(ora["flags"] & 1) > 1000
+    G.compare_records(sc, gpu, ora, pos_tol_px=1e-4)
