@@ -120,10 +120,10 @@ __device__ __forceinline__ double lerp_table(const double* __restrict__ t, int n
     double fl = 0.0;
     const bool found = floor_product64(f, 1.0, fl, k);
     double w = f - fl;
-    if (!found || k < 0 || k > n - 2) {              // off the table: its first or last value
+    if (!found || k < 0 || k > n - 2) {              // off the table: its first or last value, none where f is no number
         const bool last = found ? k > 0 : f > 0.0;
         k = last ? n - 2 : 0;
-        w = last ? 1.0 : 0.0;
+        w = isnan(f) ? f : last ? 1.0 : 0.0;
     }
     const double a = __ldg(t + k);
     return fma(w, __ldg(t + k + 1) - a, a);

@@ -11,7 +11,7 @@ from tests import gpu_helpers as G
 torch = pytest.importorskip("torch")
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
 
-VIGNETTED, MISSED, NEWTON = 1, 2, 3
+VIGNETTED, MISSED, NEWTON, NOT_CONVERTED = 1, 2, 3, 7
 BOTH = pytest.mark.parametrize("precision", [P.PLAIN_FP64, P.MIXED])
 
 
@@ -68,3 +68,13 @@ def test_screen_too_far_for_a_fraction(oracle_mod, precision, v):
     gpu, ora = G.run_gpu(sc, precision, moments=False), G.oracle_trace(oracle_mod, sc)
     assert np.sum(ora["flags"] & 1) > 1000
     G.compare_records(sc, gpu, ora, pos_tol_px=1e-4)
+
+
+def test_table_without_a_place(oracle_mod):
+    # an absorption table that starts nowhere: no length, no conversion
+    sc = scene()
+    sc.detector.ell_lam0 = np.nan
+    rec = G.run_gpu(sc, P.PLAIN_FP64, moments=False)["rec"]
+    ora = G.oracle_trace(oracle_mod, sc)
+    assert np.all((rec["flags"] == ora["flags"]) | G.boundary_mask(ora))
+    assert not np.any(rec["flags"] & 1) and np.sum(reasons(rec)[0] == NOT_CONVERTED) > 1000
