@@ -767,12 +767,22 @@ __device__ __forceinline__ uint32_t intersect(const DSurface& S, const DSurfaceS
     return why;
 }
 
-// Sellmeier index, its three fractions over one denominator
+// Sellmeier index by its three fractions: where they have a pole or no real root (NaN), or their product over- or underflows
+static __device__ __noinline__ double sellmeier_terms(const DMaterial& m, double l2) {
+    double n2 = 1.0;
+    for (int i = 0; i < 3; ++i) n2 += m.B[i] * l2 / (l2 - m.C[i]);
+    return sqrt(n2);
+}
+// the same over one denominator
 __device__ __forceinline__ double sellmeier(const DMaterial& m, double lam_nm) {
     const double l = lam_nm * 1e-3, l2 = l * l;
-    const double a = l2 - m.C[0], b = l2 - m.C[1], c = l2 - m.C[2], ab = a * b;
+    const double a = l2 - m.C[0], b = l2 - m.C[1], c = l2 - m.C[2], ab = a * b, den = ab * c;
     const double num = fma(m.B[2], ab, c * fma(m.B[0], b, m.B[1] * a));
-    return sqrt64(fma(l2 * num, rcp64(ab * c), 1.0));
+    const double n2 = fma(l2 * num, rcp64(den), 1.0);
+    // a denominator within 2^+-960 and 2^-16 < n2 < 2^32, by their high words
+    const bool plain = (uint32_t)((__double2hiint(den) & 0x7fffffff) - 0x03f00000) < 0x78000000u &&
+                       (uint32_t)(__double2hiint(n2) - 0x3ef00000) < 0x03000000u;
+    return plain ? sqrt64_pos(n2) : sellmeier_terms(m, l2);
 }
 
 // silicon index of Sec. 2.4.1, E in eV

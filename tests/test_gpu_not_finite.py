@@ -78,3 +78,21 @@ def test_table_without_a_place(oracle_mod):
     ora = G.oracle_trace(oracle_mod, sc)
     assert np.all((rec["flags"] == ora["flags"]) | G.boundary_mask(ora))
     assert not np.any(rec["flags"] & 1) and np.sum(reasons(rec)[0] == NOT_CONVERTED) > 1000
+
+
+@BOTH
+def test_glass_without_an_index(oracle_mod, precision):
+    # blue-shifted to 40 to 70 nm, where the Sellmeier formula of silica has negative squares: no index, no direction, and
+    # the next surface's aperture drops the photon; the others are the oracle's
+    sc = scene()
+    sc.sources.redshift = np.full(3, -0.9)
+    rec = G.run_gpu(sc, precision, moments=False)["rec"]
+    ora = G.oracle_trace(oracle_mod, sc)
+    l2 = (rec["lam"] * 1e-3) ** 2
+    square = 1.0 + sum(b * l2 / (l2 - c) for b, c in zip(I.FUSED_SILICA_B, I.FUSED_SILICA_C))
+    why, surface = reasons(rec)
+    met = ~((surface == 0) | ((surface == 1) & (why == VIGNETTED)))          # went into the lens
+    none = met & (square < -1e-9)
+    assert none.sum() > 3000 and np.all(why[none] == VIGNETTED) and np.all(surface[none] == 2)
+    real = square > 1e-9
+    assert real.sum() > 1000 and np.all(((rec["flags"] == ora["flags"]) | G.boundary_mask(ora))[real])
