@@ -57,10 +57,11 @@ __device__ __forceinline__ float f32_trunc(double v) {
     const uint32_t bits = __funnelshift_l((uint32_t)__double2loint(v), (uint32_t)(m - 0x38000000), 3);
     return __uint_as_float((bits & 0x7fffffffu) | ((uint32_t)hi & 0x80000000u));
 }
-// (float)v, rounded to nearest even, for 0 or 1e-37 < v < 1e38
+// (float)v, rounded to nearest even, for 0 or 1e-37 < v (infinity above 3.4e38)
 __device__ __forceinline__ float f32_rn_pos(double v) {
     const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
     if (hi < 0x38100000u) return 0.f;
+    if (hi >= 0x47f00000u) return INFINITY;
     const unsigned long long b = ((unsigned long long)(hi - 0x38000000u) << 32) | lo;
     return __uint_as_float((uint32_t)((b + 0x0fffffffull + ((lo >> 29) & 1u)) >> 29));
 }
@@ -68,6 +69,13 @@ __device__ __forceinline__ float f32_rn_pos(double v) {
 __device__ __forceinline__ double f64_exact(float f) {
     const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
     const uint32_t hi = m ? (b & 0x80000000u) | ((m >> 3) + 0x38000000u) : b;
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+// the same for any normal number, infinity or NaN
+__device__ __forceinline__ double f64_any(float f) {
+    const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
+    uint32_t hi = m ? (b & 0x80000000u) | ((m >> 3) + 0x38000000u) : b;
+    if (m >= 0x7f800000u) hi |= 0x7ff00000u;
     return __hiloint2double((int)hi, (int)(b << 29));
 }
 // (double)n of a non-negative n, exact: 2^52 + n by its bits, then 2^52 off

@@ -93,8 +93,8 @@ __device__ __forceinline__ void screen_gradient(const DScale& S, double sx, doub
         float4 A, B;
         load_block(S.g32 + 2 * node, A, B);
         const float w00 = (1.f - fx) * (1.f - fy), w10 = fx * (1.f - fy), w01 = (1.f - fx) * fy, w11 = fx * fy;
-        const double ax = f64_exact(w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z);
-        const double ay = f64_exact(w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w);
+        const double ax = f64_any(w00 * A.x + w10 * A.z + w01 * B.x + w11 * B.z);
+        const double ay = f64_any(w00 * A.y + w10 * A.w + w01 * B.y + w11 * B.w);
         gx = FIRST ? ax : gx + ax;
         gy = FIRST ? ay : gy + ay;
     } else {
@@ -564,7 +564,7 @@ __device__ __forceinline__ void trace_photon(const TraceParams& P, const DSource
             double y5 = f64_exact(powf(f32_trunc(a), -0.2f));
             const double y2 = y5 * y5, e = fma(-(a * y5), y2 * y2, 1.0);
             y5 = fma(y5 * e, fma(0.12, e, 0.2), y5);
-            kick = P.kick0 * y5;
+            kick = __double2hiint(a) < 0x47f00000 ? P.kick0 * y5 : 0.0;       // none beyond single precision
         }
 #pragma unroll 1
         for (int k = 0; k < P.n_layers; ++k) {

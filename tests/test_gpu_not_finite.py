@@ -96,3 +96,27 @@ def test_glass_without_an_index(oracle_mod, precision):
     assert none.sum() > 3000 and np.all(why[none] == VIGNETTED) and np.all(surface[none] == 2)
     real = square > 1e-9
     assert real.sum() > 1000 and np.all(((rec["flags"] == ora["flags"]) | G.boundary_mask(ora))[real])
+
+
+def test_gradients_beyond_single_precision():
+    # a band of phases of 1e300 on every screen: gradients that are infinite in single precision, or none; the photons that
+    # the FP64 path loses for their directions the mixed path loses as well
+    sc = G.test_system_scene(sources=G.mixed_sources([4000, 3000, 2000], seed=4), hf=True)
+    for q in [q for layer in sc.layers for q in layer.scales]:
+        q.phase = q.phase.copy()
+        q.phase[10:14, 20:60] = 1e300
+    full, mixed = (G.run_gpu(sc, p, moments=False)["rec"] for p in (P.PLAIN_FP64, P.MIXED))
+    why, surface = reasons(full)
+    nowhere = (why == NEWTON) & (surface == 0)
+    assert nowhere.sum() > 1000 and np.array_equal(mixed["flags"][nowhere], full["flags"][nowhere])
+    assert np.sum(full["flags"] & 1) > 1000
+
+
+@BOTH
+def test_no_kick_beyond_single_precision(oracle_mod, precision):
+    # a reference wavelength of 1e-300 nm: (lambda / lambda_ref)^(-1/5) is nothing, and no photon is deflected
+    sc = scene()
+    sc.lambda_ref = 1e-300
+    rec = G.run_gpu(sc, precision, moments=False)["rec"]
+    ora = G.oracle_trace(oracle_mod, sc)
+    assert np.all((rec["flags"] == ora["flags"]) | G.boundary_mask(ora)) and np.sum(rec["flags"] & 1) > 1000
