@@ -578,17 +578,18 @@ static __device__ __forceinline__ bool far_sag(const DSurface& S, double x, doub
 }
 
 // An aspheric or Zernike surface where the single-precision start below does not come near it: Newton's method on the sag
-// in FP64 from the conic's root along p + l d (the ray's own start is at l = -from), until the step is below 1e-8 mm.  Whether it gets there within 20 steps, and
-// whether it leaves the conic's domain on its way, is what says that a ray meets such a surface or how it is lost: steep
-// terms have roots of their own beyond the aperture, which a method with larger steps finds where this one ends.  Out of
-// line, for the rays that come in far off the aperture: those that a lens or a mirror is made for do not get here (2e7 photons
-// all FP64 6.24 ms with it, 6.33 where every ray went on from whatever start it had).
+// in FP64 from the conic's root along p + l d (the ray's own start is at l = -from), until the step is below 1e-8 mm.
+// Whether it gets there within 20 steps, and whether it leaves the conic's domain on its way, is what says that a ray meets
+// such a surface or how it is lost: steep terms have roots of their own beyond the aperture, which a method with larger
+// steps finds where this one ends.  Out of line, for the rays that come in far off the aperture: those that a lens or a
+// mirror is made for do not get here (2e7 photons all FP64 6.24 ms with it, 6.33 where every ray went on from whatever
+// start it had).
 static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, double3 p, double3 d, double from,
                                                       double* h, double* N) {
     double l = conic_root(S.c, S.kc, p.x, p.y, p.z, d.x, d.y, d.z, from);
     if (fabs(l) >= 1e300) return PHOSIM_LOST_MISSED;
     bool done = false;
-    for (int it = 0; it < 21; ++it) {
+    for (int it = 0; it < 20 || done; ++it) {             // (the last time for the point and the normal)
         const double x = fma(l, d.x, p.x), y = fma(l, d.y, p.y), z = fma(l, d.z, p.z);
         double zs, zx, zy;
         if (!far_sag(S, x, y, zs, zx, zy)) return PHOSIM_LOST_MISSED;
@@ -621,7 +622,7 @@ static __device__ __noinline__ uint32_t intersect_far(const DSurface& S, double3
 // is not that of a start near the surface, Newton's method on the sag decides (intersect_far).
 // Measured (GB300, 300 stars, 2e7 photons, all FP64): 17.6 ms with the conic's FP64 root (a root and a quotient) and two
 // to three FP64 Newton steps on the sag a mirror, 10.3 ms with this start and the savings of fp64.cuh; with the slope in
-// single precision 7.7 ms, 8.1 with an FP64 slope and its reciprocal.  On steep and aspheric lenses the position error
+// single precision 7.7 ms, 8.1 with an FP64 slope and its reciprocal (6.3 since, by savings elsewhere).  On steep and aspheric lenses the position error
 // against the oracle fell from up to 9e-10 mm to 9e-13 mm, with either slope.
 // On success h is the point and N the unit normal (along (-S_x, -S_y, 1)); way has the sign of the distance, or is 0 where
 // the single-precision start does not say it for certain (a start within 0.1 mm of the surface does beyond 1 mm).
